@@ -108,12 +108,14 @@ __device__ __forceinline__ float gv_quad(const FRec &a, const float xx[6]) {
            fmaf(a.w8.y, xx[3], fmaf(a.w8.z, xx[4], a.w8.w * xx[5])))));
 }
 
-__device__ __forceinline__ void kern(const FRec &a, float r, bool in, float &W, float &G) {
+// Kernel of particle a.  Outside gather(a), r >= h_a and t vanishes (the
+// rounding of eta leaves at most t ~ 1e-7, t^5 ~ 1e-35 of the kernel).
+__device__ __forceinline__ void kern(const FRec &a, float r, float &W, float &G) {
     float eta = r * a.w0.w;
-    float t = fmaxf(1.f - eta, 0.f);
+    float t = __saturatef(1.f - eta);
     float t2 = t * t, t5 = t2 * t2 * t;
-    W = in ? a.w1.x * t5 * t * fmaf(eta, fmaf(eta, K35_3, 6.f), 1.f) : 0.f;
-    G = in ? a.w1.y * fmaf(5.f, eta, 1.f) * t5 : 0.f;
+    W = a.w1.x * t5 * t * fmaf(eta, fmaf(eta, K35_3, 6.f), 1.f);
+    G = a.w1.y * fmaf(5.f, eta, 1.f) * t5;
 }
 
 struct PairOut {
@@ -126,10 +128,10 @@ struct PairOut {
 
 // One pair of the pair set seen from particle a; x = x_a - x_b.
 __device__ __forceinline__ void pair_force(const FRec &a, const FRec &b, const float x[3], float r2,
-                                           float r, bool in_a, bool in_b, const FParams &fp, PairOut &o) {
+                                           float r, const FParams &fp, PairOut &o) {
     float Wa, Ga, Wb, Gb;
-    kern(a, r, in_a, Wa, Ga);
-    kern(b, r, in_b, Wb, Gb);
+    kern(a, r, Wa, Ga);
+    kern(b, r, Wb, Gb);
     const float xn[3] = {-x[0], -x[1], -x[2]};
     float gRa[3], gRb[3];
     grad_rk(a, x, Wa, Ga, gRa);
@@ -243,15 +245,14 @@ struct P4 {
         s.vsig = fmaxf(s.vsig, o.vsig);
         s.qmax = fmaxf(s.qmax, o.qmax);
     }
-    __device__ static Rec load(uint32_t e, size_t, const Params &p) { return ldg_frec(p.frec + (e & 0x3fffffffu)); }
-    __device__ static void pair(IState &s, const Rec &r, uint32_t e, size_t pos, bool in_i, const Params &p) {
-        const bool in_j = in_i ? (e >> 31) != 0u : true;
+    __device__ static Rec load(uint32_t j, size_t, const Params &p) { return ldg_frec(p.frec + j); }
+    __device__ static void pair(IState &s, const Rec &r, uint32_t j, size_t pos, bool, const Params &p) {
         int dx = (int)(fq(s.me, 0) - fq(r, 0)), dy = (int)(fq(s.me, 1) - fq(r, 1)), dz = (int)(fq(s.me, 2) - fq(r, 2));
         Sep d = separation(dx, dy, dz);
         float x[3] = {d.x, d.y, d.z};
         PairOut o;
-        pair_force(s.me, r, x, d.r2, d.r, in_i, in_j, p.fp, o);
-        p.Fst[pos] = make_float4(o.F[0], o.F[1], o.F[2], __uint_as_float(e & 0x3fffffffu));   // F_ij, j
+        pair_force(s.me, r, x, d.r2, d.r, p.fp, o);
+        p.Fst[pos] = make_float4(o.F[0], o.F[1], o.F[2], __uint_as_float(j));   // F_ij, j
         float dv[3] = {r.w3.x - s.me.w3.x, r.w3.y - s.me.w3.y, r.w3.z - s.me.w3.z};
 #pragma unroll
         for (int g = 0; g < 3; g++) s.F[g].add(o.F[g]);
@@ -341,14 +342,11 @@ __global__ void __launch_bounds__(TMA_WARPS * 32) k_p4_tma(ListGeom g, typename 
     const bool valid = i < g.n;
     typename P::IState st;
     P::init(st, i, valid, prm);
-    const uint32_t *col0 = g.ent + (size_t)tile * g.kcap * 32 + lane;
-    const size_t fb = (size_t)g.fbase[tile] * 32 + lane;
-    const int len = min((int)g.len_u[tile], g.kcap);
-    const int mg = valid ? min(g.cnt_g[i], g.kcap) : 0;
-    const int my = valid ? min(g.cnt_u[i], g.kcap) : 0;
+    const LaneList<P> ll(g, tile, lane, i, valid);
+    const size_t fb = ll.fb;
+    const int len = min((int)g.len_u[tile], g.kcap), my = LB * ll.nb;   // rows of the tile, of this lane
     auto entry = [&](int k) -> uint32_t {
-        const int c = k < mg ? k : g.kcap - 1 - (k - mg);
-        return __ldg(col0 + (size_t)c * 32);
+        return __ldg(ll.tile_ent + block_at(pair_block(k / LB, ll.nbg, g.kcap), lane) + k % LB);
     };
     // the records of row j of every lane into stage s (lanes without an entry
     // fetch row 0, so that a stage always receives TMA_TX bytes)
@@ -366,13 +364,13 @@ __global__ void __launch_bounds__(TMA_WARPS * 32) k_p4_tma(ListGeom g, typename 
         __syncwarp();
     };
     uint32_t e0 = my > 0 ? entry(0) : 0u, e1 = my > 1 ? entry(1) : 0u;
-    if (len > 0) issue(0, my > 0 ? (e0 & 0x3fffffffu) : 0u);
+    if (len > 0) issue(0, my > 0 ? e0 : 0u);
     uint32_t ph = 0u;   // bit s: the phase stage s waits for next
     const unsigned char *mine = &stg[w][0][0] + (lane >> 2) * TMA_SLOT + (lane & 3) * (TMA_RF * 4);
     for (int k = 0; k < len; k++) {
         const int s = k & 1;
         const uint32_t e = e0;
-        if (k + 1 < len) issue(s ^ 1, k + 1 < my ? (e1 & 0x3fffffffu) : 0u);
+        if (k + 1 < len) issue(s ^ 1, k + 1 < my ? e1 : 0u);
         e0 = e1;
         e1 = k + 2 < my ? entry(k + 2) : 0u;
         // one decision for the warp: every lane continues, or every lane leaves
@@ -396,7 +394,7 @@ __global__ void __launch_bounds__(TMA_WARPS * 32) k_p4_tma(ListGeom g, typename 
             r.w7 = q[7];
             r.w8 = q[8];
             r.w9 = make_float4(0.f, 0.f, 0.f, 0.f);
-            P::pair(st, r, e, fb + (size_t)k * 32, k < mg, prm);
+            P::pair(st, r, e, fb + (size_t)k * 32, true, prm);
         }
         __syncwarp();
     }
@@ -485,7 +483,7 @@ __device__ __forceinline__ float compat_term(const float4 me, const float4 r, co
 template <bool COMP, bool DUAL = false>
 struct P5 {
     static constexpr bool GATHER = false;
-    static constexpr int UNROLL = 3;
+    static constexpr int UNROLL = 4;
     static constexpr bool PERSISTENT = false;
     static constexpr bool PREFETCH = false;
     static constexpr bool SKIPPABLE = true;
@@ -635,13 +633,17 @@ __device__ __forceinline__ void po_flush(const typename P::Params &prm, float (*
     for (int q = 0; q < P::NS; q++) slot[q] = 0.f;
 }
 
+// Row of a lane's entry k (gather entries, then the others) among its stored forces.
+__device__ __forceinline__ int entry_row(int k, int mg) { return k < mg ? k : LB * list_blocks(mg) + (k - mg); }
+
 // One tile of a pair-once pass.  P provides NS (floats of a share), Ent (what
 // a lane reads per list entry), Rec (the neighbour data), IState and
 //   init(IState&, int i, bool valid, const Params&)
-//   fetch(const uint32_t *col0, size_t fb, int mg, int kcap, int k, const Params&) -> Ent   (entry k)
+//   fetch(const uint32_t *ent, size_t fb, int lane, int mg, int kcap, int k, const Params&) -> Ent   (entry k:
+//     gather entries, then the others; ent: the tile's columns)
 //   jof(const Ent&) -> j
 //   load(const Ent&, const Params&) -> Rec
-//   pair(IState&, const Rec&, const Ent&, size_t pos, bool in_i, const Params&, float share[NS])
+//   pair(IState&, const Rec&, const Ent&, size_t pos, const Params&, float share[NS])
 //   add(float *slot, const float share[NS]), flush(uint32_t row, int lane, const float *slot, const Params&)
 //   finish(IState&, int i, const Params&)          (valid lanes: i's own sums)
 template <class P>
@@ -667,7 +669,7 @@ __device__ __forceinline__ void po_tile(const POGeom &g, const typename P::Param
         return c - cself < PO_CMAX ? stl[c - cself] : __ldg(g.tlist + to.x + c);
     };
     auto rv_at = [&](int c) -> uint32_t { return c - cself < PO_CMAX ? srv[c - cself] : __ldg(g.rev + to.x + c); };
-    const uint32_t *col0 = g.ent + (size_t)tile * g.kcap * 32 + lane;
+    const uint32_t *col0 = g.ent + (size_t)tile * g.kcap * 32;
     const size_t fb = (size_t)g.fbase[tile] * 32 + lane;
     const int mg = valid ? min(g.cnt_g[i], g.kcap) : 0;
     const int mu = valid ? min(g.cnt_u[i], g.kcap) : 0;
@@ -675,8 +677,8 @@ __device__ __forceinline__ void po_tile(const POGeom &g, const typename P::Param
     // owned entries: gather [kg, mg), other [ko, mu) (virtual indices)
     int kg = min(lw.x, mg), ko = mg + min(lw.y, mu - mg);
     Ent eg{}, eo{};
-    if (kg < mg) eg = P::fetch(col0, fb, mg, g.kcap, kg, prm);
-    if (ko < mu) eo = P::fetch(col0, fb, mg, g.kcap, ko, prm);
+    if (kg < mg) eg = P::fetch(col0, fb, lane, mg, g.kcap, kg, prm);
+    if (ko < mu) eo = P::fetch(col0, fb, lane, mg, g.kcap, ko, prm);
     // next owned entry in increasing j (a j is in one of the two segments only)
     auto pick = [&](int &k, Ent &e, bool &gath) -> bool {
         const uint32_t jg = kg < mg ? P::jof(eg) : PO_NONE;
@@ -684,10 +686,10 @@ __device__ __forceinline__ void po_tile(const POGeom &g, const typename P::Param
         if (jg == PO_NONE && jo == PO_NONE) return false;
         if (jg < jo) {
             k = kg; e = eg; gath = true;
-            if (++kg < mg) eg = P::fetch(col0, fb, mg, g.kcap, kg, prm);
+            if (++kg < mg) eg = P::fetch(col0, fb, lane, mg, g.kcap, kg, prm);
         } else {
             k = ko; e = eo; gath = false;
-            if (++ko < mu) eo = P::fetch(col0, fb, mg, g.kcap, ko, prm);
+            if (++ko < mu) eo = P::fetch(col0, fb, lane, mg, g.kcap, ko, prm);
         }
         return true;
     };
@@ -728,7 +730,7 @@ __device__ __forceinline__ void po_tile(const POGeom &g, const typename P::Param
             if (have2) rn = P::load(e2, prm);
         }
         float sh[P::NS];
-        if (go) P::pair(st, rc, e, fb + (size_t)k * 32, gath, prm, sh);
+        if (go) P::pair(st, rc, e, fb + (size_t)entry_row(k, mg) * 32, prm, sh);
         // j's share into the ring: lanes with the same slot add in lane order
         const uint32_t key = ((uint32_t)(c % PO_W) << 5) | (P::jof(e) & 31u);
         unsigned pend = __ballot_sync(0xffffffffu, go);
@@ -790,21 +792,20 @@ struct P4PO {
         typename P4<COMP>::Params q{p.frec, p.mass, p.fp, p.acc, p.vq, p.Fst};
         P4<COMP>::init(s, i, valid, q);
     }
-    __device__ static Ent fetch(const uint32_t *col0, size_t, int mg, int kcap, int k, const Params &) {
-        const int c = k < mg ? k : kcap - 1 - (k - mg);
-        return __ldg(col0 + (size_t)c * 32);
+    __device__ static Ent fetch(const uint32_t *ent, size_t, int lane, int mg, int kcap, int k, const Params &) {
+        const int row = entry_row(k, mg);
+        return __ldg(ent + block_at(pair_block(row / LB, list_blocks(mg), kcap), lane) + row % LB);
     }
-    __device__ static uint32_t jof(const Ent &e) { return e & 0x3fffffffu; }
-    __device__ static Rec load(const Ent &e, const Params &p) { return ldg_frec(p.frec + (e & 0x3fffffffu)); }
-    __device__ static void pair(IState &s, const Rec &r, const Ent &e, size_t pos, bool in_i, const Params &p,
+    __device__ static uint32_t jof(const Ent &e) { return e; }
+    __device__ static Rec load(const Ent &e, const Params &p) { return ldg_frec(p.frec + e); }
+    __device__ static void pair(IState &s, const Rec &r, const Ent &e, size_t pos, const Params &p,
                                 float sh[NS]) {
-        const bool in_j = in_i ? (e >> 31) != 0u : true;
         int dx = (int)(fq(s.me, 0) - fq(r, 0)), dy = (int)(fq(s.me, 1) - fq(r, 1)), dz = (int)(fq(s.me, 2) - fq(r, 2));
         Sep d = separation(dx, dy, dz);
         float x[3] = {d.x, d.y, d.z};
         PairOut o;
-        pair_force(s.me, r, x, d.r2, d.r, in_i, in_j, p.fp, o);
-        p.Fst[pos] = make_float4(o.F[0], o.F[1], o.F[2], __uint_as_float(e & 0x3fffffffu));   // F_ij, j
+        pair_force(s.me, r, x, d.r2, d.r, p.fp, o);
+        p.Fst[pos] = make_float4(o.F[0], o.F[1], o.F[2], __uint_as_float(e));   // F_ij, j
         float dv[3] = {r.w3.x - s.me.w3.x, r.w3.y - s.me.w3.y, r.w3.z - s.me.w3.z};
 #pragma unroll
         for (int g = 0; g < 3; g++) s.F[g].add(o.F[g]);
@@ -901,8 +902,8 @@ struct P5PO {
         typename P5<COMP, DUAL>::Params q{p.sig, p.Fst, p.mass, p.du, p.inv_a4, p.skip, p.du2};
         P5<COMP, DUAL>::init(s, i, valid, q);
     }
-    __device__ static Ent fetch(const uint32_t *, size_t fb, int, int, int k, const Params &p) {
-        return __ldg(p.Fst + fb + (size_t)k * 32);
+    __device__ static Ent fetch(const uint32_t *, size_t fb, int, int mg, int, int k, const Params &p) {
+        return __ldg(p.Fst + fb + (size_t)entry_row(k, mg) * 32);
     }
     __device__ static uint32_t jof(const Ent &F) { return __float_as_uint(F.w); }
     __device__ static Rec load(const Ent &F, const Params &p) {
@@ -917,8 +918,7 @@ struct P5PO {
     __device__ static float dotw(const float4 &me, const float4 &r, const float4 &F) {
         return fmaf(r.x - me.x, F.x, fmaf(r.y - me.y, F.y, (r.z - me.z) * F.z));
     }
-    __device__ static void pair(IState &s, const Rec &rec, const Ent &F, size_t, bool, const Params &,
-                                float sh[NS]) {
+    __device__ static void pair(IState &s, const Rec &rec, const Ent &F, size_t, const Params &, float sh[NS]) {
         const Part pt = partition(s.me.w, rec.sig.w);
         const bool jge = rec.sig.w >= s.me.w;   // s_j >= s_i: the partition seen from j
         const float w = dotw(s.me, rec.sig, F);

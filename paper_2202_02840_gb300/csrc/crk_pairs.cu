@@ -258,8 +258,8 @@ struct P2 {
         for (int a = 0; a < 6; a++) merge_acc(s.s1[a], o.s1[a]);
         for (int a = 0; a < 10; a++) merge_acc(s.s2[a], o.s2[a]);
     }
-    __device__ static Rec load(uint32_t e, size_t, const Params &p) { return __ldg(p.qV + (e & 0x3fffffffu)); }
-    __device__ static void pair(IState &s, const Rec &r, uint32_t, size_t, bool, const Params &) {
+    __device__ static Rec load(uint32_t j, size_t, const Params &p) { return __ldg(p.qV + j); }
+    __device__ static void pair(IState &s, const Rec &r, uint32_t, size_t, bool ok, const Params &) {
         int dx = (int)(s.q.x - r.x), dy = (int)(s.q.y - r.y), dz = (int)(s.q.z - r.z);
         const float Vj = __uint_as_float(r.w);
         Sep d = separation(dx, dy, dz);
@@ -272,7 +272,7 @@ struct P2 {
         float w = Vj * Wu, g = Vj * Gu;
         float gx[3] = {g * x[0], g * x[1], g * x[2]};
         float xx[6] = {x[0] * x[0], x[0] * x[1], x[0] * x[2], x[1] * x[1], x[1] * x[2], x[2] * x[2]};
-        s.m0.add(w);
+        if (ok) s.m0.add(w);   // a pad (x = 0) adds nothing to the other sums
 #pragma unroll
         for (int a = 0; a < 3; a++) {
             s.m1[a].add(w * x[a]);
@@ -422,8 +422,8 @@ struct P2X {
         for (int a = 0; a < 6; a++) merge_acc(s.m2[a], o.m2[a]), merge_acc(s.s1[a], o.s1[a]);
         for (int a = 0; a < 10; a++) merge_acc(s.s2[a], o.s2[a]);
     }
-    __device__ static Rec load(uint32_t e, size_t, const Params &p) { return __ldg(p.qV + (e & 0x3fffffffu)); }
-    __device__ static void pair(IState &s, const Rec &rc, uint32_t, size_t, bool, const Params &) {
+    __device__ static Rec load(uint32_t j, size_t, const Params &p) { return __ldg(p.qV + j); }
+    __device__ static void pair(IState &s, const Rec &rc, uint32_t, size_t, bool ok, const Params &) {
         const int dx = (int)(s.q.x - rc.x), dy = (int)(s.q.y - rc.y), dz = (int)(s.q.z - rc.z);
         const float Vj = __uint_as_float(rc.w);
         const FF x[3] = {ff_coord(dx), ff_coord(dy), ff_coord(dz)};
@@ -449,7 +449,7 @@ struct P2X {
         const FF w = ff_mul(FF{Vj, 0.f}, Wu);
         const FF gn = ff_mul(FF{Vj, 0.f}, Gn);
         const FF gx[3] = {ff_mul(gn, x[0]), ff_mul(gn, x[1]), ff_mul(gn, x[2])};
-        s.m0.add(w);
+        if (ok) s.m0.add(w);   // a pad (x = 0) adds nothing to the other sums
 #pragma unroll
         for (int a = 0; a < 3; a++) {
             s.m1[a].add(ff_mul(w, x[a]));
@@ -492,7 +492,7 @@ struct P2X {
 template <bool COMP>
 struct P3 {
     static constexpr bool GATHER = true;
-    static constexpr int UNROLL = 3;
+    static constexpr int UNROLL = 4;
     static constexpr bool ENTRIES = true;
     static constexpr bool PERSISTENT = false;
     static constexpr bool PREFETCH = false;
@@ -539,8 +539,7 @@ struct P3 {
         uint4 qV;
         float4 v;
     };
-    __device__ static Rec load(uint32_t e, size_t, const Params &p) {
-        const uint32_t j = e & 0x3fffffffu;
+    __device__ static Rec load(uint32_t j, size_t, const Params &p) {
         return Rec{__ldg(p.qV + j), __ldg(p.vel + j)};
     }
     __device__ static void pair(IState &s, const Rec &rec, uint32_t, size_t, bool, const Params &) {
@@ -616,11 +615,10 @@ struct PD {
     }
     __device__ static void zero(IState &s) { s.acc = 0.f; }
     __device__ static void merge(IState &s, const IState &o) { s.acc += o.acc; }
-    __device__ static Rec load(uint32_t e, size_t, const Params &p) {
-        const uint32_t j = e & 0x3fffffffu;
+    __device__ static Rec load(uint32_t j, size_t, const Params &p) {
         return Rec{__ldg(p.q4 + j), __ldg(p.mass + j)};
     }
-    __device__ static void pair(IState &s, const Rec &r, uint32_t, size_t, bool, const Params &) {
+    __device__ static void pair(IState &s, const Rec &r, uint32_t, size_t, bool ok, const Params &) {
         int dx = (int)(s.q.x - r.q.x), dy = (int)(s.q.y - r.q.y), dz = (int)(s.q.z - r.q.z);
         Sep d = separation(dx, dy, dz);
         float eta = d.r * s.inv_h;
@@ -628,7 +626,7 @@ struct PD {
         float t2 = t * t, t3 = t2 * t;
         float Wu = t3 * t3 * fmaf(eta, fmaf(eta, K35_3, 6.f), 1.f);
         float sB = fmaf(s.B[0], d.x, fmaf(s.B[1], d.y, fmaf(s.B[2], d.z, 1.f)));
-        s.acc = fmaf(r.m * sB, Wu, s.acc);
+        s.acc = fmaf(ok ? r.m * sB : 0.f, Wu, s.acc);
     }
     __device__ static void finish(IState &s, int i, const Params &p) {
         const float ih3 = s.inv_h * s.inv_h * s.inv_h;

@@ -97,34 +97,50 @@ struct Acc {
 
 
 
-// Warp per tile, lane = particle i; lane i walks its own neighbour list (entry
-// k at base + 32 k + lane).  Gather passes walk the first cnt_g[i] entries,
-// pair-set passes all cnt_u[i].  P must provide Params, IState, Rec, GATHER,
-// PREFETCH, UNROLL, PERSISTENT, ENTRIES (false: the pass reads only its stored entries,
-// and `entry` is passed as 0),
+// Per-particle lists.  A tile has kcap columns of 32 lanes, stored as blocks of
+// four columns: a lane's four entries of a block are 16 contiguous bytes and a
+// block is 512, so a warp reads a block in one coalesced 128-bit load per lane,
+// and the walk writes 16 bytes at a time.  Gather neighbours fill blocks from
+// the front, the other pair-set neighbours fill blocks from the back; a lane
+// pads the last block of either segment with its own index i.  A pair (i, i)
+// adds exactly zero to every sum of differences (x = 0, v_i - v_j = 0, F_ii = 0);
+// the passes whose self term is not zero (W(0)) get `ok` = false for a pad.
+constexpr int LB = 4;   // entries of a block
+
+__host__ __device__ __forceinline__ int list_blocks(int entries) { return (entries + LB - 1) / LB; }
+
+// word of a lane's column 0 of block b within its tile's columns
+__device__ __forceinline__ size_t block_at(int b, int lane) { return ((size_t)b * 32 + lane) * LB; }
+
+// Block b of the pair-set sequence of a lane with nbg gather blocks: its
+// gather blocks, then the others from the tile's last block down.
+__device__ __forceinline__ int pair_block(int b, int nbg, int kcap) { return b < nbg ? b : kcap / LB - 1 - (b - nbg); }
+
+// Warp per tile, lane = particle i; lane i walks its own list, block by block.
+// Gather passes walk the gather blocks, pair-set passes all blocks; entry u of
+// block b has its stored force (P4 -> P5) in row 4 b + u of the tile, pads
+// included (F = 0, j = i).  P must provide Params, IState, Rec, GATHER,
+// PREFETCH, UNROLL, PERSISTENT, ENTRIES (false: the pass reads only its stored
+// entries, and `entry` is passed as 0),
 //   init(IState&, int i, bool valid, const Params&)
 //   load(uint32_t entry, size_t pos, const Params&) -> Rec   (the neighbour's data)
-//   pair(IState&, const Rec&, uint32_t entry, size_t pos, bool in_i, const Params&)
+//   pair(IState&, const Rec&, uint32_t entry, size_t pos, bool ok, const Params&)
 //   finish(IState&, int i, const Params&)            (valid lanes only)
 struct ListGeom {
     int n, ntiles, kcap;
     const uint32_t *fbase;             // per-tile stored-force base, units of 32 entries
-    const uint32_t *len_g, *len_u;
+    const uint32_t *len_g, *len_u;     // per-tile rows of the longest lane (multiples of LB)
     const int32_t *cnt_g, *cnt_u;
     const uint32_t *ent;
 };
 
-// Entry k of a particle's list (gather neighbours k < cnt_g from the front
-// columns, the rest from the back columns) and its stored-force position.
-// The entries stream once from HBM, the longest latency of the loop, so they
-// are always read ahead.  Passes with 16-32-byte records (mostly L1 hits)
-// take P::UNROLL entries per iteration: that many independent gathers and
-// pair evaluations per lane, the next P::UNROLL entries in flight (measured
-// best: 4 for P1 and P2, 3 for P3 and P5).  P4, whose 160-byte record
-// already fills the registers, evaluates one pair at a time and instead
-// prefetches the record of entry k + 1 and the entry k + 2 (P::PREFETCH),
-// alternating two register sets for the record in flight (measured 7%
-// faster than copying the prefetched record into the current one).
+// The blocks of lists stream once from HBM (or L2, just written by the walk),
+// the longest latency of the loop, so the next block is always read ahead.
+// Passes with 16-32-byte records (mostly L1 hits) gather U neighbours' records
+// at a time (U = 1, 2 or 4; 4 is the measured best).  P4, whose record already
+// fills the registers, evaluates one pair at a time with the next record in
+// flight (P::PREFETCH), alternating two register sets (measured 7% faster than
+// copying the prefetched record into the current one).
 // passes that declare SKIPPABLE take a device flag (Params::skip, may be null)
 template <class P, class = void>
 struct has_skip : std::false_type {};
@@ -143,94 +159,118 @@ __device__ __forceinline__ bool pass_skipped(const typename P::Params &prm) {
     return false;
 }
 
-// What a lane reads ahead for entry k: its list entry (P::ENTRIES), or, for a
-// pass that reads only what an earlier pass stored per entry, that stored
-// record (P::Stored, from P::stored(pos)), which then streams from HBM.
+// What a lane reads ahead for a block: its four list entries (P::ENTRIES), or,
+// for a pass that reads only what an earlier pass stored per entry, those four
+// stored records (P::Stored, from P::stored(pos)), which then stream from HBM.
 template <class P, bool = P::ENTRIES>
-struct EntOf {
-    using type = uint32_t;
+struct BlockOf {
+    uint32_t e[LB];
 };
 template <class P>
-struct EntOf<P, false> {
-    using type = typename P::Stored;
+struct BlockOf<P, false> {
+    typename P::Stored e[LB];
 };
 
-// Entries [k0, mk) of this lane, U per iteration, the warp looping over
-// [k0, k1): U independent gathers and pair evaluations in flight per lane and
-// the next U entries (or stored records) read ahead.
-template <class P, int U, class EntryFn>
-__device__ __forceinline__ void list_loop(typename P::IState &st, const typename P::Params &prm, EntryFn entry,
-                                          size_t fb, int mg, int k0, int k1, int mk) {
-    using Ent = typename EntOf<P>::type;
-    auto fetch = [&](int k) -> Ent {
-        if constexpr (P::ENTRIES)
-            return entry(k);
-        else
-            return P::stored(fb + (size_t)k * 32, prm);
-    };
-    Ent en[U] = {};
+// One lane's list: where its blocks are and how many it has.
+template <class P>
+struct LaneList {
+    const uint32_t *tile_ent;   // the tile's columns
+    size_t fb;                  // stored-force position of row 0
+    int lane, kcap, mg, nbg, nb;
+    __device__ __forceinline__ LaneList(const ListGeom &g, int tile, int lane_, int i, bool valid) {
+        lane = lane_;
+        kcap = g.kcap;
+        tile_ent = g.ent + (size_t)tile * g.kcap * 32;
+        fb = (size_t)g.fbase[tile] * 32 + lane;
+        // counts beyond kcap only occur in a walk that overflowed (the host then
+        // grows kcap and walks again, or discards a replayed step): never read
+        // past the tile's columns
+        const int all = g.kcap / LB;
+        mg = valid ? min(g.cnt_g[i], g.kcap) : 0;
+        nbg = list_blocks(mg);
+        nb = P::GATHER ? nbg : (valid ? min(nbg + list_blocks(max(g.cnt_u[i] - g.cnt_g[i], 0)), all) : 0);
+    }
+    __device__ __forceinline__ BlockOf<P> fetch(int b, const typename P::Params &prm) const {
+        BlockOf<P> r;
+        if constexpr (P::ENTRIES) {
+            const int c = P::GATHER ? b : pair_block(b, nbg, kcap);
+            const uint4 v = __ldg(reinterpret_cast<const uint4 *>(tile_ent + block_at(c, lane)));
+            r.e[0] = v.x;
+            r.e[1] = v.y;
+            r.e[2] = v.z;
+            r.e[3] = v.w;
+        } else {
 #pragma unroll
-    for (int u = 0; u < U; u++)
-        if (k0 + u < mk) en[u] = fetch(k0 + u);
-    for (int k = k0; k < k1; k += U) {
-        Ent ec[U];
-#pragma unroll
-        for (int u = 0; u < U; u++) {
-            ec[u] = en[u];
-            if (k + U + u < mk) en[u] = fetch(k + U + u);
+            for (int u = 0; u < LB; u++) r.e[u] = P::stored(fb + (size_t)(LB * b + u) * 32, prm);
         }
-        const size_t pos = fb + (size_t)k * 32;
-        typename P::Rec r[U];
+        return r;
+    }
+    // entry u of block b is a neighbour, not a pad (gather passes)
+    __device__ __forceinline__ bool ok(int b, int u) const { return LB * b + u < mg; }
+};
+
+// Blocks [b0, b1) of this lane, the warp looping over [b0, bw): U independent
+// gathers and pair evaluations in flight per lane and the next block read ahead.
+template <class P, int U>
+__device__ __forceinline__ void list_loop(typename P::IState &st, const typename P::Params &prm,
+                                          const LaneList<P> &ll, int b0, int b1, int bw) {
+    BlockOf<P> en = {};
+    if (b0 < b1) en = ll.fetch(b0, prm);
+    for (int b = b0; b < bw; b++) {
+        const BlockOf<P> ec = en;
+        if (b + 1 < b1) en = ll.fetch(b + 1, prm);
+        if (b < b1) {
+            const size_t pos = ll.fb + (size_t)b * (LB * 32);
 #pragma unroll
-        for (int u = 0; u < U; u++)
-            if (k + u < mk) r[u] = P::load(ec[u], pos + 32 * u, prm);
+            for (int q = 0; q < LB; q += U) {
+                typename P::Rec r[U];
 #pragma unroll
-        for (int u = 0; u < U; u++)
-            if (k + u < mk) P::pair(st, r[u], ec[u], pos + 32 * u, k + u < mg, prm);
+                for (int u = 0; u < U; u++) r[u] = P::load(ec.e[q + u], pos + 32 * (q + u), prm);
+#pragma unroll
+                for (int u = 0; u < U; u++)
+                    P::pair(st, r[u], ec.e[q + u], pos + 32 * (q + u), ll.ok(b, q + u), prm);
+            }
+        }
     }
 }
 
-// list_loop with the neighbour records one iteration ahead as well (RP
-// variants): at iteration k the records of iteration k + 1 and the entries
-// (or stored records) of iteration k + 2 are in flight while the U pairs of
-// iteration k are evaluated, so a record that misses L1 is waited for only if
-// it takes longer than a whole iteration.  Same entries, same order: bitwise
-// the same sums.
-template <class P, int U, class EntryFn>
-__device__ __forceinline__ void list_loop_rp(typename P::IState &st, const typename P::Params &prm, EntryFn entry,
-                                             size_t fb, int mg, int k0, int k1, int mk) {
-    using Ent = typename EntOf<P>::type;
-    auto fetch = [&](int k) -> Ent {
-        if constexpr (P::ENTRIES)
-            return entry(k);
-        else
-            return P::stored(fb + (size_t)k * 32, prm);
-    };
-    Ent ec[U] = {}, en[U] = {};
-    typename P::Rec rc[U] = {}, rn[U] = {};
+// list_loop with the neighbour records ahead as well (RP variants): while the
+// U pairs of one group are evaluated the records of the next group are in
+// flight, so a record that misses L1 is waited for only if it takes longer
+// than a whole group.  Same entries, same order: bitwise the same sums.
+template <class P, int U>
+__device__ __forceinline__ void list_loop_rp(typename P::IState &st, const typename P::Params &prm,
+                                             const LaneList<P> &ll, int b0, int b1, int bw) {
+    BlockOf<P> ec = {}, en = {};
+    typename P::Rec rc[U] = {};
+    if (b0 < b1) {
+        ec = ll.fetch(b0, prm);
 #pragma unroll
-    for (int u = 0; u < U; u++) {
-        if (k0 + u < mk) ec[u] = fetch(k0 + u);
-        if (k0 + U + u < mk) en[u] = fetch(k0 + U + u);
+        for (int u = 0; u < U; u++) rc[u] = P::load(ec.e[u], ll.fb + (size_t)b0 * (LB * 32) + 32 * u, prm);
     }
+    if (b0 + 1 < b1) en = ll.fetch(b0 + 1, prm);
+    for (int b = b0; b < bw; b++) {
+        if (b < b1) {
+            const size_t pos = ll.fb + (size_t)b * (LB * 32);
 #pragma unroll
-    for (int u = 0; u < U; u++)
-        if (k0 + u < mk) rc[u] = P::load(ec[u], fb + (size_t)(k0 + u) * 32, prm);
-    for (int k = k0; k < k1; k += U) {
-        Ent eu[U];
+            for (int q = 0; q < LB; q += U) {
+                typename P::Rec rn[U] = {};
 #pragma unroll
-        for (int u = 0; u < U; u++) {
-            if (k + U + u < mk) rn[u] = P::load(en[u], fb + (size_t)(k + U + u) * 32, prm);
-            eu[u] = ec[u];
-            ec[u] = en[u];
-            if (k + 2 * U + u < mk) en[u] = fetch(k + 2 * U + u);
+                for (int u = 0; u < U; u++) {
+                    if (q + U < LB)
+                        rn[u] = P::load(ec.e[(q + U + u) % LB], pos + 32 * (q + U + u), prm);
+                    else if (b + 1 < b1)
+                        rn[u] = P::load(en.e[u], pos + LB * 32 + 32 * u, prm);
+                }
+#pragma unroll
+                for (int u = 0; u < U; u++)
+                    P::pair(st, rc[u], ec.e[q + u], pos + 32 * (q + u), ll.ok(b, q + u), prm);
+#pragma unroll
+                for (int u = 0; u < U; u++) rc[u] = rn[u];
+            }
         }
-        const size_t pos = fb + (size_t)k * 32;
-#pragma unroll
-        for (int u = 0; u < U; u++)
-            if (k + u < mk) P::pair(st, rc[u], eu[u], pos + 32 * u, k + u < mg, prm);
-#pragma unroll
-        for (int u = 0; u < U; u++) rc[u] = rn[u];
+        ec = en;
+        if (b + 2 < b1) en = ll.fetch(b + 2, prm);
     }
 }
 
@@ -241,45 +281,36 @@ __device__ __forceinline__ void lpass_tile(const ListGeom &g, const typename P::
     const bool valid = i < g.n;
     typename P::IState st;
     P::init(st, i, valid, prm);
-    const uint32_t *col0 = g.ent + (size_t)tile * g.kcap * 32 + lane;
-    const size_t fb = (size_t)g.fbase[tile] * 32 + lane;
-    // counts beyond kcap only occur in a walk that overflowed (the host then
-    // grows kcap and walks again, or discards a replayed step): never read
-    // past the tile's columns
-    const int len = min((int)(P::GATHER ? g.len_g[tile] : g.len_u[tile]), g.kcap);
-    const int mg = valid ? min(g.cnt_g[i], g.kcap) : 0;
-    const int my = P::GATHER ? mg : (valid ? min(g.cnt_u[i], g.kcap) : 0);
-    auto entry = [&](int k) -> uint32_t {
-        const int c = k < mg ? k : g.kcap - 1 - (k - mg);
-        return __ldg(col0 + (size_t)c * 32);
-    };
+    const LaneList<P> ll(g, tile, lane, i, valid);
+    const int bw = (int)((P::GATHER ? g.len_g[tile] : g.len_u[tile]) / LB);
     if constexpr (!P::PREFETCH) {
         if constexpr (RP)
-            list_loop_rp<P, U>(st, prm, entry, fb, mg, 0, len, my);
+            list_loop_rp<P, U>(st, prm, ll, 0, ll.nb, bw);
         else
-            list_loop<P, U>(st, prm, entry, fb, mg, 0, len, my);
+            list_loop<P, U>(st, prm, ll, 0, ll.nb, bw);
     } else {
-        // two pairs per iteration: the record in flight alternates between
-        // two register sets, so no record is copied from one to the other
-        uint32_t e1 = my > 0 ? entry(0) : 0u;
-        uint32_t e2 = my > 1 ? entry(1) : 0u;
+        // one pair at a time with the next record in flight, in alternating
+        // register sets, so no record is copied from one to the other
+        BlockOf<P> e = {};
         typename P::Rec ra{}, rb{};
-        if (my > 0) ra = P::load(e1, fb, prm);
-        for (int k = 0; k < len; k += 2) {
-            const size_t pos = fb + (size_t)k * 32;
-            if (k < my) {
-                const uint32_t e = e1;
-                if (k + 1 < my) rb = P::load(e2, pos + 32, prm);
-                e1 = e2;
-                if (k + 2 < my) e2 = entry(k + 2);
-                P::pair(st, ra, e, pos, k < mg, prm);
-            }
-            if (k + 1 < my) {
-                const uint32_t e = e1;
-                if (k + 2 < my) ra = P::load(e2, pos + 64, prm);
-                e1 = e2;
-                if (k + 3 < my) e2 = entry(k + 3);
-                P::pair(st, rb, e, pos + 32, k + 1 < mg, prm);
+        if (ll.nb > 0) {
+            e = ll.fetch(0, prm);
+            ra = P::load(e.e[0], ll.fb, prm);
+        }
+        for (int b = 0; b < bw; b++) {
+            if (b < ll.nb) {
+                const size_t pos = ll.fb + (size_t)b * (LB * 32);
+                BlockOf<P> en = e;
+                if (b + 1 < ll.nb) en = ll.fetch(b + 1, prm);
+                rb = P::load(e.e[1], pos + 32, prm);
+                P::pair(st, ra, e.e[0], pos, true, prm);
+                ra = P::load(e.e[2], pos + 64, prm);
+                P::pair(st, rb, e.e[1], pos + 32, true, prm);
+                rb = P::load(e.e[3], pos + 96, prm);
+                P::pair(st, ra, e.e[2], pos + 64, true, prm);
+                ra = P::load(en.e[0], pos + 128, prm);   // past the last block: this block's first record again
+                P::pair(st, rb, e.e[3], pos + 96, true, prm);
+                e = en;
             }
         }
     }
@@ -348,19 +379,11 @@ __global__ void __launch_bounds__(S * 32) k_lpass_split(ListGeom g, typename P::
     IS st;
     P::init(st, i, valid, prm);
     if (w > 0) P::zero(st);
-    const uint32_t *col0 = g.ent + (size_t)tile * g.kcap * 32 + lane;
-    const size_t fb = (size_t)g.fbase[tile] * 32 + lane;
-    const int len = min((int)(P::GATHER ? g.len_g[tile] : g.len_u[tile]), g.kcap);
-    const int mg = valid ? min(g.cnt_g[i], g.kcap) : 0;
-    const int my = P::GATHER ? mg : (valid ? min(g.cnt_u[i], g.kcap) : 0);
-    const int chunk = ((len + S - 1) / S + U - 1) / U * U;
-    const int k0 = w * chunk, k1 = min(len, k0 + chunk);
-    const int mk = min(my, k1);   // this warp's entries of this lane: [k0, mk)
-    auto entry = [&](int k) -> uint32_t {
-        const int c = k < mg ? k : g.kcap - 1 - (k - mg);
-        return __ldg(col0 + (size_t)c * 32);
-    };
-    list_loop<P, U>(st, prm, entry, fb, mg, k0, k1, mk);
+    const LaneList<P> ll(g, tile, lane, i, valid);
+    const int bw = (int)((P::GATHER ? g.len_g[tile] : g.len_u[tile]) / LB);
+    const int chunk = (bw + S - 1) / S;
+    const int b0 = w * chunk, b1 = min(bw, b0 + chunk);
+    list_loop<P, U>(st, prm, ll, b0, min(ll.nb, b1), b1);
     IS *sp = reinterpret_cast<IS *>(part);
     if (w > 0) sp[(w - 1) * 32 + lane] = st;
     __syncthreads();
@@ -470,10 +493,9 @@ static void launch_rp(crk_ctx *ctx, const ListGeom &g, const typename P::Params 
 
 template <class P, int W>
 static void launch_rp_u(crk_ctx *ctx, const ListGeom &g, const typename P::Params &prm, int U, cudaStream_t s) {
-    switch (U) {
+    switch (U) {   // 3 does not divide a block: it runs as 4
     case 1: launch_rp<P, W, 1>(ctx, g, prm, s); break;
     case 2: launch_rp<P, W, 2>(ctx, g, prm, s); break;
-    case 3: launch_rp<P, W, 3>(ctx, g, prm, s); break;
     default: launch_rp<P, W, 4>(ctx, g, prm, s); break;
     }
 }
@@ -517,7 +539,6 @@ static int launch_variant(crk_ctx *ctx, const ListGeom &g, const typename P::Par
         switch (lv.U) {
         case 1: launch_variant_u<P, WARPS, 1>(ctx, g, prm, lv.ord, s); break;
         case 2: launch_variant_u<P, WARPS, 2>(ctx, g, prm, lv.ord, s); break;
-        case 3: launch_variant_u<P, WARPS, 3>(ctx, g, prm, lv.ord, s); break;
         default: launch_variant_u<P, WARPS, 4>(ctx, g, prm, lv.ord, s); break;
         }
     }
