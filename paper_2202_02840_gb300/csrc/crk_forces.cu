@@ -622,6 +622,27 @@ __global__ void k_po_rev(int ntiles, const uint2 *__restrict__ tofs, const uint3
     }
 }
 
+// Per particle, the gather and the other entries with j < i: both segments of a
+// list ascend in j, so each is found by bisection.
+__global__ void k_po_low(int n, int kcap, const int32_t *__restrict__ cnt_g, const int32_t *__restrict__ cnt_u,
+                         const uint32_t *__restrict__ ent, int2 *__restrict__ lowc) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const int tile = i / TILE, lane = i % TILE;
+    const uint32_t *e = ent + (size_t)tile * kcap * 32;
+    const int mg = min(cnt_g[i], kcap), mo = min(cnt_u[i], kcap) - mg;
+    auto low = [&](int count, bool other) {
+        int a = 0, b = count;
+        while (a < b) {
+            const int m = (a + b) >> 1;
+            const int blk = other ? kcap / LB - 1 - m / LB : m / LB;
+            if (e[block_at(blk, lane) + m % LB] < (uint32_t)i) a = m + 1; else b = m;
+        }
+        return a;
+    };
+    lowc[i] = make_int2(low(mg, false), low(mo, true));
+}
+
 // Write ring row c (candidate c of this tile's list) to its tile pair's row
 // `row` and clear it; lane l takes slot l.
 template <class P>
@@ -1009,13 +1030,14 @@ static int run_forces_po(crk_ctx *ctx, const FRec *fr, const FParams &fp, cudaSt
     if (rc) return rc;
     typename P4PO<COMP>::Params p{fr, ctx->mass, fp, ctx->acc, ctx->vq, ctx->Fst, ctx->po_rowA, ctx->po_rowB};
     prof_begin(ctx, PROF_P4, s);
+    k_po_low<<<grid_for(ctx->n, 256), 256, 0, s>>>(ctx->n, ctx->kcap, ctx->cnt_g, ctx->cnt_u, ctx->ent, ctx->lowc);
     k_po_rev<<<grid_for(ctx->ntiles, 8), 256, 0, s>>>(ctx->ntiles, ctx->uofs, ctx->ulist, ctx->po_rev,
                                                        ctx->po_self, ctx->po_tofs, ctx->po_tlist,
                                                        ctx->counters + CNT_PO_MISS);
     k_po<P4PO<COMP>><<<grid_for(ctx->ntiles, PO_WARPS), PO_WARPS * 32, 0, s>>>(po_geom(ctx), p);
     k_p4po_rows<COMP><<<grid_for(ctx->n, 256), 256, 0, s>>>(ctx->n, ctx->po_tofs, ctx->po_self, ctx->po_rowA,
                                                             ctx->po_rowB, ctx->mass, fp, ctx->acc, ctx->vq);
-    ctx->launches += 3;
+    ctx->launches += 4;
     prof_end(ctx, s);
     CRK_LAUNCH_CHECK(ctx, "P4 forces (pair-once)");
     ctx->fst_po = 1;

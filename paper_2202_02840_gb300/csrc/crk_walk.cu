@@ -16,6 +16,8 @@
 namespace crk {
 
 constexpr int WALK_WARPS = 8;
+constexpr int WALK_ALL = 20;       // fewer tiles than this per SM: every tile is shared by a CTA's warps
+constexpr int WALK_HEAVY = 384;    // candidate tiles above which a tile is shared
 
 struct WalkArgs {
     int n, ntiles, kcap;
@@ -33,7 +35,9 @@ struct WalkArgs {
     const int32_t *sbox;     // batched boxes: box of each slot (BATCH only)
     const uint32_t *nbox;    // box range of each tile (BATCH only)
     const int32_t *act;      // may be null: walk the tiles act[0 .. ntiles) only
-    int2 *lowc;              // may be null: per particle, gather and other entries with j < i
+    int heavy;               // tiles with more candidate tiles than this are shared by the warps of a CTA
+    int hblocks;             // CTAs that take them (all: one per tile, every tile is shared)
+    int all;
     unsigned long long *tests;   // lane tests of the exact predicate (LISTS walk)
 };
 
@@ -47,400 +51,494 @@ __device__ __forceinline__ unsigned long long point_gap(uint32_t q, uint32_t lo,
 }
 
 // One segment of a lane's list on its way to memory: the last up to three
-// entries wait in registers (newest in p3) until their block is full.
+// entries wait in registers (newest in p3) until their block is full.  A lane
+// of a shared tile (PART) may start inside a block, `start` entries of the
+// segment coming from the warps before it: that block's and the last block's
+// entries are written singly.
+template <bool PART>
 struct Seg {
     uint32_t p1, p2, p3;
-    int n;   // entries so far
-    uint32_t *at;   // the next block
-    __device__ __forceinline__ void push(uint32_t j, int kcap, ptrdiff_t step) {
+    int n, start;   // entries of the segment so far, and before this lane's first
+    int at;         // word of the current block in the tile's columns
+    __device__ __forceinline__ void push(uint32_t j, uint32_t *cols, int kcap, int step) {
         ++n;
         if ((n & (LB - 1)) == 0) {
-            if (n <= kcap) *reinterpret_cast<uint4 *>(at) = make_uint4(p1, p2, p3, j);
+            if (n <= kcap) {
+                if (!PART || n - LB >= start) {
+                    *reinterpret_cast<uint4 *>(cols + at) = make_uint4(p1, p2, p3, j);
+                } else {
+                    if (n - 3 >= start) cols[at + 1] = p2;
+                    if (n - 2 >= start) cols[at + 2] = p3;
+                    cols[at + 3] = j;
+                }
+            }
             at += step;
         }
         p1 = p2;
         p2 = p3;
         p3 = j;
     }
-    // the last, partial block, padded with the lane's own index
-    __device__ __forceinline__ void close(uint32_t self, int kcap) {
+    // the entries of the last, partial block
+    __device__ __forceinline__ void close(uint32_t *cols, int kcap) const {
+        const int r = n & (LB - 1), m = PART ? min(r, n - start) : r;
+        if (m == 0 || n > kcap) return;
+        cols[at + r - 1] = p3;
+        if (m > 1) cols[at + r - 2] = p2;
+        if (m > 2) cols[at + r - 3] = p1;
+    }
+    // its pads: the lane's own index
+    __device__ __forceinline__ void pad(uint32_t self, uint32_t *cols, int kcap) const {
         const int r = n & (LB - 1);
         if (r == 0 || n > kcap) return;
-        *reinterpret_cast<uint4 *>(at) = r == 1 ? make_uint4(p3, self, self, self)
-                                       : (r == 2 ? make_uint4(p2, p3, self, self) : make_uint4(p1, p2, p3, self));
+        for (int k = r; k < LB; k++) cols[at + k] = self;
     }
 };
-constexpr ptrdiff_t BLOCK_WORDS = LB * 32;
+constexpr int BLOCK_WORDS = LB * 32;
 
-// Rounding margin of the walk's FP32 comparisons.  Coordinates are offsets from
-// the tile's box corner, exact integers of at most M (the two tiles' extents
-// plus the larger support, < 2^31, so an offset is the minimum image) rounded
-// to FP32: each is off by at most u M (u = 2^-24), a difference d by 3 u M, a
-// squared distance r^2 <= 3 M^2 by 2 sqrt(3) r 3 u M + 3 u r^2 <= 27 u M^2 and a
-// squared support by 3 u M^2.  A comparison of the two that clears 48 u M^2 has
-// the sign of the exact one.
-constexpr float WALK_MARGIN = 48.f / 16777216.f;
-constexpr float FAR = 1e18f;   // coordinate of the padding slots: in nobody's reach
+// Rounding margins of the walk's FP32 comparisons, u = 2^-24.
+// Relative form: a particle within reach of the tile (gap to its box below the
+// support R < 2^32 / 3) lies at an offset in (-R, E + R) of the box corner, E the
+// tile's largest extent; with E + R < 2^31 that offset is the minimum image, and
+// the differences of two such offsets are too.  Offsets are exact integers of
+// at most M = E + R rounded to FP32: each is off by at most u M, a difference d
+// by 3 u M, a squared distance r^2 <= 3 M^2 by 2 sqrt(3) r 3 u M + 3 u r^2 <=
+// 27 u M^2 and a squared support by 3 u M^2: a comparison that clears 48 u M^2
+// has the sign of the exact one.
+// Integer form (tiles with E beyond that): the minimum-image difference is an
+// exact integer rounded once, so r^2 is off by at most 5 u r^2 and a comparison
+// with H^2 that clears 16 u H^2 (H the largest support) has the exact sign.
+constexpr float MARGIN_REL = 48.f / 16777216.f, MARGIN_INT = 16.f / 16777216.f;
+constexpr int RING = 64;   // kept particles a warp holds: a batch of 32 and up to 32 more
 
-// The exact predicate of one kept particle (bits of its slot p): in gather(i), i in gather(j).
-__device__ __forceinline__ void exact_bits(const uint4 &qi, unsigned long long Hi2, const uint4 &qj, bool same_box,
-                                           int p, unsigned &gm, unsigned &jm) {
-    const unsigned long long R2 =
-        same_box ? r2_fixed((int)(qi.x - qj.x), (int)(qi.y - qj.y), (int)(qi.z - qj.z)) : ~0ull;
-    gm |= (R2 < Hi2 ? 1u : 0u) << p;
-    jm |= (R2 < (unsigned long long)qj.w * qj.w ? 1u : 0u) << p;
+// What is the same for the warp's lanes: kept in shared memory, out of the
+// loops' registers (64 a thread are four CTAs per SM).
+struct WalkBox {
+    uint4 lo;        // box corner, largest support
+    float ex, ey, ez;   // extents
+    uint32_t Ie;     // the largest
+};
+
+// Batches of masks a warp of a shared tile keeps between counting and writing.
+constexpr int MASKS = 8;
+struct WalkMasks {
+    uint32_t g[MASKS][32], j[MASKS][32], id[MASKS][32];
+};
+
+template <bool VOL, bool BATCH>
+struct WalkShm {
+    WalkBox B;
+    uint4 r[RING];                      // (x, y, z, H^2) relative, or the fixed-point record
+    uint32_t id[VOL ? 1 : RING];        // sorted index
+    int32_t box[BATCH ? RING : 1];
+};
+
+// A tile and this lane's particle of it.
+struct WalkTile {
+    int tile, i;
+    bool valid, raw;          // raw: integer form
+    float fx, fy, fz;         // this lane relative to the box corner
+    float Hf, Hf2;
+    int32_t bi;               // box of the particle, box range of the tile (batched boxes)
+    uint32_t Ib;
+};
+
+// fixed-point record of this lane's particle (0 for invalid lanes): read again
+// where the rarer paths need it, which keeps it out of the loops' registers
+__device__ __forceinline__ uint4 own_record(const WalkArgs &a, const WalkTile &T) {
+    return T.valid ? __ldg(a.q4 + T.i) : make_uint4(0, 0, 0, 0);
 }
 
-// BATCH: the particles belong to independent boxes; j can be a neighbour of i
-// only in i's box (the box ranges of tiles prune the rest).
-//
-// LISTS.  Bound by instruction issue: each lane tests every kept particle of
-// each candidate tile, and about one test in five finds an entry.  A test is
-// the FP32 difference of tile-relative coordinates against both squared
-// supports (3 add, 3 multiply-add, 2 add, a running minimum of the distance to
-// either threshold and one funnel shift per mask: 13 instructions against 27 of
-// the 64-bit integer test); the integer predicate runs only for a candidate
-// tile where some lane came within the rounding margin of a threshold (about 1
-// in 500), whose tiles span half the box or more, or which holds several
-// batched boxes, so the lists are the exact ones.  The kept particles are
-// compacted in shared memory, so the loop has no bit scans.
-//
-// VOL.  Sums n_i instead of writing lists: W vanishes beyond h_i, so every kept
-// particle is summed without the predicate, and only particles within the
-// tile's own supports are kept.
-template <bool LISTS, bool VOL, bool BATCH>
-__global__ void __launch_bounds__(WALK_WARPS * 32, 4) k_walk(WalkArgs a) {
-    __shared__ float4 sf[LISTS ? WALK_WARPS : 1][32];        // kept: x, y, z (tile-relative), H^2
-    __shared__ uint4 sq[WALK_WARPS][32];                     // kept: fixed-point record
-    __shared__ uint32_t sid[LISTS ? WALK_WARPS : 1][32];     // kept: sorted index
-    __shared__ int32_t sb[WALK_WARPS][BATCH ? 32 : 1];       // kept: box
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int tw = blockIdx.x * WALK_WARPS + w;
-    if (tw >= a.ntiles) return;
-    const int tile = a.act ? a.act[tw] : tw;
-    const int i = tile * TILE + lane;
-    const bool valid = i < a.n;
-    const uint4 qi = valid ? a.q4[i] : make_uint4(0, 0, 0, 0);
-    const unsigned long long Hi2 = (unsigned long long)qi.w * qi.w;   // 0 for invalid lanes
-    const float h = VOL && valid ? a.hs[i] : 1.f;
-    const float inv_h = 1.f / h;
-    const int kcap = a.kcap;
-    uint32_t *const col0 = LISTS ? a.ent + (size_t)tile * kcap * 32 : nullptr;
-    float acc = 0.f;
-    Seg G{0u, 0u, 0u, 0, LISTS ? col0 + block_at(0, lane) : nullptr};
-    Seg O{0u, 0u, 0u, 0, LISTS ? col0 + block_at(kcap / LB - 1, lane) : nullptr};
-    int lg = 0, lo_ = 0;   // entries with j < i: the candidate tiles come in ascending order
-    uint32_t ntest = 0;    // kept staged particles (warp-uniform)
-    const uint2 lo = a.ofs[tile];
-    const uint4 Ilo = __ldg(a.tlo + tile), Ihi = __ldg(a.thi + tile);   // this tile's box, max H
-    const int32_t bi = BATCH && valid ? a.sbox[i] : 0;
-    const uint32_t Ib = BATCH ? __ldg(a.nbox + tile) : 0u;
-    // this tile and this lane relative to the box corner
-    const uint32_t Iex = Ihi.x - Ilo.x, Iey = Ihi.y - Ilo.y, Iez = Ihi.z - Ilo.z;
-    const uint32_t Ie = max(max(Iex, Iey), Iez);
-    const float ex = (float)Iex, ey = (float)Iey, ez = (float)Iez;
-    const float fx = (float)(qi.x - Ilo.x), fy = (float)(qi.y - Ilo.y), fz = (float)(qi.z - Ilo.z);
-    const float Hf = (float)qi.w, Hf2 = Hf * Hf;
+template <bool BATCH>
+__device__ __forceinline__ WalkTile walk_tile(const WalkArgs &a, int tile, int lane, WalkBox &B) {
+    WalkTile T;
+    T.tile = tile;
+    T.i = tile * TILE + lane;
+    T.valid = T.i < a.n;
+    const uint4 qi = own_record(a, T);
+    const uint4 Ilo = __ldg(a.tlo + tile), Ihi = __ldg(a.thi + tile);
+    const uint32_t x = Ihi.x - Ilo.x, y = Ihi.y - Ilo.y, z = Ihi.z - Ilo.z, e = max(max(x, y), z);
+    T.raw = e >= 0x80000000u - 0x55555556u;   // E + R may reach 2^31
+    __syncwarp();
+    if (lane == 0) B = WalkBox{Ilo, (float)x, (float)y, (float)z, e};
+    __syncwarp();
+    T.fx = (float)(qi.x - Ilo.x);
+    T.fy = (float)(qi.y - Ilo.y);
+    T.fz = (float)(qi.z - Ilo.z);
+    T.Hf = (float)qi.w;
+    T.Hf2 = T.Hf * T.Hf;
+    T.bi = BATCH && T.valid ? a.sbox[T.i] : 0;
+    T.Ib = BATCH ? __ldg(a.nbox + tile) : 0u;
+    return T;
+}
+
+// The candidate tiles [t0, t1) of a tile's list, by one warp.  Lane jj stages
+// particle jj of a candidate and keeps it if it can be in the pair set (VOL: the
+// gather set) of some particle of the tile; the kept particles of successive
+// candidates fill batches of 32 in shared memory.  visit(gm, jm, ring, c) gets a
+// batch of c kept particles in ring[ring ..]: bit p of gm: slot p is in
+// gather(i); of jm: i is in gather(slot p) (VOL: visit(ring, c), no masks).
+// `kept` counts the kept particles: every lane tests each of them.
+template <bool VOL, bool BATCH, class Visit>
+__device__ __forceinline__ void walk_range(const WalkArgs &a, const WalkTile &T, int lane, uint2 lo, int t0, int t1,
+                                           WalkShm<VOL, BATCH> &S, uint32_t &kept, Visit &&visit) {
+    uint32_t head = 0, done = 0;   // kept particles staged, and handed on
+    uint32_t exact_to = 0;         // batches that start below take the integer predicate (mixed boxes)
+    int self = -1;                 // the staged number of this lane's own particle
+    float margin = 0.f;            // of the tests so far
+    auto batch = [&](int c) {
+        const uint32_t ring = done & (RING - 1);
+        if constexpr (VOL) {
+            visit(ring, c);
+        } else {
+            unsigned gm = 0u, jm = 0u;
+            const unsigned live = c == 32 ? 0xffffffffu : (1u << c) - 1u;
+            bool exact = done < exact_to;
+            if (!exact) {
+                float amb = 3.0e38f;
+                const int top = (c + 3) & ~3;
+                if (!T.raw) {
+                    for (int p = top - 4; p >= 0; p -= 4) {   // independent chains; slot 0 ends at bit 0
+#pragma unroll
+                        for (int u = 3; u >= 0; u--) {
+                            const float4 f = reinterpret_cast<const float4 *>(S.r)[ring + p + u];
+                            const float dx = T.fx - f.x, dy = T.fy - f.y, dz = T.fz - f.z;
+                            const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+                            const float ti = r2 - T.Hf2, tj = r2 - f.w;
+                            amb = fminf(amb, fminf(fabsf(ti), fabsf(tj)));
+                            gm = __funnelshift_l(__float_as_uint(ti), gm, 1);
+                            jm = __funnelshift_l(__float_as_uint(tj), jm, 1);
+                        }
+                    }
+                } else {
+                    const uint4 qi = own_record(a, T);
+                    for (int p = top - 4; p >= 0; p -= 4) {
+#pragma unroll
+                        for (int u = 3; u >= 0; u--) {
+                            const uint4 q = S.r[ring + p + u];
+                            const float dx = (float)(int)(qi.x - q.x), dy = (float)(int)(qi.y - q.y),
+                                        dz = (float)(int)(qi.z - q.z), H = (float)q.w;
+                            const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+                            const float ti = r2 - T.Hf2, tj = r2 - H * H;
+                            amb = fminf(amb, fminf(fabsf(ti), fabsf(tj)));
+                            gm = __funnelshift_l(__float_as_uint(ti), gm, 1);
+                            jm = __funnelshift_l(__float_as_uint(tj), jm, 1);
+                        }
+                    }
+                }
+                exact = __any_sync(0xffffffffu, T.valid && amb < margin);
+            }
+            if (exact) {
+                gm = jm = 0u;
+                const uint4 qi = own_record(a, T);
+                const unsigned long long Hi2 = (unsigned long long)qi.w * qi.w;
+                for (int p = 0; p < c; p++) {
+                    const uint4 q = __ldg(a.q4 + S.id[ring + p]);
+                    unsigned long long R2 = r2_fixed((int)(qi.x - q.x), (int)(qi.y - q.y), (int)(qi.z - q.z));
+                    if (BATCH && S.box[ring + p] != T.bi) R2 = ~0ull;
+                    gm |= (R2 < Hi2 ? 1u : 0u) << p;
+                    jm |= (R2 < (unsigned long long)q.w * q.w ? 1u : 0u) << p;
+                }
+            }
+            unsigned use = T.valid ? live : 0u;
+            const int me = self - (int)done;   // j != i
+            if (me >= 0 && me < 32) use &= ~(1u << me);
+            visit(gm & use, jm & use, ring);
+        }
+        done += (uint32_t)c;
+    };
     // software pipeline over the candidate tiles: the tile id two ahead, and
     // the box and this lane's staged particle of the next tile, are in flight
     // while the current tile is tested (each is otherwise a dependent L2 trip)
     const uint32_t *tl = a.tiles + lo.x;
-    const int nt = (int)lo.y;
-    int J1 = nt > 0 ? (int)__ldg(tl) : 0, J2 = nt > 1 ? (int)__ldg(tl + 1) : 0;
+    int J1 = t0 < t1 ? (int)__ldg(tl + t0) : 0, J2 = t0 + 1 < t1 ? (int)__ldg(tl + t0 + 1) : 0;
     uint4 lo1 = make_uint4(0, 0, 0, 0), hi1 = lo1, qn = lo1;
-    if (nt > 0) {
+    if (t0 < t1) {
         lo1 = __ldg(a.tlo + J1);
         hi1 = __ldg(a.thi + J1);
         if (J1 * TILE + lane < a.n) qn = __ldg(a.q4 + J1 * TILE + lane);
     }
-    for (int t = 0; t < nt; t++) {
+    for (int t = t0; t < t1; t++) {
         const int J = J1;
         const uint4 Jlo = lo1, Jhi = hi1, qc = qn;
         J1 = J2;
-        if (t + 2 < nt) J2 = (int)__ldg(tl + t + 2);
-        if (t + 1 < nt) {
+        if (t + 2 < t1) J2 = (int)__ldg(tl + t + 2);
+        if (t + 1 < t1) {
             lo1 = __ldg(a.tlo + J1);
             hi1 = __ldg(a.thi + J1);
             if (J1 * TILE + lane < a.n) qn = __ldg(a.q4 + J1 * TILE + lane);
         }
         const int j0 = J * TILE;
         const int cnt = min(TILE, a.n - j0);
+        const uint4 Ilo = S.B.lo;
         const uint32_t Jex = Jhi.x - Jlo.x, Jey = Jhi.y - Jlo.y, Jez = Jhi.z - Jlo.z;
         const uint32_t HJ = VOL ? 0u : Jlo.w;   // the volumes take gather(i) only
-        const uint32_t Hm = max(Ilo.w, HJ);
-        const unsigned long long M =
-            (unsigned long long)Ie + max(max(Jex, Jey), Jez) + max(Ilo.w, Jlo.w);   // warp-uniform
-        const bool wide = M >= 0x7fffffffull;   // offsets may not be the minimum image
-        const float margin = WALK_MARGIN * ((float)M * (float)M);
-        // lane jj stages particle j0 + jj and keeps it only if it can be in the
-        // pair set (VOL: the gather set) of some particle of this tile: its gap
-        // to the tile's box below the larger support.  Skip a tile that no
-        // lane's sphere touches.  Conservative, so the lists are unchanged.
+        const uint32_t R = max(Ilo.w, Jlo.w), M = S.B.Ie + R;   // warp-uniform
+        // Skip a tile that no lane's sphere touches; keep a particle whose gap to
+        // the tile's box is below the larger support.  Both conservative, so the
+        // lists are unchanged.
         bool near, keep;
         float jx = 0.f, jy = 0.f, jz = 0.f;
-        if (!wide) {
+        const float edge = T.raw ? (float)R : (float)M;
+        const float mrg = (T.raw ? MARGIN_INT : MARGIN_REL) * (edge * edge);
+        if (!T.raw) {
             const int ox = (int)(Jlo.x - Ilo.x), oy = (int)(Jlo.y - Ilo.y), oz = (int)(Jlo.z - Ilo.z);
             const float lx = (float)ox, ly = (float)oy, lz = (float)oz;
-            const float gx = fmaxf(fmaxf(lx - fx, fx - (float)(int)((uint32_t)ox + Jex)), 0.f);
-            const float gy = fmaxf(fmaxf(ly - fy, fy - (float)(int)((uint32_t)oy + Jey)), 0.f);
-            const float gz = fmaxf(fmaxf(lz - fz, fz - (float)(int)((uint32_t)oz + Jez)), 0.f);
-            const float re = fmaxf(Hf, (float)HJ);
-            near = valid && fmaf(gx, gx, fmaf(gy, gy, gz * gz)) < fmaf(re, re, margin);
+            const float gx = fmaxf(fmaxf(lx - T.fx, T.fx - (float)(int)((uint32_t)ox + Jex)), 0.f);
+            const float gy = fmaxf(fmaxf(ly - T.fy, T.fy - (float)(int)((uint32_t)oy + Jey)), 0.f);
+            const float gz = fmaxf(fmaxf(lz - T.fz, T.fz - (float)(int)((uint32_t)oz + Jez)), 0.f);
+            const float re = fmaxf(T.Hf, (float)HJ);
+            // (offsets of a box that spans much of the period may not be its nearest image)
+            near = T.valid && (M + (unsigned long long)max(max(Jex, Jey), Jez) >= 0x80000000ull ||
+                               fmaf(gx, gx, fmaf(gy, gy, gz * gz)) < fmaf(re, re, mrg));
             jx = (float)(int)(qc.x - Ilo.x);
             jy = (float)(int)(qc.y - Ilo.y);
             jz = (float)(int)(qc.z - Ilo.z);
-            const float hx = fmaxf(fmaxf(-jx, jx - ex), 0.f), hy = fmaxf(fmaxf(-jy, jy - ey), 0.f),
-                        hz = fmaxf(fmaxf(-jz, jz - ez), 0.f);
+            const float hx = fmaxf(fmaxf(-jx, jx - S.B.ex), 0.f), hy = fmaxf(fmaxf(-jy, jy - S.B.ey), 0.f),
+                        hz = fmaxf(fmaxf(-jz, jz - S.B.ez), 0.f);
             const float rj = (float)(VOL ? Ilo.w : max(qc.w, Ilo.w));
-            keep = lane < cnt && fmaf(hx, hx, fmaf(hy, hy, hz * hz)) < fmaf(rj, rj, margin);
+            keep = lane < cnt && fmaf(hx, hx, fmaf(hy, hy, hz * hz)) < fmaf(rj, rj, mrg);
         } else {
+            const uint4 qi = own_record(a, T), Ihi = __ldg(a.thi + T.tile);
             const unsigned long long gx = point_gap(qi.x, Jlo.x, Jhi.x), gy = point_gap(qi.y, Jlo.y, Jhi.y),
                                      gz = point_gap(qi.z, Jlo.z, Jhi.z);
             const unsigned long long reach = max(qi.w, HJ);
-            near = valid && gx * gx + gy * gy + gz * gz < reach * reach;
+            near = T.valid && gx * gx + gy * gy + gz * gz < reach * reach;
             const unsigned long long hx = point_gap(qc.x, Ilo.x, Ihi.x), hy = point_gap(qc.y, Ilo.y, Ihi.y),
                                      hz = point_gap(qc.z, Ilo.z, Ihi.z);
-            const unsigned long long rj = VOL ? Hm : max(qc.w, Ilo.w);
+            const unsigned long long rj = VOL ? Ilo.w : max(qc.w, Ilo.w);
             keep = lane < cnt && hx * hx + hy * hy + hz * hz < rj * rj;
         }
         bool mixed = false;   // the pair's boxes must be compared
         int32_t bj = 0;
         if constexpr (BATCH) {
             const uint32_t Jb = __ldg(a.nbox + J);
-            near = near && (uint32_t)bi >= (Jb & 0xffffu) && (uint32_t)bi <= (Jb >> 16);
-            mixed = Ib != Jb || (Ib & 0xffffu) != (Ib >> 16);
+            near = near && (uint32_t)T.bi >= (Jb & 0xffffu) && (uint32_t)T.bi <= (Jb >> 16);
+            mixed = T.Ib != Jb || (T.Ib & 0xffffu) != (T.Ib >> 16);
+            bj = (int32_t)(Jb & 0xffffu);
             if (mixed && lane < cnt) {
                 bj = __ldg(a.sbox + j0 + lane);
-                keep = keep && (uint32_t)bj >= (Ib & 0xffffu) && (uint32_t)bj <= (Ib >> 16);
+                keep = keep && (uint32_t)bj >= (T.Ib & 0xffffu) && (uint32_t)bj <= (T.Ib >> 16);
             }
         }
         if (__ballot_sync(0xffffffffu, near) == 0u) continue;
         const unsigned mask = __ballot_sync(0xffffffffu, keep);
         if (mask == 0u) continue;
-        const int nk = __popc(mask), nk4 = (nk + 3) & ~3;
-        ntest += (uint32_t)nk;   // every lane tests every kept particle
-        const int slot = __popc(mask & lanemask_lt());
+        const uint32_t at = head + (uint32_t)__popc(mask & lanemask_lt());
+        if (J == T.tile) self = (int)at;   // this tile's particles are all kept
         __syncwarp();
         if (keep) {
-            sq[w][slot] = qc;
-            if (LISTS) {
-                const float hj = (float)qc.w;
-                sf[w][slot] = make_float4(jx, jy, jz, hj * hj);
-                sid[w][slot] = (uint32_t)(j0 + lane);
-            }
-            if (BATCH) sb[w][slot] = bj;
-        }
-        if (lane < nk4 - nk) {
-            if (LISTS) sf[w][nk + lane] = make_float4(FAR, FAR, FAR, 0.f);
-            if (VOL) sq[w][nk + lane] = make_uint4(0, 0, 0, 0);
+            const uint32_t k = at & (RING - 1);
+            const float hj = (float)qc.w;
+            S.r[k] = VOL || T.raw ? qc
+                                  : make_uint4(__float_as_uint(jx), __float_as_uint(jy), __float_as_uint(jz),
+                                               __float_as_uint(hj * hj));
+            if (!VOL) S.id[k] = (uint32_t)(j0 + lane);
+            if (BATCH) S.box[k] = bj;
         }
         __syncwarp();
-        if constexpr (LISTS) {
-            // gm: j in gather(i); jm: i in gather(j); bit = slot
-            unsigned gm = 0u, jm = 0u;
-            bool exact = wide || mixed;
-            if (!exact) {
-                float amb = 3.0e38f;
-                for (int p = nk4 - 4; p >= 0; p -= 4) {   // four independent chains; slot 0 ends at bit 0
-#pragma unroll
-                    for (int u = 3; u >= 0; u--) {
-                        const float4 f = sf[w][p + u];
-                        const float dx = fx - f.x, dy = fy - f.y, dz = fz - f.z;
-                        const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                        const float ti = r2 - Hf2, tj = r2 - f.w;
-                        amb = fminf(amb, fminf(fabsf(ti), fabsf(tj)));
-                        gm = __funnelshift_l(__float_as_uint(ti), gm, 1);
-                        jm = __funnelshift_l(__float_as_uint(tj), jm, 1);
-                    }
-                }
-                exact = __any_sync(0xffffffffu, valid && amb < margin);
-            }
-            if (exact) {
-                gm = jm = 0u;
-                for (int p = 0; p < nk; p++)
-                    exact_bits(qi, Hi2, sq[w][p], !BATCH || !mixed || sb[w][p] == bi, p, gm, jm);
-            }
-            if (!valid) gm = jm = 0u;
-            if (J <= tile) {
-                unsigned below = 0xffffffffu;
-                if (J == tile) {   // j != i (particle i is kept, in slot `slot`)
-                    below = (1u << slot) - 1u;
-                    gm &= ~(1u << slot);
-                    jm &= ~(1u << slot);
-                }
-                lg = G.n + __popc(gm & below);
-                lo_ = O.n + __popc(jm & ~gm & below);
-            }
-            // each lane appends its own entries in staging order
-            jm &= ~gm;
-            while (gm) {
-                const int p = __ffs(gm) - 1;
-                gm &= gm - 1u;
-                G.push(sid[w][p], kcap, BLOCK_WORDS);
-            }
-            while (jm) {
-                const int p = __ffs(jm) - 1;
-                jm &= jm - 1u;
-                O.push(sid[w][p], kcap, -BLOCK_WORDS);
-            }
-        } else {
-            for (int p = 0; p < nk4; p += 4) {
-#pragma unroll
-                for (int u = 0; u < 4; u++) {
-                    const uint4 qj = sq[w][p + u];
-                    Sep d = separation((int)(qi.x - qj.x), (int)(qi.y - qj.y), (int)(qi.z - qj.z));
-                    const float eta = d.r * inv_h;
-                    float tt = __saturatef(1.f - eta);
-                    if (p + u >= nk) tt = 0.f;
-                    if (BATCH && mixed && p + u < nk && sb[w][p + u] != bi) tt = 0.f;
-                    const float t2 = tt * tt, t3 = t2 * tt;
-                    acc = fmaf(t3 * t3, fmaf(eta, fmaf(eta, K35_3, 6.f), 1.f), acc);
-                }
-            }
-        }
+        head += (uint32_t)__popc(mask);
+        margin = fmaxf(margin, mrg);
+        if (mixed) exact_to = head;
+        if (head - done >= 32u) batch(32);
     }
-    const int cu = G.n + O.n;
-    const int rg = LB * list_blocks(G.n), ru = rg + LB * list_blocks(O.n);   // rows with the pads
-    if (valid) {
-        if (VOL) {
-            float ih3 = inv_h * inv_h * inv_h;
-            float nsum = KW * ih3 * acc;                       // n_i, eq:vol
-            a.V[i] = 1.f / nsum;
-            if (a.Nn) a.Nn[i] = (K4PI_3 * h * h * h) * nsum;   // eq:hi
-        }
-        if (LISTS) {
-            G.close((uint32_t)i, kcap);
-            O.close((uint32_t)i, kcap);
-        }
-        a.cnt_g[i] = G.n;
-        a.cnt_u[i] = cu;
-        if (LISTS && a.lowc) a.lowc[i] = make_int2(lg, lo_);
-    }
-    uint32_t mg = __reduce_max_sync(0xffffffffu, (uint32_t)rg);
-    uint32_t mu = __reduce_max_sync(0xffffffffu, (uint32_t)ru);
-    uint32_t sg = __reduce_add_sync(0xffffffffu, (uint32_t)G.n);
-    uint32_t su = __reduce_add_sync(0xffffffffu, (uint32_t)cu);
-    if (lane == 0) {
-        a.len_g[tile] = min(mg, (uint32_t)kcap);
-        a.len_u[tile] = min(mu, (uint32_t)kcap);
-        atomicAdd(a.pairs_g, (unsigned long long)sg);
-        atomicAdd(a.pairs_u, (unsigned long long)su);
-        atomicMax(a.maxcnt, (unsigned long long)mu);
-        if (LISTS) atomicAdd(a.tests, 32ull * ntest);
-    }
+    if (head > done) batch((int)(head - done));
+    kept += head;
 }
 
-// The walk for few tiles (time bins, act set): S warps share one tile, warp w
-// testing the candidate tiles [w chunk, (w+1) chunk) of its list.  A first
-// sweep counts every lane's gather and other neighbours per warp; their
-// prefix over the warps gives each warp its columns, and a second sweep
-// writes the entries there, so every list is exactly the one-warp walk's.
-template <int S>
-__global__ void __launch_bounds__(S * 32) k_walk_split(WalkArgs a) {
-    __shared__ uint4 sq[S][32];
-    __shared__ int cnt[2][S][32];
+// Neighbour lists (LISTS) or volumes (VOL).  BATCH: the particles belong to
+// independent boxes; j can be a neighbour of i only in i's box (the box ranges
+// of tiles prune the rest).
+//
+// LISTS.  Bound by instruction issue: each lane tests every kept particle, and
+// about one test in five finds an entry.  A test is an FP32 difference against
+// both squared supports (3 add, 3 multiply-add, 2 add, a running minimum of the
+// distance to either threshold and a funnel shift per mask: 13 instructions
+// against 27 of the 64-bit integer test); the integer predicate runs only for a
+// batch where some lane came within the rounding margin of a threshold, or that
+// holds several batched boxes, so the lists are the exact ones.  Batches span
+// candidate tiles (a tile keeps about 15 of a candidate's 32), so the loops run
+// full and each lane's divergent writing of its entries runs half as often.
+//
+// VOL.  Sums n_i instead of writing lists: W vanishes beyond h_i, so every kept
+// particle is summed without the predicate, and only particles within the
+// tile's own supports are kept.
+//
+// A warp takes a tile, except where that leaves the chip waiting for a few
+// warps: tiles with more than a.heavy candidates (a run of the Morton order
+// that jumps across the box: at 64^3 clustered the largest has 16 times the
+// mean's candidates), and every tile of a set that does not fill the chip.
+// Those are shared by the eight warps of a CTA, each taking a range of the
+// candidates: a first sweep counts and keeps its masks, the prefix over the
+// warps gives each its place in the lists, and the entries are written from the
+// masks (a warp with more than MASKS batches sweeps again), so the lists are
+// exactly the one-warp walk's.
+template <bool LISTS, bool VOL, bool BATCH>
+__global__ void __launch_bounds__(WALK_WARPS * 32, 4) k_walk(WalkArgs a) {
+    __shared__ WalkShm<VOL, BATCH> shm[WALK_WARPS];
+    __shared__ int part[2][WALK_WARPS][32];
+    __shared__ WalkMasks masks[LISTS ? WALK_WARPS : 1];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int tile = a.act[blockIdx.x];
-    const int i = tile * TILE + lane;
-    const bool valid = i < a.n;
-    const uint4 qi = valid ? a.q4[i] : make_uint4(0, 0, 0, 0);
-    const unsigned long long Hi2 = (unsigned long long)qi.w * qi.w;
+    WalkShm<VOL, BATCH> &S = shm[w];
     const int kcap = a.kcap;
-    uint32_t *const col0 = a.ent + (size_t)tile * kcap * 32;
-    auto word = [&](int c) -> uint32_t * { return col0 + block_at(c / LB, lane) + c % LB; };   // gather entry c
-    auto back = [&](int c) -> uint32_t * { return col0 + block_at(kcap / LB - 1 - c / LB, lane) + c % LB; };
-    const uint2 lo = a.ofs[tile];
-    const uint4 Ilo = __ldg(a.tlo + tile), Ihi = __ldg(a.thi + tile);
-    const int nt = (int)lo.y;
-    const int chunk = (nt + S - 1) / S;
-    const int t0 = w * chunk, t1 = min(nt, t0 + chunk);
-    int base_g = 0, base_o = 0, tot_g = 0, tot_o = 0;
-    for (int phase = 0; phase < 2; phase++) {
-        int cg = 0, co = 0;
-        for (int t = t0; t < t1; t++) {
-            const int J = (int)__ldg(a.tiles + lo.x + t);
-            const uint4 Jlo = __ldg(a.tlo + J), Jhi = __ldg(a.thi + J);
-            const unsigned long long gx = point_gap(qi.x, Jlo.x, Jhi.x), gy = point_gap(qi.y, Jlo.y, Jhi.y),
-                                     gz = point_gap(qi.z, Jlo.z, Jhi.z);
-            const unsigned long long reach = qi.w > Jlo.w ? qi.w : Jlo.w;
-            const bool near = valid && gx * gx + gy * gy + gz * gz < reach * reach;
-            if (__ballot_sync(0xffffffffu, near) == 0u) continue;
-            const int j0 = J * TILE;
-            const int cj = min(TILE, a.n - j0);
-            __syncwarp();
-            bool keep = false;
-            if (lane < cj) {
-                const uint4 q = __ldg(a.q4 + j0 + lane);
-                sq[w][lane] = q;
-                const unsigned long long hx = point_gap(q.x, Ilo.x, Ihi.x), hy = point_gap(q.y, Ilo.y, Ihi.y),
-                                         hz = point_gap(q.z, Ilo.z, Ihi.z);
-                const unsigned long long rj = q.w > Ilo.w ? q.w : Ilo.w;
-                keep = hx * hx + hy * hy + hz * hz < rj * rj;
-            }
-            unsigned mask = __ballot_sync(0xffffffffu, keep);
-            __syncwarp();
-            auto visit = [&](int jj, const uint4 &qj, unsigned long long R2) {
-                const uint32_t j = (uint32_t)(j0 + jj);
-                if (valid && (int)j != i) {
-                    const bool in_i = R2 < Hi2;
-                    const bool in_j = R2 < (unsigned long long)qj.w * qj.w;
-                    if (in_i) {
-                        const int c = base_g + cg;
-                        if (phase == 1 && c < kcap) *word(c) = j;
-                        cg++;
-                    } else if (in_j) {
-                        const int c = base_o + co;
-                        if (phase == 1 && c < kcap) *back(c) = j;
-                        co++;
-                    }
-                }
-            };
-            while (mask) {   // two staged neighbours per iteration, in staging order
-                const int ja = __ffs(mask) - 1;
-                mask &= mask - 1u;
-                const bool two = mask != 0u;
-                const int jb = two ? __ffs(mask) - 1 : ja;
-                if (two) mask &= mask - 1u;
-                const uint4 qa = sq[w][ja], qb = sq[w][jb];
-                const unsigned long long Ra = r2_fixed((int)(qi.x - qa.x), (int)(qi.y - qa.y), (int)(qi.z - qa.z));
-                const unsigned long long Rb = r2_fixed((int)(qi.x - qb.x), (int)(qi.y - qb.y), (int)(qi.z - qb.z));
-                visit(ja, qa, Ra);
-                if (two) visit(jb, qb, Rb);
+    // V_i, N_i from the kernel sum of a lane
+    auto volume = [&](const WalkTile &T, float acc) {
+        const float h = a.hs[T.i], inv_h = 1.f / h;
+        const float ih3 = inv_h * inv_h * inv_h;
+        const float nsum = KW * ih3 * acc;                         // n_i, eq:vol
+        a.V[T.i] = 1.f / nsum;
+        if (a.Nn) a.Nn[T.i] = (K4PI_3 * h * h * h) * nsum;         // eq:hi
+    };
+    auto sum_batch = [&](const WalkTile &T, const uint4 &qi, float inv_h, uint32_t ring, int c, float &acc) {
+        for (int p = 0; p < c; p += 4) {
+#pragma unroll
+            for (int u = 0; u < 4; u++) {
+                const uint4 q = S.r[ring + p + u];
+                const Sep d = separation((int)(qi.x - q.x), (int)(qi.y - q.y), (int)(qi.z - q.z));
+                const float eta = d.r * inv_h;
+                float t = __saturatef(1.f - eta);
+                if (p + u >= c) t = 0.f;
+                if (BATCH && S.box[ring + p + u] != T.bi) t = 0.f;
+                const float t2 = t * t, t3 = t2 * t;
+                acc = fmaf(t3 * t3, fmaf(eta, fmaf(eta, K35_3, 6.f), 1.f), acc);
             }
         }
-        if (phase == 0) {
-            cnt[0][w][lane] = cg;
-            cnt[1][w][lane] = co;
+    };
+    // counts, per-tile rows and totals of a finished tile (one warp)
+    auto close = [&](const WalkTile &T, int cg, int co) {
+        const int rg = LB * list_blocks(cg), ru = rg + LB * list_blocks(co);   // rows with the pads
+        if (T.valid) {
+            a.cnt_g[T.i] = cg;
+            a.cnt_u[T.i] = cg + co;
+        }
+        const uint32_t mg = __reduce_max_sync(0xffffffffu, (uint32_t)rg);
+        const uint32_t mu = __reduce_max_sync(0xffffffffu, (uint32_t)ru);
+        const uint32_t sg = __reduce_add_sync(0xffffffffu, (uint32_t)cg);
+        const uint32_t su = __reduce_add_sync(0xffffffffu, (uint32_t)(cg + co));
+        if (lane == 0) {
+            a.len_g[T.tile] = min(mg, (uint32_t)kcap);
+            a.len_u[T.tile] = min(mu, (uint32_t)kcap);
+            atomicAdd(a.pairs_g, (unsigned long long)sg);
+            atomicAdd(a.pairs_u, (unsigned long long)su);
+            atomicMax(a.maxcnt, (unsigned long long)mu);
+        }
+    };
+    auto shared_tile = [&](int tile, uint2 lo) {   // by all warps of the CTA
+        const WalkTile T = walk_tile<BATCH>(a, tile, lane, S.B);
+        const int nt = (int)lo.y, chunk = (nt + WALK_WARPS - 1) / WALK_WARPS;
+        const int t0 = min(nt, w * chunk), t1 = min(nt, t0 + chunk);
+        uint32_t kept = 0;
+        if constexpr (VOL) {
+            const uint4 qi = own_record(a, T);
+            const float inv_h = 1.f / (T.valid ? a.hs[T.i] : 1.f);
+            float acc = 0.f;
+            walk_range<VOL, BATCH>(a, T, lane, lo, t0, t1, S, kept,
+                                   [&](uint32_t ring, int c) { sum_batch(T, qi, inv_h, ring, c, acc); });
+            part[0][w][lane] = __float_as_int(acc);
             __syncthreads();
-            for (int v = 0; v < S; v++) {
-                if (v < w) {
-                    base_g += cnt[0][v][lane];
-                    base_o += cnt[1][v][lane];
+            if (w == 0) {
+                for (int v = 1; v < WALK_WARPS; v++) acc += __int_as_float(part[0][v][lane]);
+                if (T.valid) volume(T, acc);
+                close(T, 0, 0);
+            }
+        } else {
+            uint32_t *const col0 = a.ent + (size_t)tile * kcap * 32;
+            WalkMasks &K = masks[w];
+            int cg = 0, co = 0, nb = 0;
+            walk_range<VOL, BATCH>(a, T, lane, lo, t0, t1, S, kept, [&](unsigned gm, unsigned jm, uint32_t ring) {
+                jm &= ~gm;
+                cg += __popc(gm);
+                co += __popc(jm);
+                if (nb < MASKS) {
+                    K.g[nb][lane] = gm;
+                    K.j[nb][lane] = jm;
+                    K.id[nb][lane] = S.id[ring + lane];
                 }
-                tot_g += cnt[0][v][lane];
-                tot_o += cnt[1][v][lane];
+                nb++;
+            });
+            if (lane == 0) atomicAdd(a.tests, 32ull * kept);
+            part[0][w][lane] = cg;
+            part[1][w][lane] = co;
+            __syncthreads();
+            int pg = 0, po = 0, tg = 0, to = 0;   // this warp's place, the totals
+            for (int v = 0; v < WALK_WARPS; v++) {
+                if (v == w) pg = tg, po = to;
+                tg += part[0][v][lane];
+                to += part[1][v][lane];
+            }
+            Seg<true> G{0u, 0u, 0u, pg, pg, (int)block_at(pg / LB, lane)};
+            Seg<true> O{0u, 0u, 0u, po, po, (int)block_at(kcap / LB - 1 - po / LB, lane)};
+            auto write = [&](unsigned gm, unsigned jm, const uint32_t *id) {
+                for (; gm; gm &= gm - 1u) G.push(id[__ffs(gm) - 1], col0, kcap, BLOCK_WORDS);
+                for (; jm; jm &= jm - 1u) O.push(id[__ffs(jm) - 1], col0, kcap, -BLOCK_WORDS);
+            };
+            if (nb <= MASKS) {
+                for (int b = 0; b < nb; b++) write(K.g[b][lane], K.j[b][lane], K.id[b]);
+            } else {
+                walk_range<VOL, BATCH>(a, T, lane, lo, t0, t1, S, kept, [&](unsigned gm, unsigned jm, uint32_t ring) {
+                    write(gm, jm & ~gm, S.id + ring);
+                });
+            }
+            if (T.valid) {
+                G.close(col0, kcap);
+                O.close(col0, kcap);
+                if (w == WALK_WARPS - 1) {   // its segments end where the lists end
+                    G.pad((uint32_t)T.i, col0, kcap);
+                    O.pad((uint32_t)T.i, col0, kcap);
+                }
+            }
+            if (w == 0) close(T, tg, to);
+        }
+        __syncthreads();   // `part` is free for the next tile
+    };
+    if ((int)blockIdx.x < a.hblocks) {
+        if (a.all) {
+            const int tile = a.act ? a.act[blockIdx.x] : (int)blockIdx.x;
+            shared_tile(tile, a.ofs[tile]);
+            return;
+        }
+        for (int t0 = (int)blockIdx.x * 32; t0 < a.ntiles; t0 += a.hblocks * 32) {
+            const int t = t0 + lane;
+            const int mine = t < a.ntiles ? (a.act ? a.act[t] : t) : -1;
+            unsigned m = __ballot_sync(0xffffffffu, mine >= 0 && (int)a.ofs[max(mine, 0)].y > a.heavy);
+            for (; m; m &= m - 1u) {
+                const int tile = __shfl_sync(0xffffffffu, mine, __ffs(m) - 1);
+                shared_tile(tile, a.ofs[tile]);
             }
         }
+        return;
     }
-    if (w != 0) return;
-    const int cu = tot_g + tot_o;
-    const int rg = LB * list_blocks(tot_g), ru = rg + LB * list_blocks(tot_o);
-    if (valid) {
-        for (int c = tot_g; c < min(rg, kcap); c++) *word(c) = (uint32_t)i;   // pads
-        for (int c = tot_o; c < min(ru - rg, kcap); c++) *back(c) = (uint32_t)i;
-        a.cnt_g[i] = tot_g;
-        a.cnt_u[i] = cu;
-    }
-    uint32_t mg = __reduce_max_sync(0xffffffffu, (uint32_t)rg);
-    uint32_t mu = __reduce_max_sync(0xffffffffu, (uint32_t)ru);
-    uint32_t sg = __reduce_add_sync(0xffffffffu, (uint32_t)tot_g);
-    uint32_t su = __reduce_add_sync(0xffffffffu, (uint32_t)cu);
-    if (lane == 0) {
-        a.len_g[tile] = min(mg, (uint32_t)kcap);
-        a.len_u[tile] = min(mu, (uint32_t)kcap);
-        atomicAdd(a.pairs_g, (unsigned long long)sg);
-        atomicAdd(a.pairs_u, (unsigned long long)su);
-        atomicMax(a.maxcnt, (unsigned long long)mu);
+    const int tw = ((int)blockIdx.x - a.hblocks) * WALK_WARPS + w;
+    if (tw >= a.ntiles) return;
+    const int tile = a.act ? a.act[tw] : tw;
+    const uint2 lo = a.ofs[tile];
+    if ((int)lo.y > a.heavy) return;
+    const WalkTile T = walk_tile<BATCH>(a, tile, lane, S.B);
+    uint32_t kept = 0;
+    if constexpr (VOL) {
+        const uint4 qi = own_record(a, T);
+        const float inv_h = 1.f / (T.valid ? a.hs[T.i] : 1.f);
+        float acc = 0.f;
+        walk_range<VOL, BATCH>(a, T, lane, lo, 0, (int)lo.y, S, kept,
+                               [&](uint32_t ring, int c) { sum_batch(T, qi, inv_h, ring, c, acc); });
+        if (T.valid) volume(T, acc);
+        close(T, 0, 0);
+    } else {
+        uint32_t *const col0 = a.ent + (size_t)tile * kcap * 32;
+        Seg<false> G{0u, 0u, 0u, 0, 0, (int)block_at(0, lane)};
+        Seg<false> O{0u, 0u, 0u, 0, 0, (int)block_at(kcap / LB - 1, lane)};
+        walk_range<VOL, BATCH>(a, T, lane, lo, 0, (int)lo.y, S, kept, [&](unsigned gm, unsigned jm, uint32_t ring) {
+            jm &= ~gm;
+            for (; gm; gm &= gm - 1u) G.push(S.id[ring + __ffs(gm) - 1], col0, kcap, BLOCK_WORDS);
+            for (; jm; jm &= jm - 1u) O.push(S.id[ring + __ffs(jm) - 1], col0, kcap, -BLOCK_WORDS);
+        });
+        if (T.valid) {
+            G.close(col0, kcap);
+            O.close(col0, kcap);
+            G.pad((uint32_t)T.i, col0, kcap);
+            O.pad((uint32_t)T.i, col0, kcap);
+        }
+        close(T, G.n, O.n);
+        if (lane == 0) atomicAdd(a.tests, 32ull * kept);
     }
 }
 
@@ -476,8 +574,11 @@ static WalkArgs walk_args(crk_ctx *ctx) {
     a.nbox = ctx->nbox > 1 ? ctx->node_box : nullptr;
     a.act = ctx->act;
     if (ctx->act) a.ntiles = ctx->nact;
-    a.lowc = ctx->volumes_only ? nullptr : ctx->lowc;
     a.tests = ctx->counters + CNT_WALK_TESTS;
+    const int nsm = ctx->nsm > 0 ? ctx->nsm : 152;
+    a.all = a.ntiles < WALK_ALL * nsm;
+    a.heavy = a.all ? -1 : WALK_HEAVY;
+    a.hblocks = a.all ? a.ntiles : nsm;
     return a;
 }
 
@@ -495,19 +596,17 @@ static int launch_walk(crk_ctx *ctx, cudaStream_t s) {
         if (ctx->nact == 0) return CRK_OK;
     }
     prof_begin(ctx, PROF_LISTS, s);
-    const int g = grid_for(ctx->act ? ctx->nact : ctx->ntiles, WALK_WARPS);
+    const WalkArgs a = walk_args(ctx);
+    const int g = a.hblocks + (a.all ? 0 : grid_for(a.ntiles, WALK_WARPS));
     const bool b = ctx->nbox > 1;
-    const int nsm = ctx->nsm > 0 ? ctx->nsm : 152;
-    if (ctx->act && !ctx->volumes_only && !b && ctx->nact < 8 * nsm)   // few tiles: 8 warps per tile
-        k_walk_split<8><<<ctx->nact, 8 * 32, 0, s>>>(walk_args(ctx));
-    else if (ctx->volumes_only && b)
-        k_walk<false, true, true><<<g, WALK_WARPS * 32, 0, s>>>(walk_args(ctx));
+    if (ctx->volumes_only && b)
+        k_walk<false, true, true><<<g, WALK_WARPS * 32, 0, s>>>(a);
     else if (ctx->volumes_only)
-        k_walk<false, true, false><<<g, WALK_WARPS * 32, 0, s>>>(walk_args(ctx));
+        k_walk<false, true, false><<<g, WALK_WARPS * 32, 0, s>>>(a);
     else if (b)
-        k_walk<true, false, true><<<g, WALK_WARPS * 32, 0, s>>>(walk_args(ctx));
+        k_walk<true, false, true><<<g, WALK_WARPS * 32, 0, s>>>(a);
     else
-        k_walk<true, false, false><<<g, WALK_WARPS * 32, 0, s>>>(walk_args(ctx));
+        k_walk<true, false, false><<<g, WALK_WARPS * 32, 0, s>>>(a);
     ++ctx->launches;
     prof_end(ctx, s);
     CRK_LAUNCH_CHECK(ctx, "neighbour walk");
