@@ -215,12 +215,15 @@ struct P4 {
         float4 *Fst;   // (F_ij, j bits) per list entry
     };
     static int launch_tma(crk_ctx *ctx, const ListGeom &g, const Params &prm, cudaStream_t s);
-    struct IState {
-        FRec me;
-        float m;
+    struct Sums {
         Acc<COMP> F[3], du;
         float vsig, qmax;
     };
+    struct IState : Sums {
+        FRec me;
+        float m;
+    };
+    __device__ static Sums sums(const IState &s) { return s; }
     __device__ static void init(IState &s, int i, bool valid, const Params &p) {
         if (valid) {
             s.me = p.frec[i];
@@ -239,7 +242,7 @@ struct P4 {
         s.du = Acc<COMP>();
         s.vsig = s.qmax = 0.f;
     }
-    __device__ static void merge(IState &s, const IState &o) {
+    __device__ static void merge(IState &s, const Sums &o) {
         for (int g = 0; g < 3; g++) merge_acc(s.F[g], o.F[g]);
         merge_acc(s.du, o.du);
         s.vsig = fmaxf(s.vsig, o.vsig);
@@ -499,11 +502,14 @@ struct P5 {
         const unsigned long long *skip;
         float *du2;
     };
-    struct IState {
-        float4 me, me2;
-        float m;
+    struct Sums {
         Acc<COMP> du, du2;
     };
+    struct IState : Sums {
+        float4 me, me2;
+        float m;
+    };
+    __device__ static Sums sums(const IState &s) { return s; }
     __device__ static void init(IState &s, int i, bool valid, const Params &p) {
         const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
         s.me = valid ? p.sig[DUAL ? 2 * (size_t)i : (size_t)i] : z;
@@ -514,7 +520,7 @@ struct P5 {
         s.du = Acc<COMP>();
         s.du2 = Acc<COMP>();
     }
-    __device__ static void merge(IState &s, const IState &o) {
+    __device__ static void merge(IState &s, const Sums &o) {
         merge_acc(s.du, o.du);
         if (DUAL) merge_acc(s.du2, o.du2);
     }

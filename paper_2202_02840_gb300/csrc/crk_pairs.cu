@@ -218,13 +218,16 @@ struct P2 {
         const float *hs;
         CorrRec *corr;
     };
-    struct IState {
-        uint4 q;
-        float h, inv_h;
-        // s1 = sum V x^a x^g Gu and s2 = sum V x^a x^b x^g Gu are symmetric
-        // tensors: only their distinct components are summed
+    // s1 = sum V x^a x^g Gu and s2 = sum V x^a x^b x^g Gu are symmetric
+    // tensors: only their distinct components are summed
+    struct Sums {
         Acc<COMP> m0, m1[3], m2[6], dm0[3], s1[6], s2[10];
     };
+    struct IState : Sums {
+        uint4 q;
+        float h, inv_h;
+    };
+    __device__ static Sums sums(const IState &s) { return s; }
     __device__ static void init(IState &s, int i, bool valid, const Params &p) {
         s.q = valid ? p.q4[i] : make_uint4(0, 0, 0, 0);
         s.h = valid ? p.hs[i] : 1.f;
@@ -248,7 +251,7 @@ struct P2 {
         for (int a = 0; a < 6; a++) s.s1[a] = Acc<COMP>();
         for (int a = 0; a < 10; a++) s.s2[a] = Acc<COMP>();
     }
-    __device__ static void merge(IState &s, const IState &o) {
+    __device__ static void merge(IState &s, const Sums &o) {
         merge_acc(s.m0, o.m0);
         for (int a = 0; a < 3; a++) {
             merge_acc(s.m1[a], o.m1[a]);
@@ -393,12 +396,15 @@ struct P2X {
     static constexpr bool NOTUNE = true;   // one accuracy mode, one loop form
     using Rec = uint4;
     using Params = P2<true, true>::Params;
-    struct IState {
+    struct Sums {
+        AccFF m0, m1[3], m2[6], dm0[3], s1[6], s2[10];
+    };
+    struct IState : Sums {
         uint4 q;
         float h;
         FF ih;                                  // 1/h as hi + lo
-        AccFF m0, m1[3], m2[6], dm0[3], s1[6], s2[10];
     };
+    __device__ static Sums sums(const IState &s) { return s; }
     __device__ static void init(IState &s, int i, bool valid, const Params &p) {
         s.q = valid ? p.q4[i] : make_uint4(0, 0, 0, 0);
         s.h = valid ? p.hs[i] : 1.f;
@@ -416,7 +422,7 @@ struct P2X {
         for (int a = 0; a < 6; a++) s.m2[a] = s.s1[a] = AccFF();
         for (int a = 0; a < 10; a++) s.s2[a] = AccFF();
     }
-    __device__ static void merge(IState &s, const IState &o) {
+    __device__ static void merge(IState &s, const Sums &o) {
         merge_acc(s.m0, o.m0);
         for (int a = 0; a < 3; a++) merge_acc(s.m1[a], o.m1[a]), merge_acc(s.dm0[a], o.dm0[a]);
         for (int a = 0; a < 6; a++) merge_acc(s.m2[a], o.m2[a]), merge_acc(s.s1[a], o.s1[a]);
@@ -505,12 +511,15 @@ struct P3 {
         GvRec *gv;
         float inv_a;        // the state holds p = a v: grad v = (1/a) grad p
     };
-    struct IState {
+    struct Sums {
+        Acc<COMP> acc[9];
+    };
+    struct IState : Sums {
         uint4 q;
         float inv_h, cW, cG;
         float A, B[3], gA[3], gB[9], v[3];
-        Acc<COMP> acc[9];
     };
+    __device__ static Sums sums(const IState &s) { return s; }
     __device__ static void init(IState &s, int i, bool valid, const Params &p) {
         s.q = valid ? p.q4[i] : make_uint4(0, 0, 0, 0);
         float h = valid ? p.hs[i] : 1.f;
@@ -532,7 +541,7 @@ struct P3 {
     __device__ static void zero(IState &s) {
         for (int k = 0; k < 9; k++) s.acc[k] = Acc<COMP>();
     }
-    __device__ static void merge(IState &s, const IState &o) {
+    __device__ static void merge(IState &s, const Sums &o) {
         for (int k = 0; k < 9; k++) merge_acc(s.acc[k], o.acc[k]);
     }
     struct Rec {
@@ -614,7 +623,9 @@ struct PD {
         s.acc = valid ? p.mass[i] : 0.f;                 // self: x = 0, W(0) / (495/(32 pi h^3)) = 1
     }
     __device__ static void zero(IState &s) { s.acc = 0.f; }
-    __device__ static void merge(IState &s, const IState &o) { s.acc += o.acc; }
+    using Sums = float;
+    __device__ static Sums sums(const IState &s) { return s.acc; }
+    __device__ static void merge(IState &s, Sums o) { s.acc += o; }
     __device__ static Rec load(uint32_t j, size_t, const Params &p) {
         return Rec{__ldg(p.q4 + j), __ldg(p.mass + j)};
     }

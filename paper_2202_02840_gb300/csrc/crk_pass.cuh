@@ -355,28 +355,29 @@ __global__ void __launch_bounds__(32) k_lpass_sm(ListGeom g, typename P::Params 
     }
 }
 
-// Split form, for passes over few tiles (time bins: the leaves ending a step
-// at a deep level): S warps share one tile, warp w walking the entry range
-// [w chunk, (w+1) chunk) of every lane's list, so a tile's pairs take 1/S of
-// the time of one warp walking them all.  Warps w > 0 start from empty sums
-// (P::zero); warp 0 merges their partial states in warp order (P::merge,
-// deterministic) and finishes.  The stored forces of P4 go to the same entry
-// positions as in the other forms; the sums differ from them by rounding.
+// Split form, for passes over few tiles (small boxes; time bins: the leaves
+// ending a step at a deep level): S warps share one tile, warp w walking one
+// contiguous range of every lane's blocks, so a tile's pairs take 1/S of the
+// time of one warp walking them all.  Warps w > 0 start from empty sums
+// (P::zero) and leave them in shared memory (P::sums); warp 0 adds them in warp
+// order (P::merge, deterministic) and finishes.  The stored forces of P4 go to
+// the same rows as in the other forms; the sums differ from them by rounding.
 template <class P>
-constexpr int split_warps() {
-    return (7 * 32 * sizeof(typename P::IState) <= 44 * 1024) ? 8
-           : ((3 * 32 * sizeof(typename P::IState) <= 44 * 1024) ? 4 : 2);
+constexpr int split_warps() {   // as many as their sums fit static shared memory (48 KB)
+    return (7 * 32 * sizeof(typename P::Sums) <= 44 * 1024) ? 8
+           : ((3 * 32 * sizeof(typename P::Sums) <= 44 * 1024) ? 4 : 2);
 }
 
 template <class P, int S, int U>
 __global__ void __launch_bounds__(S * 32) k_lpass_split(ListGeom g, typename P::Params prm, const int32_t *order) {
-    using IS = typename P::IState;
-    __shared__ __align__(16) unsigned char part[(S - 1) * 32 * sizeof(IS)];
+    using Sums = typename P::Sums;
+    __shared__ __align__(16) unsigned char part[(S - 1) * 32 * sizeof(Sums)];
+    if (pass_skipped<P>(prm)) return;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int tile = order[blockIdx.x];
+    const int tile = order ? order[blockIdx.x] : (int)blockIdx.x;
     const int i = tile * TILE + lane;
     const bool valid = i < g.n;
-    IS st;
+    typename P::IState st;
     P::init(st, i, valid, prm);
     if (w > 0) P::zero(st);
     const LaneList<P> ll(g, tile, lane, i, valid);
@@ -384,8 +385,8 @@ __global__ void __launch_bounds__(S * 32) k_lpass_split(ListGeom g, typename P::
     const int chunk = (bw + S - 1) / S;
     const int b0 = w * chunk, b1 = min(bw, b0 + chunk);
     list_loop<P, U>(st, prm, ll, b0, min(ll.nb, b1), b1);
-    IS *sp = reinterpret_cast<IS *>(part);
-    if (w > 0) sp[(w - 1) * 32 + lane] = st;
+    Sums *sp = reinterpret_cast<Sums *>(part);
+    if (w > 0) sp[(w - 1) * 32 + lane] = P::sums(st);
     __syncthreads();
     if (w == 0) {
 #pragma unroll 1
@@ -393,6 +394,13 @@ __global__ void __launch_bounds__(S * 32) k_lpass_split(ListGeom g, typename P::
         if (valid) P::finish(st, i, prm);
     }
 }
+
+// Tiles per SM below which a pass splits them: a warp per tile then leaves the
+// SMs short of warps, or the last wave of warps nearly empty.  Measured on KDK
+// steps, warp per tile against split: clustered 16^3 (0.8 tiles per SM) 0.94 ->
+// 0.52 ms, 32^3 (6.7) 1.37 -> 1.05, 40^3 (13) 1.89 -> 1.50, 48^3 (23) 2.18 -> 2.00,
+// Sedov 64^3 (54) 2.64 -> 2.67.
+constexpr int SPLIT_TILES = 40;
 
 // merge a partial pair sum into another (the compensated sum keeps the
 // partial's correction term)
@@ -569,34 +577,14 @@ int launch_lpass(crk_ctx *ctx, int prof_id, const typename P::Params &prm, cudaS
     ListGeom g{ctx->n, ctx->ntiles, ctx->kcap, ctx->tbase, ctx->len_g, ctx->len_u, ctx->cnt_g, ctx->cnt_u,
                ctx->ent};
     int rc;
-    if (ctx->act) {
-        // the tiles ctx->act[0 .. nact) only (time bins): grid form over that
-        // list, each pass's default loop form, no tuning
-        if (ctx->nact == 0) return CRK_OK;
-        g.ntiles = ctx->nact;
-        constexpr int U = P::PREFETCH ? 1 : P::UNROLL;
-        prof_begin(ctx, prof_id, s);
-        const int nsm = ctx->nsm > 0 ? ctx->nsm : 152;
-        constexpr int S = split_warps<P>();
-        if (ctx->nact < 8 * nsm)   // few tiles: S warps per tile
-            k_lpass_split<P, S, U><<<ctx->nact, S * 32, 0, s>>>(g, prm, ctx->act);
-        else
-            k_lpass<P, WARPS, U><<<grid_for(ctx->nact, WARPS), WARPS * 32, 0, s>>>(g, prm, ctx->act);
-        ++ctx->launches;
-        prof_end(ctx, s);
-        CRK_LAUNCH_CHECK(ctx, what);
-        return CRK_OK;
-    }
-    if constexpr (has_notune<P>::value) {
-        constexpr int U = P::PREFETCH ? 1 : P::UNROLL;
-        prof_begin(ctx, prof_id, s);
-        k_lpass<P, WARPS, U><<<grid_for(ctx->ntiles, WARPS), WARPS * 32, 0, s>>>(g, prm, nullptr);
-        ++ctx->launches;
-        prof_end(ctx, s);
-        CRK_LAUNCH_CHECK(ctx, what);
-        return CRK_OK;
-    }
-    if (ctx->tune_on && !ctx->tune_done[ts]) {
+    const int nsm = ctx->nsm > 0 ? ctx->nsm : 152;
+    constexpr int U = P::PREFETCH ? 1 : P::UNROLL;
+    // the tiles ctx->act[0 .. nact) only (time bins): each pass's default loop
+    // form over that list, no tuning
+    if (ctx->act) g.ntiles = ctx->nact;
+    if (g.ntiles == 0) return CRK_OK;
+    const bool forms = !ctx->act && !has_notune<P>::value;
+    if (forms && ctx->tune_on && !ctx->tune_done[ts]) {
         // time every applicable variant once (each recomputes the same outputs)
         float best = 3.0e38f;
         int bestv = default_variant<P>();
@@ -623,10 +611,18 @@ int launch_lpass(crk_ctx *ctx, int prof_id, const typename P::Params &prm, cudaS
         ctx->tune_done[ts] = 1;
     }
     const int v = ctx->tune_choice[ts] >= 0 ? ctx->tune_choice[ts] : default_variant<P>();
-    if (!variant_applies<P>(v))   // only a variant pinned by crk_tune_set can be one the pass lacks
+    if (forms && !variant_applies<P>(v))   // only a variant pinned by crk_tune_set can be one the pass lacks
         return crk_set_error(ctx, CRK_EINVAL, "%s: the pass has no variant %d", what, v);
     prof_begin(ctx, prof_id, s);
-    rc = launch_variant<P, WARPS>(ctx, g, prm, v, s);
+    rc = CRK_OK;
+    if (g.ntiles < SPLIT_TILES * nsm) {   // whatever the variant: its warps would not fill the SMs
+        constexpr int S = split_warps<P>();
+        k_lpass_split<P, S, U><<<g.ntiles, S * 32, 0, s>>>(g, prm, ctx->act);
+    } else if (forms) {
+        rc = launch_variant<P, WARPS>(ctx, g, prm, v, s);
+    } else {
+        k_lpass<P, WARPS, U><<<grid_for(g.ntiles, WARPS), WARPS * 32, 0, s>>>(g, prm, ctx->act);
+    }
     if (rc) return rc;
     ++ctx->launches;
     prof_end(ctx, s);

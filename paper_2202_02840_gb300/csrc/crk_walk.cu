@@ -719,7 +719,9 @@ struct P1 {
         s.acc = 1.f;                                   // self: W(0) / (495/(32 pi h^3)) = 1
     }
     __device__ static void zero(IState &s) { s.acc = 0.f; }
-    __device__ static void merge(IState &s, const IState &o) { s.acc += o.acc; }
+    using Sums = float;
+    __device__ static Sums sums(const IState &s) { return s.acc; }
+    __device__ static void merge(IState &s, Sums o) { s.acc += o; }
     __device__ static Rec load(uint32_t j, size_t, const Params &p) { return __ldg(p.q4 + j); }
     __device__ static void pair(IState &s, const Rec &r, uint32_t, size_t, bool ok, const Params &) {
         int dx = (int)(s.q.x - r.x), dy = (int)(s.q.y - r.y), dz = (int)(s.q.z - r.z);
