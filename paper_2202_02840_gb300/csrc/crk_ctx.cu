@@ -92,7 +92,7 @@ int crk_ensure_particles(crk_ctx *ctx, int n) {
     rc |= dalloc(ctx, &ctx->len_g, tiles);
     rc |= dalloc(ctx, &ctx->len_u, tiles);
     rc |= dalloc(ctx, &ctx->tbase, tiles);
-    rc |= dalloc(ctx, &ctx->frec, 10 * (size_t)cap);
+    rc |= dalloc(ctx, &ctx->frec, 8 * (size_t)cap);
     rc |= dalloc(ctx, &ctx->sfun, cap);
     rc |= dalloc(ctx, &ctx->sig, cap);
     rc |= dalloc(ctx, &ctx->sig2, 2 * (size_t)cap);   // two kicks' sums side by side

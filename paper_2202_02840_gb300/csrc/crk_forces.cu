@@ -22,7 +22,7 @@ namespace crk {
 struct FParams {
     float gm1, gamma;      // gamma - 1, gamma
     float inv_nh;          // 1 / n_h
-    float eps2;            // eps^2
+    float eps2n;           // (eps / n_h)^2
     float Cl, Cq;
     float eta_crit, inv_eta_fold;
     // comoving variables (Sec. 1.1): scale factor a, adot = da/dt; all 1 / 0 in a static box
@@ -31,21 +31,34 @@ struct FParams {
     float adot, adot_a;    // adot, adot / a
 };
 
-// Per-particle record of the pair-set passes: 160 bytes, five 32-byte sectors
-// (one 256-bit load each).  grad v enters the limiter only through the
-// quadratic form x . grad v . x, so its symmetric part is kept (6 numbers).
-struct __align__(32) FRec {
+// Per-particle record of the pair-set passes: 128 bytes, four 32-byte sectors
+// (one 256-bit load each).  The corrected kernel gradient of a particle with
+// separation x, eq:gRK, is affine in x up to two radial factors:
+//   grad W^R_g = t^6 (1 + 6 eta + 35/3 eta^2) (c_g + M_g . x) - 56/3 h^-2 t^5 (1 + 5 eta) (A' + B' . x) x_g,
+//   c_g = cW (dA_g + A B_g), M_ga = cW (dA_g B_a + A dB^a_g), A' = cW A, B' = cW A B, cW = 495/(32 pi h^3)
+// so the record holds c, M, A', B' (16 numbers, formed once per particle, each
+// rounded once) instead of A, B, dA, dB, cW, cG and their products per pair: four
+// gathers a pair instead of five and about a quarter fewer instructions.  P4 at
+// 128^3 clustered: 8.82 -> 7.72 ms, at 64^3 Sedov 1.03 -> 0.87 ms; it stays bound
+// by its gathers and the 12 warps an SM holds at 167 registers (16 warps at 128
+// registers with the record read at its use: 8.05 ms).  grad v enters the limiter only through the quadratic form
+// x . grad v . x, so its symmetric part is kept (6 numbers).  P and c_s follow
+// from rho and e = P / rho = (gamma - 1) u.
+//
+// In memory the four sectors of record j stand in the order c ^ (j & 3): 32
+// lanes that read sector c of 32 records spread over the four sector columns
+// of the L1 data banks (18 cycles a load; 32 when all read the same column).
+struct FRec {
     float4 w0;      // qx, qy, qz (fixed-point bits), 1/h
-    float4 w1;      // cW = 495/(32 pi h^3), cG = -1155/(4 pi h^5), h_hat = h/n_h, V
-    float4 w2;      // P, rho, c_s, A
-    float4 w3;      // vx, vy, vz, Bx
-    float4 w4;      // By, Bz, gAx, gAy
-    float4 w5;      // gAz, gB00, gB01, gB02
-    float4 w6;      // gB10, gB11, gB12, gB20
-    float4 w7;      // gB21, gB22, S_xx, S_yy
-    float4 w8;      // S_zz, S_xy, S_xz, S_yz   (S_ab = dv^a/dx^b + dv^b/dx^a for a != b)
-    float4 w9;      // unused (keeps records on 32-byte boundaries)
+    float4 w1;      // V, vx, vy, vz
+    float4 w2;      // c_x, c_y, c_z, A'
+    float4 w3;      // M_xx, M_yx, M_zx, B'_x     (coefficients of x)
+    float4 w4;      // M_xy, M_yy, M_zy, B'_y     (of y)
+    float4 w5;      // M_xz, M_yz, M_zz, B'_z     (of z)
+    float4 w6;      // S_xx, S_yy, S_zz, S_xy
+    float4 w7;      // S_xz, S_yz, rho, e   (S_ab = dv^a/dx^b + dv^b/dx^a for a != b)
 };
+constexpr int FREC_F4 = 8;
 
 __device__ __forceinline__ uint32_t fq(const FRec &r, int k) {
     return __float_as_uint(k == 0 ? r.w0.x : (k == 1 ? r.w0.y : r.w0.z));
@@ -62,142 +75,224 @@ struct FSrc {
     const GvRec *gv;
 };
 
-__device__ __forceinline__ FRec load_frec(int j, const FSrc &src, const FParams &fp) {
+// An unevaluated sum hi + lo of two floats, for the coefficients of a record:
+// each is rounded once, from products that carry about 45 bits.
+struct F2 {
+    float hi, lo;
+};
+__device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
+    const float p = __fmul_rn(a.hi, b.hi);
+    return F2{p, fmaf(a.hi, b.lo, fmaf(a.lo, b.hi, fmaf(a.hi, b.hi, -p)))};
+}
+__device__ __forceinline__ F2 f2_mul(F2 a, float b) {
+    const float p = __fmul_rn(a.hi, b);
+    return F2{p, fmaf(a.lo, b, fmaf(a.hi, b, -p))};
+}
+__device__ __forceinline__ float f2_sum(F2 a, F2 b) {   // TwoSum of the high parts
+    const float s = __fadd_rn(a.hi, b.hi), t = __fsub_rn(s, a.hi);
+    const float e = __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, t)), __fsub_rn(b.hi, t));
+    return s + (e + (a.lo + b.lo));
+}
+constexpr float KW_LO = (float)(KW_D - (double)KW);
+constexpr float KGW = (float)(-KG_D / KW_D);   // -56/3
+constexpr float KGW_LO = (float)(-KG_D / KW_D - (double)KGW);
+
+// -56/3 h^-2 as the passes form it from 1/h
+__device__ __forceinline__ float grad_factor(float ih) { return KGW * (ih * ih); }
+
+__device__ __forceinline__ FRec make_frec(int j, const FSrc &src, const FParams &fp) {
     FRec r;
     const uint4 q = src.q4[j];
-    const float h = src.hs[j], ih = 1.f / h, ih2 = ih * ih, ih3 = ih2 * ih;
+    const float h = src.hs[j], ih = 1.f / h;
     r.w0 = make_float4(__uint_as_float(q.x), __uint_as_float(q.y), __uint_as_float(q.z), ih);
-    float V = src.V[j];
-    float4 v = src.vel[j];
-    float rho = src.rho ? src.rho[j] : src.mass[j] / V;
-    float P = fp.gm1 * rho * v.w;
-    CorrRec c = src.corr[j];
-    GvRec g = src.gv[j];
+    const float V = src.V[j];
+    const float4 v = src.vel[j];
+    const float rho = src.rho ? src.rho[j] : src.mass[j] / V;
+    const CorrRec c = src.corr[j];
+    const GvRec g = src.gv[j];
+    const float B[3] = {c.c0.y, c.c0.z, c.c0.w}, dA[3] = {c.c1.x, c.c1.y, c.c1.z};
+    const float dB[9] = {c.c1.w, c.c2.x, c.c2.y, c.c2.z, c.c2.w, c.c3.x, c.c3.y, c.c3.z, c.c3.w};   // [a][g]
+    const F2 i1 = {ih, __fmul_rn(fmaf(-ih, h, 1.f), ih)}, i2 = f2_mul(i1, i1);
+    const F2 cW = f2_mul(F2{KW, KW_LO}, f2_mul(i2, i1)), cA = f2_mul(cW, c.c0.x);
+    // A', B' also carry the rounding of grad_factor: its product with them is
+    // cG A, cG A B to their own rounding
+    const float gf = grad_factor(ih);
+    const F2 g2 = f2_mul(F2{KGW, KGW_LO}, i2);
+    const float fix = ((g2.hi - gf) + g2.lo) / gf;
+    const F2 gA = F2{cA.hi, fmaf(cA.hi, fix, cA.lo)};
+    auto C = [&](int k) { return f2_sum(f2_mul(cW, dA[k]), f2_mul(cA, B[k])); };
+    auto M = [&](int k, int a) { return f2_sum(f2_mul(f2_mul(cW, dA[k]), B[a]), f2_mul(cA, dB[3 * a + k])); };
+    auto AB = [&](int a) { const F2 v = f2_mul(gA, B[a]); return v.hi + v.lo; };
+    r.w1 = make_float4(V, v.x, v.y, v.z);
+    r.w2 = make_float4(C(0), C(1), C(2), gA.hi + gA.lo);
+    r.w3 = make_float4(M(0, 0), M(1, 0), M(2, 0), AB(0));
+    r.w4 = make_float4(M(0, 1), M(1, 1), M(2, 1), AB(1));
+    r.w5 = make_float4(M(0, 2), M(1, 2), M(2, 2), AB(2));
     // grad v [a][b]: g0 = (00 01 02 10), g1 = (11 12 20 21), g2 = (22 ...)
-    r.w1 = make_float4(KW * ih3, -KG * ih3 * ih2, h * fp.inv_nh, V);
-    r.w2 = make_float4(P, rho, sqrtf(fmaxf(fp.gamma * P / rho, 0.f)), c.c0.x);
-    r.w3 = make_float4(v.x, v.y, v.z, c.c0.y);
-    r.w4 = make_float4(c.c0.z, c.c0.w, c.c1.x, c.c1.y);
-    r.w5 = make_float4(c.c1.z, c.c1.w, c.c2.x, c.c2.y);
-    r.w6 = make_float4(c.c2.z, c.c2.w, c.c3.x, c.c3.y);
-    r.w7 = make_float4(c.c3.z, c.c3.w, g.g0.x, g.g1.x);
-    r.w8 = make_float4(g.g2.x, g.g0.y + g.g0.w, g.g0.z + g.g1.z, g.g1.y + g.g1.w);
-    r.w9 = make_float4(0.f, 0.f, 0.f, 0.f);
+    r.w6 = make_float4(g.g0.x, g.g1.x, g.g2.x, g.g0.y + g.g0.w);
+    r.w7 = make_float4(g.g0.z + g.g1.z, g.g1.y + g.g1.w, rho, fp.gm1 * v.w);
     return r;
 }
 
-// eq:gRK for particle a with separation x (= x_a - x_b), kernel value W and
-// radial factor G (grad W = G x).
-__device__ __forceinline__ void grad_rk(const FRec &a, const float x[3], float W, float G, float out[3]) {
-    const float A = a.w2.w;
-    const float B[3] = {a.w3.w, a.w4.x, a.w4.y};
-    const float gA[3] = {a.w4.z, a.w4.w, a.w5.x};
-    const float gB[9] = {a.w5.y, a.w5.z, a.w5.w, a.w6.x, a.w6.y, a.w6.z, a.w6.w, a.w7.x, a.w7.y};
-    float sB = fmaf(B[0], x[0], fmaf(B[1], x[1], fmaf(B[2], x[2], 1.f)));
-    float sW = sB * W, AW = A * W, AsG = A * sB * G;
-#pragma unroll
-    for (int g = 0; g < 3; g++) {
-        float gBx = fmaf(gB[g], x[0], fmaf(gB[3 + g], x[1], gB[6 + g] * x[2]));
-        out[g] = fmaf(gA[g], sW, fmaf(AW, gBx + B[g], AsG * x[g]));
-    }
+// What only particle i's side needs, formed once per particle.
+struct FOwn {
+    float G;     // -56/3 h^-2
+    float P;     // pressure
+    float lc;    // C_l c_s
+    float k;     // 1 / (n_h h)
+};
+__device__ __forceinline__ float sqrt_approx(float v) {
+    float r;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
+}
+
+__device__ __forceinline__ FOwn own_terms(const FRec &a, const FParams &fp) {
+    FOwn o;
+    o.G = grad_factor(a.w0.w);
+    o.P = __fmul_rn(a.w7.z, a.w7.w);
+    o.lc = fp.Cl * sqrt_approx(fmaxf(fp.gamma * a.w7.w, 0.f));
+    o.k = fp.inv_nh * a.w0.w;
+    return o;
+}
+
+// Radial factors of particle a at distance r: W = t^6 (1 + 6 eta + 35/3 eta^2)
+// and G = -56/3 h^-2 t^5 (1 + 5 eta).  Outside gather(a), r >= h_a and t vanishes
+// (the rounding of eta leaves at most t ~ 1e-7, t^5 ~ 1e-35 of the kernel).
+__device__ __forceinline__ void kern(float eta, float g, float &W, float &G) {
+    const float t = __saturatef(1.f - eta);
+    const float t2 = t * t, t5 = t2 * t2 * t;
+    W = t5 * t * fmaf(eta, fmaf(eta, K35_3, 6.f), 1.f);
+    G = g * (fmaf(5.f, eta, 1.f) * t5);
+}
+
+// c + s M x and A' + s B' x (s = +1: separation x, s = -1: -x)
+template <bool NEG>
+__device__ __forceinline__ void affine(const FRec &a, const float x[3], float T[3], float &As) {
+    auto f = [](float m, float v, float c) { return NEG ? fmaf(-m, v, c) : fmaf(m, v, c); };
+    T[0] = f(a.w3.x, x[0], f(a.w4.x, x[1], f(a.w5.x, x[2], a.w2.x)));
+    T[1] = f(a.w3.y, x[0], f(a.w4.y, x[1], f(a.w5.y, x[2], a.w2.y)));
+    T[2] = f(a.w3.z, x[0], f(a.w4.z, x[1], f(a.w5.z, x[2], a.w2.z)));
+    As = f(a.w3.w, x[0], f(a.w4.w, x[1], f(a.w5.w, x[2], a.w2.w)));
 }
 
 // x . grad v . x from the symmetric part and the products xx = (x^2, y^2, z^2, xy, xz, yz)
 __device__ __forceinline__ float gv_quad(const FRec &a, const float xx[6]) {
-    return fmaf(a.w7.z, xx[0], fmaf(a.w7.w, xx[1], fmaf(a.w8.x, xx[2],
-           fmaf(a.w8.y, xx[3], fmaf(a.w8.z, xx[4], a.w8.w * xx[5])))));
-}
-
-// Kernel of particle a.  Outside gather(a), r >= h_a and t vanishes (the
-// rounding of eta leaves at most t ~ 1e-7, t^5 ~ 1e-35 of the kernel).
-__device__ __forceinline__ void kern(const FRec &a, float r, float &W, float &G) {
-    float eta = r * a.w0.w;
-    float t = __saturatef(1.f - eta);
-    float t2 = t * t, t5 = t2 * t2 * t;
-    W = a.w1.x * t5 * t * fmaf(eta, fmaf(eta, K35_3, 6.f), 1.f);
-    G = a.w1.y * fmaf(5.f, eta, 1.f) * t5;
+    return fmaf(a.w6.x, xx[0], fmaf(a.w6.y, xx[1], fmaf(a.w6.z, xx[2],
+           fmaf(a.w6.w, xx[3], fmaf(a.w7.x, xx[4], a.w7.y * xx[5])))));
 }
 
 struct PairOut {
     float F[3];    // m_a dp_ab/dt = a^2/2 V_a V_b (P~_a + P~_b)(grad W^R_ba - grad W^R_ab)
-    float D[3];    // grad W^R_ba - grad W^R_ab
-    float Pt_b;    // P_b + Q_b of this pair
-    float Q_a;     // Q_a of this pair
-    float Q_b;     // Q_b of this pair
+    float wd;      // (v_b - v_a) . (grad W^R_ba - grad W^R_ab)
+    float hvv;     // V_a V_b / 2
+    float Pt_a, Pt_b;   // P~ = P + Q of this pair
+    float Q_a, Q_b;     // Q of this pair
+    float vs;      // signal velocity of the pair (or less than 0)
 };
 
-// One pair of the pair set seen from particle a; x = x_a - x_b.
-__device__ __forceinline__ void pair_force(const FRec &a, const FRec &b, const float x[3], float r2,
-                                           float r, const FParams &fp, PairOut &o) {
+// One pair of the pair set seen from particle a.  Every operation on (a, b) has
+// its counterpart on (b, a): F_ba = -F_ab bitwise.  STATIC: a = 1, adot = 0 (the
+// same values without the factors of one and the terms of zero).
+template <bool STATIC>
+__device__ __forceinline__ void pair_force(const FRec &a, const FOwn &oa, const FRec &b, const FParams &fp,
+                                           PairOut &o) {
+    const Sep d = separation((int)(fq(a, 0) - fq(b, 0)), (int)(fq(a, 1) - fq(b, 1)), (int)(fq(a, 2) - fq(b, 2)));
+    const float x[3] = {d.x, d.y, d.z};
+    const float ea = d.r * a.w0.w, eb = d.r * b.w0.w;
     float Wa, Ga, Wb, Gb;
-    kern(a, r, Wa, Ga);
-    kern(b, r, Wb, Gb);
-    const float xn[3] = {-x[0], -x[1], -x[2]};
-    float gRa[3], gRb[3];
-    grad_rk(a, x, Wa, Ga, gRa);
-    grad_rk(b, xn, Wb, Gb, gRb);
+    kern(ea, oa.G, Wa, Ga);
+    kern(eb, grad_factor(b.w0.w), Wb, Gb);
+    float Ta[3], Tb[3], Aa, Ab;
+    affine<false>(a, x, Ta, Aa);
+    affine<true>(b, x, Tb, Ab);
+    // grad W^R_ba - grad W^R_ab; the products are rounded before the difference
+    const float s = __fmul_rn(Aa, Ga) + __fmul_rn(Ab, Gb);
+    float D[3];
 #pragma unroll
-    for (int g = 0; g < 3; g++) o.D[g] = gRb[g] - gRa[g];
+    for (int g = 0; g < 3; g++) D[g] = fmaf(-s, x[g], __fmul_rn(Wb, Tb[g]) - __fmul_rn(Wa, Ta[g]));
 
     // limiter, eq:phi .. eq:phiad (x . grad v_a . x and x . grad v_b . x)
     const float xx[6] = {x[0] * x[0], x[1] * x[1], x[2] * x[2], x[0] * x[1], x[0] * x[2], x[1] * x[2]};
-    float qa = gv_quad(a, xx);
-    float qb = gv_quad(b, xx);
-    float qs = qa + qb;
+    const float qa = gv_quad(a, xx), qb = gv_quad(b, xx);
+    const float qs = qa + qb;
     float phi = 0.f;
     if (qs != 0.f) {
-        float is = FDIV(1.f, qs);
-        phi = fminf(fmaxf(4.f * (qa * is) * (qb * is), 0.f), 1.f);
+        const float is = FDIV(1.f, qs);
+        phi = __saturatef(4.f * (qa * is) * (qb * is));
     }
-    float eta = fminf(r * a.w0.w, r * b.w0.w);
+    const float eta = fminf(ea, eb);
     if (eta < fp.eta_crit) {
-        float e = (eta - fp.eta_crit) * fp.inv_eta_fold;
+        const float e = (eta - fp.eta_crit) * fp.inv_eta_fold;
         phi *= __expf(-e * e);
     }
     // projected proper velocity difference along x, eq:hatvi (the state holds
     // p = a v; the projection acts on the peculiar part only):
     // u_ab . x = (p_a - p_b) . x / a - phi/2 (x . grad v_a . x + x . grad v_b . x) + adot r^2
-    float vx = fmaf(a.w3.x - b.w3.x, x[0], fmaf(a.w3.y - b.w3.y, x[1], (a.w3.z - b.w3.z) * x[2]));
-    float ux = fmaf(fp.adot, r2, fmaf(-0.5f * phi, qs, vx * fp.inv_a));
-    // eq:mu (h^/a), eq:visc
-    float hha = a.w1.z, hhb = b.w1.z;
-    float uxa = ux * fp.inv_a;
-    float mua = fminf(FDIV(hha * uxa, fmaf(hha * hha, fp.eps2, r2)), 0.f);
-    float mub = fminf(FDIV(hhb * uxa, fmaf(hhb * hhb, fp.eps2, r2)), 0.f);
-    float Qa = a.w2.y * mua * fmaf(fp.Cq, mua, -fp.Cl * a.w2.z);
-    float Qb = b.w2.y * mub * fmaf(fp.Cq, mub, -fp.Cl * b.w2.z);
-    float Pta = a.w2.x + Qa, Ptb = b.w2.x + Qb;
-    float cF = fp.half_a2 * (a.w1.w * b.w1.w) * (Pta + Ptb);
+    const float dv[3] = {b.w1.y - a.w1.y, b.w1.z - a.w1.z, b.w1.w - a.w1.w};
+    const float vx = -fmaf(dv[0], x[0], fmaf(dv[1], x[1], dv[2] * x[2]));
+    float ux, uxa, vr;
+    if (STATIC) {
+        ux = fmaf(-0.5f * phi, qs, vx);
+        uxa = ux;
+        vr = vx;
+    } else {
+        ux = fmaf(fp.adot, d.r2, fmaf(-0.5f * phi, qs, vx * fp.inv_a));
+        uxa = ux * fp.inv_a;
+        // (dx_a/dt - dx_b/dt + (adot/a) x).x with dx/dt = p / a^2
+        vr = fmaf(fp.adot_a, d.r2, vx * fp.inv_a2);
+    }
+    // eq:mu (h^/a), eq:visc: h^ uxa / (r^2 + eps^2 h^^2), both sides over h^2
+    const float kb = fp.inv_nh * b.w0.w;
+    const float mua = fminf(FDIV(oa.k * uxa, fmaf(ea, ea, fp.eps2n)), 0.f);
+    const float mub = fminf(FDIV(kb * uxa, fmaf(eb, eb, fp.eps2n)), 0.f);
+    const float lcb = fp.Cl * sqrt_approx(fmaxf(fp.gamma * b.w7.w, 0.f));
+    o.Q_a = __fmul_rn(a.w7.z * mua, fmaf(fp.Cq, mua, -oa.lc));
+    o.Q_b = __fmul_rn(b.w7.z * mub, fmaf(fp.Cq, mub, -lcb));
+    o.Pt_a = oa.P + o.Q_a;
+    o.Pt_b = __fmul_rn(b.w7.z, b.w7.w) + o.Q_b;
+    const float vv = a.w1.x * b.w1.x;
+    o.hvv = 0.5f * vv;
+    const float cF = (STATIC ? o.hvv : fp.half_a2 * vv) * (o.Pt_a + o.Pt_b);
 #pragma unroll
-    for (int g = 0; g < 3; g++) o.F[g] = cF * o.D[g];
-    o.Pt_b = Ptb;
-    o.Q_a = Qa;
-    o.Q_b = Qb;
+    for (int g = 0; g < 3; g++) o.F[g] = cF * D[g];
+    o.wd = fmaf(dv[0], D[0], fmaf(dv[1], D[1], dv[2] * D[2]));
+    // -vr / r; coincident particles (0 times infinity) give NaN, which fmaxf drops
+    o.vs = FDIV(-vr, d.r);
 }
 
 // Per-particle records of the pair-set passes, packed once per evaluation.
-__global__ void k_pack_frec(int n, FSrc src, FParams fp, FRec *__restrict__ out, float *__restrict__ sfun) {
+__global__ void k_pack_frec(int n, FSrc src, FParams fp, float4 *__restrict__ out, float *__restrict__ sfun) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
-    FRec r = load_frec(i, src, fp);
-    out[i] = r;
-    sfun[i] = r.w2.x / powf(r.w2.y, fp.gamma);       // s = P / rho^gamma (eq:fij)
+    const FRec r = make_frec(i, src, fp);
+    float4 *p = out + (size_t)i * FREC_F4;
+    const int s = 2 * (i & 3);
+    p[s] = r.w0;
+    p[s + 1] = r.w1;
+    p[s ^ 2] = r.w2;
+    p[(s ^ 2) + 1] = r.w3;
+    p[s ^ 4] = r.w4;
+    p[(s ^ 4) + 1] = r.w5;
+    p[s ^ 6] = r.w6;
+    p[(s ^ 6) + 1] = r.w7;
+    const float rho = r.w7.z;
+    sfun[i] = fp.gm1 * rho * src.vel[i].w / powf(rho, fp.gamma);   // s = P / rho^gamma (eq:fij)
 }
 
-__device__ __forceinline__ FRec ldg_frec(const FRec *p) {
-    const float4 *q = reinterpret_cast<const float4 *>(p);
+__device__ __forceinline__ FRec ldg_frec(const float4 *base, uint32_t j) {
+    const uintptr_t q = reinterpret_cast<uintptr_t>(base + (size_t)j * FREC_F4) + 32u * (j & 3u);
     FRec r;
-    ldg_v8(q, r.w0, r.w1);
-    ldg_v8(q + 2, r.w2, r.w3);
-    ldg_v8(q + 4, r.w4, r.w5);
-    ldg_v8(q + 6, r.w6, r.w7);
-    ldg_v8(q + 8, r.w8, r.w9);
+    ldg_v8(reinterpret_cast<const float4 *>(q), r.w0, r.w1);
+    ldg_v8(reinterpret_cast<const float4 *>(q ^ 32u), r.w2, r.w3);
+    ldg_v8(reinterpret_cast<const float4 *>(q ^ 64u), r.w4, r.w5);
+    ldg_v8(reinterpret_cast<const float4 *>(q ^ 96u), r.w6, r.w7);
     return r;
 }
 
 // ================================================================= P4 forces
 
-template <bool COMP>
+template <bool COMP, bool STATIC>
 struct P4 {
     static constexpr bool GATHER = false;
     static constexpr int UNROLL = 1;
@@ -207,7 +302,7 @@ struct P4 {
     static constexpr bool TMA = true;   // has the TMA-fed variant
     using Rec = FRec;
     struct Params {
-        const FRec *frec;
+        const float4 *frec;
         const float *mass;
         FParams fp;
         float4 *acc;   // (ax, ay, az, dudt)
@@ -221,19 +316,17 @@ struct P4 {
     };
     struct IState : Sums {
         FRec me;
-        float m;
+        FOwn own;
     };
     __device__ static Sums sums(const IState &s) { return s; }
     __device__ static void init(IState &s, int i, bool valid, const Params &p) {
         if (valid) {
-            s.me = p.frec[i];
-            s.m = p.mass[i];
+            s.me = ldg_frec(p.frec, (uint32_t)i);
         } else {
             s.me = FRec{};
             s.me.w0.w = 1.f;
-            s.me.w2.y = 1.f;
-            s.m = 1.f;
         }
+        s.own = own_terms(s.me, p.fp);
         s.vsig = 0.f;
         s.qmax = 0.f;
     }
@@ -248,26 +341,19 @@ struct P4 {
         s.vsig = fmaxf(s.vsig, o.vsig);
         s.qmax = fmaxf(s.qmax, o.qmax);
     }
-    __device__ static Rec load(uint32_t j, size_t, const Params &p) { return ldg_frec(p.frec + j); }
+    __device__ static Rec load(uint32_t j, size_t, const Params &p) { return ldg_frec(p.frec, j); }
     __device__ static void pair(IState &s, const Rec &r, uint32_t j, size_t pos, bool, const Params &p) {
-        int dx = (int)(fq(s.me, 0) - fq(r, 0)), dy = (int)(fq(s.me, 1) - fq(r, 1)), dz = (int)(fq(s.me, 2) - fq(r, 2));
-        Sep d = separation(dx, dy, dz);
-        float x[3] = {d.x, d.y, d.z};
         PairOut o;
-        pair_force(s.me, r, x, d.r2, d.r, p.fp, o);
+        pair_force<STATIC>(s.me, s.own, r, p.fp, o);
         p.Fst[pos] = make_float4(o.F[0], o.F[1], o.F[2], __uint_as_float(j));   // F_ij, j
-        float dv[3] = {r.w3.x - s.me.w3.x, r.w3.y - s.me.w3.y, r.w3.z - s.me.w3.z};
 #pragma unroll
         for (int g = 0; g < 3; g++) s.F[g].add(o.F[g]);
-        float wd = fmaf(dv[0], o.D[0], fmaf(dv[1], o.D[1], dv[2] * o.D[2]));
-        s.du.add(0.5f * (s.me.w1.w * r.w1.w) * o.Pt_b * wd);
-        // (dx_i/dt - dx_j/dt + (adot/a) x_ij).x_ij with dx/dt = p / a^2
-        float vx = fmaf(p.fp.adot_a, d.r2, -fmaf(dv[0], x[0], fmaf(dv[1], x[1], dv[2] * x[2])) * p.fp.inv_a2);
-        if (vx < 0.f && d.r > 0.f) s.vsig = fmaxf(s.vsig, FDIV(-vx, d.r));
+        s.du.add(o.hvv * o.Pt_b * o.wd);
+        s.vsig = fmaxf(s.vsig, o.vs);
         s.qmax = fmaxf(s.qmax, o.Q_a);
     }
     __device__ static void finish(IState &s, int i, const Params &p) {
-        float im = 1.f / s.m;
+        float im = 1.f / p.mass[i];
         // dp/dt, and du/dt of eq:eng: 1/(2a^2) V V P~ (dx_j/dt - dx_i/dt).D with dx/dt = p / a^2
         p.acc[i] = make_float4(s.F[0].value() * im, s.F[1].value() * im, s.F[2].value() * im,
                                s.du.value() * im * p.fp.inv_a4);
@@ -287,8 +373,8 @@ struct P4 {
 // bitwise the results of the other variants.  Every wait on the mbarrier is
 // bounded; a wait that runs out sets CNT_TMA_ERR, waits (bounded again) for
 // the copies still in flight, and the warp returns.
-constexpr int TMA_RF = 36;                     // floats of a record P4 reads (w0 .. w8)
-constexpr int TMA_SLOT = 640;                  // bytes per gather4: 4 rows of 144 B, 128-byte slots
+constexpr int TMA_RF = 4 * FREC_F4;            // floats of a record
+constexpr int TMA_SLOT = 4 * TMA_RF * 4;       // bytes per gather4: 4 rows
 constexpr int TMA_STAGE = 8 * TMA_SLOT;        // one record per lane
 constexpr uint32_t TMA_TX = 32u * TMA_RF * 4u; // bytes a stage receives
 constexpr uint32_t TMA_SPIN = 1u << 16;        // try_wait rounds before a wait is given up
@@ -314,7 +400,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, uint32_
     return ok != 0;
 }
 
-// rows r0..r3 of the record map (x = 0) into 4 x 144 contiguous bytes at dst
+// rows r0..r3 of the record map (x = 0) into 4 x 128 contiguous bytes at dst
 __device__ __forceinline__ void tma_gather4(uint32_t dst, const CUtensorMap *map, int4 r, uint32_t bar) {
     asm volatile(
         "cp.async.bulk.tensor.2d.shared::cta.global.tile::gather4.mbarrier::complete_tx::bytes"
@@ -323,8 +409,8 @@ __device__ __forceinline__ void tma_gather4(uint32_t dst, const CUtensorMap *map
         : "memory");
 }
 
-template <bool COMP>
-__global__ void __launch_bounds__(TMA_WARPS * 32) k_p4_tma(ListGeom g, typename P4<COMP>::Params prm,
+template <bool COMP, bool STATIC>
+__global__ void __launch_bounds__(TMA_WARPS * 32) k_p4_tma(ListGeom g, typename P4<COMP, STATIC>::Params prm,
                                                           const __grid_constant__ CUtensorMap map,
                                                           unsigned long long *err) {
     __shared__ alignas(128) unsigned char stg[TMA_WARPS][2][TMA_STAGE];
@@ -340,7 +426,7 @@ __global__ void __launch_bounds__(TMA_WARPS * 32) k_p4_tma(ListGeom g, typename 
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncwarp();
-    using P = P4<COMP>;
+    using P = P4<COMP, STATIC>;
     const int i = tile * TILE + lane;
     const bool valid = i < g.n;
     typename P::IState st;
@@ -386,17 +472,16 @@ __global__ void __launch_bounds__(TMA_WARPS * 32) k_p4_tma(ListGeom g, typename 
         ph ^= 1u << s;
         if (k < my) {
             const float4 *q = reinterpret_cast<const float4 *>(mine + s * TMA_STAGE);
+            const int o = 2 * (int)(e & 3u);   // sector order of record e
             FRec r;
-            r.w0 = q[0];
-            r.w1 = q[1];
-            r.w2 = q[2];
-            r.w3 = q[3];
-            r.w4 = q[4];
-            r.w5 = q[5];
-            r.w6 = q[6];
-            r.w7 = q[7];
-            r.w8 = q[8];
-            r.w9 = make_float4(0.f, 0.f, 0.f, 0.f);
+            r.w0 = q[o];
+            r.w1 = q[o + 1];
+            r.w2 = q[o ^ 2];
+            r.w3 = q[(o ^ 2) + 1];
+            r.w4 = q[o ^ 4];
+            r.w5 = q[(o ^ 4) + 1];
+            r.w6 = q[o ^ 6];
+            r.w7 = q[(o ^ 6) + 1];
             P::pair(st, r, e, fb + (size_t)k * 32, true, prm);
         }
         __syncwarp();
@@ -404,8 +489,8 @@ __global__ void __launch_bounds__(TMA_WARPS * 32) k_p4_tma(ListGeom g, typename 
     if (valid) P::finish(st, i, prm);
 }
 
-// The record map: a 2-D tensor of n rows of TMA_RF floats with a row pitch of
-// one record (160 B); a box is one row of TMA_RF floats (gather4 takes four).
+// The record map: a 2-D tensor of n rows of TMA_RF floats; a box is one row
+// (gather4 takes four).
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
                                   const cuuint64_t *, const cuuint32_t *, const cuuint32_t *, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
@@ -422,7 +507,7 @@ static int frec_tensor_map(crk_ctx *ctx) {
         encode = reinterpret_cast<EncodeTiledFn>(fn);
     }
     const cuuint64_t dims[2] = {(cuuint64_t)TMA_RF, (cuuint64_t)ctx->n};
-    const cuuint64_t strides[1] = {(cuuint64_t)sizeof(FRec)};
+    const cuuint64_t strides[1] = {(cuuint64_t)(sizeof(float) * TMA_RF)};
     const cuuint32_t box[2] = {(cuuint32_t)TMA_RF, 1u};
     const cuuint32_t estr[2] = {1u, 1u};
     CUresult r = encode(&ctx->frec_map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, (void *)ctx->frec, dims, strides, box, estr,
@@ -434,11 +519,11 @@ static int frec_tensor_map(crk_ctx *ctx) {
     return CRK_OK;
 }
 
-template <bool COMP>
-int P4<COMP>::launch_tma(crk_ctx *ctx, const ListGeom &g, const Params &prm, cudaStream_t s) {
+template <bool COMP, bool STATIC>
+int P4<COMP, STATIC>::launch_tma(crk_ctx *ctx, const ListGeom &g, const Params &prm, cudaStream_t s) {
     int rc = frec_tensor_map(ctx);
     if (rc) return rc;
-    k_p4_tma<COMP><<<grid_for(g.ntiles, TMA_WARPS), TMA_WARPS * 32, 0, s>>>(g, prm, ctx->frec_map,
+    k_p4_tma<COMP, STATIC><<<grid_for(g.ntiles, TMA_WARPS), TMA_WARPS * 32, 0, s>>>(g, prm, ctx->frec_map,
                                                                           ctx->counters + CNT_TMA_ERR);
     return CRK_OK;
 }
@@ -799,14 +884,14 @@ __global__ void __launch_bounds__(PO_WARPS * 32) k_po(POGeom g, typename P::Para
 // j's share -F_ij, 1/2 V_j V_i P~_i (dx_i/dt - dx_j/dt).(grad W^R_ij - grad W^R_ji),
 // Q_j of the pair and the pair's signal velocity, each bitwise the term the
 // directed form evaluates from j's side.
-template <bool COMP>
+template <bool COMP, bool STATIC>
 struct P4PO {
     static constexpr int NS = 6;   // F (3), du, Q, vsig
     using Ent = uint32_t;
     using Rec = FRec;
-    using IState = typename P4<COMP>::IState;
+    using IState = typename P4<COMP, STATIC>::IState;
     struct Params {
-        const FRec *frec;
+        const float4 *frec;
         const float *mass;
         FParams fp;
         float4 *acc;     // own sums (F, du) here; the row pass completes them
@@ -816,37 +901,30 @@ struct P4PO {
         float2 *rowB;    // (Q, vsig)
     };
     __device__ static void init(IState &s, int i, bool valid, const Params &p) {
-        typename P4<COMP>::Params q{p.frec, p.mass, p.fp, p.acc, p.vq, p.Fst};
-        P4<COMP>::init(s, i, valid, q);
+        typename P4<COMP, STATIC>::Params q{p.frec, p.mass, p.fp, p.acc, p.vq, p.Fst};
+        P4<COMP, STATIC>::init(s, i, valid, q);
     }
     __device__ static Ent fetch(const uint32_t *ent, size_t, int lane, int mg, int kcap, int k, const Params &) {
         const int row = entry_row(k, mg);
         return __ldg(ent + block_at(pair_block(row / LB, list_blocks(mg), kcap), lane) + row % LB);
     }
     __device__ static uint32_t jof(const Ent &e) { return e; }
-    __device__ static Rec load(const Ent &e, const Params &p) { return ldg_frec(p.frec + e); }
+    __device__ static Rec load(const Ent &e, const Params &p) { return ldg_frec(p.frec, e); }
     __device__ static void pair(IState &s, const Rec &r, const Ent &e, size_t pos, const Params &p,
                                 float sh[NS]) {
-        int dx = (int)(fq(s.me, 0) - fq(r, 0)), dy = (int)(fq(s.me, 1) - fq(r, 1)), dz = (int)(fq(s.me, 2) - fq(r, 2));
-        Sep d = separation(dx, dy, dz);
-        float x[3] = {d.x, d.y, d.z};
         PairOut o;
-        pair_force(s.me, r, x, d.r2, d.r, p.fp, o);
+        pair_force<STATIC>(s.me, s.own, r, p.fp, o);
         p.Fst[pos] = make_float4(o.F[0], o.F[1], o.F[2], __uint_as_float(e));   // F_ij, j
-        float dv[3] = {r.w3.x - s.me.w3.x, r.w3.y - s.me.w3.y, r.w3.z - s.me.w3.z};
 #pragma unroll
         for (int g = 0; g < 3; g++) s.F[g].add(o.F[g]);
-        float wd = fmaf(dv[0], o.D[0], fmaf(dv[1], o.D[1], dv[2] * o.D[2]));
-        const float hvv = 0.5f * (s.me.w1.w * r.w1.w);
-        s.du.add(hvv * o.Pt_b * wd);
-        float vx = fmaf(p.fp.adot_a, d.r2, -fmaf(dv[0], x[0], fmaf(dv[1], x[1], dv[2] * x[2])) * p.fp.inv_a2);
-        const float vs = (vx < 0.f && d.r > 0.f) ? FDIV(-vx, d.r) : 0.f;
+        s.du.add(o.hvv * o.Pt_b * o.wd);
+        const float vs = fmaxf(0.f, o.vs);
         s.vsig = fmaxf(s.vsig, vs);
         s.qmax = fmaxf(s.qmax, o.Q_a);
         sh[0] = -o.F[0];
         sh[1] = -o.F[1];
         sh[2] = -o.F[2];
-        sh[3] = hvv * (s.me.w2.x + o.Q_a) * wd;
+        sh[3] = o.hvv * o.Pt_a * o.wd;
         sh[4] = o.Q_b;
         sh[5] = vs;
     }
@@ -1004,7 +1082,7 @@ static FParams fparams(const crk_params &c) {
     f.gamma = (float)c.gamma;
     f.gm1 = (float)(c.gamma - 1.0);
     f.inv_nh = (float)(1.0 / c.n_h);
-    f.eps2 = (float)(c.eps * c.eps);
+    f.eps2n = (float)(c.eps * c.eps / (c.n_h * c.n_h));
     f.Cl = (float)c.C_l;
     f.Cq = (float)c.C_q;
     f.eta_crit = (float)c.eta_crit;
@@ -1029,18 +1107,18 @@ __global__ void k_sig(int n, const float4 *__restrict__ vb, const float4 *__rest
 
 // P4 over the whole pair set in the pair-once form: the reverse index of the
 // tile lists, the pass, and the rows pass that completes every particle's sums.
-template <bool COMP>
-static int run_forces_po(crk_ctx *ctx, const FRec *fr, const FParams &fp, cudaStream_t s) {
+template <bool COMP, bool STATIC>
+static int run_forces_po(crk_ctx *ctx, const float4 *fr, const FParams &fp, cudaStream_t s) {
     if (!ctx->lists_valid) return crk_set_error(ctx, CRK_ESTATE, "P4 forces: neighbour lists are not built");
     int rc = crk_ensure_pair_once(ctx);
     if (rc) return rc;
-    typename P4PO<COMP>::Params p{fr, ctx->mass, fp, ctx->acc, ctx->vq, ctx->Fst, ctx->po_rowA, ctx->po_rowB};
+    typename P4PO<COMP, STATIC>::Params p{fr, ctx->mass, fp, ctx->acc, ctx->vq, ctx->Fst, ctx->po_rowA, ctx->po_rowB};
     prof_begin(ctx, PROF_P4, s);
     k_po_low<<<grid_for(ctx->n, 256), 256, 0, s>>>(ctx->n, ctx->kcap, ctx->cnt_g, ctx->cnt_u, ctx->ent, ctx->lowc);
     k_po_rev<<<grid_for(ctx->ntiles, 8), 256, 0, s>>>(ctx->ntiles, ctx->uofs, ctx->ulist, ctx->po_rev,
                                                        ctx->po_self, ctx->po_tofs, ctx->po_tlist,
                                                        ctx->counters + CNT_PO_MISS);
-    k_po<P4PO<COMP>><<<grid_for(ctx->ntiles, PO_WARPS), PO_WARPS * 32, 0, s>>>(po_geom(ctx), p);
+    k_po<P4PO<COMP, STATIC>><<<grid_for(ctx->ntiles, PO_WARPS), PO_WARPS * 32, 0, s>>>(po_geom(ctx), p);
     k_p4po_rows<COMP><<<grid_for(ctx->n, 256), 256, 0, s>>>(ctx->n, ctx->po_tofs, ctx->po_self, ctx->po_rowA,
                                                             ctx->po_rowB, ctx->mass, fp, ctx->acc, ctx->vq);
     ctx->launches += 4;
@@ -1074,6 +1152,14 @@ static int p5_form(crk_ctx *ctx, bool *po) {
     return CRK_OK;
 }
 
+template <bool COMP, bool STATIC>
+static int run_p4(crk_ctx *ctx, const FParams &fp, cudaStream_t s) {
+    if (!ctx->act && ctx->p.pair_form == 1) return run_forces_po<COMP, STATIC>(ctx, ctx->frec, fp, s);
+    ctx->fst_po = 0;
+    typename P4<COMP, STATIC>::Params p{ctx->frec, ctx->mass, fp, ctx->acc, ctx->vq, ctx->Fst};
+    return launch_lpass<P4<COMP, STATIC>, 1>(ctx, PROF_P4, p, s, "P4 forces");
+}
+
 int run_forces(crk_ctx *ctx, cudaStream_t s) {
     if (ctx->n == 0) return CRK_OK;
     FParams fp = fparams(ctx->p);
@@ -1083,20 +1169,12 @@ int run_forces(crk_ctx *ctx, cudaStream_t s) {
     }
     FSrc src{ctx->q4, ctx->hs, ctx->p.density ? ctx->rho : nullptr, ctx->V, ctx->vel, ctx->mass, ctx->corr,
              ctx->gv};
-    k_pack_frec<<<grid_for(ctx->n, 256), 256, 0, s>>>(ctx->n, src, fp, reinterpret_cast<FRec *>(ctx->frec),
-                                                     ctx->sfun);
+    k_pack_frec<<<grid_for(ctx->n, 256), 256, 0, s>>>(ctx->n, src, fp, ctx->frec, ctx->sfun);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "pack pair records");
-    const FRec *fr = reinterpret_cast<const FRec *>(ctx->frec);
-    if (!ctx->act && ctx->p.pair_form == 1)
-        return ctx->p.precision >= 1 ? run_forces_po<true>(ctx, fr, fp, s) : run_forces_po<false>(ctx, fr, fp, s);
-    ctx->fst_po = 0;
-    if (ctx->p.precision >= 1) {
-        typename P4<true>::Params p{fr, ctx->mass, fp, ctx->acc, ctx->vq, ctx->Fst};
-        return launch_lpass<P4<true>, 1>(ctx, PROF_P4, p, s, "P4 forces");
-    }
-    typename P4<false>::Params p{fr, ctx->mass, fp, ctx->acc, ctx->vq, ctx->Fst};
-    return launch_lpass<P4<false>, 1>(ctx, PROF_P4, p, s, "P4 forces");
+    const bool comp = ctx->p.precision >= 1, still = ctx->p.a == 1.0 && ctx->p.adot == 0.0;
+    if (comp) return still ? run_p4<true, true>(ctx, fp, s) : run_p4<true, false>(ctx, fp, s);
+    return still ? run_p4<false, true>(ctx, fp, s) : run_p4<false, false>(ctx, fp, s);
 }
 
 // P5 for the kick vb -> va (sorted float4 arrays), with the F_ij of the last P4;

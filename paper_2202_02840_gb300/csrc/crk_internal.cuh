@@ -135,8 +135,8 @@ struct crk_ctx {
     int kcap = 384;                  // list columns per particle
     int volumes_only = 0;            // walk without writing lists (no list buffer)
     int lists_valid = 0;
-    float4 *frec = nullptr;          // packed pair-set records, 10 float4 (160 B) per particle
-    CUtensorMap frec_map;            // TMA view of frec: rows of its first 36 floats (P4's TMA variant)
+    float4 *frec = nullptr;          // packed pair-set records, 8 float4 (128 B) per particle
+    CUtensorMap frec_map;            // TMA view of frec: rows of 32 floats (P4's TMA variant)
     const void *frec_map_base = nullptr;
     int frec_map_rows = -1;
     float *sfun = nullptr;           // specific entropy of the evaluation state
