@@ -50,68 +50,122 @@ __global__ void k_keys(int n, const float4 *__restrict__ pos, uint32_t *__restri
 
 // ------------------------------------------------------------------ radix sort
 
+// Stable LSD sort.  30-bit keys take three passes of 10 bits (four of 8 above
+// RS_WIDE_MAX keys, where the 10-bit histograms would outgrow the scan), 16-bit
+// keys two of 8.  Up to RS_FUSED blocks every block of a scatter forms its own
+// offsets from the block histograms, so a pass is two launches; with more the
+// histograms are scanned in between.  A small sort is all latency: its blocks
+// take fewer keys (64 to 512 a warp), so that more warps share the serial
+// ranking.  4096 keys: 147 us in 12 launches with four 8-bit passes over 4096-key
+// blocks, 33 us in 6 now; 262144 keys 196 us in 20, 118 us in 6.
 constexpr int RS_WARPS = 8;
-constexpr int RS_PER_WARP = 512;
-constexpr int RS_ITEMS = RS_WARPS * RS_PER_WARP;   // keys per block
+constexpr int RS_FUSED = 64;
+constexpr int RS_WIDE_MAX = 32 << 20;
 
+// keys per warp of an n-key sort
+static int rs_per_warp(int n) { return n <= 16384 ? 64 : (n <= 32768 ? 128 : (n <= 65536 ? 256 : 512)); }
+
+// Block histograms of one digit: hist[block][digit] (fused) or hist[digit][block].
+template <int BITS>
 __global__ void __launch_bounds__(256) k_rs_hist(int n, const uint32_t *__restrict__ key, int shift,
-                                                 uint32_t *__restrict__ hist, int nblocks) {
-    __shared__ uint32_t cnt[256];
-    cnt[threadIdx.x] = 0;
+                                                 uint32_t *__restrict__ hist, int nblocks, int items, bool fused) {
+    constexpr int BINS = 1 << BITS;
+    __shared__ uint32_t cnt[BINS];
+    for (int d = threadIdx.x; d < BINS; d += 256) cnt[d] = 0;
     __syncthreads();
-    int base = blockIdx.x * RS_ITEMS;
-    for (int k = threadIdx.x; k < RS_ITEMS; k += 256) {
-        int i = base + k;
-        if (i < n) atomicAdd(&cnt[(key[i] >> shift) & 255u], 1u);
+    const int base = blockIdx.x * items;
+    for (int k = threadIdx.x; k < items; k += 256) {
+        const int i = base + k;
+        if (i < n) atomicAdd(&cnt[(key[i] >> shift) & (BINS - 1u)], 1u);
     }
     __syncthreads();
-    hist[threadIdx.x * nblocks + blockIdx.x] = cnt[threadIdx.x];
+    for (int d = threadIdx.x; d < BINS; d += 256)
+        hist[fused ? blockIdx.x * BINS + d : d * nblocks + blockIdx.x] = cnt[d];
 }
 
 // Stable scatter: warp w of block b owns the contiguous items
-// [b*RS_ITEMS + w*RS_PER_WARP, +RS_PER_WARP); within a warp, items are ranked in
+// [b*items + w*per_warp, +per_warp); within a warp, items are ranked in
 // index order with match_any, so equal digits keep their input order.
+template <int BITS>
 __global__ void __launch_bounds__(256) k_rs_scatter(int n, const uint32_t *__restrict__ key_in,
                                                     const int32_t *__restrict__ val_in,
                                                     uint32_t *__restrict__ key_out,
                                                     int32_t *__restrict__ val_out, int shift,
-                                                    const uint32_t *__restrict__ hist_scan,
-                                                    int nblocks) {
-    __shared__ uint32_t off[RS_WARPS][256];
-    int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int d = lane; d < 256; d += 32) off[w][d] = 0;
+                                                    const uint32_t *__restrict__ hist,
+                                                    int nblocks, int per_warp, bool fused) {
+    constexpr int BINS = 1 << BITS, DPT = BINS / 256;   // digits per thread
+    __shared__ uint32_t off[RS_WARPS][BINS];
+    __shared__ uint32_t wsum[RS_WARPS];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int d = lane; d < BINS; d += 32) off[w][d] = 0;
     __syncwarp();
-    int wbase = blockIdx.x * RS_ITEMS + w * RS_PER_WARP;
-    for (int k = 0; k < RS_PER_WARP / 32; k++) {
-        int i = wbase + k * 32 + lane;
-        bool v = i < n;
-        uint32_t d = v ? ((key_in[i] >> shift) & 255u) : 256u + lane;
-        unsigned peers = __match_any_sync(FULL, d);
+    const int wbase = (blockIdx.x * RS_WARPS + w) * per_warp;
+    for (int k = 0; k < per_warp / 32; k++) {
+        const int i = wbase + k * 32 + lane;
+        const bool v = i < n;
+        const uint32_t d = v ? ((key_in[i] >> shift) & (BINS - 1u)) : BINS + lane;
+        const unsigned peers = __match_any_sync(FULL, d);
         if (v && lane == __ffs(peers) - 1) off[w][d] += __popc(peers);
         __syncwarp();
     }
-    __syncthreads();
-    {
-        int d = threadIdx.x;
-        uint32_t run = hist_scan[d * nblocks + blockIdx.x];
+    // where this block's items of each digit go
+    const int d0 = threadIdx.x * DPT;
+    uint32_t start[DPT];
+    if (fused) {
+        uint32_t before[DPT], total[DPT], sum = 0;
+#pragma unroll
+        for (int k = 0; k < DPT; k++) before[k] = total[k] = 0u;
+        for (int b = 0; b < nblocks; b++) {
+#pragma unroll
+            for (int k = 0; k < DPT; k++) {
+                const uint32_t c = __ldg(hist + b * BINS + d0 + k);
+                total[k] += c;
+                if (b < (int)blockIdx.x) before[k] += c;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < DPT; k++) sum += total[k];
+        uint32_t x = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(FULL, x, o);
+            if (lane >= o) x += y;
+        }
+        if (lane == 31) wsum[w] = x;
+        __syncthreads();
+        uint32_t excl = x - sum;
+        for (int v = 0; v < w; v++) excl += wsum[v];
+#pragma unroll
+        for (int k = 0; k < DPT; k++) {
+            start[k] = excl + before[k];
+            excl += total[k];
+        }
+    } else {
+#pragma unroll
+        for (int k = 0; k < DPT; k++) start[k] = hist[(d0 + k) * nblocks + blockIdx.x];
+        __syncthreads();
+    }
+#pragma unroll
+    for (int k = 0; k < DPT; k++) {
+        uint32_t run = start[k];
         for (int ww = 0; ww < RS_WARPS; ww++) {
-            uint32_t c = off[ww][d];
-            off[ww][d] = run;
+            const uint32_t c = off[ww][d0 + k];
+            off[ww][d0 + k] = run;
             run += c;
         }
     }
     __syncthreads();
-    unsigned lt = lanemask_lt();
-    for (int k = 0; k < RS_PER_WARP / 32; k++) {
-        int i = wbase + k * 32 + lane;
-        bool v = i < n;
-        uint32_t kk = v ? key_in[i] : 0u;
-        uint32_t d = v ? ((kk >> shift) & 255u) : 256u + lane;
-        unsigned peers = __match_any_sync(FULL, d);
-        uint32_t base = v ? off[w][d] : 0u;
+    const unsigned lt = lanemask_lt();
+    for (int k = 0; k < per_warp / 32; k++) {
+        const int i = wbase + k * 32 + lane;
+        const bool v = i < n;
+        const uint32_t kk = v ? key_in[i] : 0u;
+        const uint32_t d = v ? ((kk >> shift) & (BINS - 1u)) : BINS + lane;
+        const unsigned peers = __match_any_sync(FULL, d);
+        const uint32_t base = v ? off[w][d] : 0u;
         __syncwarp();
         if (v) {
-            uint32_t pos = base + __popc(peers & lt);
+            const uint32_t pos = base + __popc(peers & lt);
             key_out[pos] = kk;
             val_out[pos] = val_in[i];
             if (lane == __ffs(peers) - 1) off[w][d] = base + __popc(peers);
@@ -184,26 +238,47 @@ int scan_u32(crk_ctx *ctx, const uint32_t *in, uint32_t *out, int count, cudaStr
     return CRK_OK;
 }
 
-// Stable sort of (key_a, idx_a) by the low `bits` bits of key; result in key_a/idx_a.
-static int radix_sort(crk_ctx *ctx, int n, int bits, cudaStream_t s) {
-    int nblocks = grid_for(n, RS_ITEMS);
-    int passes = (bits + 7) / 8;
-    if (passes & 1) passes++;   // even number of passes leaves the result in the _a buffers
-    uint32_t *kin = ctx->key_a, *kout = ctx->key_b;
-    int32_t *vin = ctx->idx_a, *vout = ctx->idx_b;
-    for (int p = 0; p < passes; p++) {
-        int shift = 8 * p;
-        k_rs_hist<<<nblocks, 256, 0, s>>>(n, kin, shift, ctx->hist, nblocks);
-        ++ctx->launches;
-        int rc = scan_u32(ctx, ctx->hist, ctx->hist, 256 * nblocks, s);
+template <int BITS>
+static int radix_pass(crk_ctx *ctx, int n, int shift, const uint32_t *kin, const int32_t *vin, uint32_t *kout,
+                      int32_t *vout, cudaStream_t s) {
+    const int pw = rs_per_warp(n), items = RS_WARPS * pw, nblocks = grid_for(n, items);
+    const bool fused = nblocks <= RS_FUSED;
+    k_rs_hist<BITS><<<nblocks, 256, 0, s>>>(n, kin, shift, ctx->hist, nblocks, items, fused);
+    ++ctx->launches;
+    if (!fused) {
+        int rc = scan_u32(ctx, ctx->hist, ctx->hist, (1 << BITS) * nblocks, s);
         if (rc) return rc;
-        k_rs_scatter<<<nblocks, 256, 0, s>>>(n, kin, vin, kout, vout, shift, ctx->hist, nblocks);
-        ++ctx->launches;
-        CRK_LAUNCH_CHECK(ctx, "radix sort");
-        uint32_t *tk = kin; kin = kout; kout = tk;
-        int32_t *tv = vin; vin = vout; vout = tv;
+    }
+    k_rs_scatter<BITS><<<nblocks, 256, 0, s>>>(n, kin, vin, kout, vout, shift, ctx->hist, nblocks, pw, fused);
+    ++ctx->launches;
+    CRK_LAUNCH_CHECK(ctx, "radix sort");
+    return CRK_OK;
+}
+
+// A 30-bit sort of n keys starts from the _b buffers (three passes) or the _a
+// buffers (four); its result is in key_a, idx_a.
+static bool sort30_from_b(int n) { return n <= RS_WIDE_MAX; }
+
+static int radix_sort30(crk_ctx *ctx, int n, cudaStream_t s) {
+    int rc;
+    if (sort30_from_b(n)) {
+        rc = radix_pass<10>(ctx, n, 0, ctx->key_b, ctx->idx_b, ctx->key_a, ctx->idx_a, s);
+        if (!rc) rc = radix_pass<10>(ctx, n, 10, ctx->key_a, ctx->idx_a, ctx->key_b, ctx->idx_b, s);
+        if (!rc) rc = radix_pass<10>(ctx, n, 20, ctx->key_b, ctx->idx_b, ctx->key_a, ctx->idx_a, s);
+        return rc;
+    }
+    for (int p = 0; p < 4; p += 2) {
+        rc = radix_pass<8>(ctx, n, 8 * p, ctx->key_a, ctx->idx_a, ctx->key_b, ctx->idx_b, s);
+        if (!rc) rc = radix_pass<8>(ctx, n, 8 * p + 8, ctx->key_b, ctx->idx_b, ctx->key_a, ctx->idx_a, s);
+        if (rc) return rc;
     }
     return CRK_OK;
+}
+
+// Stable sort of (key_a, idx_a) by the low 16 bits of key; result in key_a, idx_a.
+static int radix_sort16(crk_ctx *ctx, int n, cudaStream_t s) {
+    int rc = radix_pass<8>(ctx, n, 0, ctx->key_a, ctx->idx_a, ctx->key_b, ctx->idx_b, s);
+    return rc ? rc : radix_pass<8>(ctx, n, 8, ctx->key_b, ctx->idx_b, ctx->key_a, ctx->idx_a, s);
 }
 
 // ------------------------------------------------------------------ recursive coordinate bisection
@@ -470,13 +545,15 @@ static int rcb_refine(crk_ctx *ctx, int n, cudaStream_t s) {
 __global__ void k_gather_sorted(int n, const int32_t *__restrict__ idx, const uint4 *__restrict__ q_tmp,
                                 const float *__restrict__ h_tmp, const int32_t *__restrict__ base_perm,
                                 uint4 *__restrict__ q4, float *__restrict__ hs,
-                                int32_t *__restrict__ perm_out) {
+                                int32_t *__restrict__ perm_out, const uint32_t *__restrict__ key,
+                                uint32_t *__restrict__ keys_out) {
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     int i = idx[s];
     q4[s] = q_tmp[i];
     hs[s] = h_tmp[i];
     perm_out[s] = base_perm ? base_perm[i] : i;
+    if (keys_out) keys_out[s] = key[s];
 }
 
 // ------------------------------------------------------------------ tiles and tree
@@ -487,36 +564,6 @@ __global__ void k_gather_sorted(int n, const int32_t *__restrict__ idx, const ui
 // the Morton order this is its min/max box; a tile whose particles drifted
 // across the periodic boundary (time bins keep tiles between sorts) gets an
 // arc with lo > hi instead of a box spanning the whole period.
-__global__ void k_tiles(int n, int ntiles, const uint4 *__restrict__ q4, uint4 *__restrict__ lo,
-                        uint4 *__restrict__ hi, const int32_t *__restrict__ sbox, uint32_t *__restrict__ nbox) {
-    int tile = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    int lane = threadIdx.x & 31;
-    if (tile >= ntiles) return;
-    int s = tile * TILE + lane;
-    bool v = s < n;
-    uint4 q = v ? q4[s] : make_uint4(0, 0, 0, 0);
-    const uint32_t rx = __shfl_sync(FULL, q.x, 0), ry = __shfl_sync(FULL, q.y, 0), rz = __shfl_sync(FULL, q.z, 0);
-    const int dx = v ? (int)(q.x - rx) : 0, dy = v ? (int)(q.y - ry) : 0, dz = v ? (int)(q.z - rz) : 0;
-    uint32_t xl = rx + (uint32_t)__reduce_min_sync(FULL, dx);
-    uint32_t yl = ry + (uint32_t)__reduce_min_sync(FULL, dy);
-    uint32_t zl = rz + (uint32_t)__reduce_min_sync(FULL, dz);
-    uint32_t xh = rx + (uint32_t)__reduce_max_sync(FULL, dx);
-    uint32_t yh = ry + (uint32_t)__reduce_max_sync(FULL, dy);
-    uint32_t zh = rz + (uint32_t)__reduce_max_sync(FULL, dz);
-    uint32_t Hm = __reduce_max_sync(FULL, v ? q.w : 0u);
-    uint32_t c = __popc(__ballot_sync(FULL, v));
-    if (lane == 0) {
-        lo[tile] = make_uint4(xl, yl, zl, Hm);
-        hi[tile] = make_uint4(xh, yh, zh, c);
-    }
-    if (sbox) {   // batched boxes: the range of boxes the tile's particles belong to
-        uint32_t b = v ? (uint32_t)sbox[s] : 0u;
-        uint32_t bl = __reduce_min_sync(FULL, v ? b : 0xffffu);
-        uint32_t bh = __reduce_max_sync(FULL, v ? b : 0u);
-        if (lane == 0) nbox[tile] = bl | (bh << 16);
-    }
-}
-
 __device__ __forceinline__ bool box_ranges_meet(uint32_t a, uint32_t b) {
     return (a & 0xffffu) <= (b >> 16) && (b & 0xffffu) <= (a >> 16);
 }
@@ -529,27 +576,83 @@ __device__ __forceinline__ void unwrap_arcs(uint4 &l, uint4 &h) {
     if (l.z > h.z) { l.z = 0u; h.z = 0xffffffffu; }
 }
 
-__global__ void k_tree_level(const uint4 *__restrict__ clo, const uint4 *__restrict__ chi, int ccnt,
-                             uint4 *__restrict__ plo, uint4 *__restrict__ phi, int pcnt,
-                             const uint32_t *__restrict__ cbox, uint32_t *__restrict__ pbox) {
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= pcnt) return;
-    uint4 l = clo[2 * k], h = chi[2 * k];
-    uint32_t b = cbox ? cbox[2 * k] : 0u;
+// One 32-ary parent from its children, child `lane` per lane: plain intervals,
+// largest support, particle count and box range.
+__device__ __forceinline__ void reduce32(uint4 l, uint4 h, uint32_t b, bool v, uint4 &pl, uint4 &ph, uint32_t &pb) {
     unwrap_arcs(l, h);
-    if (2 * k + 1 < ccnt) {
-        uint4 l2 = clo[2 * k + 1], h2 = chi[2 * k + 1];
-        unwrap_arcs(l2, h2);
-        l = make_uint4(min(l.x, l2.x), min(l.y, l2.y), min(l.z, l2.z), max(l.w, l2.w));
-        h = make_uint4(max(h.x, h2.x), max(h.y, h2.y), max(h.z, h2.z), h.w + h2.w);
-        if (cbox) {
-            uint32_t b2 = cbox[2 * k + 1];
-            b = min(b & 0xffffu, b2 & 0xffffu) | (max(b >> 16, b2 >> 16) << 16);
+    const uint32_t U = 0xffffffffu;
+    pl = make_uint4(__reduce_min_sync(FULL, v ? l.x : U), __reduce_min_sync(FULL, v ? l.y : U),
+                    __reduce_min_sync(FULL, v ? l.z : U), __reduce_max_sync(FULL, v ? l.w : 0u));
+    ph = make_uint4(__reduce_max_sync(FULL, v ? h.x : 0u), __reduce_max_sync(FULL, v ? h.y : 0u),
+                    __reduce_max_sync(FULL, v ? h.z : 0u), __reduce_add_sync(FULL, v ? h.w : 0u));
+    pb = __reduce_min_sync(FULL, v ? (b & 0xffffu) : 0xffffu) | (__reduce_max_sync(FULL, v ? (b >> 16) : 0u) << 16);
+}
+
+// Tiles (a warp each) and, by block, the parent of the block's 32 tiles.
+__global__ void __launch_bounds__(1024) k_tiles(int n, int ntiles, const uint4 *__restrict__ q4,
+                                                uint4 *__restrict__ lo, uint4 *__restrict__ hi,
+                                                const int32_t *__restrict__ sbox, uint32_t *__restrict__ nbox,
+                                                uint4 *__restrict__ plo, uint4 *__restrict__ phi,
+                                                uint32_t *__restrict__ pbox) {
+    __shared__ uint4 sl[32], sh[32];
+    __shared__ uint32_t sb[32];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int tile = blockIdx.x * 32 + w;
+    if (tile < ntiles) {
+        const int s = tile * TILE + lane;
+        const bool v = s < n;
+        const uint4 q = v ? q4[s] : make_uint4(0, 0, 0, 0);
+        const uint32_t rx = __shfl_sync(FULL, q.x, 0), ry = __shfl_sync(FULL, q.y, 0), rz = __shfl_sync(FULL, q.z, 0);
+        const int dx = v ? (int)(q.x - rx) : 0, dy = v ? (int)(q.y - ry) : 0, dz = v ? (int)(q.z - rz) : 0;
+        const uint32_t xl = rx + (uint32_t)__reduce_min_sync(FULL, dx), yl = ry + (uint32_t)__reduce_min_sync(FULL, dy),
+                       zl = rz + (uint32_t)__reduce_min_sync(FULL, dz), xh = rx + (uint32_t)__reduce_max_sync(FULL, dx),
+                       yh = ry + (uint32_t)__reduce_max_sync(FULL, dy), zh = rz + (uint32_t)__reduce_max_sync(FULL, dz);
+        const uint32_t Hm = __reduce_max_sync(FULL, v ? q.w : 0u);
+        const uint32_t c = __popc(__ballot_sync(FULL, v));
+        uint32_t range = 0u;
+        if (sbox) {   // batched boxes: the range of boxes the tile's particles belong to
+            const uint32_t b = v ? (uint32_t)sbox[s] : 0u;
+            range = __reduce_min_sync(FULL, v ? b : 0xffffu) | (__reduce_max_sync(FULL, v ? b : 0u) << 16);
+        }
+        if (lane == 0) {
+            sl[w] = lo[tile] = make_uint4(xl, yl, zl, Hm);
+            sh[w] = hi[tile] = make_uint4(xh, yh, zh, c);
+            sb[w] = range;
+            if (sbox) nbox[tile] = range;
         }
     }
-    plo[k] = l;
-    phi[k] = h;
-    if (cbox) pbox[k] = b;
+    __syncthreads();
+    if (w == 0 && plo) {
+        const bool v = blockIdx.x * 32 + lane < ntiles;
+        const uint4 z = make_uint4(0, 0, 0, 0);
+        uint4 l, h;
+        uint32_t b;
+        reduce32(v ? sl[lane] : z, v ? sh[lane] : z, v ? sb[lane] : 0u, v, l, h, b);
+        if (lane == 0) {
+            plo[blockIdx.x] = l;
+            phi[blockIdx.x] = h;
+            if (sbox) pbox[blockIdx.x] = b;
+        }
+    }
+}
+
+// The parents of `ccnt` nodes (a warp each).
+__global__ void k_tree_up(const uint4 *__restrict__ clo, const uint4 *__restrict__ chi, int ccnt,
+                          uint4 *__restrict__ plo, uint4 *__restrict__ phi, int pcnt,
+                          const uint32_t *__restrict__ cbox, uint32_t *__restrict__ pbox) {
+    const int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (k >= pcnt) return;
+    const int c = 32 * k + lane;
+    const bool v = c < ccnt;
+    const uint4 z = make_uint4(0, 0, 0, 0);
+    uint4 l, h;
+    uint32_t b;
+    reduce32(v ? clo[c] : z, v ? chi[c] : z, v && cbox ? cbox[c] : 0u, v, l, h, b);
+    if (lane == 0) {
+        plo[k] = l;
+        phi[k] = h;
+        if (cbox) pbox[k] = b;
+    }
 }
 
 // periodic gap (fixed point) between the arcs [a0,a1] and [b0,b1] of a circle
@@ -728,23 +831,27 @@ int rebuild_lists(crk_ctx *ctx, cudaStream_t s) {
     return CRK_OK;
 }
 
-// Tiles and tree from the sorted q4 (used again when only h changes).
+// Tiles and tree from the sorted q4 (used again when only h changes).  Only the
+// levels of the 32-ary view (0, 5, 10, ..) are formed, the first two in one
+// launch: 2 to 3 launches where the binary levels took one each (13 at 64^3).
 int build_tree(crk_ctx *ctx, cudaStream_t s) {
-    int n = ctx->n, nt = ctx->ntiles;
+    const int n = ctx->n, nt = ctx->ntiles;
     if (nt == 0) return CRK_OK;
     const bool batched = ctx->nbox > 1;
-    k_tiles<<<grid_for((long long)nt * 32, 256), 256, 0, s>>>(n, nt, ctx->q4, ctx->node_lo, ctx->node_hi,
-                                                               batched ? ctx->sbox : nullptr, ctx->node_box);
+    const int *off = ctx->level_off;
+    const bool up = ctx->nlevels > 5;
+    k_tiles<<<grid_for(nt, 32), 1024, 0, s>>>(n, nt, ctx->q4, ctx->node_lo, ctx->node_hi,
+                                               batched ? ctx->sbox : nullptr, ctx->node_box,
+                                               up ? ctx->node_lo + off[5] : nullptr,
+                                               up ? ctx->node_hi + off[5] : nullptr,
+                                               up && batched ? ctx->node_box + off[5] : nullptr);
     ++ctx->launches;
-    for (int L = 1; L < ctx->nlevels; L++) {
-        int pc = ctx->level_cnt[L];
-        k_tree_level<<<grid_for(pc, 256), 256, 0, s>>>(ctx->node_lo + ctx->level_off[L - 1],
-                                                         ctx->node_hi + ctx->level_off[L - 1],
-                                                         ctx->level_cnt[L - 1],
-                                                         ctx->node_lo + ctx->level_off[L],
-                                                         ctx->node_hi + ctx->level_off[L], pc,
-                                                         batched ? ctx->node_box + ctx->level_off[L - 1] : nullptr,
-                                                         batched ? ctx->node_box + ctx->level_off[L] : nullptr);
+    for (int L = 10; L < ctx->nlevels; L += 5) {
+        const int pc = ctx->level_cnt[L];
+        k_tree_up<<<grid_for(32ll * pc, 256), 256, 0, s>>>(
+            ctx->node_lo + off[L - 5], ctx->node_hi + off[L - 5], ctx->level_cnt[L - 5], ctx->node_lo + off[L],
+            ctx->node_hi + off[L], pc, batched ? ctx->node_box + off[L - 5] : nullptr,
+            batched ? ctx->node_box + off[L] : nullptr);
         ++ctx->launches;
     }
     CRK_LAUNCH_CHECK(ctx, "tile tree");
@@ -786,42 +893,47 @@ int build_cells_sorted(crk_ctx *ctx, int n, const float4 *pos, const int32_t *ba
     uint4 *q_tmp = ctx->q_tmp;
     float *h_tmp = ctx->h_tmp;
     prof_begin(ctx, PROF_BUILD, s);
-    k_keys<<<grid_for(n, 256), 256, 0, s>>>(n, pos, ctx->key_a, ctx->idx_a, q_tmp, h_tmp, ctx->counters,
+    const bool fb = sort30_from_b(n);
+    uint32_t *key0 = fb ? ctx->key_b : ctx->key_a;
+    k_keys<<<grid_for(n, 256), 256, 0, s>>>(n, pos, key0, fb ? ctx->idx_b : ctx->idx_a, q_tmp, h_tmp, ctx->counters,
                                             ctx->p.tile_order == 1);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "keys");
     if (box_of_input && ctx->p.tile_order == 2)
         return crk_set_error(ctx, CRK_EINVAL, "the bisection order covers one box (tile_order 0 or 1 for batches)");
+    uint32_t *keys_out = ctx->p.tile_order == 0 ? ctx->keys : nullptr;   // reported for the Morton order only
     if (box_of_input) {
         // batched boxes: stable sort by Morton key, then stable sort by box,
         // which leaves the order box-major and Morton within each box
-        CRK_CUDA(ctx, cudaMemcpyAsync(ctx->mkey, ctx->key_a, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, s));
-        rc = radix_sort(ctx, n, 30, s);
+        CRK_CUDA(ctx, cudaMemcpyAsync(ctx->mkey, key0, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, s));
+        rc = radix_sort30(ctx, n, s);
         if (rc) return rc;
         k_gather_u32<<<grid_for(n, 256), 256, 0, s>>>(n, ctx->idx_a, reinterpret_cast<const uint32_t *>(box_of_input),
                                                       ctx->key_a);
         ++ctx->launches;
-        rc = radix_sort(ctx, n, ctx->nbox <= 256 ? 8 : 16, s);
+        rc = radix_sort16(ctx, n, s);
         if (rc) return rc;
         CRK_CUDA(ctx, cudaMemcpyAsync(ctx->sbox, ctx->key_a, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, s));
         k_gather_u32<<<grid_for(n, 256), 256, 0, s>>>(n, ctx->idx_a, ctx->mkey, ctx->keys);
         ++ctx->launches;
         CRK_LAUNCH_CHECK(ctx, "box sort");
+        keys_out = nullptr;
     } else {
-        rc = radix_sort(ctx, n, 30, s);
+        rc = radix_sort30(ctx, n, s);
         if (rc) return rc;
-        // sorted keys (read by the chaining-mesh table, which only the Morton order has)
-        CRK_CUDA(ctx, cudaMemcpyAsync(ctx->keys, ctx->key_a, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, s));
         if (ctx->p.tile_order == 2) {
             rc = rcb_refine(ctx, n, s);
             if (rc) return rc;
         }
     }
+    // base_perm may be the array the new order goes to: then by way of idx_b
+    int32_t *perm = base_perm == ctx->perm ? ctx->idx_b : ctx->perm;
     k_gather_sorted<<<grid_for(n, 256), 256, 0, s>>>(n, ctx->idx_a, q_tmp, h_tmp, base_perm, ctx->q4,
-                                                     ctx->hs, ctx->idx_b);
+                                                     ctx->hs, perm, ctx->key_a, keys_out);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "gather sorted");
-    CRK_CUDA(ctx, cudaMemcpyAsync(ctx->perm, ctx->idx_b, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, s));
+    if (perm != ctx->perm)
+        CRK_CUDA(ctx, cudaMemcpyAsync(ctx->perm, perm, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, s));
     if (!box_of_input && ctx->p.tile_order == 0) {   // the chaining-mesh table: one box, Morton order
         k_cell_start<<<grid_for(n + 1, 256), 256, 0, s>>>(n, ctx->keys, ctx->p.kmax, ctx->counters,
                                                           ctx->cell_start);
@@ -858,7 +970,7 @@ int tile_order_by_length(crk_ctx *ctx, cudaStream_t s) {
     }
     k_len_keys<<<grid_for(nt, 256), 256, 0, s>>>(nt, ctx->len_u, ctx->key_a, ctx->idx_a);
     ++ctx->launches;
-    int rc = radix_sort(ctx, nt, 16, s);
+    int rc = radix_sort16(ctx, nt, s);
     if (rc) return rc;
     CRK_CUDA(ctx, cudaMemcpyAsync(ctx->tile_order, ctx->idx_a, sizeof(int32_t) * (size_t)nt,
                                   cudaMemcpyDeviceToDevice, s));

@@ -99,7 +99,8 @@ int crk_ensure_particles(crk_ctx *ctx, int n) {
     rc |= dalloc(ctx, &ctx->du_next, cap);
     rc |= dalloc(ctx, &ctx->node_lo, 2 * (size_t)tiles + MAX_LEVELS);
     rc |= dalloc(ctx, &ctx->node_hi, 2 * (size_t)tiles + MAX_LEVELS);
-    rc |= dalloc(ctx, &ctx->hist, 256 * (size_t)nb);
+    const size_t nhist = 1024 * (size_t)(nb < 32 ? 32 : nb);   // 10-bit digits: 32 blocks up to 65536 keys
+    rc |= dalloc(ctx, &ctx->hist, nhist);
     rc |= dalloc(ctx, &ctx->d_red, 4096 * 8);
     if (rc) {
         ctx->cap_n = 0;
@@ -108,7 +109,7 @@ int crk_ensure_particles(crk_ctx *ctx, int n) {
     ctx->cap_n = cap;
     ctx->cap_tiles = tiles;
     ctx->cap_nodes = 2 * tiles + MAX_LEVELS;
-    ctx->cap_hist = 256 * nb;
+    ctx->cap_hist = (int)nhist;
     ctx->rates_valid = 0;
     ctx->lists_valid = 0;
     long long want = (long long)tiles * 48;

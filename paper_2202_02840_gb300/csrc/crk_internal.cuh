@@ -89,7 +89,7 @@ struct crk_ctx {
     // sort scratch
     uint32_t *key_a = nullptr, *key_b = nullptr;
     int32_t *idx_a = nullptr, *idx_b = nullptr;
-    uint32_t *hist = nullptr;        // 256 * nblocks (+ scan scratch)
+    uint32_t *hist = nullptr;        // block histograms of the sort
     uint32_t *scan_tmp = nullptr;
     int cap_hist = 0;
 

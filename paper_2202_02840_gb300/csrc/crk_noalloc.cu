@@ -56,7 +56,7 @@ constexpr Layout make_layout() {
     L.ulist = o;    o = al(o + 4ull * TMAX * TMAX);   // every tile may neighbour every tile
     L.len_g = o;    o = al(o + 4ull * TMAX);
     L.len_u = o;    o = al(o + 4ull * TMAX);
-    L.hist = o;     o = al(o + 4ull * 256 * ((NMAX + 4095) / 4096));
+    L.hist = o;     o = al(o + 4ull * 1024 * 32);      // the sort's block histograms: 32 blocks of 10-bit digits
     L.scan = o;     o = al(o + 4ull * (2 * 4096 + 64));
     L.cells = o;    o = al(o + 4ull * 9);              // chaining-mesh table at level 1
     L.counters = o; o = al(o + 8ull * crk::CNT_COUNT);
@@ -126,7 +126,7 @@ extern "C" int crk_volumes_noalloc(int n, const float *pos_h, float *V, float *N
     ctx.cap_n = NMAX;
     ctx.cap_tiles = TMAX;
     ctx.cap_nodes = 2 * TMAX + crk::MAX_LEVELS;
-    ctx.cap_hist = 256 * ((NMAX + 4095) / 4096);
+    ctx.cap_hist = 1024 * 32;
     ctx.cap_ulist = (long long)TMAX * TMAX;
 
     if (cudaMemsetAsync(ctx.counters, 0, sizeof(unsigned long long) * crk::CNT_COUNT, s) != cudaSuccess)
