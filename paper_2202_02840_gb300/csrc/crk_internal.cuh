@@ -199,6 +199,8 @@ struct crk_ctx {
     unsigned long long *box_dtmin = nullptr;   // per-box CFL minimum (float bits)
     double *box_red = nullptr;       // per-box FP64 diagnostics, 8 per box
     int32_t *fcnt = nullptr;         // occupancy of the feature grid (8^7 cells)
+    float *ftab = nullptr;           // its cells' features (8 floats each)
+    int ftab_level = 0;              // grid level the table holds
     uint32_t *sel = nullptr;         // row selection: flags and their scan (2 x cap_sel)
     int cap_sel = 0;
 

@@ -124,7 +124,7 @@ struct FeatArgs {
     const float *gradv;      // gv_stride n or null (div v = trace: entries 0, 4, 8 of a row)
     int gv_stride;           // 9 (caller's 3x3 rows) or 12 (the engine's padded records)
     const float *Nngb;       // n or null
-    const int32_t *fcnt;     // 8^kf cell counts
+    const float *ftab;       // 8^kf rows of 8 floats: features 0 .. 4 of a cell
     float dt;                // step of the state (feature 6 = dt div v)
     float log_cbrt_n;        // log(N^(1/3)) = -log(Delta)
     float inv_N_res;
@@ -137,6 +137,17 @@ __device__ __forceinline__ float h_reference(const FeatArgs &a, float h, float N
     return a.Nngb ? h * cbrtf(a.N_res / N) : h;
 }
 
+// Cell of a position in [0, 1)^3: the top kf bits of the fixed-point coordinates
+// (the product with 2^kf is exact, so its integer part is those bits).  An
+// invalid position, which is counted and refused, still names a cell of the grid.
+__device__ __forceinline__ uint32_t feat_cell(const float4 &p, int kf) {
+    const float g = (float)(1 << kf);
+    const uint32_t m = (1u << kf) - 1u;
+    const uint32_t cx = min(__float2uint_rz(p.x * g), m), cy = min(__float2uint_rz(p.y * g), m),
+                   cz = min(__float2uint_rz(p.z * g), m);
+    return (cz << (2 * kf)) | (cy << kf) | cx;
+}
+
 __global__ void k_feat_count(int n, int kf, const float4 *__restrict__ pos_h, int32_t *__restrict__ fcnt,
                              unsigned long long *err) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -147,9 +158,7 @@ __global__ void k_feat_count(int n, int kf, const float4 *__restrict__ pos_h, in
         ok = p.x >= 0.f && p.x < 1.f && p.y >= 0.f && p.y < 1.f && p.z >= 0.f && p.z < 1.f && p.w > 0.f &&
              p.w < 1.f;   // NaN fails every comparison
         if (ok) {
-            uint32_t sh = 32 - kf;
-            uint32_t cx = to_fixed(p.x) >> sh, cy = to_fixed(p.y) >> sh, cz = to_fixed(p.z) >> sh;
-            cell = (cz << (2 * kf)) | (cy << kf) | cx;
+            cell = feat_cell(p, kf);
         } else {
             atomicAdd(err, 1ull);
         }
@@ -162,51 +171,42 @@ __global__ void k_feat_count(int n, int kf, const float4 *__restrict__ pos_h, in
     }
 }
 
-// Features 2t and 2t+1 of row i for lane t (0..3) of a quad; all four lanes of
-// the quad must call it for the same row.  Lanes 0..2 each sum one z-plane of
-// the 27 cells; the class sums are combined across the quad.
+// Features 0 .. 4 depend on a particle's cell alone: one thread per cell sums the
+// counts of the 27 cells around it by class and takes the logs, once for the
+// 64 to 511 particles of the cell.
+__global__ void k_feat_table(int kf, const int32_t *__restrict__ fcnt, float *__restrict__ ftab) {
+    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (c >> (3 * kf)) return;
+    const int g = 1 << kf, cx = c & (g - 1), cy = (c >> kf) & (g - 1), cz = c >> (2 * kf);
+    float cls[4] = {0.f, 0.f, 0.f, 0.f};   // own, face, edge, corner
+#pragma unroll
+    for (int dz = -1; dz <= 1; dz++)
+#pragma unroll
+        for (int dy = -1; dy <= 1; dy++)
+#pragma unroll
+            for (int dx = -1; dx <= 1; dx++) {
+                const int x = (cx + dx + g) & (g - 1), y = (cy + dy + g) & (g - 1), z = (cz + dz + g) & (g - 1);
+                cls[(dx != 0) + (dy != 0) + (dz != 0)] +=
+                    (float)__ldg(&fcnt[((size_t)z << (2 * kf)) | ((size_t)y << kf) | (size_t)x]);
+            }
+    float4 *out = reinterpret_cast<float4 *>(ftab) + 2 * (size_t)c;   // counts are integers: 1 + c is exact
+    out[0] = make_float4(__logf(1.f + cls[0]), __logf(1.f + cls[1]), __logf(1.f + cls[2]), __logf(1.f + cls[3]));
+    out[1] = make_float4(__logf(1.f + (cls[0] + cls[1] + cls[2] + cls[3])), 0.f, 0.f, 0.f);
+}
+
+// Features 2t and 2t+1 of row i for lane t (0..3) of a quad.
 __device__ __forceinline__ float2 quad_features(const FeatArgs &a, int i, int t, float &h_out, float &N_out) {
     bool valid = i < a.n;
     float4 p = valid ? a.pos_h[i] : make_float4(0.5f, 0.5f, 0.5f, 1.f);
-    int g = 1 << a.kf;
-    uint32_t sh = 32 - a.kf;
-    int cx = (int)(to_fixed(p.x) >> sh), cy = (int)(to_fixed(p.y) >> sh), cz = (int)(to_fixed(p.z) >> sh);
-    float cls[4] = {0.f, 0.f, 0.f, 0.f};   // own, face, edge, corner
-    if (t < 3 && valid) {
-        int dz = t - 1;
-        int z = (cz + dz + g) & (g - 1);
-#pragma unroll
-        for (int dy = -1; dy <= 1; dy++) {
-            int y = (cy + dy + g) & (g - 1);
-#pragma unroll
-            for (int dx = -1; dx <= 1; dx++) {
-                int x = (cx + dx + g) & (g - 1);
-                float c = (float)__ldg(&a.fcnt[((size_t)z << (2 * a.kf)) | ((size_t)y << a.kf) | (size_t)x]);
-                int m = (dx != 0) + (dy != 0) + (dz != 0);
-                cls[m] += c;
-            }
-        }
-    }
-#pragma unroll
-    for (int k = 0; k < 4; k++) {
-        cls[k] += __shfl_xor_sync(0xffffffffu, cls[k], 1);
-        cls[k] += __shfl_xor_sync(0xffffffffu, cls[k], 2);
-    }
     float h = p.w;
     float N = (a.Nngb && valid) ? __ldg(&a.Nngb[i]) : 0.f;
     h_out = h;
     N_out = N;
     float2 f = make_float2(0.f, 0.f);
     if (!valid) return f;
-    if (t == 0) {
-        f.x = __logf(1.f + cls[0]);   // counts are integers: 1 + c is exact
-        f.y = __logf(1.f + cls[1]);
-    } else if (t == 1) {
-        f.x = __logf(1.f + cls[2]);
-        f.y = __logf(1.f + cls[3]);
-    } else if (t == 2) {
-        f.x = __logf(1.f + (cls[0] + cls[1] + cls[2] + cls[3]));
-        f.y = __logf(h) + a.log_cbrt_n;
+    if (t < 3) {
+        f = __ldg(reinterpret_cast<const float2 *>(a.ftab) + 4 * (size_t)feat_cell(p, a.kf) + t);
+        if (t == 2) f.y = __logf(h) + a.log_cbrt_n;
     } else {
         float dv = 0.f;
         if (a.gradv) {
@@ -683,8 +683,17 @@ int count_cells(crk_ctx *ctx, int n, const float4 *pos, int kf, cudaStream_t s) 
     if (!ctx->fcnt) CRK_CUDA(ctx, cudaMalloc((void **)&ctx->fcnt, sizeof(int32_t) << 21));
     CRK_CUDA(ctx, cudaMemsetAsync(ctx->fcnt, 0, sizeof(int32_t) << (3 * kf), s));
     CRK_CUDA(ctx, cudaMemsetAsync(ctx->counters + CNT_MLP_ERR, 0, sizeof(unsigned long long), s));
+    const int cells = 1 << (3 * kf);
+    if (kf > ctx->ftab_level) {
+        if (ctx->ftab) cudaFree(ctx->ftab);
+        ctx->ftab = nullptr;
+        ctx->ftab_level = 0;
+        CRK_CUDA(ctx, cudaMalloc((void **)&ctx->ftab, sizeof(float) * 8 * (size_t)cells));
+        ctx->ftab_level = kf;
+    }
     k_feat_count<<<grid_for(n, 256), 256, 0, s>>>(n, kf, pos, ctx->fcnt, ctx->counters + CNT_MLP_ERR);
-    ++ctx->launches;
+    k_feat_table<<<grid_for(cells, 128), 128, 0, s>>>(kf, ctx->fcnt, ctx->ftab);
+    ctx->launches += 2;
     CRK_LAUNCH_CHECK(ctx, "feature cell count");
     return CRK_OK;
 }
@@ -707,7 +716,7 @@ FeatArgs feat_args(const crk_ctx *ctx, int n, const float *pos_h, const float *g
     a.gradv = gradv;
     a.gv_stride = 9;
     a.Nngb = Nngb;
-    a.fcnt = ctx->fcnt;
+    a.ftab = ctx->ftab;
     a.log_cbrt_n = (float)(log((double)n) / 3.0);
     a.inv_N_res = (float)(1.0 / ctx->p.N_res);
     a.N_res = (float)ctx->p.N_res;
@@ -796,6 +805,9 @@ void crk::mlp_free(crk_ctx *ctx) {
     }
     if (ctx->fcnt) cudaFree(ctx->fcnt);
     ctx->fcnt = nullptr;
+    if (ctx->ftab) cudaFree(ctx->ftab);
+    ctx->ftab = nullptr;
+    ctx->ftab_level = 0;
     if (ctx->sel) cudaFree(ctx->sel);
     ctx->sel = nullptr;
     ctx->cap_sel = 0;
