@@ -288,9 +288,10 @@ int crk_step(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const float *mass,
  * a CUDA graph of the whole multi-pass step (two graphs: consecutive steps
  * rotate the engine's state buffers), captured once and replayed with no host
  * work between steps.  Nothing can grow inside a replayed step, so before the
- * replays the call gives the neighbour-list columns and the tile-pair lists
- * 50% headroom over the last step's needs (one more eager step applies a new
- * column width) and the stored forces their worst case; each replayed step
+ * first capture the call gives the neighbour-list columns and the tile-pair
+ * lists 50% headroom over the last step's needs (one more eager step applies a
+ * new column width; captured graphs are kept while 25% is left) and the stored
+ * forces their worst case; each replayed step
  * records whether a capacity was exceeded anyway.  If one was, the call
  * restores the positions and velocities its replays started from and redoes
  * those steps eagerly, the first of them evaluating the rates afresh at the

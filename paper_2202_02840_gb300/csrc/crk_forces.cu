@@ -32,16 +32,14 @@ struct FParams {
 };
 
 // Per-particle record of the pair-set passes: 128 bytes, four 32-byte sectors
-// (one 256-bit load each).  The corrected kernel gradient of a particle with
-// separation x, eq:gRK, is affine in x up to two radial factors:
-//   grad W^R_g = t^6 (1 + 6 eta + 35/3 eta^2) (c_g + M_g . x) - 56/3 h^-2 t^5 (1 + 5 eta) (A' + B' . x) x_g,
-//   c_g = cW (dA_g + A B_g), M_ga = cW (dA_g B_a + A dB^a_g), A' = cW A, B' = cW A B, cW = 495/(32 pi h^3)
-// so the record holds c, M, A', B' (16 numbers, formed once per particle, each
-// rounded once) instead of A, B, dA, dB, cW, cG and their products per pair: four
-// gathers a pair instead of five and about a quarter fewer instructions.  P4 at
-// 128^3 clustered: 8.82 -> 7.72 ms, at 64^3 Sedov 1.03 -> 0.87 ms; it stays bound
-// by its gathers and the 12 warps an SM holds at 167 registers (16 warps at 128
-// registers with the record read at its use: 8.05 ms).  grad v enters the limiter only through the quadratic form
+// (one 256-bit load each).  It holds the affine coefficients of the corrected
+// kernel gradient (16 numbers, formed once per particle, each rounded once)
+// instead of A, B, dA, dB, cW, cG and their products per pair: four gathers a
+// pair instead of five and about a quarter fewer instructions.  P4 at 128^3
+// clustered: 8.82 -> 7.72 ms, at 64^3 Sedov 1.03 -> 0.87 ms; it stays bound by its
+// gathers and the 12 warps an SM holds at 167 registers (16 warps at 128
+// registers with the record read at its use: 8.05 ms).  grad v enters the limiter
+// only through the quadratic form
 // x . grad v . x, so its symmetric part is kept (6 numbers).  P and c_s follow
 // from rho and e = P / rho = (gamma - 1) u.
 //
@@ -75,31 +73,6 @@ struct FSrc {
     const GvRec *gv;
 };
 
-// An unevaluated sum hi + lo of two floats, for the coefficients of a record:
-// each is rounded once, from products that carry about 45 bits.
-struct F2 {
-    float hi, lo;
-};
-__device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
-    const float p = __fmul_rn(a.hi, b.hi);
-    return F2{p, fmaf(a.hi, b.lo, fmaf(a.lo, b.hi, fmaf(a.hi, b.hi, -p)))};
-}
-__device__ __forceinline__ F2 f2_mul(F2 a, float b) {
-    const float p = __fmul_rn(a.hi, b);
-    return F2{p, fmaf(a.lo, b, fmaf(a.hi, b, -p))};
-}
-__device__ __forceinline__ float f2_sum(F2 a, F2 b) {   // TwoSum of the high parts
-    const float s = __fadd_rn(a.hi, b.hi), t = __fsub_rn(s, a.hi);
-    const float e = __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, t)), __fsub_rn(b.hi, t));
-    return s + (e + (a.lo + b.lo));
-}
-constexpr float KW_LO = (float)(KW_D - (double)KW);
-constexpr float KGW = (float)(-KG_D / KW_D);   // -56/3
-constexpr float KGW_LO = (float)(-KG_D / KW_D - (double)KGW);
-
-// -56/3 h^-2 as the passes form it from 1/h
-__device__ __forceinline__ float grad_factor(float ih) { return KGW * (ih * ih); }
-
 __device__ __forceinline__ FRec make_frec(int j, const FSrc &src, const FParams &fp) {
     FRec r;
     const uint4 q = src.q4[j];
@@ -110,24 +83,12 @@ __device__ __forceinline__ FRec make_frec(int j, const FSrc &src, const FParams 
     const float rho = src.rho ? src.rho[j] : src.mass[j] / V;
     const CorrRec c = src.corr[j];
     const GvRec g = src.gv[j];
-    const float B[3] = {c.c0.y, c.c0.z, c.c0.w}, dA[3] = {c.c1.x, c.c1.y, c.c1.z};
-    const float dB[9] = {c.c1.w, c.c2.x, c.c2.y, c.c2.z, c.c2.w, c.c3.x, c.c3.y, c.c3.z, c.c3.w};   // [a][g]
-    const F2 i1 = {ih, __fmul_rn(fmaf(-ih, h, 1.f), ih)}, i2 = f2_mul(i1, i1);
-    const F2 cW = f2_mul(F2{KW, KW_LO}, f2_mul(i2, i1)), cA = f2_mul(cW, c.c0.x);
-    // A', B' also carry the rounding of grad_factor: its product with them is
-    // cG A, cG A B to their own rounding
-    const float gf = grad_factor(ih);
-    const F2 g2 = f2_mul(F2{KGW, KGW_LO}, i2);
-    const float fix = ((g2.hi - gf) + g2.lo) / gf;
-    const F2 gA = F2{cA.hi, fmaf(cA.hi, fix, cA.lo)};
-    auto C = [&](int k) { return f2_sum(f2_mul(cW, dA[k]), f2_mul(cA, B[k])); };
-    auto M = [&](int k, int a) { return f2_sum(f2_mul(f2_mul(cW, dA[k]), B[a]), f2_mul(cA, dB[3 * a + k])); };
-    auto AB = [&](int a) { const F2 v = f2_mul(gA, B[a]); return v.hi + v.lo; };
+    const Affine f = affine_of(c, h, ih);
     r.w1 = make_float4(V, v.x, v.y, v.z);
-    r.w2 = make_float4(C(0), C(1), C(2), gA.hi + gA.lo);
-    r.w3 = make_float4(M(0, 0), M(1, 0), M(2, 0), AB(0));
-    r.w4 = make_float4(M(0, 1), M(1, 1), M(2, 1), AB(1));
-    r.w5 = make_float4(M(0, 2), M(1, 2), M(2, 2), AB(2));
+    r.w2 = make_float4(f.c[0], f.c[1], f.c[2], f.A);
+    r.w3 = make_float4(f.M[0][0], f.M[0][1], f.M[0][2], f.B[0]);
+    r.w4 = make_float4(f.M[1][0], f.M[1][1], f.M[1][2], f.B[1]);
+    r.w5 = make_float4(f.M[2][0], f.M[2][1], f.M[2][2], f.B[2]);
     // grad v [a][b]: g0 = (00 01 02 10), g1 = (11 12 20 21), g2 = (22 ...)
     r.w6 = make_float4(g.g0.x, g.g1.x, g.g2.x, g.g0.y + g.g0.w);
     r.w7 = make_float4(g.g0.z + g.g1.z, g.g1.y + g.g1.w, rho, fp.gm1 * v.w);
@@ -141,12 +102,6 @@ struct FOwn {
     float lc;    // C_l c_s
     float k;     // 1 / (n_h h)
 };
-__device__ __forceinline__ float sqrt_approx(float v) {
-    float r;
-    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
-    return r;
-}
-
 __device__ __forceinline__ FOwn own_terms(const FRec &a, const FParams &fp) {
     FOwn o;
     o.G = grad_factor(a.w0.w);

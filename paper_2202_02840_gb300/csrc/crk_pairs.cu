@@ -265,10 +265,10 @@ struct P2 {
     __device__ static void pair(IState &s, const Rec &r, uint32_t, size_t, bool ok, const Params &) {
         int dx = (int)(s.q.x - r.x), dy = (int)(s.q.y - r.y), dz = (int)(s.q.z - r.z);
         const float Vj = __uint_as_float(r.w);
-        Sep d = separation(dx, dy, dz);
+        const Sep d = separation32(dx, dy, dz);   // the sums are scaled in finish
         float x[3] = {d.x, d.y, d.z};
-        float eta = d.r * s.inv_h;
-        float t = fmaxf(1.f - eta, 0.f);
+        float eta = d.r * (TWO_M32 * s.inv_h);
+        float t = __saturatef(1.f - eta);
         float t2 = t * t, t4 = t2 * t2, t5 = t4 * t;
         float Wu = t5 * t * fmaf(eta, fmaf(eta, K35_3, 6.f), 1.f);   // W / (495/(32 pi h^3))
         float Gu = -fmaf(5.f, eta, 1.f) * t5;                        // grad W / (1155/(4 pi h^5) x)
@@ -301,22 +301,25 @@ struct P2 {
     // FP64 constants before that cancellation.
     __device__ static void finish(IState &s, int i, const Params &p) {
         CorrRec out;
+        // 2^-32 per factor x of a sum (exact)
+        constexpr double X1 = (double)TWO_M32, X2 = X1 * X1, X3 = X2 * X1;
         auto val = [](const Acc<COMP> &a) -> double { return COMP ? (double)a.s - (double)a.c : (double)a.s; };
         if (FP64_SOLVE) {
             PairSums<double> ps;
             ps.m0 = val(s.m0);
-            for (int a = 0; a < 3; a++) ps.m1[a] = val(s.m1[a]), ps.dm0[a] = val(s.dm0[a]);
-            for (int q = 0; q < 6; q++) ps.m2[q] = val(s.m2[q]), ps.s1[q] = val(s.s1[q]);
-            for (int q = 0; q < 10; q++) ps.s2[q] = val(s.s2[q]);
+            for (int a = 0; a < 3; a++) ps.m1[a] = X1 * val(s.m1[a]), ps.dm0[a] = X1 * val(s.dm0[a]);
+            for (int q = 0; q < 6; q++) ps.m2[q] = X2 * val(s.m2[q]), ps.s1[q] = X2 * val(s.s1[q]);
+            for (int q = 0; q < 10; q++) ps.s2[q] = X3 * val(s.s2[q]);
             double m0, m1[3], m2[6], dm0[3], dm1[9], dm2[18];
             moments<double>(s.h, ps, m0, m1, m2, dm0, dm1, dm2);
             rk_solve<double, double>(m0, m1, m2, dm0, dm1, dm2, out);
         } else {
+            constexpr float Y1 = (float)X1, Y2 = (float)X2, Y3 = (float)X3;
             PairSums<float> ps;
             ps.m0 = s.m0.value();
-            for (int a = 0; a < 3; a++) ps.m1[a] = s.m1[a].value(), ps.dm0[a] = s.dm0[a].value();
-            for (int q = 0; q < 6; q++) ps.m2[q] = s.m2[q].value(), ps.s1[q] = s.s1[q].value();
-            for (int q = 0; q < 10; q++) ps.s2[q] = s.s2[q].value();
+            for (int a = 0; a < 3; a++) ps.m1[a] = Y1 * s.m1[a].value(), ps.dm0[a] = Y1 * s.dm0[a].value();
+            for (int q = 0; q < 6; q++) ps.m2[q] = Y2 * s.m2[q].value(), ps.s1[q] = Y2 * s.s1[q].value();
+            for (int q = 0; q < 10; q++) ps.s2[q] = Y3 * s.s2[q].value();
             float m0, m1[3], m2[6], dm0[3], dm1[9], dm2[18];
             moments<float>(s.h, ps, m0, m1, m2, dm0, dm1, dm2);
             rk_solve<float, float>(m0, m1, m2, dm0, dm1, dm2, out);
@@ -514,26 +517,28 @@ struct P3 {
     struct Sums {
         Acc<COMP> acc[9];
     };
+    // own affine coefficients of the corrected gradient, for separations in
+    // fixed-point units: M and B times 2^-32, the radial factor g with its x too
     struct IState : Sums {
         uint4 q;
-        float inv_h, cW, cG;
-        float A, B[3], gA[3], gB[9], v[3];
+        float inv_h, g;
+        Affine f;
+        float v[3];
     };
     __device__ static Sums sums(const IState &s) { return s; }
     __device__ static void init(IState &s, int i, bool valid, const Params &p) {
         s.q = valid ? p.q4[i] : make_uint4(0, 0, 0, 0);
-        float h = valid ? p.hs[i] : 1.f;
-        s.inv_h = 1.f / h;
-        float ih2 = s.inv_h * s.inv_h, ih3 = ih2 * s.inv_h;
-        s.cW = KW * ih3;
-        s.cG = -KG * ih3 * ih2;
-        CorrRec c = valid ? p.corr[i] : CorrRec{};
-        float4 v = valid ? p.vel[i] : make_float4(0.f, 0.f, 0.f, 0.f);
-        s.A = c.c0.x;
-        s.B[0] = c.c0.y; s.B[1] = c.c0.z; s.B[2] = c.c0.w;
-        s.gA[0] = c.c1.x; s.gA[1] = c.c1.y; s.gA[2] = c.c1.z;
-        s.gB[0] = c.c1.w; s.gB[1] = c.c2.x; s.gB[2] = c.c2.y; s.gB[3] = c.c2.z; s.gB[4] = c.c2.w;
-        s.gB[5] = c.c3.x; s.gB[6] = c.c3.y; s.gB[7] = c.c3.z; s.gB[8] = c.c3.w;
+        const float h = valid ? p.hs[i] : 1.f, ih = 1.f / h;
+        s.inv_h = TWO_M32 * ih;
+        s.g = TWO_M32 * grad_factor(ih);
+        s.f = affine_of(valid ? p.corr[i] : CorrRec{}, h, ih);
+#pragma unroll
+        for (int a = 0; a < 3; a++) {
+            s.f.B[a] *= TWO_M32;
+#pragma unroll
+            for (int g = 0; g < 3; g++) s.f.M[a][g] *= TWO_M32;
+        }
+        const float4 v = valid ? p.vel[i] : make_float4(0.f, 0.f, 0.f, 0.f);
         s.v[0] = v.x; s.v[1] = v.y; s.v[2] = v.z;
 #pragma unroll
         for (int k = 0; k < 9; k++) s.acc[k] = Acc<COMP>();
@@ -556,21 +561,20 @@ struct P3 {
         const float4 vj = rec.v;
         const float Vj = __uint_as_float(r.w);
         int dx = (int)(s.q.x - r.x), dy = (int)(s.q.y - r.y), dz = (int)(s.q.z - r.z);
-        Sep d = separation(dx, dy, dz);
-        float x[3] = {d.x, d.y, d.z};
-        float eta = d.r * s.inv_h;
-        float t = fmaxf(1.f - eta, 0.f);
-        float t2 = t * t, t4 = t2 * t2, t5 = t4 * t;
-        float W = s.cW * t5 * t * fmaf(eta, fmaf(eta, K35_3, 6.f), 1.f);
-        float G = s.cG * fmaf(5.f, eta, 1.f) * t5;       // grad W = G x
-        // eq:gRK with the i-side coefficients
-        float sB = fmaf(s.B[0], x[0], fmaf(s.B[1], x[1], fmaf(s.B[2], x[2], 1.f)));
-        float sW = sB * W, AW = s.A * W, AsG = s.A * sB * G;
+        const Sep d = separation32(dx, dy, dz);
+        const float x[3] = {d.x, d.y, d.z};
+        const float eta = d.r * s.inv_h;
+        const float t = __saturatef(1.f - eta);
+        const float t2 = t * t, t4 = t2 * t2, t5 = t4 * t;
+        const float W = t5 * t * fmaf(eta, fmaf(eta, K35_3, 6.f), 1.f);
+        const Affine &f = s.f;
+        const float As = fmaf(f.B[0], x[0], fmaf(f.B[1], x[1], fmaf(f.B[2], x[2], f.A)));
+        const float G = As * (s.g * (fmaf(5.f, eta, 1.f) * t5));
         float gR[3];
 #pragma unroll
         for (int g = 0; g < 3; g++) {
-            float gBx = fmaf(s.gB[g], x[0], fmaf(s.gB[3 + g], x[1], s.gB[6 + g] * x[2]));
-            gR[g] = fmaf(s.gA[g], sW, fmaf(AW, gBx + s.B[g], AsG * x[g]));
+            const float T = fmaf(f.M[0][g], x[0], fmaf(f.M[1][g], x[1], fmaf(f.M[2][g], x[2], f.c[g])));
+            gR[g] = fmaf(W, T, G * x[g]);
         }
         float Vd[3] = {Vj * (s.v[0] - vj.x), Vj * (s.v[1] - vj.y), Vj * (s.v[2] - vj.z)};
 #pragma unroll
@@ -633,7 +637,7 @@ struct PD {
         int dx = (int)(s.q.x - r.q.x), dy = (int)(s.q.y - r.q.y), dz = (int)(s.q.z - r.q.z);
         Sep d = separation(dx, dy, dz);
         float eta = d.r * s.inv_h;
-        float t = fmaxf(1.f - eta, 0.f);
+        float t = __saturatef(1.f - eta);
         float t2 = t * t, t3 = t2 * t;
         float Wu = t3 * t3 * fmaf(eta, fmaf(eta, K35_3, 6.f), 1.f);
         float sB = fmaf(s.B[0], d.x, fmaf(s.B[1], d.y, fmaf(s.B[2], d.z, 1.f)));

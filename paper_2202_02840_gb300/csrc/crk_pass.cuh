@@ -653,6 +653,12 @@ __device__ __forceinline__ void ldg_v8(const float4 *p, float4 &a, float4 &b) {
         : "l"(p));
 }
 
+__device__ __forceinline__ float sqrt_approx(float v) {
+    float r;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+    return r;
+}
+
 struct Sep {
     float x, y, z, r2, r;
 };
@@ -663,8 +669,79 @@ __device__ __forceinline__ Sep separation(int dx, int dy, int dz) {
     s.y = (float)dy * TWO_M32;
     s.z = (float)dz * TWO_M32;
     s.r2 = fmaf(s.x, s.x, fmaf(s.y, s.y, s.z * s.z));
-    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(s.r) : "f"(s.r2));
+    s.r = sqrt_approx(s.r2);
     return s;
+}
+
+// The separation in fixed-point units, 2^32 times the above (the scaling is
+// exact, so sums of products with it are the same bits up to that power of
+// two): the passes apply 2^-32 to their constants instead of to every pair.
+__device__ __forceinline__ Sep separation32(int dx, int dy, int dz) {
+    Sep s;
+    s.x = (float)dx;
+    s.y = (float)dy;
+    s.z = (float)dz;
+    s.r2 = fmaf(s.x, s.x, fmaf(s.y, s.y, s.z * s.z));
+    s.r = sqrt_approx(s.r2);
+    return s;
+}
+__device__ __forceinline__ float distance32(int dx, int dy, int dz) { return separation32(dx, dy, dz).r; }
+
+// An unevaluated sum hi + lo of two floats, for per-particle coefficients: each
+// is rounded once, from products that carry about 45 bits.
+struct F2 {
+    float hi, lo;
+};
+__device__ __forceinline__ F2 f2_mul(F2 a, F2 b) {
+    const float p = __fmul_rn(a.hi, b.hi);
+    return F2{p, fmaf(a.hi, b.lo, fmaf(a.lo, b.hi, fmaf(a.hi, b.hi, -p)))};
+}
+__device__ __forceinline__ F2 f2_mul(F2 a, float b) {
+    const float p = __fmul_rn(a.hi, b);
+    return F2{p, fmaf(a.lo, b, fmaf(a.hi, b, -p))};
+}
+__device__ __forceinline__ float f2_sum(F2 a, F2 b) {   // TwoSum of the high parts
+    const float s = __fadd_rn(a.hi, b.hi), t = __fsub_rn(s, a.hi);
+    const float e = __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, t)), __fsub_rn(b.hi, t));
+    return s + (e + (a.lo + b.lo));
+}
+constexpr float KW_LO = (float)(KW_D - (double)KW);
+constexpr float KGW = (float)(-KG_D / KW_D);   // -56/3
+constexpr float KGW_LO = (float)(-KG_D / KW_D - (double)KGW);
+
+// -56/3 h^-2 as the passes form it from 1/h
+__device__ __forceinline__ float grad_factor(float ih) { return KGW * (ih * ih); }
+
+// The corrected kernel gradient of a particle with separation x, eq:gRK, is
+// affine in x up to two radial factors:
+//   grad W^R_g = t^6 (1 + 6 eta + 35/3 eta^2) (c_g + M_g . x) - 56/3 h^-2 t^5 (1 + 5 eta) (A' + B' . x) x_g,
+//   c_g = cW (dA_g + A B_g), M_ga = cW (dA_g B_a + A dB^a_g), A' = cW A, B' = cW A B, cW = 495/(32 pi h^3).
+struct Affine {
+    float c[3], M[3][3], A, B[3];   // M[a][g]: the coefficient of x_a in component g
+};
+__device__ __forceinline__ Affine affine_of(const CorrRec &r, float h, float ih) {
+    const float B[3] = {r.c0.y, r.c0.z, r.c0.w}, dA[3] = {r.c1.x, r.c1.y, r.c1.z};
+    const float dB[9] = {r.c1.w, r.c2.x, r.c2.y, r.c2.z, r.c2.w, r.c3.x, r.c3.y, r.c3.z, r.c3.w};   // [a][g]
+    const F2 i1 = {ih, __fmul_rn(fmaf(-ih, h, 1.f), ih)}, i2 = f2_mul(i1, i1);
+    const F2 cW = f2_mul(F2{KW, KW_LO}, f2_mul(i2, i1)), cA = f2_mul(cW, r.c0.x);
+    // A', B' also carry the rounding of grad_factor: its product with them is
+    // cG A, cG A B to their own rounding
+    const float gf = grad_factor(ih);
+    const F2 g2 = f2_mul(F2{KGW, KGW_LO}, i2);
+    const float fix = ((g2.hi - gf) + g2.lo) / gf;
+    const F2 gA = F2{cA.hi, fmaf(cA.hi, fix, cA.lo)};
+    Affine o;
+#pragma unroll
+    for (int g = 0; g < 3; g++) {
+        const F2 d = f2_mul(cW, dA[g]);
+        o.c[g] = f2_sum(d, f2_mul(cA, B[g]));
+#pragma unroll
+        for (int a = 0; a < 3; a++) o.M[a][g] = f2_sum(f2_mul(d, B[a]), f2_mul(cA, dB[3 * a + g]));
+        const F2 v = f2_mul(gA, B[g]);
+        o.B[g] = v.hi + v.lo;
+    }
+    o.A = gA.hi + gA.lo;
+    return o;
 }
 
 }  // namespace crk

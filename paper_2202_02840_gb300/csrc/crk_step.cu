@@ -833,18 +833,26 @@ static int steps_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const flo
     }
     if (done < nsteps) {
         // headroom for the replayed steps: list columns (they change only at a
-        // walk, so one more eager step applies the new width) and tile-pair lists
+        // walk, so one more eager step applies the new width) and tile-pair lists.
+        // 50% of the last step's needs before the first capture; graphs that are
+        // there are kept while 25% is left (a run that calls this every few steps
+        // with slowly growing counts would otherwise widen the columns, copy the
+        // stored forces and capture anew in every call)
+        const bool have = ctx->gexec[0] || ctx->gexec[1];
         rc = crk_sync_counters(ctx, s);
         if (rc) return rc;
         const long long maxc = (long long)ctx->h_counters[CNT_MAXCNT];
         const long long nu = (long long)ctx->h_counters[CNT_ULIST];
-        if (maxc + maxc / 2 > ctx->kcap && done < nsteps) {
-            ctx->kcap = (int)((maxc + maxc / 2 + 31) / 32 * 32);
+        if (maxc + maxc / (have ? 4 : 2) > ctx->kcap && done < nsteps) {
+            // a second widening means growing counts: twice the need, while the
+            // worst case of the stored forces stays below 32 GB
+            const bool twice = have && (double)ctx->ntiles * (2.0 * maxc) * 512.0 < 32e9;
+            ctx->kcap = (int)((maxc + (twice ? maxc : maxc / 2) + 31) / 32 * 32);
             rc = step_impl(ctx, n, pos_h, vel_u, mass, dt, nullptr, batched, s);
             if (rc) return rc;
             done++;
         }
-        if (nu + nu / 2 > ctx->cap_ulist) {
+        if (nu + nu / (have ? 4 : 2) > ctx->cap_ulist) {
             rc = crk_ensure_lists(ctx, 0, nu + nu / 2 + 1024);
             if (rc) return rc;
         }

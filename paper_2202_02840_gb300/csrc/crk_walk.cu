@@ -41,13 +41,10 @@ struct WalkArgs {
     unsigned long long *tests;   // lane tests of the exact predicate (LISTS walk)
 };
 
-// LISTS: write the lists; VOL: sum n_i in the walk (volumes-only contexts).
 // circular distance (fixed point) from coordinate q to the arc [lo, hi]
 // (which may wrap, lo > hi); differences modulo 2^32
-__device__ __forceinline__ unsigned long long point_gap(uint32_t q, uint32_t lo, uint32_t hi) {
-    if (q - lo <= hi - lo) return 0ull;
-    uint32_t d1 = lo - q, d2 = q - hi;
-    return (unsigned long long)(d1 < d2 ? d1 : d2);
+__device__ __forceinline__ float point_gap(uint32_t q, uint32_t lo, uint32_t hi) {
+    return q - lo <= hi - lo ? 0.f : (float)min(lo - q, q - hi);
 }
 
 // One segment of a lane's list on its way to memory: the last up to three
@@ -127,7 +124,7 @@ struct WalkMasks {
 template <bool VOL, bool BATCH>
 struct WalkShm {
     WalkBox B;
-    uint4 r[RING];                      // (x, y, z, H^2) relative, or the fixed-point record
+    uint4 r[RING];                      // x, y, z relative or fixed point; H^2
     uint32_t id[VOL ? 1 : RING];        // sorted index
     int32_t box[BATCH ? RING : 1];
 };
@@ -216,9 +213,9 @@ __device__ __forceinline__ void walk_range(const WalkArgs &a, const WalkTile &T,
                         for (int u = 3; u >= 0; u--) {
                             const uint4 q = S.r[ring + p + u];
                             const float dx = (float)(int)(qi.x - q.x), dy = (float)(int)(qi.y - q.y),
-                                        dz = (float)(int)(qi.z - q.z), H = (float)q.w;
+                                        dz = (float)(int)(qi.z - q.z);
                             const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                            const float ti = r2 - T.Hf2, tj = r2 - H * H;
+                            const float ti = r2 - T.Hf2, tj = r2 - __uint_as_float(q.w);
                             amb = fminf(amb, fminf(fabsf(ti), fabsf(tj)));
                             gm = __funnelshift_l(__float_as_uint(ti), gm, 1);
                             jm = __funnelshift_l(__float_as_uint(tj), jm, 1);
@@ -299,14 +296,12 @@ __device__ __forceinline__ void walk_range(const WalkArgs &a, const WalkTile &T,
             keep = lane < cnt && fmaf(hx, hx, fmaf(hy, hy, hz * hz)) < fmaf(rj, rj, mrg);
         } else {
             const uint4 qi = own_record(a, T), Ihi = __ldg(a.thi + T.tile);
-            const unsigned long long gx = point_gap(qi.x, Jlo.x, Jhi.x), gy = point_gap(qi.y, Jlo.y, Jhi.y),
-                                     gz = point_gap(qi.z, Jlo.z, Jhi.z);
-            const unsigned long long reach = max(qi.w, HJ);
-            near = T.valid && gx * gx + gy * gy + gz * gz < reach * reach;
-            const unsigned long long hx = point_gap(qc.x, Ilo.x, Ihi.x), hy = point_gap(qc.y, Ilo.y, Ihi.y),
-                                     hz = point_gap(qc.z, Ilo.z, Ihi.z);
-            const unsigned long long rj = VOL ? Ilo.w : max(qc.w, Ilo.w);
-            keep = lane < cnt && hx * hx + hy * hy + hz * hz < rj * rj;
+            const float gx = point_gap(qi.x, Jlo.x, Jhi.x), gy = point_gap(qi.y, Jlo.y, Jhi.y),
+                        gz = point_gap(qi.z, Jlo.z, Jhi.z), re = fmaxf(T.Hf, (float)HJ);
+            near = T.valid && fmaf(gx, gx, fmaf(gy, gy, gz * gz)) < fmaf(re, re, mrg);
+            const float hx = point_gap(qc.x, Ilo.x, Ihi.x), hy = point_gap(qc.y, Ilo.y, Ihi.y),
+                        hz = point_gap(qc.z, Ilo.z, Ihi.z), rj = (float)(VOL ? Ilo.w : max(qc.w, Ilo.w));
+            keep = lane < cnt && fmaf(hx, hx, fmaf(hy, hy, hz * hz)) < fmaf(rj, rj, mrg);
         }
         bool mixed = false;   // the pair's boxes must be compared
         int32_t bj = 0;
@@ -329,9 +324,9 @@ __device__ __forceinline__ void walk_range(const WalkArgs &a, const WalkTile &T,
         if (keep) {
             const uint32_t k = at & (RING - 1);
             const float hj = (float)qc.w;
-            S.r[k] = VOL || T.raw ? qc
-                                  : make_uint4(__float_as_uint(jx), __float_as_uint(jy), __float_as_uint(jz),
-                                               __float_as_uint(hj * hj));
+            const bool fix = VOL || T.raw;
+            S.r[k] = make_uint4(fix ? qc.x : __float_as_uint(jx), fix ? qc.y : __float_as_uint(jy),
+                                fix ? qc.z : __float_as_uint(jz), __float_as_uint(hj * hj));
             if (!VOL) S.id[k] = (uint32_t)(j0 + lane);
             if (BATCH) S.box[k] = bj;
         }
@@ -389,17 +384,23 @@ __global__ void __launch_bounds__(WALK_WARPS * 32, 4) k_walk(WalkArgs a) {
         if (a.Nn) a.Nn[T.i] = (K4PI_3 * h * h * h) * nsum;         // eq:hi
     };
     auto sum_batch = [&](const WalkTile &T, const uint4 &qi, float inv_h, uint32_t ring, int c, float &acc) {
-        for (int p = 0; p < c; p += 4) {
+        auto term = [&](int p, bool live) {
+            const uint4 q = S.r[ring + p];
+            const float eta = distance32((int)(qi.x - q.x), (int)(qi.y - q.y), (int)(qi.z - q.z)) * inv_h;
+            float t = __saturatef(1.f - eta);
+            if (!live || (BATCH && S.box[ring + p] != T.bi)) t = 0.f;
+            const float t2 = t * t, t3 = t2 * t;
+            acc = fmaf(t3 * t3, fmaf(eta, fmaf(eta, K35_3, 6.f), 1.f), acc);
+        };
+        if (c == 32) {
+            for (int p = 0; p < 32; p += 4) {
 #pragma unroll
-            for (int u = 0; u < 4; u++) {
-                const uint4 q = S.r[ring + p + u];
-                const Sep d = separation((int)(qi.x - q.x), (int)(qi.y - q.y), (int)(qi.z - q.z));
-                const float eta = d.r * inv_h;
-                float t = __saturatef(1.f - eta);
-                if (p + u >= c) t = 0.f;
-                if (BATCH && S.box[ring + p + u] != T.bi) t = 0.f;
-                const float t2 = t * t, t3 = t2 * t;
-                acc = fmaf(t3 * t3, fmaf(eta, fmaf(eta, K35_3, 6.f), 1.f), acc);
+                for (int u = 0; u < 4; u++) term(p + u, true);
+            }
+        } else {
+            for (int p = 0; p < c; p += 2) {
+                term(p, true);
+                term(p + 1, p + 1 < c);
             }
         }
     };
@@ -429,7 +430,7 @@ __global__ void __launch_bounds__(WALK_WARPS * 32, 4) k_walk(WalkArgs a) {
         uint32_t kept = 0;
         if constexpr (VOL) {
             const uint4 qi = own_record(a, T);
-            const float inv_h = 1.f / (T.valid ? a.hs[T.i] : 1.f);
+            const float inv_h = TWO_M32 * (1.f / (T.valid ? a.hs[T.i] : 1.f));
             float acc = 0.f;
             walk_range<VOL, BATCH>(a, T, lane, lo, t0, t1, S, kept,
                                    [&](uint32_t ring, int c) { sum_batch(T, qi, inv_h, ring, c, acc); });
@@ -516,7 +517,7 @@ __global__ void __launch_bounds__(WALK_WARPS * 32, 4) k_walk(WalkArgs a) {
     uint32_t kept = 0;
     if constexpr (VOL) {
         const uint4 qi = own_record(a, T);
-        const float inv_h = 1.f / (T.valid ? a.hs[T.i] : 1.f);
+        const float inv_h = TWO_M32 * (1.f / (T.valid ? a.hs[T.i] : 1.f));
         float acc = 0.f;
         walk_range<VOL, BATCH>(a, T, lane, lo, 0, (int)lo.y, S, kept,
                                [&](uint32_t ring, int c) { sum_batch(T, qi, inv_h, ring, c, acc); });
@@ -724,9 +725,8 @@ struct P1 {
     __device__ static void merge(IState &s, Sums o) { s.acc += o; }
     __device__ static Rec load(uint32_t j, size_t, const Params &p) { return __ldg(p.q4 + j); }
     __device__ static void pair(IState &s, const Rec &r, uint32_t, size_t, bool ok, const Params &) {
-        int dx = (int)(s.q.x - r.x), dy = (int)(s.q.y - r.y), dz = (int)(s.q.z - r.z);
-        Sep d = separation(dx, dy, dz);
-        float eta = d.r * s.inv_h;
+        const float eta =
+            distance32((int)(s.q.x - r.x), (int)(s.q.y - r.y), (int)(s.q.z - r.z)) * (TWO_M32 * s.inv_h);
         float t = ok ? __saturatef(1.f - eta) : 0.f;
         float t2 = t * t, t3 = t2 * t;
         s.acc = fmaf(t3 * t3, fmaf(eta, fmaf(eta, K35_3, 6.f), 1.f), s.acc);
