@@ -687,10 +687,13 @@ struct Tree32 {
 // child of the node being expanded; passing leaves (tiles) are emitted in
 // ascending order, passing inner nodes pushed so that the lowest pops first.
 // The reach of a node is max(Hmax_I, Hmax_node) (pair-set predicate).
-template <bool WRITE>
+// SOME: only tiles in [r0, r1) (r0 a multiple of 32).  Stops once more than
+// `stop` are found.
+template <bool WRITE, bool SOME = false>
 __device__ uint32_t walk32(const Tree32 &T, const uint4 *__restrict__ lo, const uint4 *__restrict__ hi,
                            const uint32_t *__restrict__ nbox, uint32_t Ibox, uint4 Ilo, uint4 Ihi,
-                           uint32_t *__restrict__ out, uint32_t lim, int *stL, int *stK, int lane) {
+                           uint32_t *__restrict__ out, uint32_t lim, int *stL, int *stK, int lane,
+                           uint32_t stop = 0xfffffffeu, long long r0 = 0, long long r1 = 0) {
     const unsigned lt = lanemask_lt();
     const unsigned long long HI = Ilo.w;
     uint32_t count = 0;
@@ -705,6 +708,7 @@ __device__ uint32_t walk32(const Tree32 &T, const uint4 *__restrict__ lo, const 
             unsigned long long R = HI > (unsigned long long)nlo.w ? HI : (unsigned long long)nlo.w;
             pass = box_gap2(Ilo, Ihi, nlo, nhi) < R * R &&
                    (!nbox || box_ranges_meet(Ibox, nbox[T.off[cl] + c]));
+            if (SOME) pass = pass && ((long long)c << (5 * cl)) < r1 && ((long long)(c + 1) << (5 * cl)) > r0;
         }
         const unsigned m = __ballot_sync(0xffffffffu, pass);
         const int np = __popc(m);
@@ -714,6 +718,7 @@ __device__ uint32_t walk32(const Tree32 &T, const uint4 *__restrict__ lo, const 
                 if (at < lim) out[at] = (uint32_t)c;
             }
             count += np;
+            if (count > stop) return count;
         } else if (np) {
             if (pass) {
                 const int pos = sp + (np - 1 - __popc(m & lt));
@@ -734,16 +739,21 @@ __device__ uint32_t walk32(const Tree32 &T, const uint4 *__restrict__ lo, const 
 
 constexpr uint32_t LIST_BUF = 1024;   // tiles a warp keeps in shared memory
 
+__host__ __device__ __forceinline__ long long grid_tiles(int ntiles, int parts) {
+    return ((long long)ntiles + parts - 1) / parts;
+}
+
 // One walk per tile into shared memory, then one allocation and a coalesced
-// copy; a tile with more than LIST_BUF neighbours walks a second time
-// straight into the allocated range.  act (may be null): the lists of the
-// tiles act[0 .. count) only.
+// copy; a tile with more than LIST_BUF neighbours goes to the queue of
+// k_lists_long.  act (may be null): the lists of the tiles act[0 .. count) only.
 __global__ void __launch_bounds__(LIST_WARPS * 32) k_lists32(int count, const int32_t *__restrict__ act, Tree32 T,
                                                              const uint4 *__restrict__ lo,
                                                              const uint4 *__restrict__ hi,
                                                              const uint32_t *__restrict__ nbox,
                                                              uint2 *__restrict__ ofs, uint32_t *__restrict__ list,
-                                                             long long cap, unsigned long long *counter) {
+                                                             long long cap, unsigned long long *counter,
+                                                             int32_t *__restrict__ queue,
+                                                             unsigned long long *queued) {
     __shared__ int stL[LIST_WARPS][STACK], stK[LIST_WARPS][STACK];
     __shared__ uint32_t buf[LIST_WARPS][LIST_BUF];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -752,7 +762,7 @@ __global__ void __launch_bounds__(LIST_WARPS * 32) k_lists32(int count, const in
     const int I = act ? act[t] : t;
     const uint4 Ilo = lo[I], Ihi = hi[I];
     const uint32_t Ibox = nbox ? nbox[I] : 0u;
-    uint32_t c = walk32<true>(T, lo, hi, nbox, Ibox, Ilo, Ihi, buf[w], LIST_BUF, stL[w], stK[w], lane);
+    const uint32_t c = walk32<true>(T, lo, hi, nbox, Ibox, Ilo, Ihi, buf[w], LIST_BUF, stL[w], stK[w], lane, LIST_BUF);
     unsigned long long base = 0;
     if (c == 0xffffffffu) {
         if (lane == 0) {
@@ -761,18 +771,66 @@ __global__ void __launch_bounds__(LIST_WARPS * 32) k_lists32(int count, const in
         }
         return;
     }
+    if (c > LIST_BUF) {
+        if (lane == 0) {
+            ofs[I] = make_uint2(0u, 0u);
+            queue[atomicAdd(queued, 1ull)] = I;
+        }
+        return;
+    }
     if (lane == 0) base = atomicAdd(counter, (unsigned long long)c);
     base = __shfl_sync(0xffffffffu, base, 0);
     if ((long long)(base + c) <= cap) {
         __syncwarp();
-        if (c <= LIST_BUF) {
-            for (uint32_t k = lane; k < c; k += 32) list[base + k] = buf[w][k];
-        } else {
-            walk32<true>(T, lo, hi, nbox, Ibox, Ilo, Ihi, list + base, c, stL[w], stK[w], lane);
-        }
+        for (uint32_t k = lane; k < c; k += 32) list[base + k] = buf[w][k];
         if (lane == 0) ofs[I] = make_uint2((uint32_t)base, c);
     } else if (lane == 0) {
         ofs[I] = make_uint2(0u, 0u);
+    }
+}
+
+// The queued tiles, a CTA each: warp w walks a 1/LONG_WARPS of the tiles, first
+// counting, then writing at its place.  (A tile of an evacuated region, or one
+// that jumps across the box, may neighbour every tile; one warp took 250 us for
+// the longest at 64^3 clustered, when the other tiles were done after 40.)
+constexpr int LONG_WARPS = 16;
+__global__ void __launch_bounds__(LONG_WARPS * 32) k_lists_long(int ntiles, const int32_t *__restrict__ queue,
+                                                                const unsigned long long *queued, Tree32 T,
+                                                                const uint4 *__restrict__ lo,
+                                                                const uint4 *__restrict__ hi,
+                                                                const uint32_t *__restrict__ nbox,
+                                                                uint2 *__restrict__ ofs, uint32_t *__restrict__ list,
+                                                                long long cap, unsigned long long *counter) {
+    __shared__ int stL[LONG_WARPS][STACK], stK[LONG_WARPS][STACK];
+    __shared__ uint32_t cnt[LONG_WARPS];
+    __shared__ unsigned long long base;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int end = (int)*queued;
+    const long long part = (grid_tiles(ntiles, LONG_WARPS) + 31) / 32 * 32, r0 = w * part, r1 = r0 + part;
+    for (int t = blockIdx.x; t < end; t += gridDim.x) {
+        const int I = queue[t];
+        const uint4 Ilo = lo[I], Ihi = hi[I];
+        const uint32_t Ibox = nbox ? nbox[I] : 0u;
+        const uint32_t c = walk32<false, true>(T, lo, hi, nbox, Ibox, Ilo, Ihi, nullptr, 0u, stL[w], stK[w], lane,
+                                               0xfffffffeu, r0, r1);
+        if (lane == 0) cnt[w] = c;
+        __syncthreads();
+        uint32_t before = 0, total = 0;
+        bool bad = false;
+        for (int v = 0; v < LONG_WARPS; v++) {
+            bad |= cnt[v] == 0xffffffffu;
+            if (v < w) before += cnt[v];
+            total += cnt[v];
+        }
+        // a stack overflow forces the overflow path, as in k_lists32
+        if (threadIdx.x == 0) base = atomicAdd(counter, bad ? (unsigned long long)cap + 1ull : (unsigned long long)total);
+        __syncthreads();
+        const bool fits = !bad && (long long)(base + total) <= cap;
+        if (fits)
+            walk32<true, true>(T, lo, hi, nbox, Ibox, Ilo, Ihi, list + base + before, c, stL[w], stK[w], lane,
+                               0xfffffffeu, r0, r1);
+        if (threadIdx.x == 0 && fits) ofs[I] = make_uint2((uint32_t)base, total);
+        __syncthreads();
     }
 }
 
@@ -823,10 +881,19 @@ int rebuild_lists(crk_ctx *ctx, cudaStream_t s) {
     ctx->lists_valid = 0;
     const int count = ctx->act ? ctx->nact : ctx->ntiles;
     if (count == 0) return CRK_OK;
+    const bool may_queue = ctx->ntiles > (int)LIST_BUF;   // else no tile has more neighbours than the buffer holds
+    if (may_queue) CRK_CUDA(ctx, cudaMemsetAsync(ctx->counters + CNT_LQUEUE, 0, sizeof(unsigned long long), s));
     k_lists32<<<grid_for(count, LIST_WARPS), LIST_WARPS * 32, 0, s>>>(
         count, ctx->act, T, ctx->node_lo, ctx->node_hi, ctx->nbox > 1 ? ctx->node_box : nullptr, ctx->uofs,
-        ctx->ulist, ctx->cap_ulist, ctx->counters + CNT_ULIST);
+        ctx->ulist, ctx->cap_ulist, ctx->counters + CNT_ULIST, ctx->lqueue, ctx->counters + CNT_LQUEUE);
     ++ctx->launches;
+    if (may_queue) {
+        k_lists_long<<<ctx->nsm > 0 ? ctx->nsm : 152, LONG_WARPS * 32, 0, s>>>(
+            ctx->ntiles, ctx->lqueue, ctx->counters + CNT_LQUEUE, T, ctx->node_lo, ctx->node_hi,
+            ctx->nbox > 1 ? ctx->node_box : nullptr, ctx->uofs, ctx->ulist, ctx->cap_ulist,
+            ctx->counters + CNT_ULIST);
+        ++ctx->launches;
+    }
     CRK_LAUNCH_CHECK(ctx, "interaction lists");
     return CRK_OK;
 }

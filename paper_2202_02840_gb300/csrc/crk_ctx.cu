@@ -92,6 +92,8 @@ int crk_ensure_particles(crk_ctx *ctx, int n) {
     rc |= dalloc(ctx, &ctx->len_g, tiles);
     rc |= dalloc(ctx, &ctx->len_u, tiles);
     rc |= dalloc(ctx, &ctx->tbase, tiles);
+    rc |= dalloc(ctx, &ctx->heavy, tiles);
+    rc |= dalloc(ctx, &ctx->lqueue, tiles);
     rc |= dalloc(ctx, &ctx->frec, 8 * (size_t)cap);
     rc |= dalloc(ctx, &ctx->sfun, cap);
     rc |= dalloc(ctx, &ctx->sig, cap);
@@ -541,7 +543,7 @@ extern "C" int crk_destroy(crk_ctx *ctx) {
     dfree(&ctx->node_lo); dfree(&ctx->node_hi);
     dfree(&ctx->gofs); dfree(&ctx->uofs); dfree(&ctx->glist); dfree(&ctx->ulist);
     dfree(&ctx->qV); dfree(&ctx->cnt_g); dfree(&ctx->cnt_u); dfree(&ctx->len_g); dfree(&ctx->len_u);
-    dfree(&ctx->tcap); dfree(&ctx->tbase); dfree(&ctx->ent); dfree(&ctx->Fst); dfree(&ctx->frec);
+    dfree(&ctx->heavy); dfree(&ctx->lqueue); dfree(&ctx->tcap); dfree(&ctx->tbase); dfree(&ctx->ent); dfree(&ctx->Fst); dfree(&ctx->frec);
     dfree(&ctx->lowc); dfree(&ctx->po_self); dfree(&ctx->po_rev); dfree(&ctx->po_rowA); dfree(&ctx->po_rowB);
     dfree(&ctx->po_tofs); dfree(&ctx->po_tlist);
     dfree(&ctx->sfun); dfree(&ctx->sig); dfree(&ctx->sig2); dfree(&ctx->du_next);

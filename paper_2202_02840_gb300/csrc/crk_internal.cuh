@@ -42,7 +42,9 @@ enum {
     CNT_PO_MISS = 21,   // pair-once: tile pairs (I, J) whose reverse (J, I) was not found (sticky)
     CNT_WALK_TESTS = 22,  // lane tests of the exact predicate in the last list walk
     CNT_TMA_ERR = 23,   // sticky: a TMA-fed pass gave up waiting on its copies
-    CNT_COUNT = 24
+    CNT_HEAVY = 24,     // tiles of the last walk with more than HEAVY_ROWS list rows (ctx->heavy)
+    CNT_LQUEUE = 25,    // tiles queued by the last list build (ctx->lqueue)
+    CNT_COUNT = 26
 };
 
 // Pass-input records in sorted order.
@@ -119,6 +121,8 @@ struct crk_ctx {
     uint4 *qV = nullptr;             // (qx, qy, qz, V bits)
     int32_t *cnt_g = nullptr, *cnt_u = nullptr;   // gather (j != i) and pair-set counts
     uint32_t *len_g = nullptr, *len_u = nullptr;  // per-tile max counts
+    int32_t *heavy = nullptr;        // tiles with long lists (any order)
+    int32_t *lqueue = nullptr;       // tiles the list build leaves to k_lists_long (any order)
     uint32_t *tcap = nullptr, *tbase = nullptr;   // per-tile stored-force base (units of 32)
     uint32_t *ent = nullptr;         // list entries: j | (j's kernel reaches i) << 31
     float4 *Fst = nullptr;           // F_ij per entry (P4 -> P5), compact layout

@@ -132,7 +132,13 @@ struct ListGeom {
     const uint32_t *len_g, *len_u;     // per-tile rows of the longest lane (multiples of LB)
     const int32_t *cnt_g, *cnt_u;
     const uint32_t *ent;
+    int heavy;                         // > 0: tiles with more pair-set rows are left to the split form
 };
+
+// A tile with more rows than this (a typical one has 260 to 400) is shared by the
+// warps of a CTA: a warp that walks the 1000 to 2000 neighbours of a particle in
+// an evacuated region runs on alone when the others are done.
+constexpr int HEAVY_ROWS = 576;
 
 // The blocks of lists stream once from HBM (or L2, just written by the walk),
 // the longest latency of the loop, so the next block is always read ahead.
@@ -277,6 +283,7 @@ __device__ __forceinline__ void list_loop_rp(typename P::IState &st, const typen
 template <class P, int U, bool RP = false>
 __device__ __forceinline__ void lpass_tile(const ListGeom &g, const typename P::Params &prm, int tile, int lane) {
     if (pass_skipped<P>(prm)) return;   // the sums were formed by an earlier pass
+    if (g.heavy && (int)g.len_u[tile] > g.heavy) return;
     const int i = tile * TILE + lane;
     const bool valid = i < g.n;
     typename P::IState st;
@@ -368,30 +375,37 @@ constexpr int split_warps() {   // as many as their sums fit static shared memor
            : ((3 * 32 * sizeof(typename P::Sums) <= 44 * 1024) ? 4 : 2);
 }
 
+// count null: block b takes tile order[b] (order null: tile b); else the blocks
+// share the tiles order[0 .. *count).
 template <class P, int S, int U>
-__global__ void __launch_bounds__(S * 32) k_lpass_split(ListGeom g, typename P::Params prm, const int32_t *order) {
+__global__ void __launch_bounds__(S * 32) k_lpass_split(ListGeom g, typename P::Params prm, const int32_t *order,
+                                                        const unsigned long long *count) {
     using Sums = typename P::Sums;
     __shared__ __align__(16) unsigned char part[(S - 1) * 32 * sizeof(Sums)];
     if (pass_skipped<P>(prm)) return;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int tile = order ? order[blockIdx.x] : (int)blockIdx.x;
-    const int i = tile * TILE + lane;
-    const bool valid = i < g.n;
-    typename P::IState st;
-    P::init(st, i, valid, prm);
-    if (w > 0) P::zero(st);
-    const LaneList<P> ll(g, tile, lane, i, valid);
-    const int bw = (int)((P::GATHER ? g.len_g[tile] : g.len_u[tile]) / LB);
-    const int chunk = (bw + S - 1) / S;
-    const int b0 = w * chunk, b1 = min(bw, b0 + chunk);
-    list_loop<P, U>(st, prm, ll, b0, min(ll.nb, b1), b1);
-    Sums *sp = reinterpret_cast<Sums *>(part);
-    if (w > 0) sp[(w - 1) * 32 + lane] = P::sums(st);
-    __syncthreads();
-    if (w == 0) {
+    const int end = count ? (int)*count : (int)blockIdx.x + 1;
+    for (int t = blockIdx.x; t < end; t += gridDim.x) {
+        const int tile = order ? order[t] : t;
+        const int i = tile * TILE + lane;
+        const bool valid = i < g.n;
+        typename P::IState st;
+        P::init(st, i, valid, prm);
+        if (w > 0) P::zero(st);
+        const LaneList<P> ll(g, tile, lane, i, valid);
+        const int bw = (int)((P::GATHER ? g.len_g[tile] : g.len_u[tile]) / LB);
+        const int chunk = (bw + S - 1) / S;
+        const int b0 = w * chunk, b1 = min(bw, b0 + chunk);
+        list_loop<P, U>(st, prm, ll, b0, min(ll.nb, b1), b1);
+        Sums *sp = reinterpret_cast<Sums *>(part);
+        if (w > 0) sp[(w - 1) * 32 + lane] = P::sums(st);
+        __syncthreads();
+        if (w == 0) {
 #pragma unroll 1
-        for (int v = 1; v < S; v++) P::merge(st, sp[(v - 1) * 32 + lane]);
-        if (valid) P::finish(st, i, prm);
+            for (int v = 1; v < S; v++) P::merge(st, sp[(v - 1) * 32 + lane]);
+            if (valid) P::finish(st, i, prm);
+        }
+        __syncthreads();
     }
 }
 
@@ -574,8 +588,8 @@ int launch_lpass(crk_ctx *ctx, int prof_id, const typename P::Params &prm, cudaS
     const int ts = tune_slot >= 0 ? tune_slot : prof_id;
     if (ctx->n == 0) return CRK_OK;
     if (!ctx->lists_valid) return crk_set_error(ctx, CRK_ESTATE, "%s: neighbour lists are not built", what);
-    ListGeom g{ctx->n, ctx->ntiles, ctx->kcap, ctx->tbase, ctx->len_g, ctx->len_u, ctx->cnt_g, ctx->cnt_u,
-               ctx->ent};
+    ListGeom g{ctx->n,   ctx->ntiles, ctx->kcap,  ctx->tbase, ctx->len_g,
+               ctx->len_u, ctx->cnt_g, ctx->cnt_u, ctx->ent,  0};
     int rc;
     const int nsm = ctx->nsm > 0 ? ctx->nsm : 152;
     constexpr int U = P::PREFETCH ? 1 : P::UNROLL;
@@ -615,13 +629,23 @@ int launch_lpass(crk_ctx *ctx, int prof_id, const typename P::Params &prm, cudaS
         return crk_set_error(ctx, CRK_EINVAL, "%s: the pass has no variant %d", what, v);
     prof_begin(ctx, prof_id, s);
     rc = CRK_OK;
+    constexpr int S = split_warps<P>();
     if (g.ntiles < SPLIT_TILES * nsm) {   // whatever the variant: its warps would not fill the SMs
-        constexpr int S = split_warps<P>();
-        k_lpass_split<P, S, U><<<g.ntiles, S * 32, 0, s>>>(g, prm, ctx->act);
-    } else if (forms) {
-        rc = launch_variant<P, WARPS>(ctx, g, prm, v, s);
-    } else {
+        k_lpass_split<P, S, U><<<g.ntiles, S * 32, 0, s>>>(g, prm, ctx->act, nullptr);
+    } else if (ctx->act) {
         k_lpass<P, WARPS, U><<<grid_for(g.ntiles, WARPS), WARPS * 32, 0, s>>>(g, prm, ctx->act);
+    } else {
+        // long lists first, by CTAs (a captured step does not know whether there are any)
+        if (ctx->graph_mode || ctx->h_counters[CNT_MAXCNT] > (unsigned long long)HEAVY_ROWS) {
+            g.heavy = HEAVY_ROWS;
+            k_lpass_split<P, S, U><<<2 * nsm, S * 32, 0, s>>>(g, prm, ctx->heavy, ctx->counters + CNT_HEAVY);
+            ++ctx->launches;
+            CRK_LAUNCH_CHECK(ctx, what);
+        }
+        if (forms)
+            rc = launch_variant<P, WARPS>(ctx, g, prm, v, s);
+        else
+            k_lpass<P, WARPS, U><<<grid_for(g.ntiles, WARPS), WARPS * 32, 0, s>>>(g, prm, nullptr);
     }
     if (rc) return rc;
     ++ctx->launches;

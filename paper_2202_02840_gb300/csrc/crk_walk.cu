@@ -35,6 +35,8 @@ struct WalkArgs {
     const int32_t *sbox;     // batched boxes: box of each slot (BATCH only)
     const uint32_t *nbox;    // box range of each tile (BATCH only)
     const int32_t *act;      // may be null: walk the tiles act[0 .. ntiles) only
+    int32_t *long_list;      // tiles with more than HEAVY_ROWS rows, and their count
+    unsigned long long *nlong;
     int heavy;               // tiles with more candidate tiles than this are shared by the warps of a CTA
     int hblocks;             // CTAs that take them (all: one per tile, every tile is shared)
     int all;
@@ -421,6 +423,7 @@ __global__ void __launch_bounds__(WALK_WARPS * 32, 4) k_walk(WalkArgs a) {
             atomicAdd(a.pairs_g, (unsigned long long)sg);
             atomicAdd(a.pairs_u, (unsigned long long)su);
             atomicMax(a.maxcnt, (unsigned long long)mu);
+            if (LISTS && mu > (uint32_t)HEAVY_ROWS) a.long_list[atomicAdd(a.nlong, 1ull)] = T.tile;
         }
     };
     auto shared_tile = [&](int tile, uint2 lo) {   // by all warps of the CTA
@@ -497,8 +500,9 @@ __global__ void __launch_bounds__(WALK_WARPS * 32, 4) k_walk(WalkArgs a) {
             shared_tile(tile, a.ofs[tile]);
             return;
         }
-        for (int t0 = (int)blockIdx.x * 32; t0 < a.ntiles; t0 += a.hblocks * 32) {
-            const int t = t0 + lane;
+        // neighbouring tiles, which are heavy together, go to different CTAs
+        for (int t0 = (int)blockIdx.x; t0 < a.ntiles; t0 += a.hblocks * 32) {
+            const int t = t0 + lane * a.hblocks;
             const int mine = t < a.ntiles ? (a.act ? a.act[t] : t) : -1;
             unsigned m = __ballot_sync(0xffffffffu, mine >= 0 && (int)a.ofs[max(mine, 0)].y > a.heavy);
             for (; m; m &= m - 1u) {
@@ -576,10 +580,12 @@ static WalkArgs walk_args(crk_ctx *ctx) {
     a.act = ctx->act;
     if (ctx->act) a.ntiles = ctx->nact;
     a.tests = ctx->counters + CNT_WALK_TESTS;
+    a.long_list = ctx->heavy;
+    a.nlong = ctx->counters + CNT_HEAVY;
     const int nsm = ctx->nsm > 0 ? ctx->nsm : 152;
     a.all = a.ntiles < WALK_ALL * nsm;
     a.heavy = a.all ? -1 : WALK_HEAVY;
-    a.hblocks = a.all ? a.ntiles : nsm;
+    a.hblocks = a.all ? a.ntiles : 4 * nsm;   // a full wave of CTAs
     return a;
 }
 
@@ -591,6 +597,7 @@ static int launch_walk(crk_ctx *ctx, cudaStream_t s) {
     CRK_CUDA(ctx, cudaMemsetAsync(ctx->counters + CNT_PAIRS_G, 0, 2 * sizeof(unsigned long long), s));
     CRK_CUDA(ctx, cudaMemsetAsync(ctx->counters + CNT_MAXCNT, 0, sizeof(unsigned long long), s));
     CRK_CUDA(ctx, cudaMemsetAsync(ctx->counters + CNT_WALK_TESTS, 0, sizeof(unsigned long long), s));
+    CRK_CUDA(ctx, cudaMemsetAsync(ctx->counters + CNT_HEAVY, 0, sizeof(unsigned long long), s));
     if (ctx->act) {   // tiles left out of the walk take no list columns and no stored forces
         CRK_CUDA(ctx, cudaMemsetAsync(ctx->len_g, 0, sizeof(uint32_t) * ctx->ntiles, s));
         CRK_CUDA(ctx, cudaMemsetAsync(ctx->len_u, 0, sizeof(uint32_t) * ctx->ntiles, s));
