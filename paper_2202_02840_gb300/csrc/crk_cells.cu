@@ -57,13 +57,14 @@ __global__ void k_keys(int n, const float4 *__restrict__ pos, uint32_t *__restri
 // histograms are scanned in between.  A small sort is all latency: its blocks
 // take fewer keys (64 to 512 a warp), so that more warps share the serial
 // ranking.  4096 keys: 147 us in 12 launches with four 8-bit passes over 4096-key
-// blocks, 33 us in 6 now; 262144 keys 196 us in 20, 118 us in 6.
+// blocks, 27 us in 6 now; 262144 keys 196 us in 20, 73 us in 6.
 constexpr int RS_WARPS = 8;
+constexpr int RS_ROUNDS = 16;   // keys per lane, at most
 constexpr int RS_FUSED = 64;
 constexpr int RS_WIDE_MAX = 32 << 20;
 
 // keys per warp of an n-key sort
-static int rs_per_warp(int n) { return n <= 16384 ? 64 : (n <= 32768 ? 128 : (n <= 65536 ? 256 : 512)); }
+static int rs_per_warp(int n) { return n <= 16384 ? 64 : (n <= 32768 ? 128 : (n <= 65536 ? 256 : 32 * RS_ROUNDS)); }
 
 // Block histograms of one digit: hist[block][digit] (fused) or hist[digit][block].
 template <int BITS>
@@ -73,11 +74,13 @@ __global__ void __launch_bounds__(256) k_rs_hist(int n, const uint32_t *__restri
     __shared__ uint32_t cnt[BINS];
     for (int d = threadIdx.x; d < BINS; d += 256) cnt[d] = 0;
     __syncthreads();
-    const int base = blockIdx.x * items;
-    for (int k = threadIdx.x; k < items; k += 256) {
-        const int i = base + k;
-        if (i < n) atomicAdd(&cnt[(key[i] >> shift) & (BINS - 1u)], 1u);
-    }
+    const int first = blockIdx.x * items + threadIdx.x, rounds = items / 256;
+    uint32_t kk[RS_ROUNDS];   // all loads in flight
+#pragma unroll
+    for (int k = 0; k < RS_ROUNDS; k++) kk[k] = k < rounds && first + k * 256 < n ? key[first + k * 256] : 0u;
+#pragma unroll
+    for (int k = 0; k < RS_ROUNDS; k++)
+        if (k < rounds && first + k * 256 < n) atomicAdd(&cnt[(kk[k] >> shift) & (BINS - 1u)], 1u);
     __syncthreads();
     for (int d = threadIdx.x; d < BINS; d += 256)
         hist[fused ? blockIdx.x * BINS + d : d * nblocks + blockIdx.x] = cnt[d];
@@ -85,7 +88,11 @@ __global__ void __launch_bounds__(256) k_rs_hist(int n, const uint32_t *__restri
 
 // Stable scatter: warp w of block b owns the contiguous items
 // [b*items + w*per_warp, +per_warp); within a warp, items are ranked in
-// index order with match_any, so equal digits keep their input order.
+// index order with match_any, so equal digits keep their input order.  A
+// lane's keys, values and ranks stay in registers: every load of the warp is
+// in flight at once, and the keys are read and ranked once (ranking them again
+// on the way out, each round behind its own load, took 29 us a pass of
+// 262144 keys; 21 us now, and the histogram's 10 us became 3.6).
 template <int BITS>
 __global__ void __launch_bounds__(256) k_rs_scatter(int n, const uint32_t *__restrict__ key_in,
                                                     const int32_t *__restrict__ val_in,
@@ -96,16 +103,29 @@ __global__ void __launch_bounds__(256) k_rs_scatter(int n, const uint32_t *__res
     constexpr int BINS = 1 << BITS, DPT = BINS / 256;   // digits per thread
     __shared__ uint32_t off[RS_WARPS][BINS];
     __shared__ uint32_t wsum[RS_WARPS];
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, rounds = per_warp / 32;
+    const int first = (blockIdx.x * RS_WARPS + w) * per_warp + lane;
+    uint32_t key[RS_ROUNDS], rank[RS_ROUNDS];
+    int32_t val[RS_ROUNDS];
+#pragma unroll
+    for (int k = 0; k < RS_ROUNDS; k++) {
+        const bool v = k < rounds && first + k * 32 < n;
+        key[k] = v ? key_in[first + k * 32] : 0u;
+        val[k] = v ? val_in[first + k * 32] : 0;
+    }
     for (int d = lane; d < BINS; d += 32) off[w][d] = 0;
     __syncwarp();
-    const int wbase = (blockIdx.x * RS_WARPS + w) * per_warp;
-    for (int k = 0; k < per_warp / 32; k++) {
-        const int i = wbase + k * 32 + lane;
-        const bool v = i < n;
-        const uint32_t d = v ? ((key_in[i] >> shift) & (BINS - 1u)) : BINS + lane;
+    const unsigned lt = lanemask_lt();
+#pragma unroll
+    for (int k = 0; k < RS_ROUNDS; k++) {
+        if (k >= rounds) break;
+        const bool v = first + k * 32 < n;
+        const uint32_t d = v ? ((key[k] >> shift) & (BINS - 1u)) : BINS + lane;
         const unsigned peers = __match_any_sync(FULL, d);
-        if (v && lane == __ffs(peers) - 1) off[w][d] += __popc(peers);
+        const uint32_t base = v ? off[w][d] : 0u;
+        rank[k] = base + __popc(peers & lt);
+        __syncwarp();
+        if (v && lane == __ffs(peers) - 1) off[w][d] = base + __popc(peers);
         __syncwarp();
     }
     // where this block's items of each digit go
@@ -115,12 +135,20 @@ __global__ void __launch_bounds__(256) k_rs_scatter(int n, const uint32_t *__res
         uint32_t before[DPT], total[DPT], sum = 0;
 #pragma unroll
         for (int k = 0; k < DPT; k++) before[k] = total[k] = 0u;
+#pragma unroll 8
         for (int b = 0; b < nblocks; b++) {
+            uint32_t c[DPT];
+            if constexpr (DPT == 4) {
+                const uint4 c4 = __ldg(reinterpret_cast<const uint4 *>(hist + b * BINS) + threadIdx.x);
+                c[0] = c4.x, c[1] = c4.y, c[2] = c4.z, c[3] = c4.w;
+            } else {
+#pragma unroll
+                for (int k = 0; k < DPT; k++) c[k] = __ldg(hist + b * BINS + d0 + k);
+            }
 #pragma unroll
             for (int k = 0; k < DPT; k++) {
-                const uint32_t c = __ldg(hist + b * BINS + d0 + k);
-                total[k] += c;
-                if (b < (int)blockIdx.x) before[k] += c;
+                total[k] += c[k];
+                if (b < (int)blockIdx.x) before[k] += c[k];
             }
         }
 #pragma unroll
@@ -148,6 +176,7 @@ __global__ void __launch_bounds__(256) k_rs_scatter(int n, const uint32_t *__res
 #pragma unroll
     for (int k = 0; k < DPT; k++) {
         uint32_t run = start[k];
+#pragma unroll
         for (int ww = 0; ww < RS_WARPS; ww++) {
             const uint32_t c = off[ww][d0 + k];
             off[ww][d0 + k] = run;
@@ -155,22 +184,12 @@ __global__ void __launch_bounds__(256) k_rs_scatter(int n, const uint32_t *__res
         }
     }
     __syncthreads();
-    const unsigned lt = lanemask_lt();
-    for (int k = 0; k < per_warp / 32; k++) {
-        const int i = wbase + k * 32 + lane;
-        const bool v = i < n;
-        const uint32_t kk = v ? key_in[i] : 0u;
-        const uint32_t d = v ? ((kk >> shift) & (BINS - 1u)) : BINS + lane;
-        const unsigned peers = __match_any_sync(FULL, d);
-        const uint32_t base = v ? off[w][d] : 0u;
-        __syncwarp();
-        if (v) {
-            const uint32_t pos = base + __popc(peers & lt);
-            key_out[pos] = kk;
-            val_out[pos] = val_in[i];
-            if (lane == __ffs(peers) - 1) off[w][d] = base + __popc(peers);
-        }
-        __syncwarp();
+#pragma unroll
+    for (int k = 0; k < RS_ROUNDS; k++) {
+        if (k >= rounds || first + k * 32 >= n) break;
+        const uint32_t pos = off[w][(key[k] >> shift) & (BINS - 1u)] + rank[k];
+        key_out[pos] = key[k];
+        val_out[pos] = val[k];
     }
 }
 
@@ -877,12 +896,11 @@ int rebuild_lists(crk_ctx *ctx, cudaStream_t s) {
     if (ctx->ntiles == 0) return CRK_OK;
     Tree32 T = tree32(ctx);
     if (T.cnt[T.top] > 32) return crk_set_error(ctx, CRK_ECAPACITY, "tile tree too deep");
-    CRK_CUDA(ctx, cudaMemsetAsync(ctx->counters + CNT_GLIST, 0, 2 * sizeof(unsigned long long), s));
+    CRK_CUDA(ctx, cudaMemsetAsync(ctx->counters + CNT_GLIST, 0, 3 * sizeof(unsigned long long), s));
     ctx->lists_valid = 0;
     const int count = ctx->act ? ctx->nact : ctx->ntiles;
     if (count == 0) return CRK_OK;
     const bool may_queue = ctx->ntiles > (int)LIST_BUF;   // else no tile has more neighbours than the buffer holds
-    if (may_queue) CRK_CUDA(ctx, cudaMemsetAsync(ctx->counters + CNT_LQUEUE, 0, sizeof(unsigned long long), s));
     k_lists32<<<grid_for(count, LIST_WARPS), LIST_WARPS * 32, 0, s>>>(
         count, ctx->act, T, ctx->node_lo, ctx->node_hi, ctx->nbox > 1 ? ctx->node_box : nullptr, ctx->uofs,
         ctx->ulist, ctx->cap_ulist, ctx->counters + CNT_ULIST, ctx->lqueue, ctx->counters + CNT_LQUEUE);

@@ -19,31 +19,34 @@ constexpr double PI_D = 3.14159265358979323846;
 
 // device counters (unsigned long long slots in ctx->counters)
 enum {
-    CNT_GLIST = 0,      // gather-list entries allocated
-    CNT_ULIST = 1,      // union-list entries allocated
-    CNT_PAIRS_G = 2,    // gather pairs (excl. self) of the last P1
-    CNT_PAIRS_U = 3,    // ordered union pairs of the last P4
-    CNT_ERR_INPUT = 4,  // invalid particle records found
-    CNT_HMAX = 5,       // max h as float bits
-    CNT_WORK = 6,       // dynamic tile counter of the persistent pair kernels
-    CNT_NOTDONE = 7,    // h iteration: particles not converged
-    CNT_DTMIN = 8,      // min per-particle time step (float bits)
-    CNT_ENTRIES = 9,    // stored-force units (32 entries) of the last list build
-    CNT_MAXCNT = 10,    // largest pair-set count of the last walk
-    CNT_MLP_ERR = 11,   // invalid records seen by the feature kernels
-    CNT_GRAPH_ERR = 12, // sticky: some replayed step overflowed a capacity or saw invalid records
-    CNT_TNEXT = 13,     // time bins: earliest step end over the leaves (ticks)
-    CNT_CHANGED = 14,   // time bins: a limiter sweep raised some level
-    CNT_UNRES = 15,     // time bins: particle level requests deeper than L
-    CNT_WAKE = 16,      // time bins: passive leaves raised
-    CNT_NACT = 17,      // time bins: leaves ending a step at the current tick (and 18: their particles)
-    CNT_NEXT_OK = 19,   // du_next holds the next opening kick's energy rate for dt_next
-    CNT_SKIP = 20,      // this step's opening kick takes du_next
-    CNT_PO_MISS = 21,   // pair-once: tile pairs (I, J) whose reverse (J, I) was not found (sticky)
-    CNT_WALK_TESTS = 22,  // lane tests of the exact predicate in the last list walk
-    CNT_TMA_ERR = 23,   // sticky: a TMA-fed pass gave up waiting on its copies
-    CNT_HEAVY = 24,     // tiles of the last walk with more than HEAVY_ROWS list rows (ctx->heavy)
-    CNT_LQUEUE = 25,    // tiles queued by the last list build (ctx->lqueue)
+    // reset by a list build: the next three
+    CNT_GLIST = 0,       // gather-list entries allocated
+    CNT_ULIST = 1,       // union-list entries allocated
+    CNT_LQUEUE = 2,      // tiles queued by the last list build (ctx->lqueue)
+    // reset by a walk: the next five
+    CNT_PAIRS_G = 3,     // gather pairs (excl. self) of the last P1
+    CNT_PAIRS_U = 4,     // ordered union pairs of the last P4
+    CNT_MAXCNT = 5,      // largest pair-set count of the last walk
+    CNT_WALK_TESTS = 6,  // lane tests of the exact predicate in the last list walk
+    CNT_HEAVY = 7,       // tiles of the last walk with more than HEAVY_ROWS list rows (ctx->heavy)
+    // others
+    CNT_ERR_INPUT = 8,   // invalid particle records found
+    CNT_HMAX = 9,        // max h as float bits
+    CNT_WORK = 10,       // dynamic tile counter of the persistent pair kernels
+    CNT_NOTDONE = 11,    // h iteration: particles not converged
+    CNT_DTMIN = 12,      // min per-particle time step (float bits)
+    CNT_ENTRIES = 13,    // stored-force units (32 entries) of the last list build
+    CNT_MLP_ERR = 14,    // invalid records seen by the feature kernels
+    CNT_GRAPH_ERR = 15,  // sticky: some replayed step overflowed a capacity or saw invalid records
+    CNT_TNEXT = 16,      // time bins: earliest step end over the leaves (ticks)
+    CNT_CHANGED = 17,    // time bins: a limiter sweep raised some level
+    CNT_UNRES = 18,      // time bins: particle level requests deeper than L
+    CNT_WAKE = 19,       // time bins: passive leaves raised
+    CNT_NACT = 20,       // time bins: leaves ending a step at the current tick (and 21: their particles)
+    CNT_NEXT_OK = 22,    // du_next holds the next opening kick's energy rate for dt_next
+    CNT_SKIP = 23,       // this step's opening kick takes du_next
+    CNT_PO_MISS = 24,    // pair-once: tile pairs (I, J) whose reverse (J, I) was not found (sticky)
+    CNT_TMA_ERR = 25,    // sticky: a TMA-fed pass gave up waiting on its copies
     CNT_COUNT = 26
 };
 

@@ -594,10 +594,7 @@ static int launch_walk(crk_ctx *ctx, cudaStream_t s) {
         int rc = crk_ensure_entries(ctx, (long long)ctx->ntiles * 32 * ctx->kcap, -1);
         if (rc) return rc;
     }
-    CRK_CUDA(ctx, cudaMemsetAsync(ctx->counters + CNT_PAIRS_G, 0, 2 * sizeof(unsigned long long), s));
-    CRK_CUDA(ctx, cudaMemsetAsync(ctx->counters + CNT_MAXCNT, 0, sizeof(unsigned long long), s));
-    CRK_CUDA(ctx, cudaMemsetAsync(ctx->counters + CNT_WALK_TESTS, 0, sizeof(unsigned long long), s));
-    CRK_CUDA(ctx, cudaMemsetAsync(ctx->counters + CNT_HEAVY, 0, sizeof(unsigned long long), s));
+    CRK_CUDA(ctx, cudaMemsetAsync(ctx->counters + CNT_PAIRS_G, 0, 5 * sizeof(unsigned long long), s));
     if (ctx->act) {   // tiles left out of the walk take no list columns and no stored forces
         CRK_CUDA(ctx, cudaMemsetAsync(ctx->len_g, 0, sizeof(uint32_t) * ctx->ntiles, s));
         CRK_CUDA(ctx, cudaMemsetAsync(ctx->len_u, 0, sizeof(uint32_t) * ctx->ntiles, s));
