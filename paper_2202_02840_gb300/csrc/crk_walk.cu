@@ -16,6 +16,7 @@
 namespace crk {
 
 constexpr int WALK_WARPS = 8;
+constexpr int WALK_WIDE = 8;       // fewer tiles than this per SM: CTAs of 32 warps
 constexpr int WALK_ALL = 20;       // fewer tiles than this per SM: every tile is shared by a CTA's warps
 constexpr int WALK_HEAVY = 384;    // candidate tiles above which a tile is shared
 
@@ -129,6 +130,14 @@ struct WalkShm {
     uint4 r[RING];                      // x, y, z relative or fixed point; H^2
     uint32_t id[VOL ? 1 : RING];        // sorted index
     int32_t box[BATCH ? RING : 1];
+};
+
+// Shared memory of a CTA of W warps.
+template <bool LISTS, bool VOL, bool BATCH, int W>
+struct WalkCta {
+    WalkShm<VOL, BATCH> shm[W];
+    WalkMasks masks[LISTS ? W : 1];
+    int part[2][W][32];
 };
 
 // A tile and this lane's particle of it.
@@ -250,45 +259,35 @@ __device__ __forceinline__ void walk_range(const WalkArgs &a, const WalkTile &T,
     // while the current tile is tested (each is otherwise a dependent L2 trip)
     const uint32_t *tl = a.tiles + lo.x;
     int J1 = t0 < t1 ? (int)__ldg(tl + t0) : 0, J2 = t0 + 1 < t1 ? (int)__ldg(tl + t0 + 1) : 0;
-    uint4 lo1 = make_uint4(0, 0, 0, 0), hi1 = lo1, qn = lo1;
+    uint4 qn = make_uint4(0, 0, 0, 0);
+    uint32_t H1 = 0;
     if (t0 < t1) {
-        lo1 = __ldg(a.tlo + J1);
-        hi1 = __ldg(a.thi + J1);
+        H1 = __ldg(&a.tlo[J1].w);
         if (J1 * TILE + lane < a.n) qn = __ldg(a.q4 + J1 * TILE + lane);
     }
     for (int t = t0; t < t1; t++) {
         const int J = J1;
-        const uint4 Jlo = lo1, Jhi = hi1, qc = qn;
+        const uint4 qc = qn;
+        const uint32_t JH = H1;
         J1 = J2;
         if (t + 2 < t1) J2 = (int)__ldg(tl + t + 2);
         if (t + 1 < t1) {
-            lo1 = __ldg(a.tlo + J1);
-            hi1 = __ldg(a.thi + J1);
+            H1 = __ldg(&a.tlo[J1].w);
             if (J1 * TILE + lane < a.n) qn = __ldg(a.q4 + J1 * TILE + lane);
         }
         const int j0 = J * TILE;
         const int cnt = min(TILE, a.n - j0);
         const uint4 Ilo = S.B.lo;
-        const uint32_t Jex = Jhi.x - Jlo.x, Jey = Jhi.y - Jlo.y, Jez = Jhi.z - Jlo.z;
-        const uint32_t HJ = VOL ? 0u : Jlo.w;   // the volumes take gather(i) only
-        const uint32_t R = max(Ilo.w, Jlo.w), M = S.B.Ie + R;   // warp-uniform
-        // Skip a tile that no lane's sphere touches; keep a particle whose gap to
-        // the tile's box is below the larger support.  Both conservative, so the
-        // lists are unchanged.
-        bool near, keep;
+        const uint32_t R = VOL ? Ilo.w : max(Ilo.w, JH), M = S.B.Ie + R;   // warp-uniform
+        // Keep a particle whose gap to the tile's box is below the larger support:
+        // conservative, so the lists are unchanged.  (Skipping candidates whose
+        // box no lane's sphere touches, too, took 30 instructions a candidate
+        // and dropped few: 128^3 clustered 3.80 ms with that test, 3.20 without.)
+        bool keep;
         float jx = 0.f, jy = 0.f, jz = 0.f;
         const float edge = T.raw ? (float)R : (float)M;
         const float mrg = (T.raw ? MARGIN_INT : MARGIN_REL) * (edge * edge);
         if (!T.raw) {
-            const int ox = (int)(Jlo.x - Ilo.x), oy = (int)(Jlo.y - Ilo.y), oz = (int)(Jlo.z - Ilo.z);
-            const float lx = (float)ox, ly = (float)oy, lz = (float)oz;
-            const float gx = fmaxf(fmaxf(lx - T.fx, T.fx - (float)(int)((uint32_t)ox + Jex)), 0.f);
-            const float gy = fmaxf(fmaxf(ly - T.fy, T.fy - (float)(int)((uint32_t)oy + Jey)), 0.f);
-            const float gz = fmaxf(fmaxf(lz - T.fz, T.fz - (float)(int)((uint32_t)oz + Jez)), 0.f);
-            const float re = fmaxf(T.Hf, (float)HJ);
-            // (offsets of a box that spans much of the period may not be its nearest image)
-            near = T.valid && (M + (unsigned long long)max(max(Jex, Jey), Jez) >= 0x80000000ull ||
-                               fmaf(gx, gx, fmaf(gy, gy, gz * gz)) < fmaf(re, re, mrg));
             jx = (float)(int)(qc.x - Ilo.x);
             jy = (float)(int)(qc.y - Ilo.y);
             jz = (float)(int)(qc.z - Ilo.z);
@@ -297,10 +296,7 @@ __device__ __forceinline__ void walk_range(const WalkArgs &a, const WalkTile &T,
             const float rj = (float)(VOL ? Ilo.w : max(qc.w, Ilo.w));
             keep = lane < cnt && fmaf(hx, hx, fmaf(hy, hy, hz * hz)) < fmaf(rj, rj, mrg);
         } else {
-            const uint4 qi = own_record(a, T), Ihi = __ldg(a.thi + T.tile);
-            const float gx = point_gap(qi.x, Jlo.x, Jhi.x), gy = point_gap(qi.y, Jlo.y, Jhi.y),
-                        gz = point_gap(qi.z, Jlo.z, Jhi.z), re = fmaxf(T.Hf, (float)HJ);
-            near = T.valid && fmaf(gx, gx, fmaf(gy, gy, gz * gz)) < fmaf(re, re, mrg);
+            const uint4 Ihi = __ldg(a.thi + T.tile);
             const float hx = point_gap(qc.x, Ilo.x, Ihi.x), hy = point_gap(qc.y, Ilo.y, Ihi.y),
                         hz = point_gap(qc.z, Ilo.z, Ihi.z), rj = (float)(VOL ? Ilo.w : max(qc.w, Ilo.w));
             keep = lane < cnt && fmaf(hx, hx, fmaf(hy, hy, hz * hz)) < fmaf(rj, rj, mrg);
@@ -309,7 +305,6 @@ __device__ __forceinline__ void walk_range(const WalkArgs &a, const WalkTile &T,
         int32_t bj = 0;
         if constexpr (BATCH) {
             const uint32_t Jb = __ldg(a.nbox + J);
-            near = near && (uint32_t)T.bi >= (Jb & 0xffffu) && (uint32_t)T.bi <= (Jb >> 16);
             mixed = T.Ib != Jb || (T.Ib & 0xffffu) != (T.Ib >> 16);
             bj = (int32_t)(Jb & 0xffffu);
             if (mixed && lane < cnt) {
@@ -317,7 +312,6 @@ __device__ __forceinline__ void walk_range(const WalkArgs &a, const WalkTile &T,
                 keep = keep && (uint32_t)bj >= (T.Ib & 0xffffu) && (uint32_t)bj <= (T.Ib >> 16);
             }
         }
-        if (__ballot_sync(0xffffffffu, near) == 0u) continue;
         const unsigned mask = __ballot_sync(0xffffffffu, keep);
         if (mask == 0u) continue;
         const uint32_t at = head + (uint32_t)__popc(mask & lanemask_lt());
@@ -364,18 +358,20 @@ __device__ __forceinline__ void walk_range(const WalkArgs &a, const WalkTile &T,
 // warps: tiles with more than a.heavy candidates (a run of the Morton order
 // that jumps across the box: at 64^3 clustered the largest has 16 times the
 // mean's candidates), and every tile of a set that does not fill the chip.
-// Those are shared by the eight warps of a CTA, each taking a range of the
-// candidates: a first sweep counts and keeps its masks, the prefix over the
+// Those are shared by the W warps of a CTA, each taking a range of the
+// candidates (W = 32 below WALK_WIDE tiles per SM, where the CTA of the slowest
+// tile is the time: Sedov 17^3 97 -> 43 us, 16^3 36 -> 24, the tiles of a 48^3
+// cycle 2.20 -> 1.46 ms; at 13 tiles per SM it is even, and a loss at 20): a
+// first sweep counts and keeps its masks, the prefix over the
 // warps gives each its place in the lists, and the entries are written from the
 // masks (a warp with more than MASKS batches sweeps again), so the lists are
 // exactly the one-warp walk's.
-template <bool LISTS, bool VOL, bool BATCH>
-__global__ void __launch_bounds__(WALK_WARPS * 32, 4) k_walk(WalkArgs a) {
-    __shared__ WalkShm<VOL, BATCH> shm[WALK_WARPS];
-    __shared__ int part[2][WALK_WARPS][32];
-    __shared__ WalkMasks masks[LISTS ? WALK_WARPS : 1];
+template <bool LISTS, bool VOL, bool BATCH, int W>
+__global__ void __launch_bounds__(W * 32, 32 / W) k_walk(WalkArgs a) {
+    extern __shared__ __align__(16) unsigned char walk_smem[];
+    WalkCta<LISTS, VOL, BATCH, W> &C = *reinterpret_cast<WalkCta<LISTS, VOL, BATCH, W> *>(walk_smem);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    WalkShm<VOL, BATCH> &S = shm[w];
+    WalkShm<VOL, BATCH> &S = C.shm[w];
     const int kcap = a.kcap;
     // V_i, N_i from the kernel sum of a lane
     auto volume = [&](const WalkTile &T, float acc) {
@@ -428,7 +424,7 @@ __global__ void __launch_bounds__(WALK_WARPS * 32, 4) k_walk(WalkArgs a) {
     };
     auto shared_tile = [&](int tile, uint2 lo) {   // by all warps of the CTA
         const WalkTile T = walk_tile<BATCH>(a, tile, lane, S.B);
-        const int nt = (int)lo.y, chunk = (nt + WALK_WARPS - 1) / WALK_WARPS;
+        const int nt = (int)lo.y, chunk = (nt + W - 1) / W;
         const int t0 = min(nt, w * chunk), t1 = min(nt, t0 + chunk);
         uint32_t kept = 0;
         if constexpr (VOL) {
@@ -437,16 +433,16 @@ __global__ void __launch_bounds__(WALK_WARPS * 32, 4) k_walk(WalkArgs a) {
             float acc = 0.f;
             walk_range<VOL, BATCH>(a, T, lane, lo, t0, t1, S, kept,
                                    [&](uint32_t ring, int c) { sum_batch(T, qi, inv_h, ring, c, acc); });
-            part[0][w][lane] = __float_as_int(acc);
+            C.part[0][w][lane] = __float_as_int(acc);
             __syncthreads();
             if (w == 0) {
-                for (int v = 1; v < WALK_WARPS; v++) acc += __int_as_float(part[0][v][lane]);
+                for (int v = 1; v < W; v++) acc += __int_as_float(C.part[0][v][lane]);
                 if (T.valid) volume(T, acc);
                 close(T, 0, 0);
             }
         } else {
             uint32_t *const col0 = a.ent + (size_t)tile * kcap * 32;
-            WalkMasks &K = masks[w];
+            WalkMasks &K = C.masks[w];
             int cg = 0, co = 0, nb = 0;
             walk_range<VOL, BATCH>(a, T, lane, lo, t0, t1, S, kept, [&](unsigned gm, unsigned jm, uint32_t ring) {
                 jm &= ~gm;
@@ -460,14 +456,14 @@ __global__ void __launch_bounds__(WALK_WARPS * 32, 4) k_walk(WalkArgs a) {
                 nb++;
             });
             if (lane == 0) atomicAdd(a.tests, 32ull * kept);
-            part[0][w][lane] = cg;
-            part[1][w][lane] = co;
+            C.part[0][w][lane] = cg;
+            C.part[1][w][lane] = co;
             __syncthreads();
             int pg = 0, po = 0, tg = 0, to = 0;   // this warp's place, the totals
-            for (int v = 0; v < WALK_WARPS; v++) {
+            for (int v = 0; v < W; v++) {
                 if (v == w) pg = tg, po = to;
-                tg += part[0][v][lane];
-                to += part[1][v][lane];
+                tg += C.part[0][v][lane];
+                to += C.part[1][v][lane];
             }
             Seg<true> G{0u, 0u, 0u, pg, pg, (int)block_at(pg / LB, lane)};
             Seg<true> O{0u, 0u, 0u, po, po, (int)block_at(kcap / LB - 1 - po / LB, lane)};
@@ -485,7 +481,7 @@ __global__ void __launch_bounds__(WALK_WARPS * 32, 4) k_walk(WalkArgs a) {
             if (T.valid) {
                 G.close(col0, kcap);
                 O.close(col0, kcap);
-                if (w == WALK_WARPS - 1) {   // its segments end where the lists end
+                if (w == W - 1) {   // its segments end where the lists end
                     G.pad((uint32_t)T.i, col0, kcap);
                     O.pad((uint32_t)T.i, col0, kcap);
                 }
@@ -512,7 +508,7 @@ __global__ void __launch_bounds__(WALK_WARPS * 32, 4) k_walk(WalkArgs a) {
         }
         return;
     }
-    const int tw = ((int)blockIdx.x - a.hblocks) * WALK_WARPS + w;
+    const int tw = ((int)blockIdx.x - a.hblocks) * W + w;
     if (tw >= a.ntiles) return;
     const int tile = a.act ? a.act[tw] : tw;
     const uint2 lo = a.ofs[tile];
@@ -589,6 +585,24 @@ static WalkArgs walk_args(crk_ctx *ctx) {
     return a;
 }
 
+template <bool LISTS, bool VOL, bool BATCH, int W>
+static int launch_walk_wide(crk_ctx *ctx, const WalkArgs &a, cudaStream_t s) {
+    using Cta = WalkCta<LISTS, VOL, BATCH, W>;
+    if (sizeof(Cta) > 48 * 1024)
+        CRK_CUDA(ctx, cudaFuncSetAttribute(k_walk<LISTS, VOL, BATCH, W>,
+                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Cta)));
+    const int g = a.hblocks + (a.all ? 0 : grid_for(a.ntiles, W));
+    k_walk<LISTS, VOL, BATCH, W><<<g, W * 32, sizeof(Cta), s>>>(a);
+    return CRK_OK;
+}
+
+template <bool LISTS, bool VOL, bool BATCH>
+static int launch_walk_form(crk_ctx *ctx, const WalkArgs &a, cudaStream_t s) {
+    const int nsm = ctx->nsm > 0 ? ctx->nsm : 152;
+    if (a.ntiles < WALK_WIDE * nsm) return launch_walk_wide<LISTS, VOL, BATCH, 32>(ctx, a, s);
+    return launch_walk_wide<LISTS, VOL, BATCH, WALK_WARPS>(ctx, a, s);
+}
+
 static int launch_walk(crk_ctx *ctx, cudaStream_t s) {
     if (!ctx->volumes_only) {
         int rc = crk_ensure_entries(ctx, (long long)ctx->ntiles * 32 * ctx->kcap, -1);
@@ -602,16 +616,17 @@ static int launch_walk(crk_ctx *ctx, cudaStream_t s) {
     }
     prof_begin(ctx, PROF_LISTS, s);
     const WalkArgs a = walk_args(ctx);
-    const int g = a.hblocks + (a.all ? 0 : grid_for(a.ntiles, WALK_WARPS));
     const bool b = ctx->nbox > 1;
+    int rc = CRK_OK;
     if (ctx->volumes_only && b)
-        k_walk<false, true, true><<<g, WALK_WARPS * 32, 0, s>>>(a);
+        rc = launch_walk_form<false, true, true>(ctx, a, s);
     else if (ctx->volumes_only)
-        k_walk<false, true, false><<<g, WALK_WARPS * 32, 0, s>>>(a);
+        rc = launch_walk_form<false, true, false>(ctx, a, s);
     else if (b)
-        k_walk<true, false, true><<<g, WALK_WARPS * 32, 0, s>>>(a);
+        rc = launch_walk_form<true, false, true>(ctx, a, s);
     else
-        k_walk<true, false, false><<<g, WALK_WARPS * 32, 0, s>>>(a);
+        rc = launch_walk_form<true, false, false>(ctx, a, s);
+    if (rc) return rc;
     ++ctx->launches;
     prof_end(ctx, s);
     CRK_LAUNCH_CHECK(ctx, "neighbour walk");
