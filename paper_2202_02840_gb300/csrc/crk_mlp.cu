@@ -194,44 +194,41 @@ __global__ void k_feat_table(int kf, const int32_t *__restrict__ fcnt, float *__
     out[1] = make_float4(__logf(1.f + (cls[0] + cls[1] + cls[2] + cls[3])), 0.f, 0.f, 0.f);
 }
 
-// Features 2t and 2t+1 of row i for lane t (0..3) of a quad.
-__device__ __forceinline__ float2 quad_features(const FeatArgs &a, int i, int t, float &h_out, float &N_out) {
-    bool valid = i < a.n;
-    float4 p = valid ? a.pos_h[i] : make_float4(0.5f, 0.5f, 0.5f, 1.f);
-    float h = p.w;
-    float N = (a.Nngb && valid) ? __ldg(&a.Nngb[i]) : 0.f;
-    h_out = h;
-    N_out = N;
-    float2 f = make_float2(0.f, 0.f);
-    if (!valid) return f;
-    if (t < 3) {
-        f = __ldg(reinterpret_cast<const float2 *>(a.ftab) + 4 * (size_t)feat_cell(p, a.kf) + t);
-        if (t == 2) f.y = __logf(h) + a.log_cbrt_n;
-    } else {
-        float dv = 0.f;
-        if (a.gradv) {
-            const float *gv = a.gradv + (size_t)a.gv_stride * i;
-            dv = __ldg(gv) + __ldg(gv + 4) + __ldg(gv + 8);
-        }
-        f.x = a.dt * dv;
-        f.y = a.Nngb ? __logf(N * a.inv_N_res) : 0.f;
+// h and count of row i, and its 8 features (zeros past the last row).
+__device__ __forceinline__ void row_features(const FeatArgs &a, int i, float (&f)[8], float &h, float &N) {
+#pragma unroll
+    for (int k = 0; k < 8; k++) f[k] = 0.f;
+    h = 1.f;
+    N = 0.f;
+    if (i >= a.n) return;
+    const float4 p = a.pos_h[i];
+    float dv = 0.f;
+    if (a.Nngb) N = __ldg(&a.Nngb[i]);
+    if (a.gradv) {
+        const float *gv = a.gradv + (size_t)a.gv_stride * i;
+        dv = __ldg(gv) + __ldg(gv + 4) + __ldg(gv + 8);
     }
-    return f;
+    const float4 *c = reinterpret_cast<const float4 *>(a.ftab) + 2 * (size_t)feat_cell(p, a.kf);
+    const float4 cls = __ldg(c);
+    h = p.w;
+    f[0] = cls.x, f[1] = cls.y, f[2] = cls.z, f[3] = cls.w;
+    f[4] = __ldg(&c[1].x);
+    f[5] = __logf(h) + a.log_cbrt_n;
+    f[6] = a.dt * dv;
+    f[7] = a.Nngb ? __logf(N * a.inv_N_res) : 0.f;
 }
 
 // feat[8i..8i+7] and, with pos_conv, target[i] = log(h_conv / h_prev)
 __global__ void k_features(FeatArgs a, const float4 *__restrict__ pos_conv, float *__restrict__ feat,
                            float *__restrict__ target) {
-    int lane = threadIdx.x & 31;
-    int t = lane & 3;
-    // every lane of the warp takes part in the quad shuffles; rows >= n only skip the stores
-    int i = (int)(((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 2);
-    float h, N;
-    float2 f = quad_features(a, i, t, h, N);
-    if (i < a.n) {
-        reinterpret_cast<float2 *>(feat)[4 * (size_t)i + t] = f;
-        if (t == 0 && pos_conv && target) target[i] = logf(pos_conv[i].w / h_reference(a, h, N));
-    }
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= a.n) return;
+    float f[8], h, N;
+    row_features(a, i, f, h, N);
+    float2 *out = reinterpret_cast<float2 *>(feat) + 4 * (size_t)i;   // 8-byte alignment is what forward asks for
+#pragma unroll
+    for (int t = 0; t < 4; t++) out[t] = make_float2(f[2 * t], f[2 * t + 1]);
+    if (pos_conv && target) target[i] = logf(pos_conv[i].w / h_reference(a, h, N));
 }
 
 }  // namespace
@@ -321,59 +318,90 @@ __device__ __forceinline__ float quad_sum(float v) {
 }
 
 // Inference: MODE 0 reads feat (8n, row-major) and writes y; MODE 1 computes
-// the features in place and writes the proposal into pos.w.  One warp per
-// 16-row tile, tiles strided over the grid.
+// the features in place and writes the proposal into pos.w.  A warp takes
+// `span` rows, 32 in two 16-row tiles, or 16 where that still gives every warp
+// at most one; spans are strided over the grid.  What belongs to a row alone
+// (its loads, features and the proposal from y) is one lane's work, passed to
+// and from the quads' fragments through shared memory: the 64 tanh of a tile
+// keep the SFU busy for 512 cycles, and roots, logs and conversions that the
+// quads repeated for their rows kept it for 430 more (2097152 rows 164 us so,
+// 123 us now).
+struct RowShm {
+    uint32_t x[32][4];   // features, BF16 pairs
+    float y[32];
+};
+
 template <int MODE>
-__global__ void __launch_bounds__(256, 4) k_mlp_fwd(int n, const float *__restrict__ W, const float *__restrict__ feat,
-                                                  float *__restrict__ y_out, FeatArgs fa, float4 *pos_out, float tol,
-                                                  float h_min, float h_max, float N_res) {
+__global__ void __launch_bounds__(256, 4) k_mlp_fwd(int n, int span, const float *__restrict__ W,
+                                                    const float *__restrict__ feat, float *__restrict__ y_out,
+                                                    FeatArgs fa, float4 *pos_out, float tol, float h_min,
+                                                    float h_max, float N_res) {
     __shared__ __align__(16) FwdShm S;
+    __shared__ __align__(16) RowShm rows[MODE == 1 ? 8 : 1];
     stage_fwd<256, false>(W, S);
     float b3 = W[OFF_B3];
     __syncthreads();
     int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     uint32_t w1f[8];
     load_w1f(S, g, t, w1f);
-    int wpb = blockDim.x >> 5;
-    int ntile = (n + 15) >> 4;
-    for (int tile = blockIdx.x * wpb + (threadIdx.x >> 5); tile < ntile; tile += gridDim.x * wpb) {
-        int r0 = tile * 16 + g, r1 = r0 + 8;
-        float2 x0 = make_float2(0.f, 0.f), x1 = x0;
-        float h0 = 0.f, h1 = 0.f, N0 = 0.f, N1 = 0.f;
-        if (MODE == 0) {
-            if (r0 < n) x0 = __ldg(reinterpret_cast<const float2 *>(feat) + 4 * (size_t)r0 + t);
-            if (r1 < n) x1 = __ldg(reinterpret_cast<const float2 *>(feat) + 4 * (size_t)r1 + t);
-        } else {
-            x0 = quad_features(fa, r0, t, h0, N0);
-            x1 = quad_features(fa, r1, t, h1, N1);
+    const int wpb = blockDim.x >> 5, w = threadIdx.x >> 5;
+    const int nspan = (n + span - 1) / span;
+    RowShm &R = rows[MODE == 1 ? w : 0];
+    for (int sp = blockIdx.x * wpb + w; sp < nspan; sp += gridDim.x * wpb) {
+        const int base = sp * span, row = base + lane;
+        float h = 1.f, N = 0.f;
+        if (MODE == 1) {
+            if (lane < span) {
+                float f[8];
+                row_features(fa, row, f, h, N);
+                *reinterpret_cast<uint4 *>(R.x[lane]) = make_uint4(pack_bf16(f[0], f[1]), pack_bf16(f[2], f[3]),
+                                                                   pack_bf16(f[4], f[5]), pack_bf16(f[6], f[7]));
+            }
+            __syncwarp();
         }
-        uint32_t A1[4][4];
-        float unused[8][4];
-        layer1<false>(pack_bf16(x0.x, x0.y), pack_bf16(x1.x, x1.y), w1f, S, t, A1, unused);
-        float y0 = 0.f, y1 = 0.f;
+#pragma unroll 1
+        for (int o = 0; o < span; o += 16) {
+            uint32_t xa0, xa1;
+            const int r0 = base + o + g, r1 = r0 + 8;
+            if (MODE == 0) {
+                float2 x0 = make_float2(0.f, 0.f), x1 = x0;
+                if (r0 < n) x0 = __ldg(reinterpret_cast<const float2 *>(feat) + 4 * (size_t)r0 + t);
+                if (r1 < n) x1 = __ldg(reinterpret_cast<const float2 *>(feat) + 4 * (size_t)r1 + t);
+                xa0 = pack_bf16(x0.x, x0.y);
+                xa1 = pack_bf16(x1.x, x1.y);
+            } else {
+                xa0 = R.x[o + g][t];
+                xa1 = R.x[o + g + 8][t];
+            }
+            uint32_t A1[4][4];
+            float unused[8][4];
+            layer1<false>(xa0, xa1, w1f, S, t, A1, unused);
+            float y0 = 0.f, y1 = 0.f;
 #pragma unroll
-        for (int j = 0; j < 8; j++) {
-            float d[4];
-            layer2_tile(j, A1, S, g, t, d);
-            float wa = S.w3[8 * j + 2 * t], wb = S.w3[8 * j + 2 * t + 1];
-            const float2 a01 = silu2<false>(d[0], d[1]), a23 = silu2<false>(d[2], d[3]);
-            y0 = fmaf(wa, bf16r(a01.x), fmaf(wb, bf16r(a01.y), y0));
-            y1 = fmaf(wa, bf16r(a23.x), fmaf(wb, bf16r(a23.y), y1));
+            for (int j = 0; j < 8; j++) {
+                float d[4];
+                layer2_tile(j, A1, S, g, t, d);
+                float wa = S.w3[8 * j + 2 * t], wb = S.w3[8 * j + 2 * t + 1];
+                const float2 a01 = silu2<false>(d[0], d[1]), a23 = silu2<false>(d[2], d[3]);
+                y0 = fmaf(wa, bf16r(a01.x), fmaf(wb, bf16r(a01.y), y0));
+                y1 = fmaf(wa, bf16r(a23.x), fmaf(wb, bf16r(a23.y), y1));
+            }
+            y0 = Y_SCALE * (quad_sum(y0) + b3);
+            y1 = Y_SCALE * (quad_sum(y1) + b3);
+            if (MODE == 0) {
+                if (t == 0 && r0 < n) y_out[r0] = y0;
+                if (t == 0 && r1 < n) y_out[r1] = y1;
+            } else if (t < 2) {
+                R.y[o + 8 * t + g] = t ? y1 : y0;
+            }
         }
-        y0 = Y_SCALE * (quad_sum(y0) + b3);
-        y1 = Y_SCALE * (quad_sum(y1) + b3);
-        if (t == 0 && MODE == 0) {
-            if (r0 < n) y_out[r0] = y0;
-            if (r1 < n) y_out[r1] = y1;
-        }
-        if (t == 0 && MODE == 1) {
-#pragma unroll
-            for (int e = 0; e < 2; e++) {
-                int r = e ? r1 : r0;
-                float h = e ? h1 : h0, N = e ? N1 : N0, y = e ? y1 : y0;
-                bool done = fa.Nngb && fabsf(cbrtf(N_res / N) - 1.f) <= tol;
-                float hn = done ? h : fminf(fmaxf(h_reference(fa, h, N) * expf(y), h_min), h_max);
-                if (r < n) pos_out[r].w = hn;
+        if (MODE == 1) {
+            __syncwarp();
+            if (lane < span && row < n) {
+                const float root = cbrtf(N_res / N);
+                const bool done = fa.Nngb && fabsf(root - 1.f) <= tol;
+                const float ref = fa.Nngb ? h * root : h;
+                pos_out[row].w = done ? h : fminf(fmaxf(ref * expf(R.y[lane]), h_min), h_max);
             }
         }
     }
@@ -757,11 +785,12 @@ int need_weights(crk_ctx *ctx) {
     return CRK_OK;
 }
 
-int fwd_blocks(const crk_ctx *ctx, int n) {
-    int tiles = (n + 15) / 16;
-    int b = (tiles + 7) / 8;
-    int cap = 4 * (ctx->nsm > 0 ? ctx->nsm : 152);
-    return b < 1 ? 1 : (b > cap ? cap : b);
+// grid of k_mlp_fwd and the rows a warp takes at a time
+int fwd_blocks(const crk_ctx *ctx, int n, int *span) {
+    const int cap = 4 * (ctx->nsm > 0 ? ctx->nsm : 152);
+    *span = n <= cap * 8 * 16 ? 16 : 32;
+    const int b = (n + 8 * *span - 1) / (8 * *span);
+    return b > cap ? cap : b;
 }
 
 int train_launch(crk_ctx *ctx, int n, const float *feat, const float *target, const int32_t *rows, int n_rows,
@@ -886,7 +915,7 @@ extern "C" int crk_h_features(crk_ctx *ctx, int n, const float *pos_h, const flo
     int rc = count_cells(ctx, n, reinterpret_cast<const float4 *>(pos_h), kf, s);
     if (rc) return rc;
     FeatArgs fa = feat_args(ctx, n, pos_h, gradv, Nngb, dt, kf);
-    k_features<<<grid_for(4ll * n, 256), 256, 0, s>>>(fa, reinterpret_cast<const float4 *>(pos_conv), feat, target);
+    k_features<<<grid_for(n, 256), 256, 0, s>>>(fa, reinterpret_cast<const float4 *>(pos_conv), feat, target);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "features");
     return check_records(ctx, s);
@@ -901,7 +930,9 @@ extern "C" int crk_mlp_forward(crk_ctx *ctx, int n, const float *feat, float *y,
     cudaStream_t s = (cudaStream_t)stream;
     FeatArgs none{};
     prof_begin(ctx, PROF_MLP_FWD, s);
-    k_mlp_fwd<0><<<fwd_blocks(ctx, n), 256, 0, s>>>(n, ctx->mlp_w, feat, y, none, nullptr, 0.f, 0.f, 0.f, 0.f);
+    int span;
+    const int blocks = fwd_blocks(ctx, n, &span);
+    k_mlp_fwd<0><<<blocks, 256, 0, s>>>(n, span, ctx->mlp_w, feat, y, none, nullptr, 0.f, 0.f, 0.f, 0.f);
     ++ctx->launches;
     prof_end(ctx, s);
     CRK_LAUNCH_CHECK(ctx, "mlp forward");
@@ -921,7 +952,9 @@ extern "C" int crk_h_propose(crk_ctx *ctx, int n, float *pos_h, const float *gra
     rc = count_cells(ctx, n, reinterpret_cast<const float4 *>(pos_h), kf, s);
     if (rc) return rc;
     FeatArgs fa = feat_args(ctx, n, pos_h, gradv, Nngb, dt, kf);
-    k_mlp_fwd<1><<<fwd_blocks(ctx, n), 256, 0, s>>>(n, ctx->mlp_w, nullptr, nullptr, fa,
+    int span;
+    const int blocks = fwd_blocks(ctx, n, &span);
+    k_mlp_fwd<1><<<blocks, 256, 0, s>>>(n, span, ctx->mlp_w, nullptr, nullptr, fa,
                                                      reinterpret_cast<float4 *>(pos_h), tol, (float)ctx->p.h_min,
                                                      (float)ctx->p.h_max, (float)ctx->p.N_res);
     ++ctx->launches;
@@ -946,7 +979,9 @@ int propose_sorted(crk_ctx *ctx, int n, float4 *pos, const GvRec *gv, const floa
     FeatArgs fa = feat_args(ctx, n, reinterpret_cast<const float *>(pos), reinterpret_cast<const float *>(gv), Nn,
                             dt, kf);
     fa.gv_stride = 12;
-    k_mlp_fwd<1><<<fwd_blocks(ctx, n), 256, 0, s>>>(n, ctx->mlp_w, nullptr, nullptr, fa, pos, tol,
+    int span;
+    const int blocks = fwd_blocks(ctx, n, &span);
+    k_mlp_fwd<1><<<blocks, 256, 0, s>>>(n, span, ctx->mlp_w, nullptr, nullptr, fa, pos, tol,
                                                      (float)ctx->p.h_min, (float)ctx->p.h_max, (float)ctx->p.N_res);
     ++ctx->launches;
     prof_end(ctx, s);
