@@ -124,7 +124,8 @@ struct FeatArgs {
     const float *gradv;      // gv_stride n or null (div v = trace: entries 0, 4, 8 of a row)
     int gv_stride;           // 9 (caller's 3x3 rows) or 12 (the engine's padded records)
     const float *Nngb;       // n or null
-    const float *ftab;       // 8^kf rows of 8 floats: features 0 .. 4 of a cell
+    const int32_t *fcnt;     // particles per cell
+    const float *ftab;       // 8^kf rows of 8 floats: features 0 .. 4 of a cell; or null
     float dt;                // step of the state (feature 6 = dt div v)
     float log_cbrt_n;        // log(N^(1/3)) = -log(Delta)
     float inv_N_res;
@@ -171,14 +172,11 @@ __global__ void k_feat_count(int n, int kf, const float4 *__restrict__ pos_h, in
     }
 }
 
-// Features 0 .. 4 depend on a particle's cell alone: one thread per cell sums the
-// counts of the 27 cells around it by class and takes the logs, once for the
-// 64 to 511 particles of the cell.
-__global__ void k_feat_table(int kf, const int32_t *__restrict__ fcnt, float *__restrict__ ftab) {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >> (3 * kf)) return;
+// Features 0 .. 4 of the particles of cell c: the logs of the counts of the 27
+// cells around it by class (own, face, edge, corner) and of their sum.
+__device__ __forceinline__ void cell_features(int kf, int c, const int32_t *fcnt, float (&f)[5]) {
     const int g = 1 << kf, cx = c & (g - 1), cy = (c >> kf) & (g - 1), cz = c >> (2 * kf);
-    float cls[4] = {0.f, 0.f, 0.f, 0.f};   // own, face, edge, corner
+    float cls[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
     for (int dz = -1; dz <= 1; dz++)
 #pragma unroll
@@ -189,9 +187,20 @@ __global__ void k_feat_table(int kf, const int32_t *__restrict__ fcnt, float *__
                 cls[(dx != 0) + (dy != 0) + (dz != 0)] +=
                     (float)__ldg(&fcnt[((size_t)z << (2 * kf)) | ((size_t)y << kf) | (size_t)x]);
             }
-    float4 *out = reinterpret_cast<float4 *>(ftab) + 2 * (size_t)c;   // counts are integers: 1 + c is exact
-    out[0] = make_float4(__logf(1.f + cls[0]), __logf(1.f + cls[1]), __logf(1.f + cls[2]), __logf(1.f + cls[3]));
-    out[1] = make_float4(__logf(1.f + (cls[0] + cls[1] + cls[2] + cls[3])), 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int k = 0; k < 4; k++) f[k] = __logf(1.f + cls[k]);   // counts are integers: 1 + c is exact
+    f[4] = __logf(1.f + (cls[0] + cls[1] + cls[2] + cls[3]));
+}
+
+// They depend on the cell alone: once per cell for its 64 to 511 particles.
+__global__ void k_feat_table(int kf, const int32_t *__restrict__ fcnt, float *__restrict__ ftab) {
+    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (c >> (3 * kf)) return;
+    float f[5];
+    cell_features(kf, c, fcnt, f);
+    float4 *out = reinterpret_cast<float4 *>(ftab) + 2 * (size_t)c;
+    out[0] = make_float4(f[0], f[1], f[2], f[3]);
+    out[1] = make_float4(f[4], 0.f, 0.f, 0.f);
 }
 
 // h and count of row i, and its 8 features (zeros past the last row).
@@ -208,11 +217,19 @@ __device__ __forceinline__ void row_features(const FeatArgs &a, int i, float (&f
         const float *gv = a.gradv + (size_t)a.gv_stride * i;
         dv = __ldg(gv) + __ldg(gv + 4) + __ldg(gv + 8);
     }
-    const float4 *c = reinterpret_cast<const float4 *>(a.ftab) + 2 * (size_t)feat_cell(p, a.kf);
-    const float4 cls = __ldg(c);
+    const int cell = (int)feat_cell(p, a.kf);
+    if (a.ftab) {
+        const float4 *c = reinterpret_cast<const float4 *>(a.ftab) + 2 * (size_t)cell;
+        const float4 cls = __ldg(c);
+        f[0] = cls.x, f[1] = cls.y, f[2] = cls.z, f[3] = cls.w;
+        f[4] = __ldg(&c[1].x);
+    } else {
+        float e[5];
+        cell_features(a.kf, cell, a.fcnt, e);
+#pragma unroll
+        for (int k = 0; k < 5; k++) f[k] = e[k];
+    }
     h = p.w;
-    f[0] = cls.x, f[1] = cls.y, f[2] = cls.z, f[3] = cls.w;
-    f[4] = __ldg(&c[1].x);
     f[5] = __logf(h) + a.log_cbrt_n;
     f[6] = a.dt * dv;
     f[7] = a.Nngb ? __logf(N * a.inv_N_res) : 0.f;
@@ -735,12 +752,20 @@ int feature_level(int n) {
     return k;
 }
 
+// Rows that one wave of the forward pass's warps takes at 16 each.
+int wave_rows(const crk_ctx *ctx) { return 4 * (ctx->nsm > 0 ? ctx->nsm : 152) * 8 * 16; }
+
+// Within one wave a row's own 27 counts cost less than the launch of the table
+// (8000 rows: 56 us a proposal with the table, 50 without; 262144 rows 73 with, 80 without).
+bool feature_table(const crk_ctx *ctx, int n) { return n > wave_rows(ctx); }
+
 int count_cells(crk_ctx *ctx, int n, const float4 *pos, int kf, cudaStream_t s) {
     if (!ctx->fcnt) CRK_CUDA(ctx, cudaMalloc((void **)&ctx->fcnt, sizeof(int32_t) << 21));
     CRK_CUDA(ctx, cudaMemsetAsync(ctx->fcnt, 0, sizeof(int32_t) << (3 * kf), s));
     CRK_CUDA(ctx, cudaMemsetAsync(ctx->counters + CNT_MLP_ERR, 0, sizeof(unsigned long long), s));
     const int cells = 1 << (3 * kf);
-    if (kf > ctx->ftab_level) {
+    const bool table = feature_table(ctx, n);
+    if (table && kf > ctx->ftab_level) {
         if (ctx->ftab) cudaFree(ctx->ftab);
         ctx->ftab = nullptr;
         ctx->ftab_level = 0;
@@ -748,8 +773,11 @@ int count_cells(crk_ctx *ctx, int n, const float4 *pos, int kf, cudaStream_t s) 
         ctx->ftab_level = kf;
     }
     k_feat_count<<<grid_for(n, 256), 256, 0, s>>>(n, kf, pos, ctx->fcnt, ctx->counters + CNT_MLP_ERR);
-    k_feat_table<<<grid_for(cells, 128), 128, 0, s>>>(kf, ctx->fcnt, ctx->ftab);
-    ctx->launches += 2;
+    ++ctx->launches;
+    if (table) {
+        k_feat_table<<<grid_for(cells, 128), 128, 0, s>>>(kf, ctx->fcnt, ctx->ftab);
+        ++ctx->launches;
+    }
     CRK_LAUNCH_CHECK(ctx, "feature cell count");
     return CRK_OK;
 }
@@ -772,7 +800,8 @@ FeatArgs feat_args(const crk_ctx *ctx, int n, const float *pos_h, const float *g
     a.gradv = gradv;
     a.gv_stride = 9;
     a.Nngb = Nngb;
-    a.ftab = ctx->ftab;
+    a.fcnt = ctx->fcnt;
+    a.ftab = feature_table(ctx, n) ? ctx->ftab : nullptr;
     a.log_cbrt_n = (float)(log((double)n) / 3.0);
     a.inv_N_res = (float)(1.0 / ctx->p.N_res);
     a.N_res = (float)ctx->p.N_res;
@@ -788,7 +817,7 @@ int need_weights(crk_ctx *ctx) {
 // grid of k_mlp_fwd and the rows a warp takes at a time
 int fwd_blocks(const crk_ctx *ctx, int n, int *span) {
     const int cap = 4 * (ctx->nsm > 0 ? ctx->nsm : 152);
-    *span = n <= cap * 8 * 16 ? 16 : 32;
+    *span = n <= wave_rows(ctx) ? 16 : 32;
     const int b = (n + 8 * *span - 1) / (8 * *span);
     return b > cap ? cap : b;
 }
