@@ -677,17 +677,22 @@ __global__ void k_tree_up(const uint4 *__restrict__ clo, const uint4 *__restrict
 // periodic gap (fixed point) between the arcs [a0,a1] and [b0,b1] of a circle
 // of 2^32 (an arc may wrap, a0 > a1): 0 when they meet, else the shorter way
 // round; all differences modulo 2^32
-__device__ __forceinline__ unsigned long long axis_gap(uint32_t a0, uint32_t a1, uint32_t b0, uint32_t b1) {
-    if (b0 - a0 <= a1 - a0 || a0 - b0 <= b1 - b0) return 0ull;
-    const uint32_t g1 = b0 - a1, g2 = a0 - b1;
-    return (unsigned long long)(g1 < g2 ? g1 : g2);
+__device__ __forceinline__ uint32_t axis_gap(uint32_t a0, uint32_t a1, uint32_t b0, uint32_t b1) {
+    if (b0 - a0 <= a1 - a0 || a0 - b0 <= b1 - b0) return 0u;
+    return min(b0 - a1, a0 - b1);
 }
 
-__device__ __forceinline__ unsigned long long box_gap2(uint4 alo, uint4 ahi, uint4 blo, uint4 bhi) {
-    unsigned long long gx = axis_gap(alo.x, ahi.x, blo.x, bhi.x);
-    unsigned long long gy = axis_gap(alo.y, ahi.y, blo.y, bhi.y);
-    unsigned long long gz = axis_gap(alo.z, ahi.z, blo.z, bhi.z);
-    return gx * gx + gy * gy + gz * gz;
+// squared gap of two boxes < R^2, exactly: in FP32 first, where every term is
+// within 3 u of its exact value and the sum and R^2 within 5 u (u = 2^-24), so a
+// difference above 16 u R^2 has the exact sign; in 64-bit integers otherwise
+__device__ __forceinline__ bool boxes_near(uint4 alo, uint4 ahi, uint4 blo, uint4 bhi, uint32_t R) {
+    const uint32_t gx = axis_gap(alo.x, ahi.x, blo.x, bhi.x), gy = axis_gap(alo.y, ahi.y, blo.y, bhi.y),
+                   gz = axis_gap(alo.z, ahi.z, blo.z, bhi.z);
+    const float x = (float)gx, y = (float)gy, z = (float)gz, r = (float)R, r2 = r * r;
+    const float d = fmaf(x, x, fmaf(y, y, z * z)) - r2;
+    if (fabsf(d) > (16.f / 16777216.f) * r2) return d < 0.f;
+    return (unsigned long long)gx * gx + (unsigned long long)gy * gy + (unsigned long long)gz * gz <
+           (unsigned long long)R * R;
 }
 
 // 32-ary view of the binary tile tree: 32-ary level L is binary level 5 L, and
@@ -706,51 +711,77 @@ struct Tree32 {
 // child of the node being expanded; passing leaves (tiles) are emitted in
 // ascending order, passing inner nodes pushed so that the lowest pops first.
 // The reach of a node is max(Hmax_I, Hmax_node) (pair-set predicate).
+// Bound by the latency of a node's boxes, on which the next pop waits: the
+// parents of tiles, most of the nodes, are expanded PARENTS at a time, all of
+// their loads in flight, and boxes are compared in FP32 where that decides (64^3
+// clustered: 152 us one node at a time with 64-bit squares, 69 so).
 // SOME: only tiles in [r0, r1) (r0 a multiple of 32).  Stops once more than
 // `stop` are found.
+constexpr int PARENTS = 4;
 template <bool WRITE, bool SOME = false>
 __device__ uint32_t walk32(const Tree32 &T, const uint4 *__restrict__ lo, const uint4 *__restrict__ hi,
                            const uint32_t *__restrict__ nbox, uint32_t Ibox, uint4 Ilo, uint4 Ihi,
                            uint32_t *__restrict__ out, uint32_t lim, int *stL, int *stK, int lane,
                            uint32_t stop = 0xfffffffeu, long long r0 = 0, long long r1 = 0) {
     const unsigned lt = lanemask_lt();
-    const unsigned long long HI = Ilo.w;
     uint32_t count = 0;
-    int sp = 0;
-    int L = T.top + 1, k = 0;           // virtual root: its children are the top-level nodes
-    for (;;) {
-        const int cl = L - 1;
-        const int c = k * 32 + lane;
+    int sp = 1;
+    if (lane == 0) {
+        stL[0] = T.top + 1;   // virtual root: its children are the top-level nodes
+        stK[0] = 0;
+    }
+    __syncwarp();
+    while (sp > 0) {
+        if (stL[sp - 1] == 1) {   // children are tiles; the run of such nodes on top of the stack
+            int c[PARENTS], q = 0;
+            uint4 nlo[PARENTS], nhi[PARENTS];
+            bool on[PARENTS];
+#pragma unroll
+            for (int u = 0; u < PARENTS; u++) {
+                const int at = sp - 1 - u;
+                const bool live = q == u && at >= 0 && stL[max(at, 0)] == 1;
+                c[u] = live ? stK[at] * 32 + lane : 0;
+                on[u] = live && c[u] < T.cnt[0];
+                if (live) q++;
+                nlo[u] = lo[T.off[0] + (on[u] ? c[u] : 0)];
+                nhi[u] = hi[T.off[0] + (on[u] ? c[u] : 0)];
+            }
+            sp -= q;
+#pragma unroll
+            for (int u = 0; u < PARENTS; u++) {
+                bool pass = on[u] && boxes_near(Ilo, Ihi, nlo[u], nhi[u], max(Ilo.w, nlo[u].w)) &&
+                            (!nbox || box_ranges_meet(Ibox, nbox[T.off[0] + c[u]]));
+                if (SOME) pass = pass && c[u] < r1 && c[u] >= r0;
+                const unsigned m = __ballot_sync(0xffffffffu, pass);
+                if (WRITE && pass) {
+                    const uint32_t at = count + __popc(m & lt);
+                    if (at < lim) out[at] = (uint32_t)c[u];
+                }
+                count += __popc(m);
+            }
+            if (count > stop) return count;
+            __syncwarp();
+            continue;
+        }
+        --sp;
+        const int cl = stL[sp] - 1, c = stK[sp] * 32 + lane;
         bool pass = false;
         if (c < T.cnt[cl]) {
             const uint4 nlo = lo[T.off[cl] + c], nhi = hi[T.off[cl] + c];
-            unsigned long long R = HI > (unsigned long long)nlo.w ? HI : (unsigned long long)nlo.w;
-            pass = box_gap2(Ilo, Ihi, nlo, nhi) < R * R &&
+            pass = boxes_near(Ilo, Ihi, nlo, nhi, max(Ilo.w, nlo.w)) &&
                    (!nbox || box_ranges_meet(Ibox, nbox[T.off[cl] + c]));
             if (SOME) pass = pass && ((long long)c << (5 * cl)) < r1 && ((long long)(c + 1) << (5 * cl)) > r0;
         }
         const unsigned m = __ballot_sync(0xffffffffu, pass);
         const int np = __popc(m);
-        if (cl == 0) {
-            if (WRITE && pass) {
-                const uint32_t at = count + __popc(m & lt);
-                if (at < lim) out[at] = (uint32_t)c;
-            }
-            count += np;
-            if (count > stop) return count;
-        } else if (np) {
-            if (pass) {
-                const int pos = sp + (np - 1 - __popc(m & lt));
-                if (pos < STACK) { stL[pos] = cl; stK[pos] = c; }
-            }
-            sp += np;
-        }
+        if (sp + np > STACK) return 0xffffffffu;   // stack overflow: caller reports
         __syncwarp();
-        if (sp == 0) break;
-        sp--;
-        if (sp >= STACK) return 0xffffffffu;  // stack overflow: caller reports
-        L = stL[sp];
-        k = stK[sp];
+        if (pass) {
+            const int pos = sp + (np - 1 - __popc(m & lt));
+            stL[pos] = cl;
+            stK[pos] = c;
+        }
+        sp += np;
         __syncwarp();
     }
     return count;
