@@ -1,0 +1,203 @@
+"""The kernels at the sizes where their form changes.
+
+The list walk and the list passes choose their form by the number of tiles (32
+particles each): below 8 tiles per SM a tile is walked by 32 warps, below 20 by
+8, above by one; below 40 tiles per SM a tile's list is split over warps; and
+tiles with long lists or many neighbour tiles take forms of their own at any
+size.  Each case lies just past one of these lines with a ragged last tile, and
+is compared with the oracle at targets that include every unusual particle."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import crk as O
+from oracle import mlp as M
+from paper_2202_02840_gb300 import crk, inputs
+from parity import TOL, as_np, rel_err
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _device():
+    import __graft_entry__
+    __graft_entry__.build()
+    assert torch.cuda.is_available(), "GPU tests need a CUDA device"
+    torch.cuda.set_device(0)
+
+
+def dev(a):
+    return torch.from_numpy(np.ascontiguousarray(a)).cuda()
+
+
+def octants(n, seed=3):
+    """Two dense octants, jittered lattices of spacing s and h = 3 s, and 48 lone
+    particles in the six octants between them in Morton order: the tiles of
+    these span the whole box, so every tile is their neighbour.  Five particles
+    in the middle of the first octant have h = 6.2 s (1000 neighbours, where a
+    pass sends a tile to its split form).  Returns the state and those 53 indices."""
+    r = inputs.rng(seed)
+    lone = np.array([[x, y, z] for z in (0, 1) for y in (0, 1) for x in (0, 1)][1:-1])
+    lone = (lone[:, None, :] * 0.5 + np.array([[a, b, c] for a in (0.14, 0.36) for b in (0.14, 0.36)
+                                              for c in (0.14, 0.36)])[None]).reshape(-1, 3)
+    m = n - len(lone)
+    side = int(np.ceil((m / 2) ** (1 / 3)))
+    s = 0.5 / side
+    g = (np.stack(np.meshgrid(*[np.arange(side)] * 3, indexing="ij"), -1).reshape(-1, 3) + 0.5) * s
+    pick = [np.sort(r.permutation(side ** 3)[:k]) for k in (m - m // 2, m // 2)]
+    dense = np.concatenate([g[pick[0]], g[pick[1]] + 0.5]) + r.uniform(-0.1, 0.1, (m, 3)) * s
+    pos = inputs._to_unit_f32(np.concatenate([dense, lone])).astype(np.float64)
+    h = np.full(n, 3.0 * s)
+    big = np.argsort(((pos - 0.25) ** 2).sum(1))[:5]
+    h[big] = 6.2 * s
+    order = r.permutation(n)
+    st = inputs.pack(pos[order], np.minimum(h[order], 0.3), r.normal(0, 0.3, (n, 3)), 10 ** r.normal(0, 0.5, n),
+                     r.uniform(0.5, 1.5, n) / n)
+    back = np.argsort(order)
+    return st, np.sort(back[big]), np.sort(back[np.arange(m, n)])
+
+
+@pytest.mark.parametrize("n", [1300, 39037, 97401, 194577])
+def test_lists_and_passes_in_every_form(n):
+    """Lists exactly, then each pass on the GPU's own FP32 inputs, within the bar
+    of the parity tests."""
+    st, big, lone = octants(n)
+    pos = st["pos_h"]
+    some = inputs.rng(5).choice(n, 300, replace=False)
+    tg = np.unique(np.concatenate([big, lone, some])).astype(np.int32)
+    ctx = crk.crk_create(precision=1)
+    crk.crk_build_cells(ctx, dev(pos))
+    for mode in (0, 1):
+        off, lst = crk.crk_neighbour_lists(ctx, mode)
+        off, ids = off.cpu().numpy(), lst.cpu().numpy().view(np.uint32) & np.uint32(0x7FFFFFFF)
+        oc, ol = O.neighbours(pos, mode=mode, targets=tg)
+        assert np.array_equal(np.diff(off)[tg], oc)
+        oo = np.concatenate([[0], np.cumsum(oc.astype(np.int64))])
+        for k, i in enumerate(tg):
+            assert np.array_equal(np.sort(ids[off[i]:off[i + 1]]), np.sort(ol[oo[k]:oo[k + 1]])), (mode, i)
+    V, N = crk.crk_volumes(ctx)
+    o = O.volumes(pos, targets=tg)
+    assert max(rel_err(as_np(V)[tg], o["V"][tg]), rel_err(as_np(N)[tg], o["N"][tg])) < TOL
+    if n < 30000:
+        return   # lone particles within reach of the dense ones: ill-conditioned moments
+    vel = dev(st["vel_u"])
+    A, B, gA, gB, gv = crk.crk_corrections(ctx, V, vel)
+    acc, dudt, vsig, qmax = crk.crk_forces(ctx, dev(st["mass"]), vel, V, A, B, gA, gB, gv)
+    tg = np.setdiff1d(tg, lone).astype(np.int32)   # no neighbours, no moments
+    vel64, u, m = st["vel_u"][:, :3].astype(np.float64), st["vel_u"][:, 3].astype(np.float64), \
+        st["mass"].astype(np.float64)
+    c = {k: np.nan_to_num(as_np(t), nan=0.0, posinf=0.0, neginf=0.0)
+         for k, t in (("V", V), ("A", A), ("B", B), ("gA", gA), ("gB", gB), ("gv", gv))}
+    p2 = O.corrections(pos, c["V"], targets=tg)
+    coef = (c["A"], c["B"], c["gA"], c["gB"])
+    gv_o = O.gradv(pos, c["V"], vel64, *coef, targets=tg)
+    p4 = O.forces(pos, vel64, u, m, c["V"], *coef, c["gv"], targets=tg)
+    va = (vel64 + 1e-4 * np.nan_to_num(as_np(acc))).astype(np.float32)
+    vb = st["vel_u"][:, :3].copy()
+    du = crk.crk_compatible(ctx, dev(st["mass"]), vel, V, A, B, gA, gB, gv, dev(vb), dev(va))
+    du_o = O.compatible(pos, vel64, u, m, c["V"], *coef, c["gv"], vb.astype(np.float64), va.astype(np.float64),
+                        targets=tg)
+    e = {"A": rel_err(c["A"][tg], p2["A"][tg])}
+    e.update({k: rel_err(c[k][tg], p2[k][tg], floor=p2["s" + k][tg]) for k in ("B", "gA", "gB")})
+    e["gv"] = rel_err(c["gv"][tg], gv_o[tg])
+    e["acc"] = rel_err(as_np(acc)[tg], p4["acc"][tg], floor=p4["fscale"][tg])
+    e.update({k: rel_err(as_np(t)[tg], p4[k][tg]) for k, t in (("dudt", dudt), ("vsig", vsig), ("qmax", qmax))})
+    e["du"] = rel_err(as_np(du)[tg], du_o[tg])
+    print(n, e)
+    assert max(e.values()) < TOL, e
+
+
+@pytest.mark.parametrize("n", [1300, 39037, 97401])
+def test_batched_lists_in_every_form(n):
+    """Two boxes in one set: each box's lists and volumes are those of the box."""
+    sts = [octants(n // 3, 7), octants(n - n // 3, 9)]
+    pos = np.concatenate([s[0]["pos_h"] for s in sts])
+    start = [0, n // 3, n]
+    ctx = crk.crk_create()
+    crk.crk_build_cells_batched(ctx, dev(pos), start)
+    V = as_np(crk.crk_volumes(ctx)[0])
+    off = crk.crk_neighbour_lists(ctx, 1)[0].cpu().numpy()
+    for b, (st, big, lone) in enumerate(sts):
+        tg = np.unique(np.concatenate([big, lone, np.arange(0, len(st["pos_h"]), 997)])).astype(np.int32)
+        oc, _ = O.neighbours(st["pos_h"], mode=1, targets=tg)
+        assert np.array_equal(np.diff(off)[start[b] + tg], oc)
+        assert rel_err(V[start[b] + tg], O.volumes(st["pos_h"], targets=tg)["V"][tg]) < TOL
+
+
+@pytest.mark.parametrize("side", [11, 34, 46])
+def test_volume_walk_in_every_form(side):
+    """One h update from the walk that only sums volumes: h is a smooth function
+    of the sum, whose error is bounded as for the volumes."""
+    pos = inputs.sedov(side)["pos_h"].copy()
+    pos[:, 3] *= np.float32(0.8)
+    g = dev(pos)
+    crk.crk_h_iterate(crk.crk_create(), g, tol=1e-4, max_it=1)
+    want = O.h_iterate(pos, tol=1e-4, max_it=1)
+    want = np.asarray(want[0] if isinstance(want, tuple) else want)
+    assert rel_err(g[:, 3], want if want.ndim == 1 else want[:, 3]) < TOL
+
+
+@pytest.mark.parametrize("n", [1, 512, 513, 16384, 16385, 32769, 65537, 262144, 262145])
+def test_sort_at_the_edges_of_its_blocks(n):
+    """Keys per warp change at 2^14, 2^15 and 2^16 keys, scattered offsets beyond
+    64 blocks (2^18 keys); equal keys (a third of the particles) keep their order."""
+    r = inputs.rng(n)
+    pos = r.uniform(0, 1, (n, 4)).astype(np.float32)
+    pos[::3, :3] = pos[0, :3]
+    pos[:, :3] = np.minimum(pos[:, :3], np.float32(1 - 2.0 ** -24))
+    pos[:, 3] = 0.5 / max(n, 64) ** (1 / 3)
+    pos[pos[:, 3] > 0.3, 3] = 0.3
+    ctx = crk.crk_create()
+    crk.crk_build_cells(ctx, dev(pos))
+    keys, perm, cs, k = crk.crk_cells(ctx)
+    okey, operm, ok, ocs = O.cells(pos, kmax=7)
+    assert k == ok and np.array_equal(perm.cpu().numpy(), operm)
+    assert np.array_equal(keys.cpu().numpy().view(np.uint32), okey[operm])
+    assert np.array_equal(cs.cpu().numpy(), ocs)
+
+
+@pytest.mark.parametrize("n", [77824, 77825])
+def test_features_and_proposal_across_the_table(n):
+    """Up to one wave of 16-row tiles (77824 rows at 152 SMs) a row sums its cells
+    itself, beyond it reads the table: the features within the bounds of the
+    feature test, and the proposal from them (exp and the cube root: 3e-6)."""
+    r = np.random.default_rng(n)
+    pos = r.uniform(0, 1, (n, 4)).astype(np.float32)
+    pos[:, :3] = np.minimum(pos[:, :3], np.float32(1 - 2.0 ** -24))
+    pos[:, 3] = 0.05
+    N = r.uniform(150, 400, n).astype(np.float32)
+    gradv = r.normal(0, 0.5, (n, 3, 3)).astype(np.float32)
+    ctx = crk.crk_create()
+    w = inputs.mlp_init(1)
+    crk.crk_mlp_set_weights(ctx, dev(w))
+    feat = crk.crk_h_features(ctx, dev(pos), dev(gradv), dev(N), dt=0.1)
+    f = as_np(feat)
+    o = M.features(pos, N_prev=N, divv=gradv[:, 0, 0].astype(np.float64) + gradv[:, 1, 1] + gradv[:, 2, 2],
+                   dt=np.float32(0.1))
+    np.testing.assert_allclose(f[:, :5], o[:, :5], rtol=2e-7, atol=0)
+    assert np.all(np.abs(f[:, 5] - o[:, 5]) <= 1e-6 * (1 + np.abs(o[:, 5])))
+    y = as_np(crk.crk_mlp_forward(ctx, feat)).astype(np.float64)
+    p = dev(pos)
+    crk.crk_h_propose(ctx, p, dev(gradv), dev(N), dt=0.1, tol=0.0)
+    want = np.clip(pos[:, 3].astype(np.float64) * np.cbrt(268.0 / N.astype(np.float64)) * np.exp(y), 1e-6, 0.3)
+    np.testing.assert_allclose(as_np(p)[:, 3], want, rtol=3e-6)
+
+
+@pytest.mark.parametrize("n", [1, 64, 65, 513, 4096])
+def test_gradient_at_the_edges_of_its_chunks(n):
+    """64 rows a chunk; the update sums the partials of the blocks eight at a time.
+    The bounds are those of the ragged-batch gradient test: flipped roundings of
+    the BF16 activations (2^-8 each) within 3e-2 of the gradient's norm."""
+    r = np.random.default_rng(n)
+    x = np.stack([r.uniform(0, 6, n) for _ in range(8)], 1).astype(np.float32)
+    t = r.normal(0, 0.3, n).astype(np.float32)
+    w = inputs.mlp_init(2).astype(np.float32)
+    w[4736:4800] = r.normal(0, 0.125, 64)
+    ctx = crk.crk_create()
+    crk.crk_mlp_set_weights(ctx, dev(w))
+    g, loss = crk.crk_mlp_train_step(ctx, dev(x), dev(t), lr=0.0)
+    xb = M.bf16_round(x).astype(np.float64)
+    L, go = M.loss_and_grad(M.round_weights(w), xb, t, rnd=M.bf16_round)
+    g = as_np(g).astype(np.float64)
+    assert abs(float(as_np(loss)[0]) - L) <= 1e-2 * L
+    assert np.linalg.norm(g - go) <= 3e-2 * np.linalg.norm(go)
