@@ -96,6 +96,26 @@ __device__ __forceinline__ float2 silu2(float z0, float z1, float2 *ds = nullptr
     return up2(mul2(z, sg));
 }
 
+// Dependent launches of a training step (programmatic stream serialisation): a
+// kernel may start while the one before it still runs, up to grid_wait(), behind
+// which everything that one wrote is visible in L2.  What a training kernel
+// writes is therefore read with ld_l2, never through L1.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ float ld_l2(const float *p) {
+    float v;
+    asm volatile("ld.global.cg.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ float4 ld_l2(const float4 *p) {
+    float4 v;
+    asm volatile("ld.global.cg.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "l"(p)
+                 : "memory");
+    return v;
+}
+
 // D += A (16x8, row) B (8x8, col); bf16 in, f32 accumulate
 __device__ __forceinline__ void mma_k8(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t b0) {
     asm volatile(
@@ -266,16 +286,16 @@ struct FwdShm {
 // once (a training step's block does little else, so the serial trips to L2 of
 // a scalar loop were a third of its time).
 template <int NT, bool TR>
-__device__ __forceinline__ void stage_fwd(const float *__restrict__ W, FwdShm &S, __nv_bfloat16 *w2t = nullptr) {
+__device__ __forceinline__ void stage_fwd(const float *W, FwdShm &S, __nv_bfloat16 *w2t = nullptr) {
     constexpr int Q = 1024 / NT;   // float4 of W2 per thread
     float4 v[Q];
 #pragma unroll
-    for (int q = 0; q < Q; q++) v[q] = reinterpret_cast<const float4 *>(W + OFF_W2)[q * NT + threadIdx.x];
-    for (int k = threadIdx.x; k < 512; k += NT) S.w1[k] = __float2bfloat16_rn(W[OFF_W1 + k]);
+    for (int q = 0; q < Q; q++) v[q] = ld_l2(reinterpret_cast<const float4 *>(W + OFF_W2) + q * NT + threadIdx.x);
+    for (int k = threadIdx.x; k < 512; k += NT) S.w1[k] = __float2bfloat16_rn(ld_l2(W + OFF_W1 + k));
     for (int k = threadIdx.x; k < 64; k += NT) {
-        S.b1[k] = W[OFF_B1 + k];
-        S.b2[k] = W[OFF_B2 + k];
-        S.w3[k] = bf16r(W[OFF_W3 + k]);
+        S.b1[k] = ld_l2(W + OFF_B1 + k);
+        S.b2[k] = ld_l2(W + OFF_B2 + k);
+        S.w3[k] = bf16r(ld_l2(W + OFF_W3 + k));
     }
 #pragma unroll
     for (int q = 0; q < Q; q++) {
@@ -490,10 +510,32 @@ __device__ __forceinline__ void st_bf16(__nv_bfloat16 *p, float v) { *p = __floa
 __global__ void __launch_bounds__(128) k_mlp_grad(TrainArgs a) {
     extern __shared__ __align__(16) unsigned char shm_raw[];
     GradShm &S = *reinterpret_cast<GradShm *>(shm_raw);
-    stage_fwd<128, true>(a.W, S.f, S.w2t);
-    float b3 = a.W[OFF_B3];
-    __syncthreads();
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+    const int rr0 = 16 * w + g, rr1 = rr0 + 8;     // rows of this lane within the chunk
+    const int nchunk = (a.batch + 63) >> 6;
+    float2 x0, x1;       // the lane's columns of its rows of a chunk, and their targets
+    float t0, t1;
+    auto load_rows = [&](int ch) {
+        const int b0 = ch * 64 + rr0, b1 = ch * 64 + rr1;
+        x0 = x1 = make_float2(0.f, 0.f);
+        t0 = t1 = 0.f;
+        if (b0 < a.batch) {
+            const int i = sample_row(a, b0);
+            x0 = __ldg(reinterpret_cast<const float2 *>(a.feat) + 4 * (size_t)i + t);
+            t0 = __ldg(a.target + i);
+        }
+        if (b1 < a.batch) {
+            const int i = sample_row(a, b1);
+            x1 = __ldg(reinterpret_cast<const float2 *>(a.feat) + 4 * (size_t)i + t);
+            t1 = __ldg(a.target + i);
+        }
+    };
+    load_rows(blockIdx.x);   // the data set is no step's output
+    grid_wait();
+    grid_launch_next();
+    stage_fwd<128, true>(a.W, S.f, S.w2t);
+    float b3 = ld_l2(a.W + OFF_B3);
+    __syncthreads();
     uint32_t w1f[8];
     load_w1f(S.f, g, t, w1f);
 
@@ -508,22 +550,9 @@ __global__ void __launch_bounds__(128) k_mlp_grad(TrainArgs a) {
 #pragma unroll
     for (int c = 0; c < 4; c++) gw1[c] = 0.f;
 
-    const int rr0 = 16 * w + g, rr1 = rr0 + 8;     // rows of this lane within the chunk
-    const int nchunk = (a.batch + 63) >> 6;
     for (int ch = blockIdx.x; ch < nchunk; ch += gridDim.x) {
-        const int b0 = ch * 64 + rr0, b1 = ch * 64 + rr1;
-        const bool v0 = b0 < a.batch, v1 = b1 < a.batch;
-        const int i0 = v0 ? sample_row(a, b0) : 0, i1 = v1 ? sample_row(a, b1) : 0;
-        float2 x0 = make_float2(0.f, 0.f), x1 = x0;
-        float t0 = 0.f, t1 = 0.f;
-        if (v0) {
-            x0 = __ldg(reinterpret_cast<const float2 *>(a.feat) + 4 * (size_t)i0 + t);
-            t0 = __ldg(a.target + i0);
-        }
-        if (v1) {
-            x1 = __ldg(reinterpret_cast<const float2 *>(a.feat) + 4 * (size_t)i1 + t);
-            t1 = __ldg(a.target + i1);
-        }
+        const bool v0 = ch * 64 + rr0 < a.batch, v1 = ch * 64 + rr1 < a.batch;
+        if (ch != (int)blockIdx.x) load_rows(ch);
         const uint32_t xa0 = pack_bf16(x0.x, x0.y), xa1 = pack_bf16(x1.x, x1.y);
 
         // forward, keeping silu' of both layers and the BF16 layer-2 outputs
@@ -707,16 +736,27 @@ struct AdamArgs {
 // their sums are added in row order: deterministic), then one Adam update
 // (Kingma & Ba 2015) of each master weight; lr = 0 leaves W unchanged.  Bound by
 // the latency of its loads: a thread has its eight partials of a 4096-row step
-// in flight at once (6.3 us with one thread per weight, 4.5 now).
+// in flight at once (6.3 us with one thread per weight, 4.5 so).  A step is two
+// launches of a few microseconds each, so a third of it was their starts: with
+// dependent launches the blocks are in place, and the gradient's rows and the
+// master weights read, when the kernel before ends (a 4096-row step 15.1 -> 11.6 us).
 constexpr int ADAM_ROWS = 8;
 __global__ void __launch_bounds__(32 * ADAM_ROWS) k_adam(AdamArgs a) {
     __shared__ float sum[ADAM_ROWS][32];
     const int lane = threadIdx.x & 31, q = threadIdx.x >> 5;
     const int p = blockIdx.x * 32 + lane;
+    grid_launch_next();
+    float m0 = 0.f, v0 = 0.f, w0 = 0.f;
+    if (q == 0 && p < NP) {   // written by the update before the gradient that launched this one
+        m0 = ld_l2(a.m + p);
+        v0 = ld_l2(a.v + p);
+        w0 = ld_l2(a.W + p);
+    }
+    grid_wait();
     float s = 0.f;
     if (p <= NP) {
 #pragma unroll 8
-        for (int b = q; b < a.nblk; b += ADAM_ROWS) s += a.part[(size_t)b * NPART + p];
+        for (int b = q; b < a.nblk; b += ADAM_ROWS) s += ld_l2(a.part + (size_t)b * NPART + p);
     }
     sum[q][lane] = s;
     __syncthreads();
@@ -729,11 +769,11 @@ __global__ void __launch_bounds__(32 * ADAM_ROWS) k_adam(AdamArgs a) {
     }
     if (a.grad_out) a.grad_out[p] = s;
     if (a.lr > 0.f) {
-        float m = a.beta1 * a.m[p] + (1.f - a.beta1) * s;
-        float v = a.beta2 * a.v[p] + (1.f - a.beta2) * s * s;
+        const float m = a.beta1 * m0 + (1.f - a.beta1) * s;
+        const float v = a.beta2 * v0 + (1.f - a.beta2) * s * s;
         a.m[p] = m;
         a.v[p] = v;
-        a.W[p] -= a.lr * (m * a.corr1) / (sqrtf(v * a.corr2) + a.eps);
+        a.W[p] = w0 - a.lr * (m * a.corr1) / (sqrtf(v * a.corr2) + a.eps);
     }
 }
 
@@ -822,9 +862,29 @@ int fwd_blocks(const crk_ctx *ctx, int n, int *span) {
     return b > cap ? cap : b;
 }
 
+// Launch that may start while the kernel before it in the stream still runs (early).
+template <class Args>
+cudaError_t launch_dependent(void (*kernel)(Args), int grid, int block, size_t shm, cudaStream_t s, bool early,
+                             const Args &args) {
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = shm;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = early ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, args);
+}
+
+// One step.  follows: the stream's last kernel is the update of the step before, so
+// the gradient may start early (its first rows are read meanwhile); else it waits
+// for whatever made the data set.
 int train_launch(crk_ctx *ctx, int n, const float *feat, const float *target, const int32_t *rows, int n_rows,
                  int batch, long long step, float lr, unsigned long long seed, float *grad, float *loss,
-                 cudaStream_t s) {
+                 bool follows, cudaStream_t s) {
     static bool attr_set = false;
     if (!attr_set) {
         CRK_CUDA(ctx, cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -854,7 +914,7 @@ int train_launch(crk_ctx *ctx, int n, const float *feat, const float *target, co
     ta.two_over_B = 2.f * Y_SCALE / (float)batch;   // dL/dy times dy/d(output layer)
     ta.part = ctx->mlp_part;
     prof_begin(ctx, PROF_MLP_TRAIN, s);
-    k_mlp_grad<<<nblk, 128, sizeof(GradShm), s>>>(ta);
+    CRK_CUDA(ctx, launch_dependent(k_mlp_grad, nblk, 128, sizeof(GradShm), s, follows, ta));
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "mlp gradient");
     AdamArgs aa;
@@ -874,7 +934,7 @@ int train_launch(crk_ctx *ctx, int n, const float *feat, const float *target, co
     aa.inv_B = 1.f / (float)batch;
     aa.grad_out = grad;
     aa.loss_out = loss;
-    k_adam<<<grid_for(NP + 1, 32), 32 * ADAM_ROWS, 0, s>>>(aa);
+    CRK_CUDA(ctx, launch_dependent(k_adam, grid_for(NP + 1, 32), 32 * ADAM_ROWS, 0, s, true, aa));
     ++ctx->launches;
     prof_end(ctx, s);
     CRK_LAUNCH_CHECK(ctx, "mlp adam");
@@ -1024,7 +1084,7 @@ extern "C" int crk_mlp_train_step(crk_ctx *ctx, int n, const float *feat, const 
     int rc = need_weights(ctx);
     if (rc) return rc;
     if (n < 1 || !feat || !target || !(lr >= 0.f)) return crk_set_error(ctx, CRK_EINVAL, "bad arguments");
-    return train_launch(ctx, n, feat, target, nullptr, 0, n, -1, lr, 0ull, grad, loss, (cudaStream_t)stream);
+    return train_launch(ctx, n, feat, target, nullptr, 0, n, -1, lr, 0ull, grad, loss, false, (cudaStream_t)stream);
 }
 
 extern "C" int crk_h_select(crk_ctx *ctx, int n, const float *Nngb, float tol, int base, int32_t *rows, int *count,
@@ -1077,7 +1137,7 @@ extern "C" int crk_mlp_train(crk_ctx *ctx, int n, const float *feat, const float
     }
     for (int k = 0; k < steps; k++) {
         rc = train_launch(ctx, n, feat, target, rows, rows ? n_rows : 0, batch, ctx->mlp_t, lr, seed, nullptr,
-                          ctx->mlp_hist + k, s);
+                          ctx->mlp_hist + k, k > 0, s);
         if (rc) return rc;
     }
     if (loss_hist && steps > 0) {

@@ -201,3 +201,22 @@ def test_gradient_at_the_edges_of_its_chunks(n):
     g = as_np(g).astype(np.float64)
     assert abs(float(as_np(loss)[0]) - L) <= 1e-2 * L
     assert np.linalg.norm(g - go) <= 3e-2 * np.linalg.norm(go)
+
+
+@pytest.mark.parametrize("batch", [100, 4096, 50000])
+def test_overlapped_training_steps_are_the_separate_ones(batch):
+    """Within one call a step starts while the one before it still runs; one call a
+    step has nothing to overlap with.  Losses and weights agree bit for bit."""
+    r = np.random.default_rng(batch)
+    n, steps = 20000, 40
+    x = np.stack([r.uniform(0, 6, n) for _ in range(8)], 1).astype(np.float32)
+    t = r.normal(0, 0.3, n).astype(np.float32)
+    out = []
+    for calls in (1, steps):
+        ctx = crk.crk_create()
+        crk.crk_mlp_set_weights(ctx, dev(inputs.mlp_init(4)))
+        X, T, losses = dev(x), dev(t), []
+        for _ in range(calls):
+            losses += crk.crk_mlp_train(ctx, X, T, batch=batch, steps=steps // calls, lr=1e-3, seed=3)
+        out.append((np.array(losses), as_np(crk.crk_mlp_get_weights(ctx))))
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
