@@ -26,6 +26,7 @@ constexpr unsigned FULL = 0xffffffffu;
 __global__ void k_keys(int n, const float4 *__restrict__ pos, uint32_t *__restrict__ key,
                        int32_t *__restrict__ idx, uint4 *__restrict__ q_tmp,
                        float *__restrict__ h_tmp, unsigned long long *counters, int hilbert) {
+    grid_wait();
     int t = blockIdx.x * blockDim.x + threadIdx.x;
     uint32_t hbits = 0u;
     if (t < n) {
@@ -70,6 +71,7 @@ static int rs_per_warp(int n) { return n <= 16384 ? 64 : (n <= 32768 ? 128 : (n 
 template <int BITS>
 __global__ void __launch_bounds__(256) k_rs_hist(int n, const uint32_t *__restrict__ key, int shift,
                                                  uint32_t *__restrict__ hist, int nblocks, int items, bool fused) {
+    grid_wait();
     constexpr int BINS = 1 << BITS;
     __shared__ uint32_t cnt[BINS];
     for (int d = threadIdx.x; d < BINS; d += 256) cnt[d] = 0;
@@ -100,6 +102,7 @@ __global__ void __launch_bounds__(256) k_rs_scatter(int n, const uint32_t *__res
                                                     int32_t *__restrict__ val_out, int shift,
                                                     const uint32_t *__restrict__ hist,
                                                     int nblocks, int per_warp, bool fused) {
+    grid_wait();
     constexpr int BINS = 1 << BITS, DPT = BINS / 256;   // digits per thread
     __shared__ uint32_t off[RS_WARPS][BINS];
     __shared__ uint32_t wsum[RS_WARPS];
@@ -197,6 +200,7 @@ __global__ void __launch_bounds__(256) k_rs_scatter(int n, const uint32_t *__res
 __global__ void __launch_bounds__(1024) k_scan_block(const uint32_t *__restrict__ in,
                                                      uint32_t *__restrict__ out, int count,
                                                      uint32_t *__restrict__ block_sums) {
+    grid_wait();
     __shared__ uint32_t wt[32];
     int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int base = blockIdx.x * 4096 + threadIdx.x * 4;
@@ -236,6 +240,7 @@ __global__ void __launch_bounds__(1024) k_scan_block(const uint32_t *__restrict_
 }
 
 __global__ void k_scan_add(uint32_t *__restrict__ out, int count, const uint32_t *__restrict__ offs) {
+    grid_wait();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < count) out[i] += offs[i / 4096];
 }
@@ -245,12 +250,12 @@ int scan_u32(crk_ctx *ctx, const uint32_t *in, uint32_t *out, int count, cudaStr
     uint32_t *scratch = ctx->scan_tmp;
     int nb = grid_for(count, 4096);
     if (nb > 4096) return crk_set_error(ctx, CRK_ECAPACITY, "scan of %d items exceeds 2 levels", count);
-    k_scan_block<<<nb, 1024, 0, s>>>(in, out, count, scratch);
+    launch(s, nb, 1024, 0, k_scan_block, in, out, count, scratch);
     ++ctx->launches;
     if (nb > 1) {
-        k_scan_block<<<1, 1024, 0, s>>>(scratch, scratch + 4096, nb, nullptr);
+        launch(s, 1, 1024, 0, k_scan_block, scratch, scratch + 4096, nb, nullptr);
         ++ctx->launches;
-        k_scan_add<<<grid_for(count, 256), 256, 0, s>>>(out, count, scratch + 4096);
+        launch(s, grid_for(count, 256), 256, 0, k_scan_add, out, count, scratch + 4096);
         ++ctx->launches;
     }
     CRK_LAUNCH_CHECK(ctx, "scan");
@@ -262,13 +267,13 @@ static int radix_pass(crk_ctx *ctx, int n, int shift, const uint32_t *kin, const
                       int32_t *vout, cudaStream_t s) {
     const int pw = rs_per_warp(n), items = RS_WARPS * pw, nblocks = grid_for(n, items);
     const bool fused = nblocks <= RS_FUSED;
-    k_rs_hist<BITS><<<nblocks, 256, 0, s>>>(n, kin, shift, ctx->hist, nblocks, items, fused);
+    launch(s, nblocks, 256, 0, k_rs_hist<BITS>, n, kin, shift, ctx->hist, nblocks, items, fused);
     ++ctx->launches;
     if (!fused) {
         int rc = scan_u32(ctx, ctx->hist, ctx->hist, (1 << BITS) * nblocks, s);
         if (rc) return rc;
     }
-    k_rs_scatter<BITS><<<nblocks, 256, 0, s>>>(n, kin, vin, kout, vout, shift, ctx->hist, nblocks, pw, fused);
+    launch(s, nblocks, 256, 0, k_rs_scatter<BITS>, n, kin, vin, kout, vout, shift, ctx->hist, nblocks, pw, fused);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "radix sort");
     return CRK_OK;
@@ -343,6 +348,7 @@ __device__ __forceinline__ bool rcb_segment(int n, int level, int leaf, int s, i
 __global__ void k_rcb_box(int n, int level, int leaf, const int32_t *__restrict__ perm, const uint4 *__restrict__ q,
                           int32_t *__restrict__ seg_a, int32_t *__restrict__ seg_id, uint32_t *__restrict__ blo,
                           uint32_t *__restrict__ bhi, int32_t *__restrict__ bsize) {
+    grid_wait();
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     int a = 0, size = 0, path = -1;
     bool act = false;
@@ -387,6 +393,7 @@ __device__ __forceinline__ int rcb_axis(const uint32_t *lo, const uint32_t *hi, 
 __global__ void k_rcb_hist(int n, const int32_t *__restrict__ perm, const uint4 *__restrict__ q,
                            const int32_t *__restrict__ seg_id, const uint32_t *__restrict__ blo,
                            const uint32_t *__restrict__ bhi, uint32_t *__restrict__ bin, uint32_t *__restrict__ hist) {
+    grid_wait();
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     const int path = seg_id[s];
@@ -404,6 +411,7 @@ __global__ void k_rcb_hist(int n, const int32_t *__restrict__ perm, const uint4 
 // per segment (warp): the median slice and the counts below it and in it
 __global__ void k_rcb_pick(int nseg, const int32_t *__restrict__ bsize, const uint32_t *__restrict__ hist,
                            uint32_t *__restrict__ pick) {
+    grid_wait();
     const int lane = threadIdx.x & 31;
     const int g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (g >= nseg) return;
@@ -444,6 +452,7 @@ __global__ void k_rcb_pick(int nseg, const int32_t *__restrict__ bsize, const ui
 
 __global__ void k_rcb_flags(int n, const int32_t *__restrict__ seg_id, const uint32_t *__restrict__ bin,
                             const uint32_t *__restrict__ pick, uint32_t *__restrict__ f0, uint32_t *__restrict__ f1) {
+    grid_wait();
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     const int path = seg_id[s];
@@ -462,6 +471,7 @@ __global__ void k_rcb_scatter(int n, const int32_t *__restrict__ perm, const int
                               const int32_t *__restrict__ seg_id, const uint32_t *__restrict__ bin,
                               const uint32_t *__restrict__ pick, const uint32_t *__restrict__ r0,
                               const uint32_t *__restrict__ r1, int32_t *__restrict__ out) {
+    grid_wait();
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     const int path = seg_id[s];
@@ -517,6 +527,7 @@ void rcb_free(crk_ctx *ctx) {
 }
 
 __global__ void k_fill_u32(long long count, uint32_t v, uint32_t *out) {
+    grid_wait();
     const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (k < count) out[k] = v;
 }
@@ -534,22 +545,22 @@ static int rcb_refine(crk_ctx *ctx, int n, cudaStream_t s) {
     const int g = grid_for(n, 256);
     for (int L = 0; L < levels; L++) {
         const int nseg = 1 << L;
-        k_fill_u32<<<grid_for(3ll * nseg, 256), 256, 0, s>>>(3ll * nseg, 0xffffffffu, ctx->rcb_lo);
+        launch(s, grid_for(3ll * nseg, 256), 256, 0, k_fill_u32, 3ll * nseg, 0xffffffffu, ctx->rcb_lo);
         CRK_CUDA(ctx, cudaMemsetAsync(ctx->rcb_hi, 0, sizeof(uint32_t) * 3 * (size_t)nseg, s));
         CRK_CUDA(ctx, cudaMemsetAsync(ctx->rcb_size, 0, sizeof(int32_t) * (size_t)nseg, s));
         CRK_CUDA(ctx, cudaMemsetAsync(ctx->rcb_hist, 0, sizeof(uint32_t) * RCB_BINS * (size_t)nseg, s));
-        k_rcb_box<<<g, 256, 0, s>>>(n, L, leaf, cur, ctx->q_tmp, ctx->rcb_a, ctx->rcb_id, ctx->rcb_lo, ctx->rcb_hi,
-                                    ctx->rcb_size);
-        k_rcb_hist<<<g, 256, 0, s>>>(n, cur, ctx->q_tmp, ctx->rcb_id, ctx->rcb_lo, ctx->rcb_hi, ctx->rcb_bin,
-                                     ctx->rcb_hist);
-        k_rcb_pick<<<grid_for(32ll * nseg, 256), 256, 0, s>>>(nseg, ctx->rcb_size, ctx->rcb_hist, ctx->rcb_pick);
-        k_rcb_flags<<<g, 256, 0, s>>>(n, ctx->rcb_id, ctx->rcb_bin, ctx->rcb_pick, f0, f1);
+        launch(s, g, 256, 0, k_rcb_box, n, L, leaf, cur, ctx->q_tmp, ctx->rcb_a, ctx->rcb_id, ctx->rcb_lo,
+               ctx->rcb_hi, ctx->rcb_size);
+        launch(s, g, 256, 0, k_rcb_hist, n, cur, ctx->q_tmp, ctx->rcb_id, ctx->rcb_lo, ctx->rcb_hi, ctx->rcb_bin,
+               ctx->rcb_hist);
+        launch(s, grid_for(32ll * nseg, 256), 256, 0, k_rcb_pick, nseg, ctx->rcb_size, ctx->rcb_hist, ctx->rcb_pick);
+        launch(s, g, 256, 0, k_rcb_flags, n, ctx->rcb_id, ctx->rcb_bin, ctx->rcb_pick, f0, f1);
         ctx->launches += 5;
         CRK_LAUNCH_CHECK(ctx, "bisection");
         rc = scan_u32(ctx, f0, r0, n, s);
         if (!rc) rc = scan_u32(ctx, f1, r1, n, s);
         if (rc) return rc;
-        k_rcb_scatter<<<g, 256, 0, s>>>(n, cur, ctx->rcb_a, ctx->rcb_id, ctx->rcb_bin, ctx->rcb_pick, r0, r1, nxt);
+        launch(s, g, 256, 0, k_rcb_scatter, n, cur, ctx->rcb_a, ctx->rcb_id, ctx->rcb_bin, ctx->rcb_pick, r0, r1, nxt);
         ++ctx->launches;
         CRK_LAUNCH_CHECK(ctx, "bisection");
         int32_t *t = cur; cur = nxt; nxt = t;
@@ -566,6 +577,7 @@ __global__ void k_gather_sorted(int n, const int32_t *__restrict__ idx, const ui
                                 uint4 *__restrict__ q4, float *__restrict__ hs,
                                 int32_t *__restrict__ perm_out, const uint32_t *__restrict__ key,
                                 uint32_t *__restrict__ keys_out) {
+    grid_wait();
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     int i = idx[s];
@@ -613,6 +625,7 @@ __global__ void __launch_bounds__(1024) k_tiles(int n, int ntiles, const uint4 *
                                                 const int32_t *__restrict__ sbox, uint32_t *__restrict__ nbox,
                                                 uint4 *__restrict__ plo, uint4 *__restrict__ phi,
                                                 uint32_t *__restrict__ pbox) {
+    grid_wait();
     __shared__ uint4 sl[32], sh[32];
     __shared__ uint32_t sb[32];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -659,6 +672,7 @@ __global__ void __launch_bounds__(1024) k_tiles(int n, int ntiles, const uint4 *
 __global__ void k_tree_up(const uint4 *__restrict__ clo, const uint4 *__restrict__ chi, int ccnt,
                           uint4 *__restrict__ plo, uint4 *__restrict__ phi, int pcnt,
                           const uint32_t *__restrict__ cbox, uint32_t *__restrict__ pbox) {
+    grid_wait();
     const int k = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
     if (k >= pcnt) return;
     const int c = 32 * k + lane;
@@ -804,6 +818,7 @@ __global__ void __launch_bounds__(LIST_WARPS * 32) k_lists32(int count, const in
                                                              long long cap, unsigned long long *counter,
                                                              int32_t *__restrict__ queue,
                                                              unsigned long long *queued) {
+    grid_wait();
     __shared__ int stL[LIST_WARPS][STACK], stK[LIST_WARPS][STACK];
     __shared__ uint32_t buf[LIST_WARPS][LIST_BUF];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -851,6 +866,7 @@ __global__ void __launch_bounds__(LONG_WARPS * 32) k_lists_long(int ntiles, cons
                                                                 const uint32_t *__restrict__ nbox,
                                                                 uint2 *__restrict__ ofs, uint32_t *__restrict__ list,
                                                                 long long cap, unsigned long long *counter) {
+    grid_wait();
     __shared__ int stL[LONG_WARPS][STACK], stK[LONG_WARPS][STACK];
     __shared__ uint32_t cnt[LONG_WARPS];
     __shared__ unsigned long long base;
@@ -896,6 +912,7 @@ __device__ __forceinline__ int cell_level(unsigned long long hbits, int kmax) {
 
 __global__ void k_cell_start(int n, const uint32_t *__restrict__ keys, int kmax,
                              const unsigned long long *__restrict__ counters, int32_t *__restrict__ cs) {
+    grid_wait();
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     int k = cell_level(counters[CNT_HMAX], kmax);
     int sh = 30 - 3 * k;
@@ -932,15 +949,14 @@ int rebuild_lists(crk_ctx *ctx, cudaStream_t s) {
     const int count = ctx->act ? ctx->nact : ctx->ntiles;
     if (count == 0) return CRK_OK;
     const bool may_queue = ctx->ntiles > (int)LIST_BUF;   // else no tile has more neighbours than the buffer holds
-    k_lists32<<<grid_for(count, LIST_WARPS), LIST_WARPS * 32, 0, s>>>(
-        count, ctx->act, T, ctx->node_lo, ctx->node_hi, ctx->nbox > 1 ? ctx->node_box : nullptr, ctx->uofs,
-        ctx->ulist, ctx->cap_ulist, ctx->counters + CNT_ULIST, ctx->lqueue, ctx->counters + CNT_LQUEUE);
+    launch(s, grid_for(count, LIST_WARPS), LIST_WARPS * 32, 0, k_lists32, count, ctx->act, T, ctx->node_lo,
+           ctx->node_hi, ctx->nbox > 1 ? ctx->node_box : nullptr, ctx->uofs, ctx->ulist, ctx->cap_ulist,
+           ctx->counters + CNT_ULIST, ctx->lqueue, ctx->counters + CNT_LQUEUE);
     ++ctx->launches;
     if (may_queue) {
-        k_lists_long<<<ctx->nsm > 0 ? ctx->nsm : 152, LONG_WARPS * 32, 0, s>>>(
-            ctx->ntiles, ctx->lqueue, ctx->counters + CNT_LQUEUE, T, ctx->node_lo, ctx->node_hi,
-            ctx->nbox > 1 ? ctx->node_box : nullptr, ctx->uofs, ctx->ulist, ctx->cap_ulist,
-            ctx->counters + CNT_ULIST);
+        launch(s, ctx->nsm > 0 ? ctx->nsm : 152, LONG_WARPS * 32, 0, k_lists_long, ctx->ntiles, ctx->lqueue,
+               ctx->counters + CNT_LQUEUE, T, ctx->node_lo, ctx->node_hi, ctx->nbox > 1 ? ctx->node_box : nullptr,
+               ctx->uofs, ctx->ulist, ctx->cap_ulist, ctx->counters + CNT_ULIST);
         ++ctx->launches;
     }
     CRK_LAUNCH_CHECK(ctx, "interaction lists");
@@ -956,18 +972,15 @@ int build_tree(crk_ctx *ctx, cudaStream_t s) {
     const bool batched = ctx->nbox > 1;
     const int *off = ctx->level_off;
     const bool up = ctx->nlevels > 5;
-    k_tiles<<<grid_for(nt, 32), 1024, 0, s>>>(n, nt, ctx->q4, ctx->node_lo, ctx->node_hi,
-                                               batched ? ctx->sbox : nullptr, ctx->node_box,
-                                               up ? ctx->node_lo + off[5] : nullptr,
-                                               up ? ctx->node_hi + off[5] : nullptr,
-                                               up && batched ? ctx->node_box + off[5] : nullptr);
+    launch(s, grid_for(nt, 32), 1024, 0, k_tiles, n, nt, ctx->q4, ctx->node_lo, ctx->node_hi,
+           batched ? ctx->sbox : nullptr, ctx->node_box, up ? ctx->node_lo + off[5] : nullptr,
+           up ? ctx->node_hi + off[5] : nullptr, up && batched ? ctx->node_box + off[5] : nullptr);
     ++ctx->launches;
     for (int L = 10; L < ctx->nlevels; L += 5) {
         const int pc = ctx->level_cnt[L];
-        k_tree_up<<<grid_for(32ll * pc, 256), 256, 0, s>>>(
-            ctx->node_lo + off[L - 5], ctx->node_hi + off[L - 5], ctx->level_cnt[L - 5], ctx->node_lo + off[L],
-            ctx->node_hi + off[L], pc, batched ? ctx->node_box + off[L - 5] : nullptr,
-            batched ? ctx->node_box + off[L] : nullptr);
+        launch(s, grid_for(32ll * pc, 256), 256, 0, k_tree_up, ctx->node_lo + off[L - 5], ctx->node_hi + off[L - 5],
+               ctx->level_cnt[L - 5], ctx->node_lo + off[L], ctx->node_hi + off[L], pc,
+               batched ? ctx->node_box + off[L - 5] : nullptr, batched ? ctx->node_box + off[L] : nullptr);
         ++ctx->launches;
     }
     CRK_LAUNCH_CHECK(ctx, "tile tree");
@@ -979,6 +992,7 @@ int build_tree(crk_ctx *ctx, cudaStream_t s) {
 // for every new sorted slot, its index in the input order.
 __global__ void k_gather_u32(int n, const int32_t *__restrict__ idx, const uint32_t *__restrict__ in,
                              uint32_t *__restrict__ out) {
+    grid_wait();
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s < n) out[s] = in[idx[s]];
 }
@@ -1011,8 +1025,8 @@ int build_cells_sorted(crk_ctx *ctx, int n, const float4 *pos, const int32_t *ba
     prof_begin(ctx, PROF_BUILD, s);
     const bool fb = sort30_from_b(n);
     uint32_t *key0 = fb ? ctx->key_b : ctx->key_a;
-    k_keys<<<grid_for(n, 256), 256, 0, s>>>(n, pos, key0, fb ? ctx->idx_b : ctx->idx_a, q_tmp, h_tmp, ctx->counters,
-                                            ctx->p.tile_order == 1);
+    launch(s, grid_for(n, 256), 256, 0, k_keys, n, pos, key0, fb ? ctx->idx_b : ctx->idx_a, q_tmp, h_tmp,
+           ctx->counters, ctx->p.tile_order == 1);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "keys");
     if (box_of_input && ctx->p.tile_order == 2)
@@ -1024,13 +1038,13 @@ int build_cells_sorted(crk_ctx *ctx, int n, const float4 *pos, const int32_t *ba
         CRK_CUDA(ctx, cudaMemcpyAsync(ctx->mkey, key0, sizeof(uint32_t) * n, cudaMemcpyDeviceToDevice, s));
         rc = radix_sort30(ctx, n, s);
         if (rc) return rc;
-        k_gather_u32<<<grid_for(n, 256), 256, 0, s>>>(n, ctx->idx_a, reinterpret_cast<const uint32_t *>(box_of_input),
-                                                      ctx->key_a);
+        launch(s, grid_for(n, 256), 256, 0, k_gather_u32, n, ctx->idx_a,
+               reinterpret_cast<const uint32_t *>(box_of_input), ctx->key_a);
         ++ctx->launches;
         rc = radix_sort16(ctx, n, s);
         if (rc) return rc;
         CRK_CUDA(ctx, cudaMemcpyAsync(ctx->sbox, ctx->key_a, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, s));
-        k_gather_u32<<<grid_for(n, 256), 256, 0, s>>>(n, ctx->idx_a, ctx->mkey, ctx->keys);
+        launch(s, grid_for(n, 256), 256, 0, k_gather_u32, n, ctx->idx_a, ctx->mkey, ctx->keys);
         ++ctx->launches;
         CRK_LAUNCH_CHECK(ctx, "box sort");
         keys_out = nullptr;
@@ -1044,15 +1058,15 @@ int build_cells_sorted(crk_ctx *ctx, int n, const float4 *pos, const int32_t *ba
     }
     // base_perm may be the array the new order goes to: then by way of idx_b
     int32_t *perm = base_perm == ctx->perm ? ctx->idx_b : ctx->perm;
-    k_gather_sorted<<<grid_for(n, 256), 256, 0, s>>>(n, ctx->idx_a, q_tmp, h_tmp, base_perm, ctx->q4,
-                                                     ctx->hs, perm, ctx->key_a, keys_out);
+    launch(s, grid_for(n, 256), 256, 0, k_gather_sorted, n, ctx->idx_a, q_tmp, h_tmp, base_perm, ctx->q4, ctx->hs,
+           perm, ctx->key_a, keys_out);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "gather sorted");
     if (perm != ctx->perm)
         CRK_CUDA(ctx, cudaMemcpyAsync(ctx->perm, perm, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, s));
     if (!box_of_input && ctx->p.tile_order == 0) {   // the chaining-mesh table: one box, Morton order
-        k_cell_start<<<grid_for(n + 1, 256), 256, 0, s>>>(n, ctx->keys, ctx->p.kmax, ctx->counters,
-                                                          ctx->cell_start);
+        launch(s, grid_for(n + 1, 256), 256, 0, k_cell_start, n, ctx->keys, ctx->p.kmax, ctx->counters,
+               ctx->cell_start);
         ++ctx->launches;
         CRK_LAUNCH_CHECK(ctx, "cell table");
     }
@@ -1067,6 +1081,7 @@ int build_cells_sorted(crk_ctx *ctx, int n, const float4 *pos, const int32_t *ba
 
 __global__ void k_len_keys(int nt, const uint32_t *__restrict__ len, uint32_t *__restrict__ key,
                            int32_t *__restrict__ idx) {
+    grid_wait();
     int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= nt) return;
     key[t] = 0xffffu - min(len[t], 0xffffu);
@@ -1084,7 +1099,7 @@ int tile_order_by_length(crk_ctx *ctx, cudaStream_t s) {
         CRK_CUDA(ctx, cudaMalloc((void **)&ctx->tile_order, sizeof(int32_t) * (size_t)nt));
         ctx->cap_order = nt;
     }
-    k_len_keys<<<grid_for(nt, 256), 256, 0, s>>>(nt, ctx->len_u, ctx->key_a, ctx->idx_a);
+    launch(s, grid_for(nt, 256), 256, 0, k_len_keys, nt, ctx->len_u, ctx->key_a, ctx->idx_a);
     ++ctx->launches;
     int rc = radix_sort16(ctx, nt, s);
     if (rc) return rc;

@@ -235,6 +235,7 @@ int crk_sync_counters(crk_ctx *ctx, cudaStream_t s) {
 
 __global__ void k_gather_rows(long long total, int w, const int32_t *__restrict__ perm,
                               const uint32_t *__restrict__ in, uint32_t *__restrict__ out) {
+    grid_wait();
     long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= total) return;
     long long s = t / w;
@@ -244,6 +245,7 @@ __global__ void k_gather_rows(long long total, int w, const int32_t *__restrict_
 
 __global__ void k_scatter_rows(long long total, int w, const int32_t *__restrict__ perm,
                                const uint32_t *__restrict__ in, uint32_t *__restrict__ out) {
+    grid_wait();
     long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= total) return;
     long long s = t / w;
@@ -255,6 +257,7 @@ __global__ void k_scatter_rows(long long total, int w, const int32_t *__restrict
 __global__ void k_pack_corr(int n, const int32_t *__restrict__ perm, const float *__restrict__ A,
                             const float *__restrict__ B, const float *__restrict__ gA,
                             const float *__restrict__ gB, CorrRec *__restrict__ out) {
+    grid_wait();
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     long long i = perm[s];
@@ -270,6 +273,7 @@ __global__ void k_pack_corr(int n, const int32_t *__restrict__ perm, const float
 __global__ void k_unpack_corr(int n, const int32_t *__restrict__ perm, const CorrRec *__restrict__ in,
                               float *__restrict__ A, float *__restrict__ B, float *__restrict__ gA,
                               float *__restrict__ gB) {
+    grid_wait();
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     long long i = perm[s];
@@ -284,6 +288,7 @@ __global__ void k_unpack_corr(int n, const int32_t *__restrict__ perm, const Cor
 
 __global__ void k_pack_gv(int n, const int32_t *__restrict__ perm, const float *__restrict__ g,
                           GvRec *__restrict__ out) {
+    grid_wait();
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     const float *a = g + 9 * (long long)perm[s];
@@ -296,6 +301,7 @@ __global__ void k_pack_gv(int n, const int32_t *__restrict__ perm, const float *
 
 __global__ void k_unpack_gv(int n, const int32_t *__restrict__ perm, const GvRec *__restrict__ in,
                             float *__restrict__ g) {
+    grid_wait();
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     float *a = g + 9 * (long long)perm[s];
@@ -308,6 +314,7 @@ __global__ void k_unpack_gv(int n, const int32_t *__restrict__ perm, const GvRec
 // caller float[3n] -> sorted float4 (w = 0)
 __global__ void k_pack_v3(int n, const int32_t *__restrict__ perm, const float *__restrict__ v,
                           float4 *__restrict__ out) {
+    grid_wait();
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     const float *a = v + 3 * (long long)perm[s];
@@ -318,6 +325,7 @@ __global__ void k_pack_v3(int n, const int32_t *__restrict__ perm, const float *
 __global__ void k_unpack_forces(int n, const int32_t *__restrict__ perm, const float4 *__restrict__ acc,
                                 const float2 *__restrict__ vq, float *__restrict__ accel,
                                 float *__restrict__ dudt, float *__restrict__ vsig, float *__restrict__ qmax) {
+    grid_wait();
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     long long i = perm[s];
@@ -333,6 +341,7 @@ __global__ void k_unpack_forces(int n, const int32_t *__restrict__ perm, const f
 
 // (q, V) records of the gather passes from the sorted V
 __global__ void k_make_qV(int n, const uint4 *__restrict__ q4, const float *__restrict__ V, uint4 *__restrict__ qV) {
+    grid_wait();
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     uint4 q = q4[s];
@@ -343,7 +352,7 @@ namespace crk {
 int gather_rows(crk_ctx *ctx, const void *in, void *out, int w, cudaStream_t s) {
     long long total = (long long)ctx->n * w;
     if (total == 0) return CRK_OK;
-    k_gather_rows<<<grid_for(total, 256), 256, 0, s>>>(total, w, ctx->perm, (const uint32_t *)in, (uint32_t *)out);
+    launch(s, grid_for(total, 256), 256, 0, k_gather_rows, total, w, ctx->perm, (const uint32_t *)in, (uint32_t *)out);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "gather rows");
     return CRK_OK;
@@ -351,7 +360,7 @@ int gather_rows(crk_ctx *ctx, const void *in, void *out, int w, cudaStream_t s) 
 int scatter_rows(crk_ctx *ctx, const void *in, void *out, int w, cudaStream_t s) {
     long long total = (long long)ctx->n * w;
     if (total == 0) return CRK_OK;
-    k_scatter_rows<<<grid_for(total, 256), 256, 0, s>>>(total, w, ctx->perm, (const uint32_t *)in, (uint32_t *)out);
+    launch(s, grid_for(total, 256), 256, 0, k_scatter_rows, total, w, ctx->perm, (const uint32_t *)in, (uint32_t *)out);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "scatter rows");
     return CRK_OK;
@@ -608,6 +617,7 @@ extern "C" int crk_build_cells(crk_ctx *ctx, int n, const float *pos_h, void *st
 
 // box of caller row t: the b with box_start[b] <= t < box_start[b+1]
 __global__ void k_box_of(int n, int nbox, const int32_t *__restrict__ start, int32_t *__restrict__ box) {
+    grid_wait();
     int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n) return;
     int lo = 0, hi = nbox - 1;
@@ -655,7 +665,7 @@ int crk::load_boxes(crk_ctx *ctx, int n, int nbox, const int32_t *box_start, cud
     if (rc) return rc;
     CRK_CUDA(ctx, cudaMemcpyAsync(ctx->box_start, box_start, sizeof(int32_t) * ((size_t)nbox + 1),
                                   cudaMemcpyHostToDevice, s));
-    k_box_of<<<grid_for(n, 256), 256, 0, s>>>(n, nbox, ctx->box_start, ctx->box_in);
+    launch(s, grid_for(n, 256), 256, 0, k_box_of, n, nbox, ctx->box_start, ctx->box_in);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "box ids");
     CRK_CUDA(ctx, cudaStreamSynchronize(s));   // the host table may be freed after the call
@@ -790,17 +800,17 @@ extern "C" int crk_corrections(crk_ctx *ctx, const float *V, const float *vel_u,
     if (!rc && vel_u) rc = gather_rows(ctx, vel_u, ctx->vel, 4, s);
     if (rc) return rc;
     if (n) {
-        k_make_qV<<<grid_for(n, 256), 256, 0, s>>>(n, ctx->q4, ctx->V, ctx->qV);
+        launch(s, grid_for(n, 256), 256, 0, k_make_qV, n, ctx->q4, ctx->V, ctx->qV);
         ++ctx->launches;
         CRK_LAUNCH_CHECK(ctx, "gather records");
     }
     rc = run_corrections(ctx, gradv != nullptr, s);
     if (rc) return rc;
     if (n) {
-        k_unpack_corr<<<grid_for(n, 256), 256, 0, s>>>(n, ctx->perm, ctx->corr, A, B, gradA, gradB);
+        launch(s, grid_for(n, 256), 256, 0, k_unpack_corr, n, ctx->perm, ctx->corr, A, B, gradA, gradB);
         ++ctx->launches;
         if (gradv) {
-            k_unpack_gv<<<grid_for(n, 256), 256, 0, s>>>(n, ctx->perm, ctx->gv, gradv);
+            launch(s, grid_for(n, 256), 256, 0, k_unpack_gv, n, ctx->perm, ctx->gv, gradv);
             ++ctx->launches;
         }
         CRK_LAUNCH_CHECK(ctx, "unpack corrections");
@@ -818,9 +828,9 @@ static int pack_force_inputs(crk_ctx *ctx, const float *mass, const float *vel_u
     if (!rc) rc = gather_rows(ctx, V, ctx->V, 1, s);
     if (rc) return rc;
     if (n) {
-        k_pack_corr<<<grid_for(n, 256), 256, 0, s>>>(n, ctx->perm, A, B, gradA, gradB, ctx->corr);
+        launch(s, grid_for(n, 256), 256, 0, k_pack_corr, n, ctx->perm, A, B, gradA, gradB, ctx->corr);
         ++ctx->launches;
-        k_pack_gv<<<grid_for(n, 256), 256, 0, s>>>(n, ctx->perm, gradv, ctx->gv);
+        launch(s, grid_for(n, 256), 256, 0, k_pack_gv, n, ctx->perm, gradv, ctx->gv);
         ++ctx->launches;
         CRK_LAUNCH_CHECK(ctx, "pack force inputs");
     }
@@ -841,7 +851,7 @@ extern "C" int crk_forces(crk_ctx *ctx, const float *mass, const float *vel_u, c
     if (rc) return rc;
     int n = ctx->n;
     if (n) {
-        k_unpack_forces<<<grid_for(n, 256), 256, 0, s>>>(n, ctx->perm, ctx->acc, ctx->vq, accel, dudt, vsig, qmax);
+        launch(s, grid_for(n, 256), 256, 0, k_unpack_forces, n, ctx->perm, ctx->acc, ctx->vq, accel, dudt, vsig, qmax);
         ++ctx->launches;
         CRK_LAUNCH_CHECK(ctx, "unpack forces");
     }
@@ -866,9 +876,9 @@ extern "C" int crk_compatible(crk_ctx *ctx, const float *mass, const float *vel_
     if (rc) return rc;
     int n = ctx->n;
     if (n) {
-        k_pack_v3<<<grid_for(n, 256), 256, 0, s>>>(n, ctx->perm, vel_before, ctx->vb);
+        launch(s, grid_for(n, 256), 256, 0, k_pack_v3, n, ctx->perm, vel_before, ctx->vb);
         ++ctx->launches;
-        k_pack_v3<<<grid_for(n, 256), 256, 0, s>>>(n, ctx->perm, vel_after, ctx->va);
+        launch(s, grid_for(n, 256), 256, 0, k_pack_v3, n, ctx->perm, vel_after, ctx->va);
         ++ctx->launches;
         CRK_LAUNCH_CHECK(ctx, "pack kick velocities");
     }

@@ -218,6 +218,7 @@ __device__ __forceinline__ void pair_force(const FRec &a, const FOwn &oa, const 
 
 // Per-particle records of the pair-set passes, packed once per evaluation.
 __global__ void k_pack_frec(int n, FSrc src, FParams fp, float4 *__restrict__ out, float *__restrict__ sfun) {
+    grid_wait();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const FRec r = make_frec(i, src, fp);
@@ -368,6 +369,7 @@ template <bool COMP, bool STATIC>
 __global__ void __launch_bounds__(TMA_WARPS * 32) k_p4_tma(ListGeom g, typename P4<COMP, STATIC>::Params prm,
                                                           const __grid_constant__ CUtensorMap map,
                                                           unsigned long long *err) {
+    grid_wait();
     __shared__ alignas(128) unsigned char stg[TMA_WARPS][2][TMA_STAGE];
     __shared__ alignas(16) int rows[TMA_WARPS][32];
     __shared__ alignas(8) unsigned long long bar[TMA_WARPS][2];
@@ -478,8 +480,8 @@ template <bool COMP, bool STATIC>
 int P4<COMP, STATIC>::launch_tma(crk_ctx *ctx, const ListGeom &g, const Params &prm, cudaStream_t s) {
     int rc = frec_tensor_map(ctx);
     if (rc) return rc;
-    k_p4_tma<COMP, STATIC><<<grid_for(g.ntiles, TMA_WARPS), TMA_WARPS * 32, 0, s>>>(g, prm, ctx->frec_map,
-                                                                          ctx->counters + CNT_TMA_ERR);
+    launch(s, grid_for(g.ntiles, TMA_WARPS), TMA_WARPS * 32, 0, k_p4_tma<COMP, STATIC>, g, prm, ctx->frec_map,
+           ctx->counters + CNT_TMA_ERR);
     return CRK_OK;
 }
 
@@ -637,6 +639,7 @@ struct POGeom {
 __global__ void k_po_rev(int ntiles, const uint2 *__restrict__ tofs, const uint32_t *__restrict__ tlist,
                          uint32_t *__restrict__ rev, int32_t *__restrict__ self, uint2 *__restrict__ copy_ofs,
                          uint32_t *__restrict__ copy_list, unsigned long long *miss) {
+    grid_wait();
     const int lane = threadIdx.x & 31;
     const int I = (int)((blockIdx.x * (size_t)blockDim.x + threadIdx.x) >> 5);
     if (I >= ntiles) return;
@@ -672,6 +675,7 @@ __global__ void k_po_rev(int ntiles, const uint2 *__restrict__ tofs, const uint3
 // list ascend in j, so each is found by bisection.
 __global__ void k_po_low(int n, int kcap, const int32_t *__restrict__ cnt_g, const int32_t *__restrict__ cnt_u,
                          const uint32_t *__restrict__ ent, int2 *__restrict__ lowc) {
+    grid_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int tile = i / TILE, lane = i % TILE;
@@ -822,6 +826,7 @@ __device__ __forceinline__ void po_tile(const POGeom &g, const typename P::Param
 
 template <class P>
 __global__ void __launch_bounds__(PO_WARPS * 32) k_po(POGeom g, typename P::Params prm) {
+    grid_wait();
     __shared__ float ring[PO_WARPS][PO_W * 32][P::NS];
     __shared__ uint32_t stl[PO_WARPS][PO_CMAX], srv[PO_WARPS][PO_CMAX];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -908,6 +913,7 @@ __global__ void k_p4po_rows(int n, const uint2 *__restrict__ tofs, const int32_t
                             const float4 *__restrict__ rowA, const float2 *__restrict__ rowB,
                             const float *__restrict__ mass, FParams fp, float4 *__restrict__ acc,
                             float2 *__restrict__ vq) {
+    grid_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int tile = i / TILE, lane = i % TILE;
@@ -1008,6 +1014,7 @@ template <bool COMP, bool DUAL>
 __global__ void k_p5po_rows(int n, const uint2 *__restrict__ tofs, const int32_t *__restrict__ self,
                             const float2 *__restrict__ rowB, const float *__restrict__ mass, float inv_a4,
                             const unsigned long long *skip, float *__restrict__ du, float *__restrict__ du2) {
+    grid_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     if (skip && *(volatile const unsigned long long *)skip) return;
@@ -1054,6 +1061,7 @@ static FParams fparams(const crk_params &c) {
 // kick velocities (w unused) -> sig = (vb + va, s)
 __global__ void k_sig(int n, const float4 *__restrict__ vb, const float4 *__restrict__ va,
                       const float *__restrict__ sfun, float4 *__restrict__ sig) {
+    grid_wait();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     float4 b = vb[i], a = va[i];
@@ -1069,13 +1077,12 @@ static int run_forces_po(crk_ctx *ctx, const float4 *fr, const FParams &fp, cuda
     if (rc) return rc;
     typename P4PO<COMP, STATIC>::Params p{fr, ctx->mass, fp, ctx->acc, ctx->vq, ctx->Fst, ctx->po_rowA, ctx->po_rowB};
     prof_begin(ctx, PROF_P4, s);
-    k_po_low<<<grid_for(ctx->n, 256), 256, 0, s>>>(ctx->n, ctx->kcap, ctx->cnt_g, ctx->cnt_u, ctx->ent, ctx->lowc);
-    k_po_rev<<<grid_for(ctx->ntiles, 8), 256, 0, s>>>(ctx->ntiles, ctx->uofs, ctx->ulist, ctx->po_rev,
-                                                       ctx->po_self, ctx->po_tofs, ctx->po_tlist,
-                                                       ctx->counters + CNT_PO_MISS);
-    k_po<P4PO<COMP, STATIC>><<<grid_for(ctx->ntiles, PO_WARPS), PO_WARPS * 32, 0, s>>>(po_geom(ctx), p);
-    k_p4po_rows<COMP><<<grid_for(ctx->n, 256), 256, 0, s>>>(ctx->n, ctx->po_tofs, ctx->po_self, ctx->po_rowA,
-                                                            ctx->po_rowB, ctx->mass, fp, ctx->acc, ctx->vq);
+    launch(s, grid_for(ctx->n, 256), 256, 0, k_po_low, ctx->n, ctx->kcap, ctx->cnt_g, ctx->cnt_u, ctx->ent, ctx->lowc);
+    launch(s, grid_for(ctx->ntiles, 8), 256, 0, k_po_rev, ctx->ntiles, ctx->uofs, ctx->ulist, ctx->po_rev,
+           ctx->po_self, ctx->po_tofs, ctx->po_tlist, ctx->counters + CNT_PO_MISS);
+    launch(s, grid_for(ctx->ntiles, PO_WARPS), PO_WARPS * 32, 0, k_po<P4PO<COMP, STATIC>>, po_geom(ctx), p);
+    launch(s, grid_for(ctx->n, 256), 256, 0, k_p4po_rows<COMP>, ctx->n, ctx->po_tofs, ctx->po_self, ctx->po_rowA,
+           ctx->po_rowB, ctx->mass, fp, ctx->acc, ctx->vq);
     ctx->launches += 4;
     prof_end(ctx, s);
     CRK_LAUNCH_CHECK(ctx, "P4 forces (pair-once)");
@@ -1090,9 +1097,9 @@ static int run_compat_po(crk_ctx *ctx, const float4 *sig, float ia4, const unsig
     if (!ctx->lists_valid) return crk_set_error(ctx, CRK_ESTATE, "%s: neighbour lists are not built", what);
     typename P5PO<COMP, DUAL>::Params p{sig, ctx->Fst, ctx->mass, ctx->du, ia4, skip, du2, ctx->po_rowB};
     prof_begin(ctx, PROF_P5, s);
-    k_po<P5PO<COMP, DUAL>><<<grid_for(ctx->ntiles, PO_WARPS), PO_WARPS * 32, 0, s>>>(po_geom(ctx), p);
-    k_p5po_rows<COMP, DUAL><<<grid_for(ctx->n, 256), 256, 0, s>>>(ctx->n, ctx->po_tofs, ctx->po_self, ctx->po_rowB,
-                                                                  ctx->mass, ia4, skip, ctx->du, du2);
+    launch(s, grid_for(ctx->ntiles, PO_WARPS), PO_WARPS * 32, 0, k_po<P5PO<COMP, DUAL>>, po_geom(ctx), p);
+    launch(s, grid_for(ctx->n, 256), 256, 0, k_p5po_rows<COMP, DUAL>, ctx->n, ctx->po_tofs, ctx->po_self,
+           ctx->po_rowB, ctx->mass, ia4, skip, ctx->du, du2);
     ctx->launches += 2;
     prof_end(ctx, s);
     CRK_LAUNCH_CHECK(ctx, what);
@@ -1124,7 +1131,7 @@ int run_forces(crk_ctx *ctx, cudaStream_t s) {
     }
     FSrc src{ctx->q4, ctx->hs, ctx->p.density ? ctx->rho : nullptr, ctx->V, ctx->vel, ctx->mass, ctx->corr,
              ctx->gv};
-    k_pack_frec<<<grid_for(ctx->n, 256), 256, 0, s>>>(ctx->n, src, fp, ctx->frec, ctx->sfun);
+    launch(s, grid_for(ctx->n, 256), 256, 0, k_pack_frec, ctx->n, src, fp, ctx->frec, ctx->sfun);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "pack pair records");
     const bool comp = ctx->p.precision >= 1, still = ctx->p.a == 1.0 && ctx->p.adot == 0.0;
@@ -1136,7 +1143,7 @@ int run_forces(crk_ctx *ctx, cudaStream_t s) {
 // skip (device flag, may be null) makes the pass read nothing when set.
 int run_compatible(crk_ctx *ctx, cudaStream_t s, const unsigned long long *skip) {
     if (ctx->n == 0) return CRK_OK;
-    k_sig<<<grid_for(ctx->n, 256), 256, 0, s>>>(ctx->n, ctx->vb, ctx->va, ctx->sfun, ctx->sig);
+    launch(s, grid_for(ctx->n, 256), 256, 0, k_sig, ctx->n, ctx->vb, ctx->va, ctx->sfun, ctx->sig);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "kick sums");
     const float ia4 = (float)(1.0 / (ctx->p.a * ctx->p.a * ctx->p.a * ctx->p.a));
@@ -1161,6 +1168,7 @@ int run_compatible(crk_ctx *ctx, cudaStream_t s, const unsigned long long *skip)
 __global__ void k_sig_dual(int n, const double *dtn, const int32_t *__restrict__ sbox,
                            const float4 *__restrict__ vb, const float4 *__restrict__ va,
                            const float4 *__restrict__ acc, const float *__restrict__ sfun, float4 *__restrict__ sig2) {
+    grid_wait();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     float h = (float)(0.5 * dtn[sbox ? sbox[i] : 0]);
@@ -1174,8 +1182,8 @@ __global__ void k_sig_dual(int n, const double *dtn, const int32_t *__restrict__
 // kick (its dt per box in dtn; into du_next) in one pass over the stored forces.
 int run_compatible_dual(crk_ctx *ctx, const double *dtn, const int32_t *sbox, cudaStream_t s) {
     if (ctx->n == 0) return CRK_OK;
-    k_sig_dual<<<grid_for(ctx->n, 256), 256, 0, s>>>(ctx->n, dtn, sbox, ctx->vb, ctx->va, ctx->acc, ctx->sfun,
-                                                      ctx->sig2);
+    launch(s, grid_for(ctx->n, 256), 256, 0, k_sig_dual, ctx->n, dtn, sbox, ctx->vb, ctx->va, ctx->acc, ctx->sfun,
+           ctx->sig2);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "kick sums");
     const float ia4 = (float)(1.0 / (ctx->p.a * ctx->p.a * ctx->p.a * ctx->p.a));

@@ -51,6 +51,7 @@ __device__ __forceinline__ bool tile_active(const int32_t *tt0, const int32_t *t
 // with its doubled step.  Writes the tentative level.
 __global__ void k_htb_req(int count, const int32_t *__restrict__ act, int n, const float *__restrict__ dt,
                           HtbConsts c, int mid, int t, int32_t *__restrict__ tlev, unsigned long long *cnt) {
+    grid_wait();
     const int lane = threadIdx.x & 31;
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (w >= count) return;
@@ -78,6 +79,7 @@ __global__ void k_htb_req(int count, const int32_t *__restrict__ act, int n, con
 __global__ void k_htb_limit(int count, const int32_t *__restrict__ act, const uint2 *__restrict__ ofs,
                             const uint32_t *__restrict__ list, int f_l, int32_t *tlev,
                             unsigned long long *changed) {
+    grid_wait();
     const int lane = threadIdx.x & 31;
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (w >= count) return;
@@ -98,6 +100,7 @@ __global__ void k_htb_wake(int count, const int32_t *__restrict__ act, const uin
                            const uint32_t *__restrict__ list, const int32_t *__restrict__ tlev,
                            const int32_t *__restrict__ tt0, const int32_t *__restrict__ tlen, int t, int f_l,
                            int32_t *twake) {
+    grid_wait();
     const int lane = threadIdx.x & 31;
     const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (w >= count) return;
@@ -117,6 +120,7 @@ __global__ void k_htb_wake(int count, const int32_t *__restrict__ act, const uin
 __global__ void k_htb_apply_wake(int ntiles, int n, HtbConsts c, int t, int32_t *tlev, const int32_t *tt0,
                                  int32_t *tlen, int32_t *twake, const float4 *__restrict__ acc,
                                  const float *__restrict__ du_open, float4 *st_half, unsigned long long *cnt) {
+    grid_wait();
     const int lane = threadIdx.x & 31;
     const int T = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (T >= ntiles) return;
@@ -158,6 +162,7 @@ __global__ void k_htb_drift(int n, HtbConsts c, int t, int t1, const int32_t *__
                             const float4 *__restrict__ acc, const float *__restrict__ du_open,
                             float4 *__restrict__ vel, uint4 *__restrict__ q4, float *__restrict__ hs,
                             float *__restrict__ hc) {
+    grid_wait();
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     const int T = s / TILE;
@@ -185,6 +190,7 @@ __global__ void k_htb_drift(int n, HtbConsts c, int t, int t1, const int32_t *__
 
 // fixed-point records and h of the state (refit without a sort)
 __global__ void k_htb_records(int n, const float4 *__restrict__ st_pos, uint4 *__restrict__ q4, float *__restrict__ hs) {
+    grid_wait();
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     const float4 p = st_pos[s];
@@ -198,6 +204,7 @@ __global__ void k_htb_close(int n, HtbConsts c, int t, const int32_t *__restrict
                             const int32_t *__restrict__ tlen, const float4 *__restrict__ st_half,
                             const float4 *__restrict__ acc, const float4 *__restrict__ vel, float4 *__restrict__ vb,
                             float4 *__restrict__ va) {
+    grid_wait();
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     const int T = s / TILE;
@@ -218,6 +225,7 @@ __global__ void k_htb_close(int n, HtbConsts c, int t, const int32_t *__restrict
 __global__ void k_htb_after_close(int n, HtbConsts c, int t, const int32_t *__restrict__ tt0,
                                   const int32_t *__restrict__ tlen, float4 *st_half, const float4 *__restrict__ va,
                                   const float *__restrict__ du, const float *__restrict__ Nn, float4 *st_pos) {
+    grid_wait();
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     const int T = s / TILE;
@@ -239,6 +247,7 @@ __global__ void k_htb_open(int n, HtbConsts c, int t, const int32_t *__restrict_
                            const int32_t *__restrict__ tt0, const int32_t *__restrict__ tlen,
                            const float4 *__restrict__ st_half, const float4 *__restrict__ acc,
                            const float4 *__restrict__ vel, float4 *__restrict__ vb, float4 *__restrict__ va) {
+    grid_wait();
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     const int T = s / TILE;
@@ -260,6 +269,7 @@ __global__ void k_htb_after_open(int n, HtbConsts c, int t, const int32_t *__res
                                  const int32_t *__restrict__ tt0, const int32_t *__restrict__ tlen, float4 *st_half,
                                  const float4 *__restrict__ va, const float *__restrict__ du,
                                  float *__restrict__ du_open) {
+    grid_wait();
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     const int T = s / TILE;
@@ -274,6 +284,7 @@ __global__ void k_htb_after_open(int n, HtbConsts c, int t, const int32_t *__res
 // the active leaves start their new step at t
 __global__ void k_htb_set_steps(int ntiles, HtbConsts c, int t, const int32_t *__restrict__ tlev, int32_t *tt0,
                                 int32_t *tlen) {
+    grid_wait();
     const int T = blockIdx.x * blockDim.x + threadIdx.x;
     if (T >= ntiles || !tile_active(tt0, tlen, T, t)) return;
     tt0[T] = t;
@@ -283,6 +294,7 @@ __global__ void k_htb_set_steps(int ntiles, HtbConsts c, int t, const int32_t *_
 // earliest step end over the tiles
 __global__ void k_htb_tnext(int ntiles, const int32_t *__restrict__ tt0, const int32_t *__restrict__ tlen,
                             unsigned long long *cnt) {
+    grid_wait();
     const int T = blockIdx.x * blockDim.x + threadIdx.x;
     const unsigned e = T < ntiles ? (unsigned)(tt0[T] + tlen[T]) : 0xffffffffu;
     const unsigned m = __reduce_min_sync(FULLM, e);
@@ -291,6 +303,7 @@ __global__ void k_htb_tnext(int ntiles, const int32_t *__restrict__ tt0, const i
 
 __global__ void k_htb_flags(int ntiles, const int32_t *__restrict__ tt0, const int32_t *__restrict__ tlen, int t,
                             uint32_t *__restrict__ flag) {
+    grid_wait();
     const int T = blockIdx.x * blockDim.x + threadIdx.x;
     if (T < ntiles) flag[T] = tile_active(tt0, tlen, T, t) ? 1u : 0u;
 }
@@ -298,6 +311,7 @@ __global__ void k_htb_flags(int ntiles, const int32_t *__restrict__ tt0, const i
 // active tiles in ascending order, their count and their particles
 __global__ void k_htb_compact(int ntiles, int n, const uint32_t *__restrict__ flag, const uint32_t *__restrict__ ofs,
                               int32_t *__restrict__ act, unsigned long long *cnt) {
+    grid_wait();
     const int T = blockIdx.x * blockDim.x + threadIdx.x;
     unsigned parts = 0;
     if (T < ntiles && flag[T]) {
@@ -311,6 +325,7 @@ __global__ void k_htb_compact(int ntiles, int n, const uint32_t *__restrict__ fl
 
 // each slot takes its tile's level (for the caller's per-particle view)
 __global__ void k_htb_slot_level(int n, const int32_t *__restrict__ tlev, int32_t *__restrict__ out) {
+    grid_wait();
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s < n) out[s] = tlev[s / TILE];
 }
@@ -320,6 +335,7 @@ __global__ void k_htb_permute(int n, const int32_t *__restrict__ idx, const floa
                               float4 *__restrict__ ao, const float4 *__restrict__ b, float4 *__restrict__ bo,
                               const float4 *__restrict__ c, float4 *__restrict__ co, const float *__restrict__ d,
                               float *__restrict__ dout) {
+    grid_wait();
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     const int o = idx[s];
@@ -333,6 +349,7 @@ __global__ void k_htb_permute(int n, const int32_t *__restrict__ idx, const floa
 // vb = p_1/2, va = p_1/2 + a hc
 __global__ void k_htb_close_all(int n, const float *__restrict__ hc, const float4 *__restrict__ st_half,
                                 const float4 *__restrict__ acc, float4 *__restrict__ vb, float4 *__restrict__ va) {
+    grid_wait();
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     const float h = hc[s];
@@ -344,6 +361,7 @@ __global__ void k_htb_close_all(int n, const float *__restrict__ hc, const float
 __global__ void k_htb_finish_all(int n, HtbConsts c, const float *__restrict__ hc, const float4 *__restrict__ st_half,
                                  const float4 *__restrict__ va, const float *__restrict__ du,
                                  const float *__restrict__ Nn, float4 *__restrict__ st_vel, float4 *st_pos) {
+    grid_wait();
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     const float4 a = va[s];
@@ -406,6 +424,7 @@ static int ensure_htb(crk_ctx *ctx) {
 
 // tile t holds a particle whose eq:hi solve is not yet done (flags[s] == 0)
 __global__ void k_unconv_flags(int ntiles, int n, const int32_t *__restrict__ flags, uint32_t *__restrict__ tflag) {
+    grid_wait();
     const int T = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
     if (T >= ntiles) return;
     const int s = T * TILE + (int)(threadIdx.x & 31);
@@ -422,11 +441,11 @@ int unconverged_tiles(crk_ctx *ctx, cudaStream_t s) {
     if (rc) return rc;
     const int nt = ctx->ntiles;
     CRK_CUDA(ctx, cudaMemsetAsync(ctx->counters + CNT_NACT, 0, 2 * sizeof(unsigned long long), s));
-    k_unconv_flags<<<grid_for((long long)nt * 32, 256), 256, 0, s>>>(nt, ctx->n, ctx->flags, ctx->tflag);
+    launch(s, grid_for((long long)nt * 32, 256), 256, 0, k_unconv_flags, nt, ctx->n, ctx->flags, ctx->tflag);
     ++ctx->launches;
     rc = scan_u32(ctx, ctx->tflag, ctx->tscan, nt, s);
     if (rc) return rc;
-    k_htb_compact<<<grid_for(nt, 256), 256, 0, s>>>(nt, ctx->n, ctx->tflag, ctx->tscan, ctx->tact, ctx->counters);
+    launch(s, grid_for(nt, 256), 256, 0, k_htb_compact, nt, ctx->n, ctx->tflag, ctx->tscan, ctx->tact, ctx->counters);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "unconverged tiles");
     return CRK_OK;
@@ -476,8 +495,8 @@ static int limit(crk_ctx *ctx, const int32_t *act, int count, int f_l, int L, cu
     for (long long it = 0; it < cap; it += 4) {
         CRK_CUDA(ctx, cudaMemsetAsync(ctx->counters + CNT_CHANGED, 0, sizeof(unsigned long long), s));
         for (int k = 0; k < 4; k++) {
-            k_htb_limit<<<grid_for((long long)count * 32, 256), 256, 0, s>>>(count, act, ctx->uofs, ctx->ulist, f_l,
-                                                                         ctx->tlev, ctx->counters + CNT_CHANGED);
+            launch(s, grid_for((long long)count * 32, 256), 256, 0, k_htb_limit, count, act, ctx->uofs, ctx->ulist,
+                   f_l, ctx->tlev, ctx->counters + CNT_CHANGED);
             ++ctx->launches;
         }
         CRK_LAUNCH_CHECK(ctx, "level limiter");
@@ -493,7 +512,7 @@ static int next_tick(crk_ctx *ctx, int *t_next, cudaStream_t s) {
     const int nt = ctx->ntiles;
     const unsigned long long big = 0xffffffffull;
     CRK_CUDA(ctx, cudaMemcpyAsync(ctx->counters + CNT_TNEXT, &big, sizeof(big), cudaMemcpyHostToDevice, s));
-    k_htb_tnext<<<grid_for(nt, 256), 256, 0, s>>>(nt, ctx->tt0, ctx->tlen, ctx->counters);
+    launch(s, grid_for(nt, 256), 256, 0, k_htb_tnext, nt, ctx->tt0, ctx->tlen, ctx->counters);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "next tick");
     int rc = crk_sync_counters(ctx, s);
@@ -505,11 +524,11 @@ static int next_tick(crk_ctx *ctx, int *t_next, cudaStream_t s) {
 static int active_list(crk_ctx *ctx, int t, long long *parts, cudaStream_t s) {
     const int nt = ctx->ntiles;
     CRK_CUDA(ctx, cudaMemsetAsync(ctx->counters + CNT_NACT, 0, 2 * sizeof(unsigned long long), s));
-    k_htb_flags<<<grid_for(nt, 256), 256, 0, s>>>(nt, ctx->tt0, ctx->tlen, t, ctx->tflag);
+    launch(s, grid_for(nt, 256), 256, 0, k_htb_flags, nt, ctx->tt0, ctx->tlen, t, ctx->tflag);
     ++ctx->launches;
     int rc = scan_u32(ctx, ctx->tflag, ctx->tscan, nt, s);
     if (rc) return rc;
-    k_htb_compact<<<grid_for(nt, 256), 256, 0, s>>>(nt, ctx->n, ctx->tflag, ctx->tscan, ctx->tact, ctx->counters);
+    launch(s, grid_for(nt, 256), 256, 0, k_htb_compact, nt, ctx->n, ctx->tflag, ctx->tscan, ctx->tact, ctx->counters);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "active leaves");
     rc = crk_sync_counters(ctx, s);
@@ -551,15 +570,15 @@ static int cycle_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const flo
     if (rc) return rc;
     const int nt = ctx->ntiles;
     // leaf boxes and interaction lists at the state (current h)
-    k_htb_records<<<g, b, 0, s>>>(n, ctx->st_pos, ctx->q4, ctx->hs);
+    launch(s, g, b, 0, k_htb_records, n, ctx->st_pos, ctx->q4, ctx->hs);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "leaf records");
     rc = refit_lists(ctx, s);
     if (rc) return rc;
     // levels at the cycle start: requirement, then the limiter's fixed point
     CRK_CUDA(ctx, cudaMemsetAsync(ctx->counters + CNT_UNRES, 0, 2 * sizeof(unsigned long long), s));
-    k_htb_req<<<grid_for((long long)nt * 32, 256), 256, 0, s>>>(nt, nullptr, n, ctx->d_dt, c, 0, 0, ctx->tlev,
-                                                              ctx->counters);
+    launch(s, grid_for((long long)nt * 32, 256), 256, 0, k_htb_req, nt, nullptr, n, ctx->d_dt, c, 0, 0, ctx->tlev,
+           ctx->counters);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "leaf levels");
     rc = limit(ctx, nullptr, nt, c.f_l, c.L, s);
@@ -578,15 +597,15 @@ static int cycle_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const flo
     std::vector<int32_t> none(nt, NO_LEVEL);
     CRK_CUDA(ctx, cudaMemcpyAsync(ctx->twake, none.data(), sizeof(int32_t) * nt, cudaMemcpyHostToDevice, s));
     CRK_CUDA(ctx, cudaMemcpyAsync(ctx->st_half, ctx->st_vel, sizeof(float4) * n, cudaMemcpyDeviceToDevice, s));
-    k_htb_open<<<g, b, 0, s>>>(n, c, 0, ctx->tlev, ctx->tt0, ctx->tlen, ctx->st_half, ctx->acc, ctx->vel, ctx->vb,
-                               ctx->va);
+    launch(s, g, b, 0, k_htb_open, n, c, 0, ctx->tlev, ctx->tt0, ctx->tlen, ctx->st_half, ctx->acc, ctx->vel, ctx->vb,
+           ctx->va);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "opening kick");
     rc = run_compatible(ctx, s);
     if (rc) return rc;
-    k_htb_after_open<<<g, b, 0, s>>>(n, c, 0, ctx->tlev, ctx->tt0, ctx->tlen, ctx->st_half, ctx->va, ctx->du,
-                                     ctx->du_open);
-    k_htb_set_steps<<<grid_for(nt, 256), 256, 0, s>>>(nt, c, 0, ctx->tlev, ctx->tt0, ctx->tlen);
+    launch(s, g, b, 0, k_htb_after_open, n, c, 0, ctx->tlev, ctx->tt0, ctx->tlen, ctx->st_half, ctx->va, ctx->du,
+           ctx->du_open);
+    launch(s, grid_for(nt, 256), 256, 0, k_htb_set_steps, nt, c, 0, ctx->tlev, ctx->tt0, ctx->tlen);
     ctx->launches += 2;
     CRK_LAUNCH_CHECK(ctx, "opening kick");
     long long evals = 0;
@@ -600,8 +619,8 @@ static int cycle_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const flo
         if (t1 <= t || t1 > T) return crk_set_error(ctx, CRK_ESTATE, "time bins: bad next tick %d after %d", t1, t);
         ++ticks;
         if (t1 == T) {
-            k_htb_drift<<<g, b, 0, s>>>(n, c, t, t1, ctx->tt0, ctx->tlen, ctx->st_pos, ctx->st_half, ctx->acc,
-                                        ctx->du_open, ctx->vel, ctx->q4, ctx->hs, ctx->hc);
+            launch(s, g, b, 0, k_htb_drift, n, c, t, t1, ctx->tt0, ctx->tlen, ctx->st_pos, ctx->st_half, ctx->acc,
+                   ctx->du_open, ctx->vel, ctx->q4, ctx->hs, ctx->hc);
             ++ctx->launches;
             CRK_LAUNCH_CHECK(ctx, "stream");
             break;
@@ -610,8 +629,8 @@ static int cycle_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const flo
         rc = active_list(ctx, t1, &parts, s);
         if (rc) return rc;
         evals += parts;
-        k_htb_drift<<<g, b, 0, s>>>(n, c, t, t1, ctx->tt0, ctx->tlen, ctx->st_pos, ctx->st_half, ctx->acc,
-                                    ctx->du_open, ctx->vel, ctx->q4, ctx->hs, nullptr);
+        launch(s, g, b, 0, k_htb_drift, n, c, t, t1, ctx->tt0, ctx->tlen, ctx->st_pos, ctx->st_half, ctx->acc,
+               ctx->du_open, ctx->vel, ctx->q4, ctx->hs, nullptr);
         ++ctx->launches;
         CRK_LAUNCH_CHECK(ctx, "stream");
         t = t1;
@@ -626,18 +645,19 @@ static int cycle_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const flo
             return rc;
         }
         // closing kick, its compatible energy, h
-        k_htb_close<<<g, b, 0, s>>>(n, c, t, ctx->tt0, ctx->tlen, ctx->st_half, ctx->acc, ctx->vel, ctx->vb, ctx->va);
+        launch(s, g, b, 0, k_htb_close, n, c, t, ctx->tt0, ctx->tlen, ctx->st_half, ctx->acc, ctx->vel, ctx->vb,
+               ctx->va);
         ++ctx->launches;
         rc = run_compatible(ctx, s);
         if (rc) {
             leave_active_mode(ctx);
             return rc;
         }
-        k_htb_after_close<<<g, b, 0, s>>>(n, c, t, ctx->tt0, ctx->tlen, ctx->st_half, ctx->va, ctx->du, ctx->Nn,
-                                          ctx->st_pos);
+        launch(s, g, b, 0, k_htb_after_close, n, c, t, ctx->tt0, ctx->tlen, ctx->st_half, ctx->va, ctx->du, ctx->Nn,
+               ctx->st_pos);
         // new levels of the active leaves, limiter over them, wake-ups
-        k_htb_req<<<grid_for((long long)ctx->nact * 32, 256), 256, 0, s>>>(ctx->nact, ctx->tact, n, ctx->d_dt, c, 1,
-                                                                           t, ctx->tlev, ctx->counters);
+        launch(s, grid_for((long long)ctx->nact * 32, 256), 256, 0, k_htb_req, ctx->nact, ctx->tact, n, ctx->d_dt, c,
+               1, t, ctx->tlev, ctx->counters);
         ctx->launches += 2;
         CRK_LAUNCH_CHECK(ctx, "leaf levels");
         rc = limit(ctx, ctx->tact, ctx->nact, c.f_l, c.L, s);
@@ -645,24 +665,21 @@ static int cycle_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const flo
             leave_active_mode(ctx);
             return rc;
         }
-        k_htb_wake<<<grid_for((long long)ctx->nact * 32, 256), 256, 0, s>>>(ctx->nact, ctx->tact, ctx->uofs,
-                                                                            ctx->ulist, ctx->tlev, ctx->tt0,
-                                                                            ctx->tlen, t, c.f_l, ctx->twake);
-        k_htb_apply_wake<<<grid_for((long long)nt * 32, 256), 256, 0, s>>>(nt, n, c, t, ctx->tlev, ctx->tt0,
-                                                                           ctx->tlen, ctx->twake, ctx->acc,
-                                                                           ctx->du_open, ctx->st_half,
-                                                                           ctx->counters);
+        launch(s, grid_for((long long)ctx->nact * 32, 256), 256, 0, k_htb_wake, ctx->nact, ctx->tact, ctx->uofs,
+               ctx->ulist, ctx->tlev, ctx->tt0, ctx->tlen, t, c.f_l, ctx->twake);
+        launch(s, grid_for((long long)nt * 32, 256), 256, 0, k_htb_apply_wake, nt, n, c, t, ctx->tlev, ctx->tt0,
+               ctx->tlen, ctx->twake, ctx->acc, ctx->du_open, ctx->st_half, ctx->counters);
         // opening kick of the new step
-        k_htb_open<<<g, b, 0, s>>>(n, c, t, ctx->tlev, ctx->tt0, ctx->tlen, ctx->st_half, ctx->acc, ctx->vel,
-                                   ctx->vb, ctx->va);
+        launch(s, g, b, 0, k_htb_open, n, c, t, ctx->tlev, ctx->tt0, ctx->tlen, ctx->st_half, ctx->acc, ctx->vel,
+               ctx->vb, ctx->va);
         ctx->launches += 3;
         CRK_LAUNCH_CHECK(ctx, "wake-ups and opening kick");
         rc = run_compatible(ctx, s);
         leave_active_mode(ctx);
         if (rc) return rc;
-        k_htb_after_open<<<g, b, 0, s>>>(n, c, t, ctx->tlev, ctx->tt0, ctx->tlen, ctx->st_half, ctx->va, ctx->du,
-                                         ctx->du_open);
-        k_htb_set_steps<<<grid_for(nt, 256), 256, 0, s>>>(nt, c, t, ctx->tlev, ctx->tt0, ctx->tlen);
+        launch(s, g, b, 0, k_htb_after_open, n, c, t, ctx->tlev, ctx->tt0, ctx->tlen, ctx->st_half, ctx->va, ctx->du,
+               ctx->du_open);
+        launch(s, grid_for(nt, 256), 256, 0, k_htb_set_steps, nt, c, t, ctx->tlev, ctx->tt0, ctx->tlen);
         ctx->launches += 2;
         CRK_LAUNCH_CHECK(ctx, "opening kick");
     }
@@ -671,8 +688,8 @@ static int cycle_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const flo
     rc = build_cells_sorted(ctx, n, ctx->st_pos, ctx->perm, s);
     if (!rc) rc = finish_build(ctx, s);
     if (rc) return rc;
-    k_htb_permute<<<g, b, 0, s>>>(n, ctx->idx_a, ctx->st_pos, ctx->st_tmp, ctx->vel, ctx->vb, ctx->st_half, ctx->va,
-                                  ctx->hc, ctx->st_tmp1);
+    launch(s, g, b, 0, k_htb_permute, n, ctx->idx_a, ctx->st_pos, ctx->st_tmp, ctx->vel, ctx->vb, ctx->st_half,
+           ctx->va, ctx->hc, ctx->st_tmp1);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "permute state");
     float4 *tp;
@@ -684,12 +701,13 @@ static int cycle_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const flo
     if (!rc) rc = evaluate(ctx, s);
     if (rc) return rc;
     evals += n;
-    k_htb_close_all<<<g, b, 0, s>>>(n, ctx->hc, ctx->st_half, ctx->acc, ctx->vb, ctx->va);
+    launch(s, g, b, 0, k_htb_close_all, n, ctx->hc, ctx->st_half, ctx->acc, ctx->vb, ctx->va);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "closing kick");
     rc = run_compatible(ctx, s);
     if (rc) return rc;
-    k_htb_finish_all<<<g, b, 0, s>>>(n, c, ctx->hc, ctx->st_half, ctx->va, ctx->du, ctx->Nn, ctx->st_vel, ctx->st_pos);
+    launch(s, g, b, 0, k_htb_finish_all, n, c, ctx->hc, ctx->st_half, ctx->va, ctx->du, ctx->Nn, ctx->st_vel,
+           ctx->st_pos);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "finish cycle");
     rc = scatter_rows(ctx, ctx->st_pos, pos_h, 4, s);
@@ -745,13 +763,13 @@ extern "C" int crk_htb_levels(crk_ctx *ctx, int n, const float *pos_h, const flo
     const HtbConsts c = htb_consts(ctx, Delta, L, f_l);
     const int nt = ctx->ntiles;
     CRK_CUDA(ctx, cudaMemsetAsync(ctx->counters + CNT_UNRES, 0, sizeof(unsigned long long), s));
-    k_htb_req<<<grid_for((long long)nt * 32, 256), 256, 0, s>>>(nt, nullptr, n, ctx->d_dt, c, 0, 0, ctx->tlev,
-                                                              ctx->counters);
+    launch(s, grid_for((long long)nt * 32, 256), 256, 0, k_htb_req, nt, nullptr, n, ctx->d_dt, c, 0, 0, ctx->tlev,
+           ctx->counters);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "leaf levels");
     rc = limit(ctx, nullptr, nt, f_l, L, s);
     if (rc) return rc;
-    k_htb_slot_level<<<grid_for(n, 256), 256, 0, s>>>(n, ctx->tlev, reinterpret_cast<int32_t *>(ctx->st_tmp1));
+    launch(s, grid_for(n, 256), 256, 0, k_htb_slot_level, n, ctx->tlev, reinterpret_cast<int32_t *>(ctx->st_tmp1));
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "leaf levels");
     rc = scatter_rows(ctx, ctx->st_tmp1, level, 1, s);

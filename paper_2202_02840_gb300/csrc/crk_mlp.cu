@@ -96,11 +96,10 @@ __device__ __forceinline__ float2 silu2(float z0, float z1, float2 *ds = nullptr
     return up2(mul2(z, sg));
 }
 
-// Dependent launches of a training step (programmatic stream serialisation): a
-// kernel may start while the one before it still runs, up to grid_wait(), behind
-// which everything that one wrote is visible in L2.  What a training kernel
-// writes is therefore read with ld_l2, never through L1.
-__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// The two kernels of a training step also let the next one start while they run
+// (grid_launch_next), so it may be in place, and have read what no training kernel
+// writes, when they end.  What a training kernel writes is read with ld_l2, never
+// through L1.
 __device__ __forceinline__ void grid_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ float ld_l2(const float *p) {
     float v;
@@ -171,6 +170,7 @@ __device__ __forceinline__ uint32_t feat_cell(const float4 &p, int kf) {
 
 __global__ void k_feat_count(int n, int kf, const float4 *__restrict__ pos_h, int32_t *__restrict__ fcnt,
                              unsigned long long *err) {
+    grid_wait();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     bool ok = false;
     uint32_t cell = 0;
@@ -214,6 +214,7 @@ __device__ __forceinline__ void cell_features(int kf, int c, const int32_t *fcnt
 
 // They depend on the cell alone: once per cell for its 64 to 511 particles.
 __global__ void k_feat_table(int kf, const int32_t *__restrict__ fcnt, float *__restrict__ ftab) {
+    grid_wait();
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c >> (3 * kf)) return;
     float f[5];
@@ -258,6 +259,7 @@ __device__ __forceinline__ void row_features(const FeatArgs &a, int i, float (&f
 // feat[8i..8i+7] and, with pos_conv, target[i] = log(h_conv / h_prev)
 __global__ void k_features(FeatArgs a, const float4 *__restrict__ pos_conv, float *__restrict__ feat,
                            float *__restrict__ target) {
+    grid_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= a.n) return;
     float f[8], h, N;
@@ -373,10 +375,11 @@ __global__ void __launch_bounds__(256, 4) k_mlp_fwd(int n, int span, const float
                                                     const float *__restrict__ feat, float *__restrict__ y_out,
                                                     FeatArgs fa, float4 *pos_out, float tol, float h_min,
                                                     float h_max, float N_res) {
+    grid_wait();
     __shared__ __align__(16) FwdShm S;
     __shared__ __align__(16) RowShm rows[MODE == 1 ? 8 : 1];
     stage_fwd<256, false>(W, S);
-    float b3 = W[OFF_B3];
+    float b3 = ld_l2(W + OFF_B3);
     __syncthreads();
     int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     uint32_t w1f[8];
@@ -490,12 +493,14 @@ __device__ __forceinline__ int sample_row(const TrainArgs &a, int r) {
 // flag[i] = 1 where the judge hands particle i to the proposal
 __global__ void k_select_flags(int n, const float *__restrict__ Nngb, float N_res, float tol,
                                uint32_t *__restrict__ flag) {
+    grid_wait();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) flag[i] = fabsf(cbrtf(N_res / Nngb[i]) - 1.f) > tol ? 1u : 0u;
 }
 
 __global__ void k_select_rows(int n, int base, const uint32_t *__restrict__ flag, const uint32_t *__restrict__ ofs,
                               int32_t *__restrict__ rows, int *count) {
+    grid_wait();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     if (flag[i]) rows[ofs[i]] = base + i;
@@ -739,7 +744,7 @@ struct AdamArgs {
 // in flight at once (6.3 us with one thread per weight, 4.5 so).  A step is two
 // launches of a few microseconds each, so a third of it was their starts: with
 // dependent launches the blocks are in place, and the gradient's rows and the
-// master weights read, when the kernel before ends (a 4096-row step 15.1 -> 11.6 us).
+// master weights read, when the kernel before ends (a 4096-row step 15.1 -> 10.7 us).
 constexpr int ADAM_ROWS = 8;
 __global__ void __launch_bounds__(32 * ADAM_ROWS) k_adam(AdamArgs a) {
     __shared__ float sum[ADAM_ROWS][32];
@@ -812,10 +817,10 @@ int count_cells(crk_ctx *ctx, int n, const float4 *pos, int kf, cudaStream_t s) 
         CRK_CUDA(ctx, cudaMalloc((void **)&ctx->ftab, sizeof(float) * 8 * (size_t)cells));
         ctx->ftab_level = kf;
     }
-    k_feat_count<<<grid_for(n, 256), 256, 0, s>>>(n, kf, pos, ctx->fcnt, ctx->counters + CNT_MLP_ERR);
+    launch(s, grid_for(n, 256), 256, 0, k_feat_count, n, kf, pos, ctx->fcnt, ctx->counters + CNT_MLP_ERR);
     ++ctx->launches;
     if (table) {
-        k_feat_table<<<grid_for(cells, 128), 128, 0, s>>>(kf, ctx->fcnt, ctx->ftab);
+        launch(s, grid_for(cells, 128), 128, 0, k_feat_table, kf, ctx->fcnt, ctx->ftab);
         ++ctx->launches;
     }
     CRK_LAUNCH_CHECK(ctx, "feature cell count");
@@ -862,23 +867,6 @@ int fwd_blocks(const crk_ctx *ctx, int n, int *span) {
     return b > cap ? cap : b;
 }
 
-// Launch that may start while the kernel before it in the stream still runs (early).
-template <class Args>
-cudaError_t launch_dependent(void (*kernel)(Args), int grid, int block, size_t shm, cudaStream_t s, bool early,
-                             const Args &args) {
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)grid);
-    cfg.blockDim = dim3((unsigned)block);
-    cfg.dynamicSmemBytes = shm;
-    cfg.stream = s;
-    cfg.attrs = &attr;
-    cfg.numAttrs = early ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, args);
-}
-
 // One step.  follows: the stream's last kernel is the update of the step before, so
 // the gradient may start early (its first rows are read meanwhile); else it waits
 // for whatever made the data set.
@@ -914,7 +902,7 @@ int train_launch(crk_ctx *ctx, int n, const float *feat, const float *target, co
     ta.two_over_B = 2.f * Y_SCALE / (float)batch;   // dL/dy times dy/d(output layer)
     ta.part = ctx->mlp_part;
     prof_begin(ctx, PROF_MLP_TRAIN, s);
-    CRK_CUDA(ctx, launch_dependent(k_mlp_grad, nblk, 128, sizeof(GradShm), s, follows, ta));
+    launch_as(follows, s, nblk, 128, sizeof(GradShm), k_mlp_grad, ta);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "mlp gradient");
     AdamArgs aa;
@@ -934,7 +922,7 @@ int train_launch(crk_ctx *ctx, int n, const float *feat, const float *target, co
     aa.inv_B = 1.f / (float)batch;
     aa.grad_out = grad;
     aa.loss_out = loss;
-    CRK_CUDA(ctx, launch_dependent(k_adam, grid_for(NP + 1, 32), 32 * ADAM_ROWS, 0, s, true, aa));
+    launch(s, grid_for(NP + 1, 32), 32 * ADAM_ROWS, 0, k_adam, aa);
     ++ctx->launches;
     prof_end(ctx, s);
     CRK_LAUNCH_CHECK(ctx, "mlp adam");
@@ -1004,7 +992,7 @@ extern "C" int crk_h_features(crk_ctx *ctx, int n, const float *pos_h, const flo
     int rc = count_cells(ctx, n, reinterpret_cast<const float4 *>(pos_h), kf, s);
     if (rc) return rc;
     FeatArgs fa = feat_args(ctx, n, pos_h, gradv, Nngb, dt, kf);
-    k_features<<<grid_for(n, 256), 256, 0, s>>>(fa, reinterpret_cast<const float4 *>(pos_conv), feat, target);
+    launch(s, grid_for(n, 256), 256, 0, k_features, fa, reinterpret_cast<const float4 *>(pos_conv), feat, target);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "features");
     return check_records(ctx, s);
@@ -1021,7 +1009,7 @@ extern "C" int crk_mlp_forward(crk_ctx *ctx, int n, const float *feat, float *y,
     prof_begin(ctx, PROF_MLP_FWD, s);
     int span;
     const int blocks = fwd_blocks(ctx, n, &span);
-    k_mlp_fwd<0><<<blocks, 256, 0, s>>>(n, span, ctx->mlp_w, feat, y, none, nullptr, 0.f, 0.f, 0.f, 0.f);
+    launch(s, blocks, 256, 0, k_mlp_fwd<0>, n, span, ctx->mlp_w, feat, y, none, nullptr, 0.f, 0.f, 0.f, 0.f);
     ++ctx->launches;
     prof_end(ctx, s);
     CRK_LAUNCH_CHECK(ctx, "mlp forward");
@@ -1043,9 +1031,8 @@ extern "C" int crk_h_propose(crk_ctx *ctx, int n, float *pos_h, const float *gra
     FeatArgs fa = feat_args(ctx, n, pos_h, gradv, Nngb, dt, kf);
     int span;
     const int blocks = fwd_blocks(ctx, n, &span);
-    k_mlp_fwd<1><<<blocks, 256, 0, s>>>(n, span, ctx->mlp_w, nullptr, nullptr, fa,
-                                                     reinterpret_cast<float4 *>(pos_h), tol, (float)ctx->p.h_min,
-                                                     (float)ctx->p.h_max, (float)ctx->p.N_res);
+    launch(s, blocks, 256, 0, k_mlp_fwd<1>, n, span, ctx->mlp_w, nullptr, nullptr, fa,
+           reinterpret_cast<float4 *>(pos_h), tol, (float)ctx->p.h_min, (float)ctx->p.h_max, (float)ctx->p.N_res);
     ++ctx->launches;
     prof_end(ctx, s);
     CRK_LAUNCH_CHECK(ctx, "h proposal");
@@ -1070,8 +1057,8 @@ int propose_sorted(crk_ctx *ctx, int n, float4 *pos, const GvRec *gv, const floa
     fa.gv_stride = 12;
     int span;
     const int blocks = fwd_blocks(ctx, n, &span);
-    k_mlp_fwd<1><<<blocks, 256, 0, s>>>(n, span, ctx->mlp_w, nullptr, nullptr, fa, pos, tol,
-                                                     (float)ctx->p.h_min, (float)ctx->p.h_max, (float)ctx->p.N_res);
+    launch(s, blocks, 256, 0, k_mlp_fwd<1>, n, span, ctx->mlp_w, nullptr, nullptr, fa, pos, tol, (float)ctx->p.h_min,
+           (float)ctx->p.h_max, (float)ctx->p.N_res);
     ++ctx->launches;
     prof_end(ctx, s);
     CRK_LAUNCH_CHECK(ctx, "h proposal");
@@ -1105,13 +1092,13 @@ extern "C" int crk_h_select(crk_ctx *ctx, int n, const float *Nngb, float tol, i
     }
     uint32_t *flag = ctx->sel, *ofs = ctx->sel + n;
     int rc;
-    k_select_flags<<<grid_for(n, 256), 256, 0, s>>>(n, Nngb, (float)ctx->p.N_res, tol, flag);
+    launch(s, grid_for(n, 256), 256, 0, k_select_flags, n, Nngb, (float)ctx->p.N_res, tol, flag);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "select flags");
     rc = scan_u32(ctx, flag, ofs, n, s);
     if (rc) return rc;
     int *d_count = reinterpret_cast<int *>(ctx->counters + CNT_MLP_ERR);
-    k_select_rows<<<grid_for(n, 256), 256, 0, s>>>(n, base, flag, ofs, rows, d_count);
+    launch(s, grid_for(n, 256), 256, 0, k_select_rows, n, base, flag, ofs, rows, d_count);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "select rows");
     rc = crk_sync_counters(ctx, s);

@@ -30,6 +30,7 @@ struct PassGeom {
 //   count(const IState&) -> pairs of this lane
 template <class P, int WARPS>
 __global__ void __launch_bounds__(WARPS * 32) k_pass(PassGeom g, typename P::Params prm) {
+    grid_wait();
     __shared__ typename P::JRec sj[WARPS][32];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int tile = blockIdx.x * WARPS + w;
@@ -67,7 +68,7 @@ int launch_pass(crk_ctx *ctx, int prof_id, bool union_list, const typename P::Pa
     g.list = union_list ? ctx->ulist : ctx->glist;
     g.pairs = pairs;
     prof_begin(ctx, prof_id, s);
-    k_pass<P, WARPS><<<grid_for(ctx->ntiles, WARPS), WARPS * 32, 0, s>>>(g, prm);
+    launch(s, grid_for(ctx->ntiles, WARPS), WARPS * 32, 0, k_pass<P, WARPS>, g, prm);
     ++ctx->launches;
     prof_end(ctx, s);
     CRK_LAUNCH_CHECK(ctx, what);
@@ -328,6 +329,7 @@ __device__ __forceinline__ void lpass_tile(const ListGeom &g, const typename P::
 // tiles in Morton order).
 template <class P, int WARPS, int U, bool RP = false>
 __global__ void __launch_bounds__(WARPS * 32) k_lpass(ListGeom g, typename P::Params prm, const int32_t *order) {
+    grid_wait();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int t = blockIdx.x * WARPS + w;
     if (t >= g.ntiles) return;
@@ -344,6 +346,7 @@ __global__ void __launch_bounds__(WARPS * 32) k_lpass(ListGeom g, typename P::Pa
 template <class P, int U, bool RP = false>
 __global__ void __launch_bounds__(32) k_lpass_sm(ListGeom g, typename P::Params prm, uint32_t *next, int nrange,
                                                  int chunk) {
+    grid_wait();
     const int lane = threadIdx.x & 31;
     unsigned smid;
     asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
@@ -380,6 +383,7 @@ constexpr int split_warps() {   // as many as their sums fit static shared memor
 template <class P, int S, int U>
 __global__ void __launch_bounds__(S * 32) k_lpass_split(ListGeom g, typename P::Params prm, const int32_t *order,
                                                         const unsigned long long *count) {
+    grid_wait();
     using Sums = typename P::Sums;
     __shared__ __align__(16) unsigned char part[(S - 1) * 32 * sizeof(Sums)];
     if (pass_skipped<P>(prm)) return;
@@ -478,10 +482,10 @@ static void launch_variant_u(crk_ctx *ctx, const ListGeom &g, const typename P::
         const int nrange = ctx->nsm > 0 ? (ctx->nsm < 1024 ? ctx->nsm : 1024) : 1;
         const int chunk = (ctx->ntiles + nrange - 1) / nrange;
         cudaMemsetAsync(ctx->sm_next, 0, sizeof(uint32_t) * nrange, s);
-        k_lpass_sm<P, U><<<nrange * per_sm, 32, 0, s>>>(g, prm, ctx->sm_next, nrange, chunk);
+        launch(s, nrange * per_sm, 32, 0, k_lpass_sm<P, U>, g, prm, ctx->sm_next, nrange, chunk);
     } else {
-        k_lpass<P, WARPS, U><<<grid_for(ctx->ntiles, WARPS), WARPS * 32, 0, s>>>(
-            g, prm, ord == ORD_LONGEST ? ctx->tile_order : nullptr);
+        launch(s, grid_for(ctx->ntiles, WARPS), WARPS * 32, 0, k_lpass<P, WARPS, U>, g, prm,
+               ord == ORD_LONGEST ? ctx->tile_order : nullptr);
     }
 }
 
@@ -499,18 +503,18 @@ static void launch_sm_rp(crk_ctx *ctx, const ListGeom &g, const typename P::Para
     const int nrange = ctx->nsm > 0 ? (ctx->nsm < 1024 ? ctx->nsm : 1024) : 1;
     const int chunk = (ctx->ntiles + nrange - 1) / nrange;
     cudaMemsetAsync(ctx->sm_next, 0, sizeof(uint32_t) * nrange, s);
-    k_lpass_sm<P, U, true><<<nrange * per_sm, 32, 0, s>>>(g, prm, ctx->sm_next, nrange, chunk);
+    launch(s, nrange * per_sm, 32, 0, k_lpass_sm<P, U, true>, g, prm, ctx->sm_next, nrange, chunk);
 }
 
 template <class P, int W>
 static void launch_width(crk_ctx *ctx, const ListGeom &g, const typename P::Params &prm, cudaStream_t s) {
     constexpr int U = P::PREFETCH ? 1 : P::UNROLL;
-    k_lpass<P, W, U><<<grid_for(ctx->ntiles, W), W * 32, 0, s>>>(g, prm, nullptr);
+    launch(s, grid_for(ctx->ntiles, W), W * 32, 0, k_lpass<P, W, U>, g, prm, nullptr);
 }
 
 template <class P, int W, int U>
 static void launch_rp(crk_ctx *ctx, const ListGeom &g, const typename P::Params &prm, cudaStream_t s) {
-    k_lpass<P, W, U, true><<<grid_for(ctx->ntiles, W), W * 32, 0, s>>>(g, prm, nullptr);
+    launch(s, grid_for(ctx->ntiles, W), W * 32, 0, k_lpass<P, W, U, true>, g, prm, nullptr);
 }
 
 template <class P, int W>
@@ -631,21 +635,21 @@ int launch_lpass(crk_ctx *ctx, int prof_id, const typename P::Params &prm, cudaS
     rc = CRK_OK;
     constexpr int S = split_warps<P>();
     if (g.ntiles < SPLIT_TILES * nsm) {   // whatever the variant: its warps would not fill the SMs
-        k_lpass_split<P, S, U><<<g.ntiles, S * 32, 0, s>>>(g, prm, ctx->act, nullptr);
+        launch(s, g.ntiles, S * 32, 0, k_lpass_split<P, S, U>, g, prm, ctx->act, nullptr);
     } else if (ctx->act) {
-        k_lpass<P, WARPS, U><<<grid_for(g.ntiles, WARPS), WARPS * 32, 0, s>>>(g, prm, ctx->act);
+        launch(s, grid_for(g.ntiles, WARPS), WARPS * 32, 0, k_lpass<P, WARPS, U>, g, prm, ctx->act);
     } else {
         // long lists first, by CTAs (a captured step does not know whether there are any)
         if (ctx->graph_mode || ctx->h_counters[CNT_MAXCNT] > (unsigned long long)HEAVY_ROWS) {
             g.heavy = HEAVY_ROWS;
-            k_lpass_split<P, S, U><<<2 * nsm, S * 32, 0, s>>>(g, prm, ctx->heavy, ctx->counters + CNT_HEAVY);
+            launch(s, 2 * nsm, S * 32, 0, k_lpass_split<P, S, U>, g, prm, ctx->heavy, ctx->counters + CNT_HEAVY);
             ++ctx->launches;
             CRK_LAUNCH_CHECK(ctx, what);
         }
         if (forms)
             rc = launch_variant<P, WARPS>(ctx, g, prm, v, s);
         else
-            k_lpass<P, WARPS, U><<<grid_for(g.ntiles, WARPS), WARPS * 32, 0, s>>>(g, prm, nullptr);
+            launch(s, grid_for(g.ntiles, WARPS), WARPS * 32, 0, k_lpass<P, WARPS, U>, g, prm, nullptr);
     }
     if (rc) return rc;
     ++ctx->launches;

@@ -59,6 +59,7 @@ __global__ void k_cfl(int n, StepConsts c, const float *__restrict__ hs, const f
                       const float4 *__restrict__ acc, const float2 *__restrict__ vq,
                       const GvRec *__restrict__ gv, unsigned long long *dtmin, const int32_t *__restrict__ sbox,
                       float *__restrict__ dt_out, const float *__restrict__ rho_in) {
+    grid_wait();
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     float dt = 3.0e38f;
     if (s < n) {
@@ -93,6 +94,7 @@ __global__ void k_cfl(int n, StepConsts c, const float *__restrict__ hs, const f
 }
 
 __global__ void k_fill_ull(int count, unsigned long long v, unsigned long long *out) {
+    grid_wait();
     int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k < count) out[k] = v;
 }
@@ -101,6 +103,7 @@ __global__ void k_fill_ull(int count, unsigned long long v, unsigned long long *
 // req (device, one per box) may be null, dt_req then applies to every box
 __global__ void k_pick_dt(int nbox, double dt_req, const double *req, double dt_max,
                           const unsigned long long *dtmin, double *dtb) {
+    grid_wait();
     int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= nbox) return;
     double dt = req ? req[b] : dt_req;
@@ -116,6 +119,7 @@ __global__ void k_pick_dt(int nbox, double dt_req, const double *req, double dt_
 // for exactly this step's dt in every box; the flag is consumed either way.
 __global__ void k_next_check(int nbox, const double *__restrict__ dtb, const double *__restrict__ dtn,
                              unsigned long long *cnt) {
+    grid_wait();
     __shared__ int differ;
     if (threadIdx.x == 0) differ = 0;
     __syncthreads();
@@ -131,12 +135,14 @@ __global__ void k_next_check(int nbox, const double *__restrict__ dtb, const dou
 // the opening kick's energy rates when its P5 pass was skipped
 __global__ void k_take_next(int n, const unsigned long long *cnt, const float *__restrict__ du_next,
                             float *__restrict__ du) {
+    grid_wait();
     if (!cnt[CNT_SKIP]) return;
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s < n) du[s] = du_next[s];
 }
 
-__global__ void k_set_next_ok(unsigned long long *cnt) { cnt[CNT_NEXT_OK] = 1ull; }
+__global__ void k_set_next_ok(unsigned long long *cnt) {
+    grid_wait(); cnt[CNT_NEXT_OK] = 1ull; }
 
 // dt of slot s: its box's (one box: dtb[0])
 __device__ __forceinline__ double slot_dt(const double *dtb, const int32_t *sbox, int s) {
@@ -146,6 +152,7 @@ __device__ __forceinline__ double slot_dt(const double *dtb, const int32_t *sbox
 // first half kick of eq:verletOP: p_1/2 = p + a dt/2; vb = p, va = p_1/2
 __global__ void k_kick1(int n, const double *sc, const int32_t *__restrict__ sbox, const float4 *__restrict__ st_vel, const float4 *__restrict__ acc,
                         float4 *__restrict__ vb, float4 *__restrict__ va) {
+    grid_wait();
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     float h = (float)(0.5 * slot_dt(sc, sbox, s));
@@ -163,6 +170,7 @@ __global__ void k_half_drift(int n, const double *sc, const int32_t *__restrict_
                              float4 *__restrict__ st_pos, float4 *__restrict__ st_vel,
                              float4 *__restrict__ st_half, const float4 *__restrict__ va,
                              const float4 *__restrict__ acc, const float *__restrict__ du) {
+    grid_wait();
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     float dt = (float)slot_dt(sc, sbox, s), h = 0.5f * dt;
@@ -187,6 +195,7 @@ __global__ void k_half_drift(int n, const double *sc, const int32_t *__restrict_
 __global__ void k_permute3(int n, const int32_t *__restrict__ idx, const float4 *__restrict__ a,
                            float4 *__restrict__ ao, const float4 *__restrict__ b, float4 *__restrict__ bo,
                            const float4 *__restrict__ c, float4 *__restrict__ co) {
+    grid_wait();
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     int o = idx[s];
@@ -198,6 +207,7 @@ __global__ void k_permute3(int n, const int32_t *__restrict__ idx, const float4 
 // second half kick: p1 = p_1/2 + a1 dt/2; vb = p_1/2, va = p1
 __global__ void k_kick2(int n, const double *sc, const int32_t *__restrict__ sbox, const float4 *__restrict__ st_half, const float4 *__restrict__ acc,
                         float4 *__restrict__ vb, float4 *__restrict__ va) {
+    grid_wait();
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     float h = (float)(0.5 * slot_dt(sc, sbox, s));
@@ -210,6 +220,7 @@ __global__ void k_kick2(int n, const double *sc, const int32_t *__restrict__ sbo
 __global__ void k_finish(int n, const double *sc, const int32_t *__restrict__ sbox, StepConsts c, const float4 *__restrict__ st_half,
                          const float4 *__restrict__ va, const float *__restrict__ du, const float *__restrict__ Nn,
                          const float *__restrict__ hs, float4 *__restrict__ st_vel, float4 *__restrict__ st_pos) {
+    grid_wait();
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     float h = (float)(0.5 * slot_dt(sc, sbox, s));
@@ -229,6 +240,7 @@ __global__ void k_finish(int n, const double *sc, const int32_t *__restrict__ sb
 constexpr int RED_BLOCKS = 1024;
 __global__ void k_energy_partials(int n, const float4 *__restrict__ vel, const float *__restrict__ mass,
                                   double *__restrict__ part) {
+    grid_wait();
     __shared__ double sh[5][256];
     double a[5] = {0, 0, 0, 0, 0};
     for (int s = blockIdx.x * blockDim.x + threadIdx.x; s < n; s += gridDim.x * blockDim.x) {
@@ -254,6 +266,7 @@ __global__ void k_energy_partials(int n, const float4 *__restrict__ vel, const f
 // the same sums per box: block b over the sorted slots of box b (box-major order)
 __global__ void k_energy_box(const int32_t *__restrict__ start, const float4 *__restrict__ vel,
                              const float *__restrict__ mass, double *__restrict__ out) {
+    grid_wait();
     __shared__ double sh[5][256];
     const int b = blockIdx.x;
     double a[5] = {0, 0, 0, 0, 0};
@@ -278,6 +291,7 @@ __global__ void k_energy_box(const int32_t *__restrict__ start, const float4 *__
 }
 
 __global__ void k_energy_final(int nb, const double *__restrict__ part, double *__restrict__ out) {
+    grid_wait();
     if (threadIdx.x < 5) {
         double s = 0;
         for (int b = 0; b < nb; b++) s += part[b * 8 + threadIdx.x];
@@ -288,6 +302,7 @@ __global__ void k_energy_final(int nb, const double *__restrict__ part, double *
 // h iteration: Thacker update of every particle not yet converged (eq:thacker)
 __global__ void k_h_iter(int n, StepConsts c, float tol, const float *__restrict__ Nn, float *__restrict__ hs,
                          uint4 *__restrict__ q4, int32_t *__restrict__ flags, unsigned long long *notdone) {
+    grid_wait();
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     unsigned nd = 0;
     if (s < n && !flags[s]) {
@@ -311,6 +326,7 @@ __global__ void k_h_iter(int n, StepConsts c, float tol, const float *__restrict
 
 // after the proposal wrote st_pos.w: the sorted h and the fixed-point support
 __global__ void k_take_h(int n, const float4 *__restrict__ st_pos, float *__restrict__ hs, uint4 *__restrict__ q4) {
+    grid_wait();
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     const float h = st_pos[s].w;
@@ -319,6 +335,7 @@ __global__ void k_take_h(int n, const float4 *__restrict__ st_pos, float *__rest
 }
 
 __global__ void k_put_h(int n, const float *__restrict__ hs, float4 *__restrict__ st_pos) {
+    grid_wait();
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     st_pos[s].w = hs[s];
@@ -328,12 +345,14 @@ __global__ void k_put_h(int n, const float *__restrict__ hs, float4 *__restrict_
 // takes old slot idx[s])
 __global__ void k_permute_gv(int n, const int32_t *__restrict__ idx, const GvRec *__restrict__ in,
                              GvRec *__restrict__ out) {
+    grid_wait();
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     out[s] = in[idx[s]];
 }
 
 __global__ void k_write_h(int n, const int32_t *__restrict__ perm, const float *__restrict__ hs, float4 *pos_h) {
+    grid_wait();
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     pos_h[perm[s]].w = hs[s];
@@ -344,6 +363,7 @@ __global__ void k_write_h(int n, const int32_t *__restrict__ perm, const float *
 // qV = (q, V) of every slot: after a P1 over some tiles only (time bins), the
 // other slots keep their last V at their current position
 __global__ void k_qv_refresh(int n, const uint4 *__restrict__ q4, const float *__restrict__ V, uint4 *__restrict__ qV) {
+    grid_wait();
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     uint4 q = q4[s];
@@ -356,7 +376,7 @@ __global__ void k_qv_refresh(int n, const uint4 *__restrict__ q4, const float *_
 int evaluate(crk_ctx *ctx, cudaStream_t s) {
     int rc = run_volumes(ctx, s);
     if (!rc && ctx->act) {
-        k_qv_refresh<<<grid_for(ctx->n, 256), 256, 0, s>>>(ctx->n, ctx->q4, ctx->V, ctx->qV);
+        launch(s, grid_for(ctx->n, 256), 256, 0, k_qv_refresh, ctx->n, ctx->q4, ctx->V, ctx->qV);
         ++ctx->launches;
         CRK_LAUNCH_CHECK(ctx, "pass records");
     }
@@ -367,10 +387,9 @@ int evaluate(crk_ctx *ctx, cudaStream_t s) {
     const bool batched = ctx->nbox > 1;
     unsigned long long *dtmin = batched ? ctx->box_dtmin : ctx->counters + CNT_DTMIN;
     const int nb = batched ? ctx->nbox : 1;
-    k_fill_ull<<<grid_for(nb, 256), 256, 0, s>>>(nb, 0x7f7fffffull, dtmin);   // FLT_MAX bits
-    k_cfl<<<grid_for(ctx->n, 256), 256, 0, s>>>(ctx->n, c, ctx->hs, ctx->V, ctx->mass, ctx->vel, ctx->acc,
-                                                  ctx->vq, ctx->gv, dtmin, batched ? ctx->sbox : nullptr,
-                                                  ctx->d_dt, ctx->p.density ? ctx->rho : nullptr);
+    launch(s, grid_for(nb, 256), 256, 0, k_fill_ull, nb, 0x7f7fffffull, dtmin);   // FLT_MAX bits
+    launch(s, grid_for(ctx->n, 256), 256, 0, k_cfl, ctx->n, c, ctx->hs, ctx->V, ctx->mass, ctx->vel, ctx->acc,
+           ctx->vq, ctx->gv, dtmin, batched ? ctx->sbox : nullptr, ctx->d_dt, ctx->p.density ? ctx->rho : nullptr);
     ctx->launches += 2;
     CRK_LAUNCH_CHECK(ctx, "CFL");
     return CRK_OK;
@@ -403,8 +422,8 @@ extern "C" int crk_reset_rates(crk_ctx *ctx) {
 static int h_update(crk_ctx *ctx, const StepConsts &c, float tol, cudaStream_t s, unsigned long long *nd) {
     const int n = ctx->n;
     CRK_CUDA(ctx, cudaMemsetAsync(ctx->counters + CNT_NOTDONE, 0, sizeof(unsigned long long), s));
-    k_h_iter<<<grid_for(n, 256), 256, 0, s>>>(n, c, tol, ctx->Nn, ctx->hs, ctx->q4, ctx->flags,
-                                              ctx->counters + CNT_NOTDONE);
+    launch(s, grid_for(n, 256), 256, 0, k_h_iter, n, c, tol, ctx->Nn, ctx->hs, ctx->q4, ctx->flags,
+           ctx->counters + CNT_NOTDONE);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "h iteration");
     int rc = unconverged_tiles(ctx, s);
@@ -423,7 +442,7 @@ static int solve_h(crk_ctx *ctx, int n, const int32_t *idx, cudaStream_t s, int 
     const int b = 256, g = grid_for(n, b);
     int rc = CRK_OK;
     if (ctx->p.h_mode == 2) {   // the last evaluation's grad v, in the new order (frec is free until P4)
-        k_permute_gv<<<g, b, 0, s>>>(n, idx, ctx->gv, reinterpret_cast<GvRec *>(ctx->frec));
+        launch(s, g, b, 0, k_permute_gv, n, idx, ctx->gv, reinterpret_cast<GvRec *>(ctx->frec));
         ++ctx->launches;
         CRK_LAUNCH_CHECK(ctx, "permute grad v");
     }
@@ -442,7 +461,7 @@ static int solve_h(crk_ctx *ctx, int n, const int32_t *idx, cudaStream_t s, int 
             rc = propose_sorted(ctx, n, ctx->st_pos, reinterpret_cast<const GvRec *>(ctx->frec), ctx->Nn, (float)dt,
                                 tol, s);
             if (rc) break;
-            k_take_h<<<g, b, 0, s>>>(n, ctx->st_pos, ctx->hs, ctx->q4);
+            launch(s, g, b, 0, k_take_h, n, ctx->st_pos, ctx->hs, ctx->q4);
             ++ctx->launches;
             CRK_LAUNCH_CHECK(ctx, "proposed h");
             ctx->act = nullptr;   // every particle may have moved: the next pass walks all tiles
@@ -467,7 +486,7 @@ static int solve_h(crk_ctx *ctx, int n, const int32_t *idx, cudaStream_t s, int 
     if (rc) return rc;
     *iters = it > max_it ? max_it : it;
     *unconv = (long long)nd;
-    k_put_h<<<g, b, 0, s>>>(n, ctx->hs, ctx->st_pos);
+    launch(s, g, b, 0, k_put_h, n, ctx->hs, ctx->st_pos);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "solved h");
     return CRK_OK;
@@ -507,20 +526,21 @@ static int step_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const floa
     double *dtb = batched ? ctx->dtb : ctx->d_scalars;
     double *dtn = batched ? ctx->dtb_next : ctx->d_scalars + 16;   // the next step's dt
     if (fresh) CRK_CUDA(ctx, cudaMemsetAsync(ctx->counters + CNT_NEXT_OK, 0, 2 * sizeof(unsigned long long), s));
-    k_pick_dt<<<grid_for(nb, 64), 64, 0, s>>>(nb, dt_req, dt_box, c.dt_max,
-                                               batched ? ctx->box_dtmin : ctx->counters + CNT_DTMIN, dtb);
-    k_next_check<<<1, 256, 0, s>>>(nb, dtb, dtn, ctx->counters);
+    launch(s, grid_for(nb, 64), 64, 0, k_pick_dt, nb, dt_req, dt_box, c.dt_max,
+           batched ? ctx->box_dtmin : ctx->counters + CNT_DTMIN, dtb);
+    launch(s, 1, 256, 0, k_next_check, nb, dtb, dtn, ctx->counters);
     ctx->launches += 2;
     // first half kick with the cached rates, compatible energy of that kick
     // (formed ahead by the previous step's dual pass when its dt matches)
-    k_kick1<<<g, b, 0, s>>>(n, dtb, sbox, ctx->st_vel, ctx->acc, ctx->vb, ctx->va);
+    launch(s, g, b, 0, k_kick1, n, dtb, sbox, ctx->st_vel, ctx->acc, ctx->vb, ctx->va);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "kick");
     rc = run_compatible(ctx, s, ctx->counters + CNT_SKIP);
     if (rc) return rc;
-    k_take_next<<<g, b, 0, s>>>(n, ctx->counters, ctx->du_next, ctx->du);
+    launch(s, g, b, 0, k_take_next, n, ctx->counters, ctx->du_next, ctx->du);
     ++ctx->launches;
-    k_half_drift<<<g, b, 0, s>>>(n, dtb, sbox, c, ctx->st_pos, ctx->st_vel, ctx->st_half, ctx->va, ctx->acc, ctx->du);
+    launch(s, g, b, 0, k_half_drift, n, dtb, sbox, c, ctx->st_pos, ctx->st_vel, ctx->st_half, ctx->va, ctx->acc,
+           ctx->du);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "drift");
     // rebuild at x1 (input order = current sorted order; boxes keep their particles)
@@ -531,7 +551,8 @@ static int step_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const floa
         ctx->rates_valid = 0;
         return rc;
     }
-    k_permute3<<<g, b, 0, s>>>(n, ctx->idx_a, ctx->st_pos, ctx->st_tmp, ctx->st_vel, ctx->vb, ctx->st_half, ctx->va);
+    launch(s, g, b, 0, k_permute3, n, ctx->idx_a, ctx->st_pos, ctx->st_tmp, ctx->st_vel, ctx->vb, ctx->st_half,
+           ctx->va);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "permute state");
     float4 *t;
@@ -558,19 +579,19 @@ static int step_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const floa
     }
     // second half kick and its compatible energy (the boxes' dt of this step;
     // the permutation kept every particle in its box)
-    k_kick2<<<g, b, 0, s>>>(n, dtb, sbox, ctx->st_half, ctx->acc, ctx->vb, ctx->va);
+    launch(s, g, b, 0, k_kick2, n, dtb, sbox, ctx->st_half, ctx->acc, ctx->vb, ctx->va);
     // the next step's dt under the same request, and both kicks' compatible
     // energy (this closing kick, the next opening kick) in one pass
-    k_pick_dt<<<grid_for(nb, 64), 64, 0, s>>>(nb, dt_req, dt_box, c.dt_max,
-                                               batched ? ctx->box_dtmin : ctx->counters + CNT_DTMIN, dtn);
+    launch(s, grid_for(nb, 64), 64, 0, k_pick_dt, nb, dt_req, dt_box, c.dt_max,
+           batched ? ctx->box_dtmin : ctx->counters + CNT_DTMIN, dtn);
     ctx->launches += 2;
     CRK_LAUNCH_CHECK(ctx, "kick");
     rc = run_compatible_dual(ctx, dtn, sbox, s);
     if (rc) return rc;
-    k_set_next_ok<<<1, 1, 0, s>>>(ctx->counters);
+    launch(s, 1, 1, 0, k_set_next_ok, ctx->counters);
     ++ctx->launches;
-    k_finish<<<g, b, 0, s>>>(n, dtb, sbox, c, ctx->st_half, ctx->va, ctx->du, ctx->Nn, ctx->hs, ctx->st_vel,
-                             ctx->st_pos);
+    launch(s, g, b, 0, k_finish, n, dtb, sbox, c, ctx->st_half, ctx->va, ctx->du, ctx->Nn, ctx->hs, ctx->st_vel,
+           ctx->st_pos);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "finish step");
     rc = scatter_rows(ctx, ctx->st_pos, pos_h, 4, s);
@@ -585,9 +606,9 @@ extern "C" int crk_step(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const f
     cudaStream_t s = (cudaStream_t)stream;
     int rc = step_impl(ctx, n, pos_h, vel_u, mass, dt, nullptr, false, s);
     if (rc || !diag) return rc;
-    k_energy_partials<<<RED_BLOCKS, 256, 0, s>>>(n, ctx->st_vel, ctx->mass, ctx->d_red);
+    launch(s, RED_BLOCKS, 256, 0, k_energy_partials, n, ctx->st_vel, ctx->mass, ctx->d_red);
     ++ctx->launches;
-    k_energy_final<<<1, 32, 0, s>>>(RED_BLOCKS, ctx->d_red, ctx->d_scalars + 2);
+    launch(s, 1, 32, 0, k_energy_final, RED_BLOCKS, ctx->d_red, ctx->d_scalars + 2);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "diagnostics");
     double h[8];
@@ -645,7 +666,7 @@ extern "C" int crk_step_batched(crk_ctx *ctx, int n, int nbox, const int32_t *bo
     std::vector<double> red(8 * (size_t)nb), dts(nb);
     std::vector<unsigned long long> dtn(nb);
     if (nbox > 1) {
-        k_energy_box<<<nb, 256, 0, s>>>(ctx->box_start, ctx->st_vel, ctx->mass, ctx->box_red);
+        launch(s, nb, 256, 0, k_energy_box, ctx->box_start, ctx->st_vel, ctx->mass, ctx->box_red);
         ++ctx->launches;
         CRK_LAUNCH_CHECK(ctx, "diagnostics");
         CRK_CUDA(ctx, cudaMemcpyAsync(red.data(), ctx->box_red, sizeof(double) * 8 * nb, cudaMemcpyDeviceToHost, s));
@@ -653,8 +674,8 @@ extern "C" int crk_step_batched(crk_ctx *ctx, int n, int nbox, const int32_t *bo
         CRK_CUDA(ctx, cudaMemcpyAsync(dtn.data(), ctx->box_dtmin, sizeof(unsigned long long) * nb,
                                       cudaMemcpyDeviceToHost, s));
     } else {
-        k_energy_partials<<<RED_BLOCKS, 256, 0, s>>>(n, ctx->st_vel, ctx->mass, ctx->d_red);
-        k_energy_final<<<1, 32, 0, s>>>(RED_BLOCKS, ctx->d_red, ctx->d_scalars + 2);
+        launch(s, RED_BLOCKS, 256, 0, k_energy_partials, n, ctx->st_vel, ctx->mass, ctx->d_red);
+        launch(s, 1, 32, 0, k_energy_final, RED_BLOCKS, ctx->d_red, ctx->d_scalars + 2);
         ctx->launches += 2;
         CRK_LAUNCH_CHECK(ctx, "diagnostics");
         double h[8];
@@ -688,6 +709,7 @@ namespace {
 
 // sticky overflow / invalid-input flag of a replayed step
 __global__ void k_graph_check(unsigned long long *cnt, long long cap_ulist, int kcap) {
+    grid_wait();
     if (cnt[CNT_ERR_INPUT] || cnt[CNT_PO_MISS] || cnt[CNT_TMA_ERR] || (long long)cnt[CNT_ULIST] > cap_ulist ||
         (long long)cnt[CNT_MAXCNT] > kcap)
         cnt[CNT_GRAPH_ERR] = 1ull;
@@ -717,8 +739,8 @@ void drop_graphs(crk_ctx *ctx) {
 }
 
 int run_diag(crk_ctx *ctx, int n, crk_diag *diag, cudaStream_t s) {
-    k_energy_partials<<<RED_BLOCKS, 256, 0, s>>>(n, ctx->st_vel, ctx->mass, ctx->d_red);
-    k_energy_final<<<1, 32, 0, s>>>(RED_BLOCKS, ctx->d_red, ctx->d_scalars + 2);
+    launch(s, RED_BLOCKS, 256, 0, k_energy_partials, n, ctx->st_vel, ctx->mass, ctx->d_red);
+    launch(s, 1, 32, 0, k_energy_final, RED_BLOCKS, ctx->d_red, ctx->d_scalars + 2);
     ctx->launches += 2;
     CRK_LAUNCH_CHECK(ctx, "diagnostics");
     double h[8];
@@ -789,7 +811,7 @@ static bool capture_step(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const 
     if (e == cudaSuccess) {
         rc = step_impl(ctx, n, pos_h, vel_u, mass, dt, nullptr, batched, ctx->gstream);
         if (!rc) {
-            k_graph_check<<<1, 1, 0, ctx->gstream>>>(ctx->counters, ctx->cap_ulist, ctx->kcap);
+            launch(ctx->gstream, 1, 1, 0, k_graph_check, ctx->counters, ctx->cap_ulist, ctx->kcap);
             ++ctx->launches;
         }
         e = cudaStreamEndCapture(ctx->gstream, &graph);
@@ -1001,7 +1023,7 @@ static int h_iterate(crk_ctx *ctx, int n, float *pos_h, float tol, int max_it, i
     ctx->nact = 0;
     if (rc) return rc;
     if (iterations) *iterations = it > max_it ? max_it : it;
-    k_write_h<<<grid_for(n, 256), 256, 0, s>>>(n, ctx->perm, ctx->hs, (float4 *)pos_h);
+    launch(s, grid_for(n, 256), 256, 0, k_write_h, n, ctx->perm, ctx->hs, (float4 *)pos_h);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "write h");
     CRK_CUDA(ctx, cudaStreamSynchronize(s));

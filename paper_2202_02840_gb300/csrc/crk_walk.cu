@@ -368,6 +368,7 @@ __device__ __forceinline__ void walk_range(const WalkArgs &a, const WalkTile &T,
 // exactly the one-warp walk's.
 template <bool LISTS, bool VOL, bool BATCH, int W>
 __global__ void __launch_bounds__(W * 32, 32 / W) k_walk(WalkArgs a) {
+    grid_wait();
     extern __shared__ __align__(16) unsigned char walk_smem[];
     WalkCta<LISTS, VOL, BATCH, W> &C = *reinterpret_cast<WalkCta<LISTS, VOL, BATCH, W> *>(walk_smem);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -546,6 +547,7 @@ __global__ void __launch_bounds__(W * 32, 32 / W) k_walk(WalkArgs a) {
 // total stored-force units (32 entries each) = base[last] + len_u[last]
 __global__ void k_total(int ntiles, const uint32_t *__restrict__ base, const uint32_t *__restrict__ len,
                         unsigned long long *out) {
+    grid_wait();
     *out = ntiles ? (unsigned long long)base[ntiles - 1] + len[ntiles - 1] : 0ull;
 }
 
@@ -592,7 +594,7 @@ static int launch_walk_wide(crk_ctx *ctx, const WalkArgs &a, cudaStream_t s) {
         CRK_CUDA(ctx, cudaFuncSetAttribute(k_walk<LISTS, VOL, BATCH, W>,
                                            cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Cta)));
     const int g = a.hblocks + (a.all ? 0 : grid_for(a.ntiles, W));
-    k_walk<LISTS, VOL, BATCH, W><<<g, W * 32, sizeof(Cta), s>>>(a);
+    launch(s, g, W * 32, sizeof(Cta), k_walk<LISTS, VOL, BATCH, W>, a);
     return CRK_OK;
 }
 
@@ -648,7 +650,7 @@ int run_lists(crk_ctx *ctx, cudaStream_t s) {
         if (rc) return rc;
         rc = scan_u32(ctx, ctx->len_u, ctx->tbase, nt, s);
         if (rc) return rc;
-        k_total<<<1, 1, 0, s>>>(nt, ctx->tbase, ctx->len_u, ctx->counters + CNT_ENTRIES);
+        launch(s, 1, 1, 0, k_total, nt, ctx->tbase, ctx->len_u, ctx->counters + CNT_ENTRIES);
         ++ctx->launches;
         CRK_LAUNCH_CHECK(ctx, "list layout");
         if (ctx->graph_mode) {   // captured step: capacities were fixed beforehand, overflow checked after
@@ -679,6 +681,7 @@ __global__ void k_export_lists(int n, int kcap, int mode, const int32_t *__restr
                                const int32_t *__restrict__ cnt_g, const int32_t *__restrict__ cnt_u,
                                const uint32_t *__restrict__ ent, const uint4 *__restrict__ q4,
                                const long long *__restrict__ off, int32_t *__restrict__ out) {
+    grid_wait();
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     const int tile = s / TILE, lane = s % TILE;
@@ -707,8 +710,8 @@ int run_export_lists(crk_ctx *ctx, int mode, const long long *off, int32_t *out,
     if (ctx->n == 0) return CRK_OK;
     int rc = run_lists(ctx, s);
     if (rc) return rc;
-    k_export_lists<<<grid_for(ctx->n, 256), 256, 0, s>>>(ctx->n, ctx->kcap, mode, ctx->perm, ctx->cnt_g, ctx->cnt_u,
-                                                          ctx->ent, ctx->q4, off, out);
+    launch(s, grid_for(ctx->n, 256), 256, 0, k_export_lists, ctx->n, ctx->kcap, mode, ctx->perm, ctx->cnt_g,
+           ctx->cnt_u, ctx->ent, ctx->q4, off, out);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "export lists");
     return CRK_OK;
