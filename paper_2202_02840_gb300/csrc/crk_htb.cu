@@ -440,7 +440,7 @@ int unconverged_tiles(crk_ctx *ctx, cudaStream_t s) {
     int rc = ensure_htb(ctx);
     if (rc) return rc;
     const int nt = ctx->ntiles;
-    CRK_CUDA(ctx, cudaMemsetAsync(ctx->counters + CNT_NACT, 0, 2 * sizeof(unsigned long long), s));
+    zero_async(ctx, ctx->counters + CNT_NACT, 2 * sizeof(unsigned long long), s);
     launch(s, grid_for((long long)nt * 32, 256), 256, 0, k_unconv_flags, nt, ctx->n, ctx->flags, ctx->tflag);
     ++ctx->launches;
     rc = scan_u32(ctx, ctx->tflag, ctx->tscan, nt, s);
@@ -493,7 +493,7 @@ static int limit(crk_ctx *ctx, const int32_t *act, int count, int f_l, int L, cu
     if (count == 0) return CRK_OK;
     const long long cap = (long long)ctx->ntiles * (L + 1) + 2;
     for (long long it = 0; it < cap; it += 4) {
-        CRK_CUDA(ctx, cudaMemsetAsync(ctx->counters + CNT_CHANGED, 0, sizeof(unsigned long long), s));
+        zero_async(ctx, ctx->counters + CNT_CHANGED, sizeof(unsigned long long), s);
         for (int k = 0; k < 4; k++) {
             launch(s, grid_for((long long)count * 32, 256), 256, 0, k_htb_limit, count, act, ctx->uofs, ctx->ulist,
                    f_l, ctx->tlev, ctx->counters + CNT_CHANGED);
@@ -507,11 +507,16 @@ static int limit(crk_ctx *ctx, const int32_t *act, int count, int f_l, int L, cu
     return crk_set_error(ctx, CRK_ENONCONV, "level limiter did not converge");
 }
 
+static __global__ void k_set_u64(unsigned long long *p, unsigned long long v) {
+    grid_wait();
+    if (threadIdx.x == 0) *p = v;
+}
+
 // earliest step end, and the active list of that tick (synchronises)
 static int next_tick(crk_ctx *ctx, int *t_next, cudaStream_t s) {
     const int nt = ctx->ntiles;
-    const unsigned long long big = 0xffffffffull;
-    CRK_CUDA(ctx, cudaMemcpyAsync(ctx->counters + CNT_TNEXT, &big, sizeof(big), cudaMemcpyHostToDevice, s));
+    launch(s, 1, 32, 0, k_set_u64, ctx->counters + CNT_TNEXT, 0xffffffffull);
+    ++ctx->launches;
     launch(s, grid_for(nt, 256), 256, 0, k_htb_tnext, nt, ctx->tt0, ctx->tlen, ctx->counters);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "next tick");
@@ -523,7 +528,7 @@ static int next_tick(crk_ctx *ctx, int *t_next, cudaStream_t s) {
 
 static int active_list(crk_ctx *ctx, int t, long long *parts, cudaStream_t s) {
     const int nt = ctx->ntiles;
-    CRK_CUDA(ctx, cudaMemsetAsync(ctx->counters + CNT_NACT, 0, 2 * sizeof(unsigned long long), s));
+    zero_async(ctx, ctx->counters + CNT_NACT, 2 * sizeof(unsigned long long), s);
     launch(s, grid_for(nt, 256), 256, 0, k_htb_flags, nt, ctx->tt0, ctx->tlen, t, ctx->tflag);
     ++ctx->launches;
     int rc = scan_u32(ctx, ctx->tflag, ctx->tscan, nt, s);
@@ -555,7 +560,7 @@ static int cycle_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const flo
         if (!rc) rc = gather_rows(ctx, vel_u, ctx->st_vel, 4, s);
         if (!rc) rc = gather_rows(ctx, mass, ctx->mass, 1, s);
         if (rc) return rc;
-        CRK_CUDA(ctx, cudaMemcpyAsync(ctx->vel, ctx->st_vel, sizeof(float4) * n, cudaMemcpyDeviceToDevice, s));
+        copy_async(ctx, ctx->vel, ctx->st_vel, sizeof(float4) * n, s);
         rc = evaluate(ctx, s);
         if (rc) return rc;
         ctx->rates_valid = 1;
@@ -576,7 +581,7 @@ static int cycle_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const flo
     rc = refit_lists(ctx, s);
     if (rc) return rc;
     // levels at the cycle start: requirement, then the limiter's fixed point
-    CRK_CUDA(ctx, cudaMemsetAsync(ctx->counters + CNT_UNRES, 0, 2 * sizeof(unsigned long long), s));
+    zero_async(ctx, ctx->counters + CNT_UNRES, 2 * sizeof(unsigned long long), s);
     launch(s, grid_for((long long)nt * 32, 256), 256, 0, k_htb_req, nt, nullptr, n, ctx->d_dt, c, 0, 0, ctx->tlev,
            ctx->counters);
     ++ctx->launches;
@@ -592,11 +597,11 @@ static int cycle_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const flo
         st->leaves = nt;
     }
     // every leaf opens its first step at tick 0 (t0 = len = 0 marks it active)
-    CRK_CUDA(ctx, cudaMemsetAsync(ctx->tt0, 0, sizeof(int32_t) * nt, s));
-    CRK_CUDA(ctx, cudaMemsetAsync(ctx->tlen, 0, sizeof(int32_t) * nt, s));
+    zero_async(ctx, ctx->tt0, sizeof(int32_t) * nt, s);
+    zero_async(ctx, ctx->tlen, sizeof(int32_t) * nt, s);
     std::vector<int32_t> none(nt, NO_LEVEL);
     CRK_CUDA(ctx, cudaMemcpyAsync(ctx->twake, none.data(), sizeof(int32_t) * nt, cudaMemcpyHostToDevice, s));
-    CRK_CUDA(ctx, cudaMemcpyAsync(ctx->st_half, ctx->st_vel, sizeof(float4) * n, cudaMemcpyDeviceToDevice, s));
+    copy_async(ctx, ctx->st_half, ctx->st_vel, sizeof(float4) * n, s);
     launch(s, g, b, 0, k_htb_open, n, c, 0, ctx->tlev, ctx->tt0, ctx->tlen, ctx->st_half, ctx->acc, ctx->vel, ctx->vb,
            ctx->va);
     ++ctx->launches;
@@ -696,7 +701,7 @@ static int cycle_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const flo
     tp = ctx->st_pos; ctx->st_pos = ctx->st_tmp; ctx->st_tmp = tp;
     tp = ctx->vel; ctx->vel = ctx->vb; ctx->vb = tp;
     tp = ctx->st_half; ctx->st_half = ctx->va; ctx->va = tp;
-    CRK_CUDA(ctx, cudaMemcpyAsync(ctx->hc, ctx->st_tmp1, sizeof(float) * n, cudaMemcpyDeviceToDevice, s));
+    copy_async(ctx, ctx->hc, ctx->st_tmp1, sizeof(float) * n, s);
     rc = gather_rows(ctx, mass, ctx->mass, 1, s);
     if (!rc) rc = evaluate(ctx, s);
     if (rc) return rc;
@@ -712,7 +717,7 @@ static int cycle_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const flo
     CRK_LAUNCH_CHECK(ctx, "finish cycle");
     rc = scatter_rows(ctx, ctx->st_pos, pos_h, 4, s);
     if (!rc) rc = scatter_rows(ctx, ctx->st_vel, vel_u, 4, s);
-    if (!rc) CRK_CUDA(ctx, cudaMemsetAsync(ctx->counters + CNT_NEXT_OK, 0, sizeof(unsigned long long), s));
+    if (!rc) zero_async(ctx, ctx->counters + CNT_NEXT_OK, sizeof(unsigned long long), s);
     if (!rc) rc = crk_sync_counters(ctx, s);
     if (rc) return rc;
     ctx->rates_valid = 1;
@@ -762,7 +767,7 @@ extern "C" int crk_htb_levels(crk_ctx *ctx, int n, const float *pos_h, const flo
     ctx->rates_valid = 0;
     const HtbConsts c = htb_consts(ctx, Delta, L, f_l);
     const int nt = ctx->ntiles;
-    CRK_CUDA(ctx, cudaMemsetAsync(ctx->counters + CNT_UNRES, 0, sizeof(unsigned long long), s));
+    zero_async(ctx, ctx->counters + CNT_UNRES, sizeof(unsigned long long), s);
     launch(s, grid_for((long long)nt * 32, 256), 256, 0, k_htb_req, nt, nullptr, n, ctx->d_dt, c, 0, 0, ctx->tlev,
            ctx->counters);
     ++ctx->launches;

@@ -350,6 +350,8 @@ int run_compatible_dual(crk_ctx *ctx, const double *dtn, const int32_t *sbox, cu
 int evaluate(crk_ctx *ctx, cudaStream_t s);   // P1..P4 and per-particle time steps (crk_step.cu)
 int propose_sorted(crk_ctx *ctx, int n, float4 *pos, const GvRec *gv, const float *Nn, float dt, float tol,
                    cudaStream_t s);   // learned h proposal in sorted order (crk_mlp.cu)
+void zero_async(crk_ctx *ctx, void *p, size_t bytes, cudaStream_t s);   // whole 32-bit words (crk_ctx.cu)
+void copy_async(crk_ctx *ctx, void *to, const void *from, size_t bytes, cudaStream_t s);
 int gather_rows(crk_ctx *ctx, const void *in, void *out, int width_words, cudaStream_t s);
 int scatter_rows(crk_ctx *ctx, const void *in, void *out, int width_words, cudaStream_t s);
 inline int grid_for(long long n, int block) { return (int)((n + block - 1) / block); }

@@ -481,7 +481,7 @@ static void launch_variant_u(crk_ctx *ctx, const ListGeom &g, const typename P::
         }
         const int nrange = ctx->nsm > 0 ? (ctx->nsm < 1024 ? ctx->nsm : 1024) : 1;
         const int chunk = (ctx->ntiles + nrange - 1) / nrange;
-        cudaMemsetAsync(ctx->sm_next, 0, sizeof(uint32_t) * nrange, s);
+        zero_async(ctx, ctx->sm_next, sizeof(uint32_t) * nrange, s);
         launch(s, nrange * per_sm, 32, 0, k_lpass_sm<P, U>, g, prm, ctx->sm_next, nrange, chunk);
     } else {
         launch(s, grid_for(ctx->ntiles, WARPS), WARPS * 32, 0, k_lpass<P, WARPS, U>, g, prm,
@@ -502,7 +502,7 @@ static void launch_sm_rp(crk_ctx *ctx, const ListGeom &g, const typename P::Para
     }
     const int nrange = ctx->nsm > 0 ? (ctx->nsm < 1024 ? ctx->nsm : 1024) : 1;
     const int chunk = (ctx->ntiles + nrange - 1) / nrange;
-    cudaMemsetAsync(ctx->sm_next, 0, sizeof(uint32_t) * nrange, s);
+    zero_async(ctx, ctx->sm_next, sizeof(uint32_t) * nrange, s);
     launch(s, nrange * per_sm, 32, 0, k_lpass_sm<P, U, true>, g, prm, ctx->sm_next, nrange, chunk);
 }
 

@@ -421,7 +421,7 @@ extern "C" int crk_reset_rates(crk_ctx *ctx) {
 // *nd = particles updated (0: all converged).
 static int h_update(crk_ctx *ctx, const StepConsts &c, float tol, cudaStream_t s, unsigned long long *nd) {
     const int n = ctx->n;
-    CRK_CUDA(ctx, cudaMemsetAsync(ctx->counters + CNT_NOTDONE, 0, sizeof(unsigned long long), s));
+    zero_async(ctx, ctx->counters + CNT_NOTDONE, sizeof(unsigned long long), s);
     launch(s, grid_for(n, 256), 256, 0, k_h_iter, n, c, tol, ctx->Nn, ctx->hs, ctx->q4, ctx->flags,
            ctx->counters + CNT_NOTDONE);
     ++ctx->launches;
@@ -446,7 +446,7 @@ static int solve_h(crk_ctx *ctx, int n, const int32_t *idx, cudaStream_t s, int 
         ++ctx->launches;
         CRK_LAUNCH_CHECK(ctx, "permute grad v");
     }
-    CRK_CUDA(ctx, cudaMemsetAsync(ctx->flags, 0, sizeof(int32_t) * n, s));
+    zero_async(ctx, ctx->flags, sizeof(int32_t) * n, s);
     const int vo = ctx->volumes_only;
     ctx->volumes_only = 1;
     int it = 0;
@@ -511,7 +511,7 @@ static int step_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const floa
         if (!rc) rc = gather_rows(ctx, vel_u, ctx->st_vel, 4, s);
         if (!rc) rc = gather_rows(ctx, mass, ctx->mass, 1, s);
         if (rc) return rc;
-        CRK_CUDA(ctx, cudaMemcpyAsync(ctx->vel, ctx->st_vel, sizeof(float4) * n, cudaMemcpyDeviceToDevice, s));
+        copy_async(ctx, ctx->vel, ctx->st_vel, sizeof(float4) * n, s);
         rc = evaluate(ctx, s);
         if (rc) return rc;
         ctx->rates_valid = 1;
@@ -525,7 +525,7 @@ static int step_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const floa
     const int32_t *sbox = batched ? ctx->sbox : nullptr;
     double *dtb = batched ? ctx->dtb : ctx->d_scalars;
     double *dtn = batched ? ctx->dtb_next : ctx->d_scalars + 16;   // the next step's dt
-    if (fresh) CRK_CUDA(ctx, cudaMemsetAsync(ctx->counters + CNT_NEXT_OK, 0, 2 * sizeof(unsigned long long), s));
+    if (fresh) zero_async(ctx, ctx->counters + CNT_NEXT_OK, 2 * sizeof(unsigned long long), s);
     launch(s, grid_for(nb, 64), 64, 0, k_pick_dt, nb, dt_req, dt_box, c.dt_max,
            batched ? ctx->box_dtmin : ctx->counters + CNT_DTMIN, dtb);
     launch(s, 1, 256, 0, k_next_check, nb, dtb, dtn, ctx->counters);
@@ -544,7 +544,7 @@ static int step_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const floa
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "drift");
     // rebuild at x1 (input order = current sorted order; boxes keep their particles)
-    if (batched) CRK_CUDA(ctx, cudaMemcpyAsync(ctx->sbox_tmp, ctx->sbox, sizeof(int32_t) * n, cudaMemcpyDeviceToDevice, s));
+    if (batched) copy_async(ctx, ctx->sbox_tmp, ctx->sbox, sizeof(int32_t) * n, s);
     rc = build_cells_sorted(ctx, n, ctx->st_pos, ctx->perm, s, batched ? ctx->sbox_tmp : nullptr);
     if (!rc) rc = finish_build(ctx, s);
     if (rc) {
@@ -571,7 +571,7 @@ static int step_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const floa
         }
     }
     // evaluation at (x1, p_p, u_p)
-    CRK_CUDA(ctx, cudaMemcpyAsync(ctx->vel, ctx->st_vel, sizeof(float4) * n, cudaMemcpyDeviceToDevice, s));
+    copy_async(ctx, ctx->vel, ctx->st_vel, sizeof(float4) * n, s);
     rc = evaluate(ctx, s);
     if (rc) {
         ctx->rates_valid = 0;
@@ -904,9 +904,9 @@ static int steps_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const flo
             CRK_CUDA(ctx, cudaEventCreateWithFlags(&ctx->gev[0], cudaEventDisableTiming));
             CRK_CUDA(ctx, cudaEventCreateWithFlags(&ctx->gev[1], cudaEventDisableTiming));
         }
-        CRK_CUDA(ctx, cudaMemcpyAsync(ctx->bk_pos, pos_h, sizeof(float4) * (size_t)n, cudaMemcpyDeviceToDevice, s));
-        CRK_CUDA(ctx, cudaMemcpyAsync(ctx->bk_vel, vel_u, sizeof(float4) * (size_t)n, cudaMemcpyDeviceToDevice, s));
-        CRK_CUDA(ctx, cudaMemsetAsync(ctx->counters + CNT_GRAPH_ERR, 0, sizeof(unsigned long long), s));
+        copy_async(ctx, ctx->bk_pos, pos_h, sizeof(float4) * (size_t)n, s);
+        copy_async(ctx, ctx->bk_vel, vel_u, sizeof(float4) * (size_t)n, s);
+        zero_async(ctx, ctx->counters + CNT_GRAPH_ERR, sizeof(unsigned long long), s);
         CRK_CUDA(ctx, cudaEventRecord(ctx->gev[0], s));
         CRK_CUDA(ctx, cudaStreamWaitEvent(ctx->gstream, ctx->gev[0], 0));
         bool eager = false;
@@ -948,8 +948,8 @@ static int steps_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const flo
             // positions and velocities this run of replays started from and redo
             // its steps eagerly (their first step evaluates the rates afresh there)
             ctx->grecoveries++;
-            CRK_CUDA(ctx, cudaMemcpyAsync(pos_h, ctx->bk_pos, sizeof(float4) * (size_t)n, cudaMemcpyDeviceToDevice, s));
-            CRK_CUDA(ctx, cudaMemcpyAsync(vel_u, ctx->bk_vel, sizeof(float4) * (size_t)n, cudaMemcpyDeviceToDevice, s));
+            copy_async(ctx, pos_h, ctx->bk_pos, sizeof(float4) * (size_t)n, s);
+            copy_async(ctx, vel_u, ctx->bk_vel, sizeof(float4) * (size_t)n, s);
             drop_graphs(ctx);
             ctx->rates_valid = 0;
             for (int k = done; k < nsteps; k++) {
@@ -1007,7 +1007,7 @@ static int h_iterate(crk_ctx *ctx, int n, float *pos_h, float tol, int max_it, i
     if (!rc) rc = finish_build(ctx, s);
     if (rc) return rc;
     StepConsts c = step_consts(ctx->p);
-    CRK_CUDA(ctx, cudaMemsetAsync(ctx->flags, 0, sizeof(int32_t) * n, s));
+    zero_async(ctx, ctx->flags, sizeof(int32_t) * n, s);
     int it = 0;
     unsigned long long nd = 1;
     for (it = 1; it <= max_it; it++) {

@@ -610,10 +610,10 @@ static int launch_walk(crk_ctx *ctx, cudaStream_t s) {
         int rc = crk_ensure_entries(ctx, (long long)ctx->ntiles * 32 * ctx->kcap, -1);
         if (rc) return rc;
     }
-    CRK_CUDA(ctx, cudaMemsetAsync(ctx->counters + CNT_PAIRS_G, 0, 5 * sizeof(unsigned long long), s));
+    zero_async(ctx, ctx->counters + CNT_PAIRS_G, 5 * sizeof(unsigned long long), s);
     if (ctx->act) {   // tiles left out of the walk take no list columns and no stored forces
-        CRK_CUDA(ctx, cudaMemsetAsync(ctx->len_g, 0, sizeof(uint32_t) * ctx->ntiles, s));
-        CRK_CUDA(ctx, cudaMemsetAsync(ctx->len_u, 0, sizeof(uint32_t) * ctx->ntiles, s));
+        zero_async(ctx, ctx->len_g, sizeof(uint32_t) * ctx->ntiles, s);
+        zero_async(ctx, ctx->len_u, sizeof(uint32_t) * ctx->ntiles, s);
         if (ctx->nact == 0) return CRK_OK;
     }
     prof_begin(ctx, PROF_LISTS, s);
