@@ -40,17 +40,18 @@ WORKLOAD = "zeldovich-128^3: clustered gas, Zel'dovich lattice displacement, P(k
 FLOPS_PER_UNIT = {"P1 volumes": 20, "P2 corrections": 88, "P3 grad v": 92, "P4 forces": 281,
                   "P5 compatible energy": 259}
 # DRAM bytes (read + write) per unit measured by ncu for the current P4 kernel on
-# zeldovich-64^3 in the Hilbert order (0.65 GB read + 1.20 GB written for
-# 39.1 M unordered pairs); a full 128^3 launch is too large to capture, so the
-# traffic is scaled by units.
+# zeldovich-64^3 in the Hilbert order (0.67 GB read + 1.23 GB written for
+# 38 M unordered pairs: 16 B per ordered entry written); a full 128^3 launch is
+# too large to capture, so the traffic is scaled by units.
 TRAFFIC_PER_UNIT = {"P4 forces": 50.0}
-# the walk's exact predicate per lane test, in 32-bit integer operations:
-# dx, dy, dz (3), the widening squares and H_j^2 (4), two 64-bit additions
-# (4), the two 64-bit comparisons (4), the gather / other / reach bits (4)
-WALK_INT_OPS = 19
-# INT32 issue: 152 SMs x 64 lanes per clock x 2070 MHz (max SM clock)
-INT32_PEAK_TOPS = 152 * 64 * 2.07e9 / 1e12
-BUILD_BYTES_PER_PARTICLE = 44 + 4 * 20 + 52 + 16
+# the walk's test of one staged particle by one lane, in 32-bit instructions:
+# three differences, a product and two multiply-adds (r^2), two differences
+# (r^2 - H_i^2, r^2 - H_j^2), two minima (the distance to the nearer
+# threshold) and two funnel shifts (the masks)
+WALK_OPS = 12
+# 32-bit issue: 152 SMs x 128 lanes per clock x 2070 MHz (max SM clock)
+ISSUE_PEAK_TOPS = 152 * 128 * 2.07e9 / 1e12
+BUILD_BYTES_PER_PARTICLE = 44 + 3 * 20 + 52 + 16
 PRECISION_NAMES = ["plain", "mixed", "mixed+compensated moments", "mixed+float-float moments"]
 
 
@@ -923,32 +924,31 @@ def run_gpu(args):
                                                  "frac": a / hbm, "peak": hbm,
                                                  "bytes": "16 B per ordered pair-set entry, read once for two kicks"}
     # the cell build: keys (read pos_h 16 B; write fixed point 16, key 4, index 4,
-    # h 4), four stable radix passes (histogram reads the 4-B key; the scatter
+    # h 4), three stable radix passes (histogram reads the 4-B key; the scatter
     # reads and writes key and index, 16 B), the gather into sorted order (read
     # index, fixed point, h: 24 B; write q4 16, h 4, perm 4, key 4), tile boxes
-    # (read q4 16 B): 192 B per particle, against the measured HBM copy bandwidth
+    # (read q4 16 B): 172 B per particle, against the measured HBM copy bandwidth
     tb = prof_ms.get("cell build", 0.0) / args.steps
     if tb > 0:
         a = BUILD_BYTES_PER_PARTICLE * n / (tb / 1e3) / 1e9
         pass_roofline["cell build"] = {"bound": "hbm", "ms_per_step": tb, "achieved": a, "unit": "GB/s",
                                        "frac": a / hbm, "peak": hbm,
-                                       "bytes": "%d B per particle per rebuild (keys, 4 radix passes, gather, "
+                                       "bytes": "%d B per particle per rebuild (keys, 3 radix passes, gather, "
                                                 "tile boxes)" % BUILD_BYTES_PER_PARTICLE}
-    # the neighbour-list walk: integer work, WALK_INT_OPS 32-bit integer
-    # operations per lane test of the exact predicate, lane tests counted by
-    # the walk itself (crk_walk_stats; one walk per step), against the INT32
-    # issue rate (64 lanes per SM per clock)
+    # the neighbour-list walk: WALK_OPS 32-bit instructions per lane test, lane
+    # tests counted by the walk itself (crk_walk_stats; one walk per step),
+    # against the issue rate (128 lanes per SM per clock); choosing and staging
+    # the tested particles and writing the entries come on top
     tw = prof_ms.get("neighbour lists", 0.0) / args.steps
     tests = walk_tests
     if tw > 0 and tests > 0:
-        a = WALK_INT_OPS * tests / (tw / 1e3) / 1e12
+        a = WALK_OPS * tests / (tw / 1e3) / 1e12
         pass_roofline["neighbour lists"] = {"bound": "alu", "ms_per_step": tw, "achieved": a, "unit": "Tops/s",
-                                            "frac": a / INT32_PEAK_TOPS, "peak": INT32_PEAK_TOPS,
+                                            "frac": a / ISSUE_PEAK_TOPS, "peak": ISSUE_PEAK_TOPS,
                                             "lane_tests_per_step": tests,
                                             "useful_fraction": u_pairs / tests,
-                                            "ops": "%d INT32 ops per lane test (3 subtractions, 4 widening "
-                                                   "products, two 64-bit sums and two 64-bit compares, 4 mask "
-                                                   "updates)" % WALK_INT_OPS}
+                                            "ops": "%d 32-bit instructions per lane test (5 differences, 3 for r^2, "
+                                                   "2 minima, 2 mask shifts)" % WALK_OPS}
     roofline["passes"] = pass_roofline
 
     if rank == 0:

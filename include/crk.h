@@ -217,8 +217,8 @@ int crk_neighbours(crk_ctx *ctx, int mode, int32_t *count, uint32_t *hash, void 
  * (device, offsets[n] ints) receives particle i's set in
  * lists[offsets[i] .. offsets[i+1]), in the order the passes visit it:
  *   mode 0: gather(i) (eq:vol; self first), each entry the caller index of j
- *           with bit 31 set when i is in gather(j) too (the "j's kernel
- *           reaches i" flag P4 uses);
+ *           with bit 31 set when i is in gather(j) too (j's kernel
+ *           reaches i);
  *   mode 1: the pair set of i (the gather neighbours, then the others),
  *           caller indices.
  * CRK_ESTATE in a context without lists (the allocation-free volumes). */
@@ -445,12 +445,14 @@ int crk_profile_read(crk_ctx *ctx, double *ms, long long *counts, long long *tot
 
 /* Autotuner of the list passes (P1, P2, P3, P4, P5).  Each pass has variants
  * that differ only in how its work is laid out on the GPU: how many list
- * entries a lane takes per iteration (1-4, for the passes with small
+ * entries a lane has in flight (1, 2 or 4, for the passes with small
  * neighbour records), the order tiles are taken in (Morton order over the
  * grid; contiguous tile ranges per SM in a persistent launch; longest
  * pair-set list first) and how many 32-particle tiles share a CTA (1, 2, 4
  * or 8: 32-256 particles).  Every variant visits each particle's list in the
- * same order, so all produce bitwise identical results.  enable = 1 makes the
+ * same order, so all produce bitwise identical results.  Sets of fewer than 40
+ * tiles per SM, and tiles with very long lists, are shared by the warps of
+ * a CTA whatever the variant.  enable = 1 makes the
  * next call of each pass time every variant once (on the stream, with CUDA
  * events; the call synchronises while tuning) and keep the fastest for the
  * context; enable = 0 keeps the choices made and stops tuning. */
@@ -458,7 +460,8 @@ int crk_autotune(crk_ctx *ctx, int enable);
 
 /* The variant chosen for each pass k (CRK_PROF_NPASS entries, numbering as in
  * crk_profile_read; -1 = not tuned, the built-in default runs) and its time in
- * ms.  Variants 0-3: Morton order, 1-4 entries per iteration; 4-7: longest
+ * ms.  Lists are stored in blocks of four entries, so "3 entries" runs as 4.
+ * Variants 0-3: Morton order, 1-4 entries per iteration; 4-7: longest
  * list first, 1-4 entries; 8: per-SM tile ranges, 1 entry; 9-12: Morton order
  * with the pass's own entries per iteration and CTAs of 1, 2, 4, 8 tiles;
  * 13-16: 1-4 entries per iteration with the neighbour records of the next

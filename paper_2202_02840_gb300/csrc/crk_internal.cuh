@@ -120,7 +120,7 @@ struct crk_ctx {
     unsigned long long *counters = nullptr;
     unsigned long long *h_counters = nullptr;   // pinned host mirror
 
-    // per-particle neighbour lists (column layout per tile) and stored pair forces
+    // per-particle neighbour lists (blocks of four columns per tile) and stored pair forces
     uint4 *qV = nullptr;             // (qx, qy, qz, V bits)
     int32_t *cnt_g = nullptr, *cnt_u = nullptr;   // gather (j != i) and pair-set counts
     uint32_t *len_g = nullptr, *len_u = nullptr;  // per-tile max counts
