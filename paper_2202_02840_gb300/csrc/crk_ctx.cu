@@ -233,46 +233,90 @@ int crk_sync_counters(crk_ctx *ctx, cudaStream_t s) {
 
 // ------------------------------------------------------------------ pack / unpack kernels
 
-__global__ void k_gather_rows(long long total, int w, const int32_t *__restrict__ perm,
-                              const uint32_t *__restrict__ in, uint32_t *__restrict__ out) {
+// Rows of up to three arrays between caller and sorted order in one launch, an
+// element a thread: 16 bytes for four-word rows on 16-byte boundaries, else one word.
+struct RowMoves {
+    const void *in[3];
+    void *out[3];
+    int per_row[3];   // elements of a row; 0: 16-byte rows
+    int sets;
+};
+template <bool GATHER>
+__global__ void k_move_rows(int n, const int32_t *__restrict__ perm, RowMoves m) {
     grid_wait();
-    long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= total) return;
-    long long s = t / w;
-    int c = (int)(t - s * w);
-    out[t] = in[(long long)perm[s] * w + c];
+    long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        if (k >= m.sets) return;
+        const int w = m.per_row[k];
+        const long long count = (long long)n * (w ? w : 1);
+        if (t < count) {
+            if (w == 0) {
+                const uint4 *in = (const uint4 *)m.in[k];
+                uint4 *out = (uint4 *)m.out[k];
+                if (GATHER)
+                    out[t] = in[perm[t]];
+                else
+                    out[perm[t]] = in[t];
+            } else {
+                const uint32_t *in = (const uint32_t *)m.in[k];
+                uint32_t *out = (uint32_t *)m.out[k];
+                const long long s = t / w, c = t - s * w, at = (long long)perm[s] * w + c;
+                if (GATHER)
+                    out[t] = in[at];
+                else
+                    out[at] = in[t];
+            }
+            return;
+        }
+        t -= count;
+    }
 }
 
-__global__ void k_scatter_rows(long long total, int w, const int32_t *__restrict__ perm,
-                               const uint32_t *__restrict__ in, uint32_t *__restrict__ out) {
-    grid_wait();
-    long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= total) return;
-    long long s = t / w;
-    int c = (int)(t - s * w);
-    out[(long long)perm[s] * w + c] = in[t];
-}
-
-// caller-order (A, B, gA, gB) -> sorted CorrRec
-__global__ void k_pack_corr(int n, const int32_t *__restrict__ perm, const float *__restrict__ A,
-                            const float *__restrict__ B, const float *__restrict__ gA,
-                            const float *__restrict__ gB, CorrRec *__restrict__ out) {
+// The caller's inputs of P4 (and P5, with vb and va) -> sorted records, one launch.
+struct ForceInputs {
+    const float *mass, *vel_u, *V, *A, *B, *gA, *gB, *g, *vb, *va;   // vb, va: null or float[3n]
+};
+struct ForceRecords {
+    float *mass, *V;
+    float4 *vel;
+    CorrRec *corr;
+    GvRec *gv;
+    float4 *vb, *va;   // w = 0
+};
+__global__ void k_pack_forces(int n, const int32_t *__restrict__ perm, ForceInputs in, ForceRecords out) {
     grid_wait();
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
-    long long i = perm[s];
-    const float *b = B + 3 * i, *ga = gA + 3 * i, *gb = gB + 9 * i;
+    const long long i = perm[s];
+    const float *v = in.vel_u + 4 * i, *b = in.B + 3 * i, *ga = in.gA + 3 * i, *gb = in.gB + 9 * i, *a = in.g + 9 * i;
+    const float mass = in.mass[i], V = in.V[i];   // every load before the first store
+    const float4 vel = make_float4(v[0], v[1], v[2], v[3]);
     CorrRec c;
-    c.c0 = make_float4(A[i], b[0], b[1], b[2]);
+    c.c0 = make_float4(in.A[i], b[0], b[1], b[2]);
     c.c1 = make_float4(ga[0], ga[1], ga[2], gb[0]);
     c.c2 = make_float4(gb[1], gb[2], gb[3], gb[4]);
     c.c3 = make_float4(gb[5], gb[6], gb[7], gb[8]);
-    out[s] = c;
+    GvRec r;
+    r.g0 = make_float4(a[0], a[1], a[2], a[3]);
+    r.g1 = make_float4(a[4], a[5], a[6], a[7]);
+    r.g2 = make_float4(a[8], 0.f, 0.f, 0.f);
+    out.mass[s] = mass;
+    out.V[s] = V;
+    out.vel[s] = vel;
+    out.corr[s] = c;
+    out.gv[s] = r;
+    if (in.vb) {
+        const float *x = in.vb + 3 * i, *y = in.va + 3 * i;
+        out.vb[s] = make_float4(x[0], x[1], x[2], 0.f);
+        out.va[s] = make_float4(y[0], y[1], y[2], 0.f);
+    }
 }
 
+// sorted CorrRec (and, with g, grad v) -> caller order
 __global__ void k_unpack_corr(int n, const int32_t *__restrict__ perm, const CorrRec *__restrict__ in,
                               float *__restrict__ A, float *__restrict__ B, float *__restrict__ gA,
-                              float *__restrict__ gB) {
+                              float *__restrict__ gB, const GvRec *__restrict__ gv, float *__restrict__ g) {
     grid_wait();
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
@@ -284,41 +328,12 @@ __global__ void k_unpack_corr(int n, const int32_t *__restrict__ perm, const Cor
     ga[0] = c.c1.x; ga[1] = c.c1.y; ga[2] = c.c1.z;
     gb[0] = c.c1.w; gb[1] = c.c2.x; gb[2] = c.c2.y; gb[3] = c.c2.z; gb[4] = c.c2.w;
     gb[5] = c.c3.x; gb[6] = c.c3.y; gb[7] = c.c3.z; gb[8] = c.c3.w;
-}
-
-__global__ void k_pack_gv(int n, const int32_t *__restrict__ perm, const float *__restrict__ g,
-                          GvRec *__restrict__ out) {
-    grid_wait();
-    int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n) return;
-    const float *a = g + 9 * (long long)perm[s];
-    GvRec r;
-    r.g0 = make_float4(a[0], a[1], a[2], a[3]);
-    r.g1 = make_float4(a[4], a[5], a[6], a[7]);
-    r.g2 = make_float4(a[8], 0.f, 0.f, 0.f);
-    out[s] = r;
-}
-
-__global__ void k_unpack_gv(int n, const int32_t *__restrict__ perm, const GvRec *__restrict__ in,
-                            float *__restrict__ g) {
-    grid_wait();
-    int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n) return;
-    float *a = g + 9 * (long long)perm[s];
-    GvRec r = in[s];
+    if (!g) return;
+    float *a = g + 9 * i;
+    GvRec r = gv[s];
     a[0] = r.g0.x; a[1] = r.g0.y; a[2] = r.g0.z; a[3] = r.g0.w;
     a[4] = r.g1.x; a[5] = r.g1.y; a[6] = r.g1.z; a[7] = r.g1.w;
     a[8] = r.g2.x;
-}
-
-// caller float[3n] -> sorted float4 (w = 0)
-__global__ void k_pack_v3(int n, const int32_t *__restrict__ perm, const float *__restrict__ v,
-                          float4 *__restrict__ out) {
-    grid_wait();
-    int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n) return;
-    const float *a = v + 3 * (long long)perm[s];
-    out[s] = make_float4(a[0], a[1], a[2], 0.f);
 }
 
 // sorted (ax, ay, az, dudt) and (vsig, qmax) -> caller arrays
@@ -339,13 +354,22 @@ __global__ void k_unpack_forces(int n, const int32_t *__restrict__ perm, const f
     if (qmax) qmax[i] = q.y;
 }
 
-// (q, V) records of the gather passes from the sorted V
-__global__ void k_make_qV(int n, const uint4 *__restrict__ q4, const float *__restrict__ V, uint4 *__restrict__ qV) {
+// The caller's V, and velocities if given, -> sorted V, (q, V) records and velocities
+__global__ void k_pack_volumes(int n, const int32_t *__restrict__ perm, const uint4 *__restrict__ q4,
+                               const float *__restrict__ V, float *__restrict__ Vs, uint4 *__restrict__ qV,
+                               const float *__restrict__ vel_u, float4 *__restrict__ vel) {
     grid_wait();
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
-    uint4 q = q4[s];
-    qV[s] = make_uint4(q.x, q.y, q.z, __float_as_uint(V[s]));
+    const long long i = perm[s];
+    const float v = V[i];
+    const uint4 q = q4[s];
+    Vs[s] = v;
+    qV[s] = make_uint4(q.x, q.y, q.z, __float_as_uint(v));
+    if (vel_u) {
+        const float *a = vel_u + 4 * i;
+        vel[s] = make_float4(a[0], a[1], a[2], a[3]);
+    }
 }
 
 __global__ void k_zero(long long words, uint32_t *__restrict__ p) {
@@ -387,21 +411,27 @@ void zero_async(crk_ctx *ctx, void *p, size_t bytes, cudaStream_t s) {
     ++ctx->launches;
 }
 
-int gather_rows(crk_ctx *ctx, const void *in, void *out, int w, cudaStream_t s) {
-    long long total = (long long)ctx->n * w;
+static int move_rows(crk_ctx *ctx, bool gather, std::initializer_list<Rows> rows, cudaStream_t s, const char *what) {
+    RowMoves m = {};
+    long long total = 0;
+    for (const Rows &r : rows) {
+        const bool wide = r.words == 4 && (((uintptr_t)r.in | (uintptr_t)r.out) & 15) == 0;
+        m.in[m.sets] = r.in;
+        m.out[m.sets] = r.out;
+        m.per_row[m.sets++] = wide ? 0 : r.words;
+        total += (long long)ctx->n * (wide ? 1 : r.words);
+    }
     if (total == 0) return CRK_OK;
-    launch(s, grid_for(total, 256), 256, 0, k_gather_rows, total, w, ctx->perm, (const uint32_t *)in, (uint32_t *)out);
+    launch(s, grid_for(total, 256), 256, 0, gather ? k_move_rows<true> : k_move_rows<false>, ctx->n, ctx->perm, m);
     ++ctx->launches;
-    CRK_LAUNCH_CHECK(ctx, "gather rows");
+    CRK_LAUNCH_CHECK(ctx, what);
     return CRK_OK;
 }
-int scatter_rows(crk_ctx *ctx, const void *in, void *out, int w, cudaStream_t s) {
-    long long total = (long long)ctx->n * w;
-    if (total == 0) return CRK_OK;
-    launch(s, grid_for(total, 256), 256, 0, k_scatter_rows, total, w, ctx->perm, (const uint32_t *)in, (uint32_t *)out);
-    ++ctx->launches;
-    CRK_LAUNCH_CHECK(ctx, "scatter rows");
-    return CRK_OK;
+int gather_rows(crk_ctx *ctx, std::initializer_list<Rows> rows, cudaStream_t s) {
+    return move_rows(ctx, true, rows, s, "gather");
+}
+int scatter_rows(crk_ctx *ctx, std::initializer_list<Rows> rows, cudaStream_t s) {
+    return move_rows(ctx, false, rows, s, "scatter");
 }
 }  // namespace crk
 
@@ -791,8 +821,7 @@ extern "C" int crk_neighbours(crk_ctx *ctx, int mode, int32_t *count, uint32_t *
         return crk_set_error(ctx, CRK_EINVAL, "bad arguments");
     cudaStream_t s = (cudaStream_t)stream;
     rc = run_neighbours(ctx, mode, ctx->flags, reinterpret_cast<uint32_t *>(ctx->st_tmp1), s);
-    if (!rc) rc = scatter_rows(ctx, ctx->flags, count, 1, s);
-    if (!rc) rc = scatter_rows(ctx, ctx->st_tmp1, hash, 1, s);
+    if (!rc) rc = scatter_rows(ctx, {{ctx->flags, count, 1}, {ctx->st_tmp1, hash, 1}}, s);
     return rc;
 }
 
@@ -813,8 +842,7 @@ extern "C" int crk_volumes(crk_ctx *ctx, float *V, float *Nngb, long long *pairs
     cudaStream_t s = (cudaStream_t)stream;
     rc = run_volumes(ctx, s);
     if (rc) return rc;
-    rc = scatter_rows(ctx, ctx->V, V, 1, s);
-    if (!rc && Nngb) rc = scatter_rows(ctx, ctx->Nn, Nngb, 1, s);
+    rc = Nngb ? scatter_rows(ctx, {{ctx->V, V, 1}, {ctx->Nn, Nngb, 1}}, s) : scatter_rows(ctx, {{ctx->V, V, 1}}, s);
     if (rc) return rc;
     if (pairs) {
         rc = crk_sync_counters(ctx, s);
@@ -834,41 +862,29 @@ extern "C" int crk_corrections(crk_ctx *ctx, const float *V, const float *vel_u,
     int n = ctx->n;
     rc = need_lists(ctx, s);
     if (rc) return rc;
-    rc = gather_rows(ctx, V, ctx->V, 1, s);
-    if (!rc && vel_u) rc = gather_rows(ctx, vel_u, ctx->vel, 4, s);
-    if (rc) return rc;
     if (n) {
-        launch(s, grid_for(n, 256), 256, 0, k_make_qV, n, ctx->q4, ctx->V, ctx->qV);
+        launch(s, grid_for(n, 256), 256, 0, k_pack_volumes, n, ctx->perm, ctx->q4, V, ctx->V, ctx->qV, vel_u, ctx->vel);
         ++ctx->launches;
         CRK_LAUNCH_CHECK(ctx, "gather records");
     }
     rc = run_corrections(ctx, gradv != nullptr, s);
     if (rc) return rc;
     if (n) {
-        launch(s, grid_for(n, 256), 256, 0, k_unpack_corr, n, ctx->perm, ctx->corr, A, B, gradA, gradB);
+        launch(s, grid_for(n, 256), 256, 0, k_unpack_corr, n, ctx->perm, ctx->corr, A, B, gradA, gradB, ctx->gv,
+               gradv);
         ++ctx->launches;
-        if (gradv) {
-            launch(s, grid_for(n, 256), 256, 0, k_unpack_gv, n, ctx->perm, ctx->gv, gradv);
-            ++ctx->launches;
-        }
         CRK_LAUNCH_CHECK(ctx, "unpack corrections");
     }
     return CRK_OK;
 }
 
-static int pack_force_inputs(crk_ctx *ctx, const float *mass, const float *vel_u, const float *V, const float *A,
-                             const float *B, const float *gradA, const float *gradB, const float *gradv,
-                             cudaStream_t s) {
+static int pack_force_inputs(crk_ctx *ctx, const ForceInputs &in, cudaStream_t s) {
     int n = ctx->n;
     int rc = need_lists(ctx, s);
-    if (!rc) rc = gather_rows(ctx, mass, ctx->mass, 1, s);
-    if (!rc) rc = gather_rows(ctx, vel_u, ctx->vel, 4, s);
-    if (!rc) rc = gather_rows(ctx, V, ctx->V, 1, s);
     if (rc) return rc;
     if (n) {
-        launch(s, grid_for(n, 256), 256, 0, k_pack_corr, n, ctx->perm, A, B, gradA, gradB, ctx->corr);
-        ++ctx->launches;
-        launch(s, grid_for(n, 256), 256, 0, k_pack_gv, n, ctx->perm, gradv, ctx->gv);
+        const ForceRecords out{ctx->mass, ctx->V, ctx->vel, ctx->corr, ctx->gv, ctx->vb, ctx->va};
+        launch(s, grid_for(n, 256), 256, 0, k_pack_forces, n, ctx->perm, in, out);
         ++ctx->launches;
         CRK_LAUNCH_CHECK(ctx, "pack force inputs");
     }
@@ -883,7 +899,7 @@ extern "C" int crk_forces(crk_ctx *ctx, const float *mass, const float *vel_u, c
     if (ctx->n > 0 && (!mass || !vel_u || !V || !A || !B || !gradA || !gradB || !gradv || !accel || !dudt))
         return crk_set_error(ctx, CRK_EINVAL, "NULL argument");
     cudaStream_t s = (cudaStream_t)stream;
-    rc = pack_force_inputs(ctx, mass, vel_u, V, A, B, gradA, gradB, gradv, s);
+    rc = pack_force_inputs(ctx, {mass, vel_u, V, A, B, gradA, gradB, gradv, nullptr, nullptr}, s);
     if (rc) return rc;
     rc = run_forces(ctx, s);
     if (rc) return rc;
@@ -910,18 +926,10 @@ extern "C" int crk_compatible(crk_ctx *ctx, const float *mass, const float *vel_
         (!mass || !vel_u || !V || !A || !B || !gradA || !gradB || !gradv || !vel_before || !vel_after || !du))
         return crk_set_error(ctx, CRK_EINVAL, "NULL argument");
     cudaStream_t s = (cudaStream_t)stream;
-    rc = pack_force_inputs(ctx, mass, vel_u, V, A, B, gradA, gradB, gradv, s);
+    rc = pack_force_inputs(ctx, {mass, vel_u, V, A, B, gradA, gradB, gradv, vel_before, vel_after}, s);
     if (rc) return rc;
-    int n = ctx->n;
-    if (n) {
-        launch(s, grid_for(n, 256), 256, 0, k_pack_v3, n, ctx->perm, vel_before, ctx->vb);
-        ++ctx->launches;
-        launch(s, grid_for(n, 256), 256, 0, k_pack_v3, n, ctx->perm, vel_after, ctx->va);
-        ++ctx->launches;
-        CRK_LAUNCH_CHECK(ctx, "pack kick velocities");
-    }
     rc = run_forces(ctx, s);     // F_ij of this evaluation state
     if (!rc) rc = run_compatible(ctx, s);
     if (rc) return rc;
-    return scatter_rows(ctx, ctx->du, du, 1, s);
+    return scatter_rows(ctx, {{ctx->du, du, 1}}, s);
 }

@@ -556,9 +556,7 @@ static int cycle_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const flo
     if (fresh) {
         rc = build_cells_sorted(ctx, n, (const float4 *)pos_h, nullptr, s);
         if (!rc) rc = finish_build(ctx, s);
-        if (!rc) rc = gather_rows(ctx, pos_h, ctx->st_pos, 4, s);
-        if (!rc) rc = gather_rows(ctx, vel_u, ctx->st_vel, 4, s);
-        if (!rc) rc = gather_rows(ctx, mass, ctx->mass, 1, s);
+        if (!rc) rc = gather_rows(ctx, {{pos_h, ctx->st_pos, 4}, {vel_u, ctx->st_vel, 4}, {mass, ctx->mass, 1}}, s);
         if (rc) return rc;
         copy_async(ctx, ctx->vel, ctx->st_vel, sizeof(float4) * n, s);
         rc = evaluate(ctx, s);
@@ -566,8 +564,7 @@ static int cycle_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const flo
         ctx->rates_valid = 1;
         ctx->step_n = n;
     } else {
-        rc = gather_rows(ctx, pos_h, ctx->st_pos, 4, s);
-        if (!rc) rc = gather_rows(ctx, vel_u, ctx->st_vel, 4, s);
+        rc = gather_rows(ctx, {{pos_h, ctx->st_pos, 4}, {vel_u, ctx->st_vel, 4}}, s);
         if (rc) return rc;
     }
     ctx->rates_valid = 0;   // until the cycle completes
@@ -702,7 +699,7 @@ static int cycle_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const flo
     tp = ctx->vel; ctx->vel = ctx->vb; ctx->vb = tp;
     tp = ctx->st_half; ctx->st_half = ctx->va; ctx->va = tp;
     copy_async(ctx, ctx->hc, ctx->st_tmp1, sizeof(float) * n, s);
-    rc = gather_rows(ctx, mass, ctx->mass, 1, s);
+    rc = gather_rows(ctx, {{mass, ctx->mass, 1}}, s);
     if (!rc) rc = evaluate(ctx, s);
     if (rc) return rc;
     evals += n;
@@ -715,8 +712,7 @@ static int cycle_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const flo
            ctx->st_pos);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "finish cycle");
-    rc = scatter_rows(ctx, ctx->st_pos, pos_h, 4, s);
-    if (!rc) rc = scatter_rows(ctx, ctx->st_vel, vel_u, 4, s);
+    rc = scatter_rows(ctx, {{ctx->st_pos, pos_h, 4}, {ctx->st_vel, vel_u, 4}}, s);
     if (!rc) zero_async(ctx, ctx->counters + CNT_NEXT_OK, sizeof(unsigned long long), s);
     if (!rc) rc = crk_sync_counters(ctx, s);
     if (rc) return rc;
@@ -762,7 +758,7 @@ extern "C" int crk_htb_levels(crk_ctx *ctx, int n, const float *pos_h, const flo
     int rc = build_cells_sorted(ctx, n, (const float4 *)pos_h, nullptr, s);
     if (!rc) rc = finish_build(ctx, s);
     if (!rc) rc = ensure_htb(ctx);
-    if (!rc) rc = gather_rows(ctx, dt, ctx->d_dt, 1, s);
+    if (!rc) rc = gather_rows(ctx, {{dt, ctx->d_dt, 1}}, s);
     if (rc) return rc;
     ctx->rates_valid = 0;
     const HtbConsts c = htb_consts(ctx, Delta, L, f_l);
@@ -777,7 +773,7 @@ extern "C" int crk_htb_levels(crk_ctx *ctx, int n, const float *pos_h, const flo
     launch(s, grid_for(n, 256), 256, 0, k_htb_slot_level, n, ctx->tlev, reinterpret_cast<int32_t *>(ctx->st_tmp1));
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "leaf levels");
-    rc = scatter_rows(ctx, ctx->st_tmp1, level, 1, s);
+    rc = scatter_rows(ctx, {{ctx->st_tmp1, level, 1}}, s);
     if (!rc) rc = crk_sync_counters(ctx, s);
     if (rc) return rc;
     if (unresolved) *unresolved = (long long)ctx->h_counters[CNT_UNRES];

@@ -8,6 +8,8 @@
 #include <stdio.h>
 #include <stdarg.h>
 
+#include <initializer_list>
+
 #include "crk.h"
 
 namespace crk {
@@ -352,8 +354,13 @@ int propose_sorted(crk_ctx *ctx, int n, float4 *pos, const GvRec *gv, const floa
                    cudaStream_t s);   // learned h proposal in sorted order (crk_mlp.cu)
 void zero_async(crk_ctx *ctx, void *p, size_t bytes, cudaStream_t s);   // whole 32-bit words (crk_ctx.cu)
 void copy_async(crk_ctx *ctx, void *to, const void *from, size_t bytes, cudaStream_t s);
-int gather_rows(crk_ctx *ctx, const void *in, void *out, int width_words, cudaStream_t s);
-int scatter_rows(crk_ctx *ctx, const void *in, void *out, int width_words, cudaStream_t s);
+struct Rows {   // of `words` 32-bit words
+    const void *in;
+    void *out;
+    int words;
+};
+int gather_rows(crk_ctx *ctx, std::initializer_list<Rows> rows, cudaStream_t s);    // caller -> sorted order, up to 3
+int scatter_rows(crk_ctx *ctx, std::initializer_list<Rows> rows, cudaStream_t s);   // sorted -> caller order
 inline int grid_for(long long n, int block) { return (int)((n + block - 1) / block); }
 }  // namespace crk
 

@@ -141,8 +141,9 @@ extern "C" int crk_volumes_noalloc(int n, const float *pos_h, float *V, float *N
     if (hc[crk::CNT_ERR_INPUT]) return CRK_EINVAL;
     if ((long long)hc[crk::CNT_ULIST] > ctx.cap_ulist) return CRK_ECAPACITY;
     rc = crk::run_volumes(&ctx, s);
-    if (!rc) rc = crk::scatter_rows(&ctx, ctx.V, V, 1, s);
-    if (!rc && Nngb) rc = crk::scatter_rows(&ctx, ctx.Nn, Nngb, 1, s);
+    if (!rc)
+        rc = Nngb ? crk::scatter_rows(&ctx, {{ctx.V, V, 1}, {ctx.Nn, Nngb, 1}}, s)
+                  : crk::scatter_rows(&ctx, {{ctx.V, V, 1}}, s);
     // Every buffer above was sized for NMAX, so nothing may have been grown;
     // a later change to the build or the pass that did grow one would have
     // swapped in library-allocated memory: report it rather than return.

@@ -507,9 +507,7 @@ static int step_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const floa
         rc = build_cells_sorted(ctx, n, (const float4 *)pos_h, nullptr, s, batched ? ctx->box_in : nullptr);
         if (!rc) rc = finish_build(ctx, s);
         if (rc) return rc;
-        rc = gather_rows(ctx, pos_h, ctx->st_pos, 4, s);
-        if (!rc) rc = gather_rows(ctx, vel_u, ctx->st_vel, 4, s);
-        if (!rc) rc = gather_rows(ctx, mass, ctx->mass, 1, s);
+        rc = gather_rows(ctx, {{pos_h, ctx->st_pos, 4}, {vel_u, ctx->st_vel, 4}, {mass, ctx->mass, 1}}, s);
         if (rc) return rc;
         copy_async(ctx, ctx->vel, ctx->st_vel, sizeof(float4) * n, s);
         rc = evaluate(ctx, s);
@@ -517,8 +515,7 @@ static int step_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const floa
         ctx->rates_valid = 1;
         ctx->step_n = n;
     } else {
-        rc = gather_rows(ctx, pos_h, ctx->st_pos, 4, s);
-        if (!rc) rc = gather_rows(ctx, vel_u, ctx->st_vel, 4, s);
+        rc = gather_rows(ctx, {{pos_h, ctx->st_pos, 4}, {vel_u, ctx->st_vel, 4}}, s);
         if (rc) return rc;
     }
     const int nb = batched ? ctx->nbox : 1;
@@ -559,7 +556,7 @@ static int step_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const floa
     t = ctx->st_pos; ctx->st_pos = ctx->st_tmp; ctx->st_tmp = t;
     t = ctx->st_vel; ctx->st_vel = ctx->vb; ctx->vb = t;
     t = ctx->st_half; ctx->st_half = ctx->va; ctx->va = t;
-    rc = gather_rows(ctx, mass, ctx->mass, 1, s);
+    rc = gather_rows(ctx, {{mass, ctx->mass, 1}}, s);
     if (rc) return rc;
     ctx->h_iters = 0;
     ctx->h_unconv = 0;
@@ -594,8 +591,7 @@ static int step_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const floa
            ctx->st_pos);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "finish step");
-    rc = scatter_rows(ctx, ctx->st_pos, pos_h, 4, s);
-    if (!rc) rc = scatter_rows(ctx, ctx->st_vel, vel_u, 4, s);
+    rc = scatter_rows(ctx, {{ctx->st_pos, pos_h, 4}, {ctx->st_vel, vel_u, 4}}, s);
     return rc;
 }
 
