@@ -132,17 +132,10 @@ __global__ void k_next_check(int nbox, const double *__restrict__ dtb, const dou
     }
 }
 
-// the opening kick's energy rates when its P5 pass was skipped
-__global__ void k_take_next(int n, const unsigned long long *cnt, const float *__restrict__ du_next,
-                            float *__restrict__ du) {
-    grid_wait();
-    if (!cnt[CNT_SKIP]) return;
-    int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s < n) du[s] = du_next[s];
-}
-
 __global__ void k_set_next_ok(unsigned long long *cnt) {
-    grid_wait(); cnt[CNT_NEXT_OK] = 1ull; }
+    grid_wait();
+    cnt[CNT_NEXT_OK] = 1ull;
+}
 
 // dt of slot s: its box's (one box: dtb[0])
 __device__ __forceinline__ double slot_dt(const double *dtb, const int32_t *sbox, int s) {
@@ -165,20 +158,23 @@ __global__ void k_kick1(int n, const double *sc, const int32_t *__restrict__ sbo
 // u_p = (u_1/2 + du dt/2) / (1 + E dt/2); drift x1 = x + p_1/2 dt / a^2
 // (periodic wrap into [0,1)).  The expansion term -E u of eq:CosmoEngEqn
 // enters the opening half kick explicitly and the closing ones implicitly:
-// the trapezoidal rule over the step (E = 0 in a static box).
+// the trapezoidal rule over the step (E = 0 in a static box).  du comes from du_next,
+// formed by the last step, where this step's opening P5 was skipped for it.
 __global__ void k_half_drift(int n, const double *sc, const int32_t *__restrict__ sbox, StepConsts c,
                              float4 *__restrict__ st_pos, float4 *__restrict__ st_vel,
                              float4 *__restrict__ st_half, const float4 *__restrict__ va,
-                             const float4 *__restrict__ acc, const float *__restrict__ du) {
+                             const float4 *__restrict__ acc, const float *__restrict__ du,
+                             const float *__restrict__ du_next, const unsigned long long *__restrict__ cnt) {
     grid_wait();
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     float dt = (float)slot_dt(sc, sbox, s), h = 0.5f * dt;
     float4 v = st_vel[s], ph = va[s], a = acc[s];
-    float uh = fmaf(h, fmaf(-c.E, v.w, du[s]), v.w);
+    const float d = cnt[CNT_SKIP] ? du_next[s] : du[s];
+    float uh = fmaf(h, fmaf(-c.E, v.w, d), v.w);
     st_half[s] = make_float4(ph.x, ph.y, ph.z, uh);
     st_vel[s] = make_float4(fmaf(h, a.x, ph.x), fmaf(h, a.y, ph.y), fmaf(h, a.z, ph.z),
-                            fmaf(h, du[s], uh) / fmaf(h, c.E, 1.f));
+                            fmaf(h, d, uh) / fmaf(h, c.E, 1.f));
     float4 p = st_pos[s];
     const float dx = dt * c.inv_a2;
     float x[3] = {fmaf(dx, ph.x, p.x), fmaf(dx, ph.y, p.y), fmaf(dx, ph.z, p.z)};
@@ -191,17 +187,23 @@ __global__ void k_half_drift(int n, const double *sc, const int32_t *__restrict_
     st_pos[s] = make_float4(x[0], x[1], x[2], p.w);
 }
 
-// new slot s takes old slot idx[s]
-__global__ void k_permute3(int n, const int32_t *__restrict__ idx, const float4 *__restrict__ a,
-                           float4 *__restrict__ ao, const float4 *__restrict__ b, float4 *__restrict__ bo,
-                           const float4 *__restrict__ c, float4 *__restrict__ co) {
+// new slot s takes old slot idx[s] and the mass of the caller's particle perm[s];
+// the velocities also go to vel, if given
+__global__ void k_permute_state(int n, const int32_t *__restrict__ idx, const float4 *__restrict__ a,
+                                float4 *__restrict__ ao, const float4 *__restrict__ b, float4 *__restrict__ bo,
+                                const float4 *__restrict__ c, float4 *__restrict__ co,
+                                const int32_t *__restrict__ perm, const float *__restrict__ mass,
+                                float *__restrict__ mo, float4 *__restrict__ vel) {
     grid_wait();
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= n) return;
     int o = idx[s];
+    const float4 v = b[o];
     ao[s] = a[o];
-    bo[s] = b[o];
+    bo[s] = v;
     co[s] = c[o];
+    mo[s] = mass[perm[s]];
+    if (vel) vel[s] = v;
 }
 
 // second half kick: p1 = p_1/2 + a1 dt/2; vb = p_1/2, va = p1
@@ -534,10 +536,8 @@ static int step_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const floa
     CRK_LAUNCH_CHECK(ctx, "kick");
     rc = run_compatible(ctx, s, ctx->counters + CNT_SKIP);
     if (rc) return rc;
-    launch(s, g, b, 0, k_take_next, n, ctx->counters, ctx->du_next, ctx->du);
-    ++ctx->launches;
     launch(s, g, b, 0, k_half_drift, n, dtb, sbox, c, ctx->st_pos, ctx->st_vel, ctx->st_half, ctx->va, ctx->acc,
-           ctx->du);
+           ctx->du, ctx->du_next, ctx->counters);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "drift");
     // rebuild at x1 (input order = current sorted order; boxes keep their particles)
@@ -548,16 +548,14 @@ static int step_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const floa
         ctx->rates_valid = 0;
         return rc;
     }
-    launch(s, g, b, 0, k_permute3, n, ctx->idx_a, ctx->st_pos, ctx->st_tmp, ctx->st_vel, ctx->vb, ctx->st_half,
-           ctx->va);
+    launch(s, g, b, 0, k_permute_state, n, ctx->idx_a, ctx->st_pos, ctx->st_tmp, ctx->st_vel, ctx->vb, ctx->st_half,
+           ctx->va, ctx->perm, mass, ctx->mass, ctx->p.h_mode >= 1 ? nullptr : ctx->vel);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "permute state");
     float4 *t;
     t = ctx->st_pos; ctx->st_pos = ctx->st_tmp; ctx->st_tmp = t;
     t = ctx->st_vel; ctx->st_vel = ctx->vb; ctx->vb = t;
     t = ctx->st_half; ctx->st_half = ctx->va; ctx->va = t;
-    rc = gather_rows(ctx, {{mass, ctx->mass, 1}}, s);
-    if (rc) return rc;
     ctx->h_iters = 0;
     ctx->h_unconv = 0;
     if (ctx->p.h_mode >= 1) {   // eq:hi at x1 before the evaluation
@@ -566,9 +564,9 @@ static int step_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const floa
             ctx->rates_valid = 0;
             return rc;
         }
+        copy_async(ctx, ctx->vel, ctx->st_vel, sizeof(float4) * n, s);
     }
     // evaluation at (x1, p_p, u_p)
-    copy_async(ctx, ctx->vel, ctx->st_vel, sizeof(float4) * n, s);
     rc = evaluate(ctx, s);
     if (rc) {
         ctx->rates_valid = 0;
