@@ -323,6 +323,67 @@ __global__ void k_htb_compact(int ntiles, int n, const uint32_t *__restrict__ fl
     if (T == ntiles - 1) cnt[CNT_NACT] = ofs[T] + flag[T];
 }
 
+// The same by one CTA straight from a predicate, without flags, scan and reset:
+// warp w takes 256 consecutive tiles of each 8192.  Up to COMPACT_ONE tiles (a
+// scan's three launches and the rest took 16 us a pass at 8192 tiles, this 4.3).
+constexpr int COMPACT_ONE = 65536;
+struct FlaggedTiles {
+    const uint32_t *flag;
+    __device__ bool operator()(int T) const { return flag[T] != 0u; }
+};
+struct DueTiles {   // tiles that end a step at tick t
+    const int32_t *tt0, *tlen;
+    int t;
+    __device__ bool operator()(int T) const { return tile_active(tt0, tlen, T, t); }
+};
+template <class F>
+__global__ void __launch_bounds__(1024) k_compact_tiles(int ntiles, int n, F listed, int32_t *__restrict__ act,
+                                                        unsigned long long *cnt) {
+    grid_wait();
+    __shared__ int found[32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    int out = 0, parts = 0;
+    for (int t0 = 0; t0 < ntiles; t0 += 8192) {
+        unsigned m[8];
+        int c = 0;
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+            const int T = t0 + w * 256 + k * 32 + lane;
+            const bool on = T < ntiles && listed(T);
+            m[k] = __ballot_sync(FULLM, on);
+            c += __popc(m[k]);
+            if (on) parts += min(TILE, n - T * TILE);
+        }
+        if (lane == 0) found[w] = c;
+        __syncthreads();
+        const int v = found[lane];
+        int x = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(FULLM, x, o);
+            if (lane >= o) x += y;
+        }
+        int at = out + __shfl_sync(FULLM, x - v, w);
+        out += __shfl_sync(FULLM, x, 31);
+#pragma unroll
+        for (int k = 0; k < 8; k++) {
+            if (m[k] >> lane & 1u) act[at + __popc(m[k] & lanemask_lt())] = t0 + w * 256 + k * 32 + lane;
+            at += __popc(m[k]);
+        }
+        __syncthreads();   // `found` is free for the next round
+    }
+    parts = __reduce_add_sync(FULLM, parts);
+    if (lane == 0) found[w] = parts;
+    __syncthreads();
+    if (w == 0) {
+        parts = __reduce_add_sync(FULLM, found[lane]);
+        if (lane == 0) {
+            cnt[CNT_NACT] = (unsigned long long)out;
+            cnt[CNT_NACT + 1] = (unsigned long long)parts;
+        }
+    }
+}
+
 // each slot takes its tile's level (for the caller's per-particle view)
 __global__ void k_htb_slot_level(int n, const int32_t *__restrict__ tlev, int32_t *__restrict__ out) {
     grid_wait();
@@ -397,7 +458,7 @@ static int grow(crk_ctx *ctx, T **p, size_t count) {
     return CRK_OK;
 }
 
-static int ensure_htb(crk_ctx *ctx) {
+int ensure_htb(crk_ctx *ctx) {
     const int nt = ctx->ntiles, n = ctx->n;
     int rc = CRK_OK;
     if (nt > ctx->cap_htb) {
@@ -422,32 +483,22 @@ static int ensure_htb(crk_ctx *ctx) {
     return CRK_OK;
 }
 
-// tile t holds a particle whose eq:hi solve is not yet done (flags[s] == 0)
-__global__ void k_unconv_flags(int ntiles, int n, const int32_t *__restrict__ flags, uint32_t *__restrict__ tflag) {
-    grid_wait();
-    const int T = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (T >= ntiles) return;
-    const int s = T * TILE + (int)(threadIdx.x & 31);
-    const bool open = s < n && flags[s] == 0;
-    const unsigned m = __ballot_sync(FULLM, open);
-    if ((threadIdx.x & 31) == 0) tflag[T] = m != 0u;
-}
-
-// The tiles that hold a particle not yet converged (ctx->flags == 0), in tile
-// order, into ctx->tact; their count lands in ctx->counters[CNT_NACT] (read
-// after the caller's next sync).  The h solves walk only these tiles.
-int unconverged_tiles(crk_ctx *ctx, cudaStream_t s) {
-    int rc = ensure_htb(ctx);
-    if (rc) return rc;
+// The tiles flagged in ctx->tflag into ctx->tact, in tile order; their count and their
+// particles' land in ctx->counters[CNT_NACT] (read after the caller's next sync).
+int flagged_tiles(crk_ctx *ctx, cudaStream_t s) {
     const int nt = ctx->ntiles;
-    zero_async(ctx, ctx->counters + CNT_NACT, 2 * sizeof(unsigned long long), s);
-    launch(s, grid_for((long long)nt * 32, 256), 256, 0, k_unconv_flags, nt, ctx->n, ctx->flags, ctx->tflag);
+    if (nt <= COMPACT_ONE) {
+        launch(s, 1, 1024, 0, k_compact_tiles<FlaggedTiles>, nt, ctx->n, FlaggedTiles{ctx->tflag}, ctx->tact,
+               ctx->counters);
+    } else {
+        zero_async(ctx, ctx->counters + CNT_NACT, 2 * sizeof(unsigned long long), s);
+        int rc = scan_u32(ctx, ctx->tflag, ctx->tscan, nt, s);
+        if (rc) return rc;
+        launch(s, grid_for(nt, 256), 256, 0, k_htb_compact, nt, ctx->n, ctx->tflag, ctx->tscan, ctx->tact,
+               ctx->counters);
+    }
     ++ctx->launches;
-    rc = scan_u32(ctx, ctx->tflag, ctx->tscan, nt, s);
-    if (rc) return rc;
-    launch(s, grid_for(nt, 256), 256, 0, k_htb_compact, nt, ctx->n, ctx->tflag, ctx->tscan, ctx->tact, ctx->counters);
-    ++ctx->launches;
-    CRK_LAUNCH_CHECK(ctx, "unconverged tiles");
+    CRK_LAUNCH_CHECK(ctx, "tile list");
     return CRK_OK;
 }
 
@@ -528,15 +579,17 @@ static int next_tick(crk_ctx *ctx, int *t_next, cudaStream_t s) {
 
 static int active_list(crk_ctx *ctx, int t, long long *parts, cudaStream_t s) {
     const int nt = ctx->ntiles;
-    zero_async(ctx, ctx->counters + CNT_NACT, 2 * sizeof(unsigned long long), s);
-    launch(s, grid_for(nt, 256), 256, 0, k_htb_flags, nt, ctx->tt0, ctx->tlen, t, ctx->tflag);
-    ++ctx->launches;
-    int rc = scan_u32(ctx, ctx->tflag, ctx->tscan, nt, s);
-    if (rc) return rc;
-    launch(s, grid_for(nt, 256), 256, 0, k_htb_compact, nt, ctx->n, ctx->tflag, ctx->tscan, ctx->tact, ctx->counters);
+    int rc = CRK_OK;
+    if (nt <= COMPACT_ONE) {
+        launch(s, 1, 1024, 0, k_compact_tiles<DueTiles>, nt, ctx->n, DueTiles{ctx->tt0, ctx->tlen, t}, ctx->tact,
+               ctx->counters);
+    } else {
+        launch(s, grid_for(nt, 256), 256, 0, k_htb_flags, nt, ctx->tt0, ctx->tlen, t, ctx->tflag);
+        rc = flagged_tiles(ctx, s);
+    }
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "active leaves");
-    rc = crk_sync_counters(ctx, s);
+    if (!rc) rc = crk_sync_counters(ctx, s);
     if (rc) return rc;
     ctx->nact = (int)ctx->h_counters[CNT_NACT];
     *parts = (long long)ctx->h_counters[CNT_NACT + 1];

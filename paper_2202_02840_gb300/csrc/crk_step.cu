@@ -301,9 +301,11 @@ __global__ void k_energy_final(int nb, const double *__restrict__ part, double *
     }
 }
 
-// h iteration: Thacker update of every particle not yet converged (eq:thacker)
+// h iteration: Thacker update of every particle not yet converged (eq:thacker);
+// tflag: tiles that still hold one
 __global__ void k_h_iter(int n, StepConsts c, float tol, const float *__restrict__ Nn, float *__restrict__ hs,
-                         uint4 *__restrict__ q4, int32_t *__restrict__ flags, unsigned long long *notdone) {
+                         uint4 *__restrict__ q4, int32_t *__restrict__ flags, uint32_t *__restrict__ tflag,
+                         unsigned long long *notdone) {
     grid_wait();
     int s = blockIdx.x * blockDim.x + threadIdx.x;
     unsigned nd = 0;
@@ -323,7 +325,10 @@ __global__ void k_h_iter(int n, StepConsts c, float tol, const float *__restrict
         }
     }
     nd = __reduce_add_sync(0xffffffffu, nd);
-    if ((threadIdx.x & 31) == 0 && nd) atomicAdd(notdone, (unsigned long long)nd);
+    if ((threadIdx.x & 31) == 0) {
+        if (s < n) tflag[s / TILE] = nd != 0u;
+        if (nd) atomicAdd(notdone, (unsigned long long)nd);
+    }
 }
 
 // after the proposal wrote st_pos.w: the sorted h and the fixed-point support
@@ -423,12 +428,14 @@ extern "C" int crk_reset_rates(crk_ctx *ctx) {
 // *nd = particles updated (0: all converged).
 static int h_update(crk_ctx *ctx, const StepConsts &c, float tol, cudaStream_t s, unsigned long long *nd) {
     const int n = ctx->n;
+    int rc = ensure_htb(ctx);
+    if (rc) return rc;
     zero_async(ctx, ctx->counters + CNT_NOTDONE, sizeof(unsigned long long), s);
-    launch(s, grid_for(n, 256), 256, 0, k_h_iter, n, c, tol, ctx->Nn, ctx->hs, ctx->q4, ctx->flags,
+    launch(s, grid_for(n, 256), 256, 0, k_h_iter, n, c, tol, ctx->Nn, ctx->hs, ctx->q4, ctx->flags, ctx->tflag,
            ctx->counters + CNT_NOTDONE);
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "h iteration");
-    int rc = unconverged_tiles(ctx, s);
+    rc = flagged_tiles(ctx, s);
     if (!rc) rc = crk_sync_counters(ctx, s);
     if (rc) return rc;
     *nd = ctx->h_counters[CNT_NOTDONE];

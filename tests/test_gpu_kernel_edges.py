@@ -220,3 +220,21 @@ def test_overlapped_training_steps_are_the_separate_ones(batch):
             losses += crk.crk_mlp_train(ctx, X, T, batch=batch, steps=steps // calls, lr=1e-3, seed=3)
         out.append((np.array(losses), as_np(crk.crk_mlp_get_weights(ctx))))
     assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])
+
+
+@pytest.mark.parametrize("side", [14, 64, 65])
+def test_h_solve_over_the_open_tiles(side):
+    """The tiles that later passes walk are listed by one CTA, 8192 at a time
+    (64^3 particles: exactly one round; 65^3: a second, ragged one): the solve
+    converges every particle, which an unlisted tile would not."""
+    pos = inputs.sedov(side)["pos_h"].copy()
+    pos[:, 3] *= np.float32(0.9)
+    g = dev(pos)
+    ctx = crk.crk_create()
+    it, ok = crk.crk_h_iterate(ctx, g, tol=1e-4, max_it=60)
+    assert ok and it > 2
+    crk.crk_build_cells(ctx, g)
+    N = as_np(crk.crk_volumes(ctx)[1]).astype(np.float64)
+    h = as_np(g)[:, 3]
+    held = (h >= 0.3) | (h <= 1e-6)
+    assert np.all(np.abs(np.cbrt(268.0 / N[~held]) - 1.0) <= 1.01e-4)   # N rounded to FP32
