@@ -320,7 +320,7 @@ struct P4 {
 // ================================================================= P4 fed by TMA
 //
 // The same pass as P4's list loop, with each lane's neighbour record brought
-// into shared memory by the tensor-memory accelerator instead of five 256-bit
+// into shared memory by the tensor-memory accelerator instead of four 256-bit
 // gathers through L1: per iteration one lane issues eight tile::gather4 loads
 // (four records each) of the next entries of all 32 lanes from L2, into the
 // other of two stages, and an mbarrier counts their bytes.  The lanes read
@@ -375,7 +375,7 @@ __global__ void __launch_bounds__(TMA_WARPS * 32) k_p4_tma(ListGeom g, typename 
     __shared__ alignas(8) unsigned long long bar[TMA_WARPS][2];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int tile = blockIdx.x * TMA_WARPS + w;
-    if (tile >= g.ntiles) return;
+    if (tile >= g.ntiles || (g.heavy && (int)g.len_u[tile] > g.heavy)) return;   // the split form has the long lists
     const uint32_t bar0 = smem_u32(&bar[w][0]), stg0 = smem_u32(&stg[w][0][0]);   // stage s: + 8 s, + TMA_STAGE s
     if (lane == 0) {
         mbar_init(bar0);

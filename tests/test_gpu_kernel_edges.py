@@ -238,3 +238,46 @@ def test_h_solve_over_the_open_tiles(side):
     h = as_np(g)[:, 3]
     held = (h >= 0.3) | (h <= 1e-6)
     assert np.all(np.abs(np.cbrt(268.0 / N[~held]) - 1.0) <= 1.01e-4)   # N rounded to FP32
+
+
+PASSES = ("P1 volumes", "P2 corrections", "P3 grad v", "P4 forces", "P5 compatible energy")
+
+
+def above_the_split_line(nsm):
+    """Past 40 tiles an SM, where the pass variants run (58^3 at 152 SMs: 6098 tiles,
+    the last ragged), cold with a blast; eight particles have h = 6.2 spacings
+    (1000 neighbours), whose tiles the split form takes."""
+    side = int(np.ceil((40 * 32 * nsm + 1) ** (1 / 3)))
+    st = inputs.sedov(side)
+    st["pos_h"][::side ** 3 // 8, 3] = 6.2 / side
+    return st
+
+
+def every_pass(ctx, st, steps=2):
+    """The outputs of each pass and of two KDK steps, as bit patterns."""
+    pos, vel, mass = dev(st["pos_h"]), dev(st["vel_u"]), dev(st["mass"])
+    crk.crk_build_cells(ctx, pos)
+    V, N = crk.crk_volumes(ctx)
+    cor = crk.crk_corrections(ctx, V, vel)
+    f = crk.crk_forces(ctx, mass, vel, V, *cor)
+    du = crk.crk_compatible(ctx, mass, vel, V, *cor, vel[:, :3].contiguous(), (vel[:, :3] + f[0] * 1e-4).contiguous())
+    for _ in range(steps):
+        crk.crk_step(ctx, pos, vel, mass, 0.0)
+    return [t.view(torch.int32).clone() for t in (V, N, *cor, *f, du, pos, vel)]
+
+
+def test_every_pass_variant_where_it_runs():
+    """Each variant pinned on a set above the split line, some of its lists longer
+    than a warp takes alone: bitwise the default run, two KDK steps included."""
+    st = above_the_split_line(torch.cuda.get_device_properties(0).multi_processor_count)
+    ref = every_pass(crk.crk_create(), st)
+    ctx = crk.crk_create()
+    crk.crk_build_cells(ctx, dev(st["pos_h"]))
+    assert crk.crk_neighbours(ctx, 1)[0].max() > 900
+    for v in range(crk.CRK_TUNE_NVARIANT):
+        ctx = crk.crk_create()
+        for name in PASSES:   # P4 has 0, 4, 8 to 12 and 21 (records by TMA), the others all but 21
+            if v in (0, 4, 8, 9, 10, 11, 12) or (v == 21) == (name == "P4 forces"):
+                crk.crk_tune_set(ctx, name, v)
+        for k, (a, b) in enumerate(zip(ref, every_pass(ctx, st))):
+            assert torch.equal(a, b), (v, k)
