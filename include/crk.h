@@ -455,7 +455,9 @@ int crk_profile_read(crk_ctx *ctx, double *ms, long long *counts, long long *tot
  * a CTA whatever the variant.  enable = 1 makes the
  * next call of each pass time every variant once (on the stream, with CUDA
  * events; the call synchronises while tuning) and keep the fastest for the
- * context; enable = 0 keeps the choices made and stops tuning. */
+ * context; on a set of fewer than 40 tiles per SM it times the one form such
+ * sets have and reports the built-in default, and the next call on a larger set
+ * times the variants.  enable = 0 keeps the choices made and stops tuning. */
 int crk_autotune(crk_ctx *ctx, int enable);
 
 /* The variant chosen for each pass k (CRK_PROF_NPASS entries, numbering as in

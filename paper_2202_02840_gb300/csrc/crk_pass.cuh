@@ -436,7 +436,10 @@ __device__ __forceinline__ void merge_acc(Acc<C> &d, const Acc<C> &o) {
 // longest list first in the grid).  Every variant visits each particle's list
 // in the same order, so all give bitwise identical results; the tuner times
 // each once on the first evaluation after crk_autotune(ctx, 1) and keeps the
-// fastest per pass.
+// fastest per pass.  A set below SPLIT_TILES tiles per SM has one form whatever
+// the variant: that one is timed and the default reported (TUNED_SPLIT), and the
+// first evaluation above the line still sweeps.
+enum { TUNED = 1, TUNED_SPLIT = 2 };   // crk_ctx::tune_done (0: not tuned)
 enum { ORD_GRID = 0, ORD_SM = 1, ORD_LONGEST = 2 };
 struct LVariant {
     int U, ord;
@@ -584,6 +587,13 @@ constexpr bool variant_applies(int v) {
     return P::PREFETCH ? (lvariant(v).U <= 1) : true;
 }
 
+// the time between the tuner's events
+inline int tune_time(crk_ctx *ctx, float *ms) {
+    CRK_CUDA(ctx, cudaEventSynchronize(ctx->tune_ev[1]));
+    CRK_CUDA(ctx, cudaEventElapsedTime(ms, ctx->tune_ev[0], ctx->tune_ev[1]));
+    return CRK_OK;
+}
+
 // tune_slot: the autotuner's record for this pass (default: its profiling id;
 // a pass with a different record layout, such as the two-kick P5, keeps its own)
 template <class P, int WARPS, int MINB = 1>
@@ -602,7 +612,14 @@ int launch_lpass(crk_ctx *ctx, int prof_id, const typename P::Params &prm, cudaS
     if (ctx->act) g.ntiles = ctx->nact;
     if (g.ntiles == 0) return CRK_OK;
     const bool forms = !ctx->act && !has_notune<P>::value;
-    if (forms && ctx->tune_on && !ctx->tune_done[ts]) {
+    const bool split = g.ntiles < SPLIT_TILES * nsm;   // whatever the variant: its warps would not fill the SMs
+    // long lists by CTAs (a captured step does not know whether there are any)
+    const bool heavy = !split && !ctx->act &&
+                       (ctx->graph_mode || ctx->h_counters[CNT_MAXCNT] > (unsigned long long)HEAVY_ROWS);
+    if (heavy) g.heavy = HEAVY_ROWS;
+    const bool tuning = forms && ctx->tune_on && !ctx->graph_mode && ctx->tune_done[ts] != TUNED;
+    float ms = 0.f;
+    if (tuning && !split) {
         // time every applicable variant once (each recomputes the same outputs)
         float best = 3.0e38f;
         int bestv = default_variant<P>();
@@ -616,9 +633,8 @@ int launch_lpass(crk_ctx *ctx, int prof_id, const typename P::Params &prm, cudaS
             CRK_CUDA(ctx, cudaEventRecord(ctx->tune_ev[1], s));
             ++ctx->launches;
             CRK_LAUNCH_CHECK(ctx, what);
-            CRK_CUDA(ctx, cudaEventSynchronize(ctx->tune_ev[1]));
-            float ms = 0.f;
-            CRK_CUDA(ctx, cudaEventElapsedTime(&ms, ctx->tune_ev[0], ctx->tune_ev[1]));
+            rc = tune_time(ctx, &ms);
+            if (rc) return rc;
             if (ms < best) {
                 best = ms;
                 bestv = v;
@@ -626,7 +642,7 @@ int launch_lpass(crk_ctx *ctx, int prof_id, const typename P::Params &prm, cudaS
         }
         ctx->tune_choice[ts] = bestv;
         ctx->tune_ms[ts] = best;
-        ctx->tune_done[ts] = 1;
+        ctx->tune_done[ts] = TUNED;
     }
     const int v = ctx->tune_choice[ts] >= 0 ? ctx->tune_choice[ts] : default_variant<P>();
     if (forms && !variant_applies<P>(v))   // only a variant pinned by crk_tune_set can be one the pass lacks
@@ -634,14 +650,14 @@ int launch_lpass(crk_ctx *ctx, int prof_id, const typename P::Params &prm, cudaS
     prof_begin(ctx, prof_id, s);
     rc = CRK_OK;
     constexpr int S = split_warps<P>();
-    if (g.ntiles < SPLIT_TILES * nsm) {   // whatever the variant: its warps would not fill the SMs
+    if (split) {
+        if (tuning) CRK_CUDA(ctx, cudaEventRecord(ctx->tune_ev[0], s));
         launch(s, g.ntiles, S * 32, 0, k_lpass_split<P, S, U>, g, prm, ctx->act, nullptr);
+        if (tuning) CRK_CUDA(ctx, cudaEventRecord(ctx->tune_ev[1], s));
     } else if (ctx->act) {
         launch(s, grid_for(g.ntiles, WARPS), WARPS * 32, 0, k_lpass<P, WARPS, U>, g, prm, ctx->act);
     } else {
-        // long lists first, by CTAs (a captured step does not know whether there are any)
-        if (ctx->graph_mode || ctx->h_counters[CNT_MAXCNT] > (unsigned long long)HEAVY_ROWS) {
-            g.heavy = HEAVY_ROWS;
+        if (heavy) {
             launch(s, 2 * nsm, S * 32, 0, k_lpass_split<P, S, U>, g, prm, ctx->heavy, ctx->counters + CNT_HEAVY);
             ++ctx->launches;
             CRK_LAUNCH_CHECK(ctx, what);
@@ -655,6 +671,13 @@ int launch_lpass(crk_ctx *ctx, int prof_id, const typename P::Params &prm, cudaS
     ++ctx->launches;
     prof_end(ctx, s);
     CRK_LAUNCH_CHECK(ctx, what);
+    if (tuning && split) {   // the one form such a set has; a later set above the line is still swept
+        rc = tune_time(ctx, &ms);
+        if (rc) return rc;
+        ctx->tune_choice[ts] = default_variant<P>();
+        ctx->tune_ms[ts] = ms;
+        ctx->tune_done[ts] = TUNED_SPLIT;
+    }
     return CRK_OK;
 }
 

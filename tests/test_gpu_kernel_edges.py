@@ -281,3 +281,23 @@ def test_every_pass_variant_where_it_runs():
                 crk.crk_tune_set(ctx, name, v)
         for k, (a, b) in enumerate(zip(ref, every_pass(ctx, st))):
             assert torch.equal(a, b), (v, k)
+
+
+def test_tuner_times_what_runs():
+    """Below the split line the tuner times the one form there and launches nothing
+    more; the same context then sweeps the variants on a set above it, whose
+    outputs stay those of the default."""
+    st = above_the_split_line(torch.cuda.get_device_properties(0).multi_processor_count)
+    small = inputs.uniform(15)
+    ctx, plain = crk.crk_create(), crk.crk_create()
+    crk.crk_autotune(ctx, True)
+    for a, b in zip(every_pass(ctx, small), every_pass(plain, small)):
+        assert torch.equal(a, b)
+    assert crk.crk_launches(ctx) == crk.crk_launches(plain)
+    t = crk.crk_tuning(ctx)
+    assert set(t) >= set(PASSES) and all(ms > 0 for _, ms in t.values())
+    before = crk.crk_launches(ctx), crk.crk_launches(plain)
+    for a, b in zip(every_pass(ctx, st), every_pass(plain, st)):
+        assert torch.equal(a, b)
+    swept = (crk.crk_launches(ctx) - before[0]) - (crk.crk_launches(plain) - before[1])
+    assert swept >= 5 * 7, swept   # P4 has 7 variants in the sweep, the other passes more
