@@ -375,7 +375,7 @@ __global__ void __launch_bounds__(TMA_WARPS * 32) k_p4_tma(ListGeom g, typename 
     __shared__ alignas(8) unsigned long long bar[TMA_WARPS][2];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int tile = blockIdx.x * TMA_WARPS + w;
-    if (tile >= g.ntiles || (g.heavy && (int)g.len_u[tile] > g.heavy)) return;   // the split form has the long lists
+    if (tile >= g.ntiles || (g.heavy && g.len_u[tile] > *g.heavy)) return;   // the split form has the long lists
     const uint32_t bar0 = smem_u32(&bar[w][0]), stg0 = smem_u32(&stg[w][0][0]);   // stage s: + 8 s, + TMA_STAGE s
     if (lane == 0) {
         mbar_init(bar0);

@@ -49,7 +49,8 @@ enum {
     CNT_SKIP = 23,       // this step's opening kick takes du_next
     CNT_PO_MISS = 24,    // pair-once: tile pairs (I, J) whose reverse (J, I) was not found (sticky)
     CNT_TMA_ERR = 25,    // sticky: a TMA-fed pass gave up waiting on its copies
-    CNT_COUNT = 26
+    CNT_LONG_ROWS = 26,  // rows above which the passes take a tile of the last list build for a long one
+    CNT_COUNT = 27
 };
 
 // Pass-input records in sorted order.

@@ -133,13 +133,18 @@ struct ListGeom {
     const uint32_t *len_g, *len_u;     // per-tile rows of the longest lane (multiples of LB)
     const int32_t *cnt_g, *cnt_u;
     const uint32_t *ent;
-    int heavy;                         // > 0: tiles with more pair-set rows are left to the split form
+    const unsigned long long *heavy;   // set: tiles with more pair-set rows than *heavy are left to the split form
 };
 
-// A tile with more rows than this (a typical one has 260 to 400) is shared by the
-// warps of a CTA: a warp that walks the 1000 to 2000 neighbours of a particle in
-// an evacuated region runs on alone when the others are done.
+// A tile with more rows than HEAVY_ROWS and than HEAVY_MEANS times the mean tile's
+// (CNT_LONG_ROWS) is shared by the warps of a CTA: a warp that walks the 1000 to
+// 2000 neighbours of a particle in an evacuated region runs on alone when the
+// others are done.  P1 to P5 of Sedov 64^3 after 500 steps (mean 320 entries, longest
+// 1460): no tile shared 2.96 ms, beyond 576 rows and 1.5, 2, 2.5, 3 means 2.60, 2.61,
+// 2.66, 2.89.  Where all lists are long the warps are even, and sharing every tile
+// only costs: 80^3 with 600 neighbours each 6.80 ms, 9.64 with a fixed line of 576.
 constexpr int HEAVY_ROWS = 576;
+constexpr int HEAVY_MEANS = 2;
 
 // The blocks of lists stream once from HBM (or L2, just written by the walk),
 // the longest latency of the loop, so the next block is always read ahead.
@@ -284,7 +289,7 @@ __device__ __forceinline__ void list_loop_rp(typename P::IState &st, const typen
 template <class P, int U, bool RP = false>
 __device__ __forceinline__ void lpass_tile(const ListGeom &g, const typename P::Params &prm, int tile, int lane) {
     if (pass_skipped<P>(prm)) return;   // the sums were formed by an earlier pass
-    if (g.heavy && (int)g.len_u[tile] > g.heavy) return;
+    if (g.heavy && g.len_u[tile] > *g.heavy) return;
     const int i = tile * TILE + lane;
     const bool valid = i < g.n;
     typename P::IState st;
@@ -391,6 +396,7 @@ __global__ void __launch_bounds__(S * 32) k_lpass_split(ListGeom g, typename P::
     const int end = count ? (int)*count : (int)blockIdx.x + 1;
     for (int t = blockIdx.x; t < end; t += gridDim.x) {
         const int tile = order ? order[t] : t;
+        if (g.heavy && g.len_u[tile] <= *g.heavy) continue;
         const int i = tile * TILE + lane;
         const bool valid = i < g.n;
         typename P::IState st;
@@ -603,7 +609,7 @@ int launch_lpass(crk_ctx *ctx, int prof_id, const typename P::Params &prm, cudaS
     if (ctx->n == 0) return CRK_OK;
     if (!ctx->lists_valid) return crk_set_error(ctx, CRK_ESTATE, "%s: neighbour lists are not built", what);
     ListGeom g{ctx->n,   ctx->ntiles, ctx->kcap,  ctx->tbase, ctx->len_g,
-               ctx->len_u, ctx->cnt_g, ctx->cnt_u, ctx->ent,  0};
+               ctx->len_u, ctx->cnt_g, ctx->cnt_u, ctx->ent,  nullptr};
     int rc;
     const int nsm = ctx->nsm > 0 ? ctx->nsm : 152;
     constexpr int U = P::PREFETCH ? 1 : P::UNROLL;
@@ -615,8 +621,8 @@ int launch_lpass(crk_ctx *ctx, int prof_id, const typename P::Params &prm, cudaS
     const bool split = g.ntiles < SPLIT_TILES * nsm;   // whatever the variant: its warps would not fill the SMs
     // long lists by CTAs (a captured step does not know whether there are any)
     const bool heavy = !split && !ctx->act &&
-                       (ctx->graph_mode || ctx->h_counters[CNT_MAXCNT] > (unsigned long long)HEAVY_ROWS);
-    if (heavy) g.heavy = HEAVY_ROWS;
+                       (ctx->graph_mode || ctx->h_counters[CNT_MAXCNT] > ctx->h_counters[CNT_LONG_ROWS]);
+    if (heavy) g.heavy = ctx->counters + CNT_LONG_ROWS;
     const bool tuning = forms && ctx->tune_on && !ctx->graph_mode && ctx->tune_done[ts] != TUNED;
     float ms = 0.f;
     if (tuning && !split) {

@@ -36,7 +36,7 @@ struct WalkArgs {
     const int32_t *sbox;     // batched boxes: box of each slot (BATCH only)
     const uint32_t *nbox;    // box range of each tile (BATCH only)
     const int32_t *act;      // may be null: walk the tiles act[0 .. ntiles) only
-    int32_t *long_list;      // tiles with more than HEAVY_ROWS rows, and their count
+    int32_t *long_list;      // tiles with more than HEAVY_ROWS rows (the passes take the long ones), and their count
     unsigned long long *nlong;
     int heavy;               // tiles with more candidate tiles than this are shared by the warps of a CTA
     int hblocks;             // CTAs that take them (all: one per tile, every tile is shared)
@@ -544,11 +544,15 @@ __global__ void __launch_bounds__(W * 32, 32 / W) k_walk(WalkArgs a) {
     }
 }
 
-// total stored-force units (32 entries each) = base[last] + len_u[last]
+// total stored-force units (32 entries each) = base[last] + len_u[last], and the
+// rows above which a tile's list is a long one
 __global__ void k_total(int ntiles, const uint32_t *__restrict__ base, const uint32_t *__restrict__ len,
-                        unsigned long long *out) {
+                        unsigned long long *counters) {
     grid_wait();
-    *out = ntiles ? (unsigned long long)base[ntiles - 1] + len[ntiles - 1] : 0ull;
+    const unsigned long long total = (unsigned long long)base[ntiles - 1] + len[ntiles - 1];
+    counters[CNT_ENTRIES] = total;
+    counters[CNT_LONG_ROWS] =
+        max((unsigned long long)HEAVY_ROWS, HEAVY_MEANS * total / (unsigned long long)ntiles);
 }
 
 static WalkArgs walk_args(crk_ctx *ctx) {
@@ -650,7 +654,7 @@ int run_lists(crk_ctx *ctx, cudaStream_t s) {
         if (rc) return rc;
         rc = scan_u32(ctx, ctx->len_u, ctx->tbase, nt, s);
         if (rc) return rc;
-        launch(s, 1, 1, 0, k_total, nt, ctx->tbase, ctx->len_u, ctx->counters + CNT_ENTRIES);
+        launch(s, 1, 1, 0, k_total, nt, ctx->tbase, ctx->len_u, ctx->counters);
         ++ctx->launches;
         CRK_LAUNCH_CHECK(ctx, "list layout");
         if (ctx->graph_mode) {   // captured step: capacities were fixed beforehand, overflow checked after

@@ -301,3 +301,22 @@ def test_tuner_times_what_runs():
         assert torch.equal(a, b)
     swept = (crk.crk_launches(ctx) - before[0]) - (crk.crk_launches(plain) - before[1])
     assert swept >= 5 * 7, swept   # P4 has 7 variants in the sweep, the other passes more
+
+
+@pytest.mark.parametrize("far, extra", [(1.0, 0), (1.3, 0), (1.55, 1)])
+def test_long_lists_are_those_longer_than_most(far, extra):
+    """A tile's list is long for its set: with 270 or with 600 neighbours everywhere
+    P1 is one kernel; with 270 and a few of 1000 it is one more, for their tiles."""
+    st = above_the_split_line(torch.cuda.get_device_properties(0).multi_processor_count)
+    h = st["pos_h"][:, 3]
+    h[h > 1.1 * h.min()] = h.min() * (far if extra else 1.0)
+    if not extra:
+        h *= np.float32(far)
+    ctx = crk.crk_create()
+    crk.crk_build_cells(ctx, dev(st["pos_h"]))
+    V = as_np(crk.crk_volumes(ctx)[0])
+    before = crk.crk_launches(ctx)
+    crk.crk_volumes(ctx)
+    assert crk.crk_launches(ctx) - before == 2 + extra   # the pass and the copy out
+    tg = np.unique(np.concatenate([np.argsort(h)[-8:], np.arange(0, len(h), 9973)])).astype(np.int32)
+    assert rel_err(V[tg], O.volumes(st["pos_h"], targets=tg)["V"][tg]) < TOL
