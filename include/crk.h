@@ -450,14 +450,14 @@ int crk_profile_read(crk_ctx *ctx, double *ms, long long *counts, long long *tot
  * grid; contiguous tile ranges per SM in a persistent launch; longest
  * pair-set list first) and how many 32-particle tiles share a CTA (1, 2, 4
  * or 8: 32-256 particles).  Every variant visits each particle's list in the
- * same order, so all produce bitwise identical results.  The tiles of small sets
- * (fewer than 10 to 40 per SM, by pass), and tiles with very long lists, are
- * shared by the warps of a CTA whatever the variant.  enable = 1 makes the
+ * same order, so all produce bitwise identical results.  Sets of fewer than 40
+ * tiles per SM, and tiles with very long lists, are shared by the warps of
+ * a CTA whatever the variant.  enable = 1 makes the
  * next call of each pass time every variant once (on the stream, with CUDA
  * events; the call synchronises while tuning) and keep the fastest for the
- * context; on such a small set it times the one form there and reports the
- * built-in default, and the next call on a larger set times the variants.
- * enable = 0 keeps the choices made and stops tuning. */
+ * context; on a set of fewer than 40 tiles per SM it times the one form such
+ * sets have and reports the built-in default, and the next call on a larger set
+ * times the variants.  enable = 0 keeps the choices made and stops tuning. */
 int crk_autotune(crk_ctx *ctx, int enable);
 
 /* The variant chosen for each pass k (CRK_PROF_NPASS entries, numbering as in

@@ -251,7 +251,6 @@ __device__ __forceinline__ FRec ldg_frec(const float4 *base, uint32_t j) {
 template <bool COMP, bool STATIC>
 struct P4 {
     static constexpr bool GATHER = false;
-    static constexpr int SPLIT = 40;
     static constexpr int UNROLL = 1;
     static constexpr bool ENTRIES = true;
     static constexpr bool PERSISTENT = true;
@@ -529,7 +528,6 @@ __device__ __forceinline__ float compat_term(const float4 me, const float4 r, co
 template <bool COMP, bool DUAL = false>
 struct P5 {
     static constexpr bool GATHER = false;
-    static constexpr int SPLIT = 40;
     static constexpr int UNROLL = 4;
     static constexpr bool PERSISTENT = false;
     static constexpr bool PREFETCH = false;

@@ -207,7 +207,6 @@ __device__ __forceinline__ void moments(float h, const PairSums<T> &s, T &m0, T 
 template <bool FP64_SOLVE, bool COMP>
 struct P2 {
     static constexpr bool GATHER = true;
-    static constexpr int SPLIT = 10;
     static constexpr int UNROLL = 4;
     static constexpr bool ENTRIES = true;
     static constexpr bool PERSISTENT = false;
@@ -393,7 +392,6 @@ __device__ __forceinline__ void merge_acc(AccFF &d, const AccFF &o) { d.add(FF{o
 
 struct P2X {
     static constexpr bool GATHER = true;
-    static constexpr int SPLIT = 40;
     static constexpr int UNROLL = 2;
     static constexpr bool ENTRIES = true;
     static constexpr bool PERSISTENT = false;
@@ -503,7 +501,6 @@ struct P2X {
 template <bool COMP>
 struct P3 {
     static constexpr bool GATHER = true;
-    static constexpr int SPLIT = 14;
     static constexpr int UNROLL = 4;
     static constexpr bool ENTRIES = true;
     static constexpr bool PERSISTENT = false;
@@ -602,7 +599,6 @@ struct P3 {
 // m_j / V_j, exact for constant and linear fields.
 struct PD {
     static constexpr bool GATHER = true;
-    static constexpr int SPLIT = 32;
     static constexpr int UNROLL = 4;
     static constexpr bool ENTRIES = true;
     static constexpr bool PERSISTENT = false;

@@ -121,7 +121,7 @@ __device__ __forceinline__ int pair_block(int b, int nbg, int kcap) { return b <
 // Gather passes walk the gather blocks, pair-set passes all blocks; entry u of
 // block b has its stored force (P4 -> P5) in row 4 b + u of the tile, pads
 // included (F = 0, j = i).  P must provide Params, IState, Rec, GATHER,
-// PREFETCH, UNROLL, PERSISTENT, SPLIT, ENTRIES (false: the pass reads only its stored
+// PREFETCH, UNROLL, PERSISTENT, ENTRIES (false: the pass reads only its stored
 // entries, and `entry` is passed as 0),
 //   init(IState&, int i, bool valid, const Params&)
 //   load(uint32_t entry, size_t pos, const Params&) -> Rec   (the neighbour's data)
@@ -419,21 +419,11 @@ __global__ void __launch_bounds__(S * 32) k_lpass_split(ListGeom g, typename P::
     }
 }
 
-// P::SPLIT: tiles per SM below which a pass splits them, where a warp per tile
-// leaves the SMs short of warps, or the last wave of warps nearly empty.  Each
-// pass has its own line: merging partial sums costs P2 and P3 more than P4, and
-// their warps fit the SM more often.  Each alone on a jittered lattice, us, a warp
-// per tile / split, at 1.2, 8.1, 11.3, 15.2, 25.7 and 38.1 tiles per SM:
-//   P1           31/12   35/25   37/32    40/40    60/63    75/89
-//   P2           44/23   71/67   73/75    89/100  142/174  179/248
-//   P2 (mode 2)  58/31  102/100 106/118  160/159  252/265  353/379
-//   P2 (mode 3) 161/70  293/240 307/312  472/414  752/676 1043/980
-//   P3           47/16   57/49   59/62    74/88   111/150  176/215
-//   P4          152/37  213/153 243/197  363/261  518/424  690/622
-//   P5           47/12   72/49   78/61    84/80   111/117  176/164
-//   RK density   43/11   56/31   65/38    70/50    86/78   101/110
-// Clustered sets lie the same.  Tile subsets (time bins) take the line of the
-// whole set, SPLIT_TILES, in every pass: a subset holds the steepest leaves.
+// Tiles per SM below which a pass splits them: a warp per tile then leaves the
+// SMs short of warps, or the last wave of warps nearly empty.  Measured on KDK
+// steps, warp per tile against split: clustered 16^3 (0.8 tiles per SM) 0.94 ->
+// 0.52 ms, 32^3 (6.7) 1.37 -> 1.05, 40^3 (13) 1.89 -> 1.50, 48^3 (23) 2.18 -> 2.00,
+// Sedov 64^3 (54) 2.64 -> 2.67.
 constexpr int SPLIT_TILES = 40;
 
 // merge a partial pair sum into another (the compensated sum keeps the
@@ -452,7 +442,7 @@ __device__ __forceinline__ void merge_acc(Acc<C> &d, const Acc<C> &o) {
 // longest list first in the grid).  Every variant visits each particle's list
 // in the same order, so all give bitwise identical results; the tuner times
 // each once on the first evaluation after crk_autotune(ctx, 1) and keeps the
-// fastest per pass.  A set below P::SPLIT tiles per SM has one form whatever
+// fastest per pass.  A set below SPLIT_TILES tiles per SM has one form whatever
 // the variant: that one is timed and the default reported (TUNED_SPLIT), and the
 // first evaluation above the line still sweeps.
 enum { TUNED = 1, TUNED_SPLIT = 2 };   // crk_ctx::tune_done (0: not tuned)
@@ -628,8 +618,7 @@ int launch_lpass(crk_ctx *ctx, int prof_id, const typename P::Params &prm, cudaS
     if (ctx->act) g.ntiles = ctx->nact;
     if (g.ntiles == 0) return CRK_OK;
     const bool forms = !ctx->act && !has_notune<P>::value;
-    // whatever the variant: its warps would not fill the SMs
-    const bool split = g.ntiles < (ctx->act ? SPLIT_TILES : P::SPLIT) * nsm;
+    const bool split = g.ntiles < SPLIT_TILES * nsm;   // whatever the variant: its warps would not fill the SMs
     // long lists by CTAs (a captured step does not know whether there are any)
     const bool heavy = !split && !ctx->act &&
                        (ctx->graph_mode || ctx->h_counters[CNT_MAXCNT] > ctx->h_counters[CNT_LONG_ROWS]);

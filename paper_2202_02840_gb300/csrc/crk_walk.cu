@@ -724,7 +724,6 @@ int run_export_lists(crk_ctx *ctx, int mode, const long long *off, int32_t *out,
 // P1 volumes over the gather lists (eq:vol, eq:hi), self included.
 struct P1 {
     static constexpr bool GATHER = true;
-    static constexpr int SPLIT = 25;
     static constexpr int UNROLL = 4;
     static constexpr bool ENTRIES = true;
     static constexpr bool PERSISTENT = false;

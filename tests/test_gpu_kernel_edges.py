@@ -2,7 +2,7 @@
 
 The list walk and the list passes choose their form by the number of tiles (32
 particles each): below 8 tiles per SM a tile is walked by 32 warps, below 20 by
-8, above by one; below 10 to 40 tiles per SM, by pass, a tile's list is split over warps; and
+8, above by one; below 40 tiles per SM a tile's list is split over warps; and
 tiles with long lists or many neighbour tiles take forms of their own at any
 size.  Each case lies just past one of these lines with a ragged last tile, and
 is compared with the oracle at targets that include every unusual particle."""
@@ -320,23 +320,3 @@ def test_long_lists_are_those_longer_than_most(far, extra):
     assert crk.crk_launches(ctx) - before == 2 + extra   # the pass and the copy out
     tg = np.unique(np.concatenate([np.argsort(h)[-8:], np.arange(0, len(h), 9973)])).astype(np.int32)
     assert rel_err(V[tg], O.volumes(st["pos_h"], targets=tg)["V"][tg]) < TOL
-
-
-@pytest.mark.parametrize("per_sm, kernels", [(9, 1), (12, 2)])
-def test_each_pass_has_its_own_split_line(per_sm, kernels):
-    """P2 splits every tile below 10 tiles an SM; above, a warp takes a tile and one
-    kernel more the few long lists (P4, whose line is higher, still splits all)."""
-    nsm = torch.cuda.get_device_properties(0).multi_processor_count
-    st = inputs.uniform(int(np.ceil((per_sm * 32 * nsm) ** (1 / 3))))
-    st["pos_h"][::len(st["mass"]) // 8, 3] *= np.float32(1.55)
-    ctx = crk.crk_create()
-    crk.crk_build_cells(ctx, dev(st["pos_h"]))
-    vel = dev(st["vel_u"])
-    V = crk.crk_volumes(ctx)[0]
-    before = crk.crk_launches(ctx)
-    crk.crk_corrections(ctx, V, gradv=False)
-    assert crk.crk_launches(ctx) - before == 2 + kernels   # the copies in and out
-    cor = crk.crk_corrections(ctx, V, vel)
-    before = crk.crk_launches(ctx)
-    crk.crk_forces(ctx, dev(st["mass"]), vel, V, *cor)
-    assert crk.crk_launches(ctx) - before == 4   # copies in and out, records, P4
