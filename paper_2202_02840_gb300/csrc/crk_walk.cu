@@ -552,7 +552,7 @@ __global__ void k_total(int ntiles, const uint32_t *__restrict__ base, const uin
     const unsigned long long total = (unsigned long long)base[ntiles - 1] + len[ntiles - 1];
     counters[CNT_ENTRIES] = total;
     counters[CNT_LONG_ROWS] =
-        max((unsigned long long)HEAVY_ROWS, HEAVY_MEANS * total / (unsigned long long)ntiles);
+        max((unsigned long long)HEAVY_ROWS, 3ull * total / (2ull * (unsigned long long)ntiles));
 }
 
 static WalkArgs walk_args(crk_ctx *ctx) {
