@@ -231,6 +231,7 @@ struct crk_ctx {
     long long glaunch[2] = {0, 0};   // kernels in each graph
     long long gcaptures = 0, greplays = 0, grecoveries = 0;
     unsigned long long gkey[2] = {0, 0};   // fingerprint of what each graph captured
+    unsigned long long gcall = 0;    // fingerprint of the call they were captured for (its arguments)
     float4 *bk_pos = nullptr, *bk_vel = nullptr;   // state before a run of replayed steps
     int cap_bk = 0;
     unsigned long long alloc_gen = 0;   // bumped by every device (re)allocation

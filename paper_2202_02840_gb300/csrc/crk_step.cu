@@ -838,6 +838,13 @@ static bool capture_step(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const 
 static int steps_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const float *mass, int nsteps, double dt,
                       int use_graph, bool batched, cudaStream_t s) {
     int rc, done = 0;
+    unsigned long long call = 1469598103934665603ull;   // the arguments a captured graph holds
+    unsigned long long dtbits;
+    memcpy(&dtbits, &dt, sizeof(dtbits));
+    for (unsigned long long v :
+         {(unsigned long long)n, (unsigned long long)(uintptr_t)pos_h, (unsigned long long)(uintptr_t)vel_u,
+          (unsigned long long)(uintptr_t)mass, dtbits, (unsigned long long)batched * 7919ull + (unsigned long long)ctx->nbox})
+        call = fnv(call, v);
     // eager steps: without graphs, from a fresh state (its first step sizes
     // every buffer a captured step uses) and while the passes are being tuned
     for (;;) {
@@ -858,10 +865,10 @@ static int steps_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const flo
         // headroom for the replayed steps: list columns (they change only at a
         // walk, so one more eager step applies the new width) and tile-pair lists.
         // 50% of the last step's needs before the first capture; graphs that are
-        // there are kept while 25% is left (a run that calls this every few steps
-        // with slowly growing counts would otherwise widen the columns, copy the
-        // stored forces and capture anew in every call)
-        const bool have = ctx->gexec[0] || ctx->gexec[1];
+        // there, captured for these arguments, are kept while 25% is left (a run
+        // that calls this every few steps with slowly growing counts would otherwise
+        // widen the columns, copy the stored forces and capture anew in every call)
+        const bool have = (ctx->gexec[0] || ctx->gexec[1]) && ctx->gcall == call;
         rc = crk_sync_counters(ctx, s);
         if (rc) return rc;
         const long long maxc = (long long)ctx->h_counters[CNT_MAXCNT];
@@ -914,20 +921,16 @@ static int steps_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const flo
         for (int k = done; k < nsteps; k++) {
             // which of the two buffer rotations the state is in
             const int p = (uintptr_t)ctx->st_pos < (uintptr_t)ctx->st_tmp ? 0 : 1;
-            unsigned long long key = 1469598103934665603ull;
-            unsigned long long dtbits;
-            memcpy(&dtbits, &dt, sizeof(dtbits));
-            const unsigned long long parts[] = {
-                (unsigned long long)n, (unsigned long long)(uintptr_t)pos_h, (unsigned long long)(uintptr_t)vel_u,
-                (unsigned long long)(uintptr_t)mass, ctx->alloc_gen, (unsigned long long)ctx->kcap,
-                (unsigned long long)ctx->cap_ulist, (unsigned long long)(uintptr_t)ctx->st_pos, dtbits,
-                (unsigned long long)batched * 7919ull + (unsigned long long)ctx->nbox};
-            for (unsigned long long v : parts) key = fnv(key, v);
+            unsigned long long key = call;
+            for (unsigned long long v : {ctx->alloc_gen, (unsigned long long)ctx->kcap, (unsigned long long)ctx->cap_ulist,
+                                         (unsigned long long)(uintptr_t)ctx->st_pos})
+                key = fnv(key, v);
             const int tuned[] = {PROF_P1, PROF_P2, PROF_P3, PROF_P4, PROF_P5, TUNE_P5_DUAL, PROF_DENS};
             for (int t : tuned) key = fnv(key, (unsigned long long)(long long)ctx->tune_choice[t]);
             if (!eager && (!ctx->gexec[p] || ctx->gkey[p] != key)) {
                 // capturing runs the step's host logic (its buffer rotation) but not its kernels
                 if (!capture_step(ctx, n, pos_h, vel_u, mass, dt, p, key, batched)) eager = true;
+                ctx->gcall = call;
             } else if (!eager) {
                 swap_state(ctx);
             }
