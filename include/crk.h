@@ -291,7 +291,8 @@ int crk_step(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const float *mass,
  * first capture the call gives the neighbour-list columns and the tile-pair
  * lists 50% headroom over the last step's needs (one more eager step applies a
  * new column width; graphs captured for the same arguments are kept while 25% is
- * left) and the stored forces their worst case; each replayed step
+ * left, and then the columns get 100% where memory allows) and the stored
+ * forces their worst case; each replayed step
  * records whether a capacity was exceeded anyway.  If one was, the call
  * restores the positions and velocities its replays started from and redoes
  * those steps eagerly, the first of them evaluating the rates afresh at the

@@ -731,6 +731,15 @@ unsigned long long fnv(unsigned long long h, unsigned long long v) {
     return h;
 }
 
+// The list columns and the worst case of the stored forces at `cols` columns, beside
+// the present ones, take no more than half of the free memory and an eighth of the card.
+bool columns_fit(const crk_ctx *ctx, long long cols) {
+    size_t left = 0, total = 0;
+    if (cudaMemGetInfo(&left, &total) != cudaSuccess) return false;
+    const double need = 32.0 * ctx->ntiles * ((double)cols + 31.0) * (sizeof(uint32_t) + sizeof(float4));
+    return need < 0.5 * (double)left && need < (double)total / 8.0;
+}
+
 void drop_graphs(crk_ctx *ctx) {
     for (int k = 0; k < 2; k++) {
         if (ctx->gexec[k]) cudaGraphExecDestroy(ctx->gexec[k]);
@@ -874,9 +883,8 @@ static int steps_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const flo
         const long long maxc = (long long)ctx->h_counters[CNT_MAXCNT];
         const long long nu = (long long)ctx->h_counters[CNT_ULIST];
         if (maxc + maxc / (have ? 4 : 2) > ctx->kcap && done < nsteps) {
-            // a second widening means growing counts: twice the need, while the
-            // worst case of the stored forces stays below 32 GB
-            const bool twice = have && (double)ctx->ntiles * (2.0 * maxc) * 512.0 < 32e9;
+            // a second widening means growing counts: twice the need, where there is room
+            const bool twice = have && columns_fit(ctx, 2 * maxc);
             ctx->kcap = (int)((maxc + (twice ? maxc : maxc / 2) + 31) / 32 * 32);
             rc = step_impl(ctx, n, pos_h, vel_u, mass, dt, nullptr, batched, s);
             if (rc) return rc;

@@ -341,3 +341,23 @@ def test_each_run_of_replays_starts_with_its_headroom():
         crk.crk_steps(ctx, *still_lattice(16, 4.2), 6)
         replays.append(crk.crk_graph_stats(ctx)[1] - r)
     assert replays == [4, 4], replays
+
+
+def test_wider_columns_look_at_free_memory():
+    """A second widening doubles the columns only where that fits: at 64^3 from 480
+    columns to 704 (3.7 GB with the forces, 0.5 of them given back), not to 928 (4.9), with
+    3.3 GB left."""
+    pos, vel, mass = still_lattice(64, 4.2)
+    ctx = crk.crk_create()
+    crk.crk_steps(ctx, pos, vel, mass, 4)
+    pos[:, 3] = 4.7 / 64
+    crk.crk_reset_rates(ctx)
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    rest = torch.empty(torch.cuda.mem_get_info()[0] - int(3.3e9), dtype=torch.uint8, device="cuda")
+    try:
+        crk.crk_steps(ctx, pos, vel, mass, 4)
+    finally:
+        del rest
+        torch.cuda.empty_cache()
+    assert torch.isfinite(pos).all()
