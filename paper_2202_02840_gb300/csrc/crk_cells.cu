@@ -546,9 +546,9 @@ static int rcb_refine(crk_ctx *ctx, int n, cudaStream_t s) {
     for (int L = 0; L < levels; L++) {
         const int nseg = 1 << L;
         launch(s, grid_for(3ll * nseg, 256), 256, 0, k_fill_u32, 3ll * nseg, 0xffffffffu, ctx->rcb_lo);
-        zero_async(ctx, ctx->rcb_hi, sizeof(uint32_t) * 3 * (size_t)nseg, s);
-        zero_async(ctx, ctx->rcb_size, sizeof(int32_t) * (size_t)nseg, s);
-        zero_async(ctx, ctx->rcb_hist, sizeof(uint32_t) * RCB_BINS * (size_t)nseg, s);
+        CRK_TRY(zero_async(ctx, ctx->rcb_hi, sizeof(uint32_t) * 3 * (size_t)nseg, s));
+        CRK_TRY(zero_async(ctx, ctx->rcb_size, sizeof(int32_t) * (size_t)nseg, s));
+        CRK_TRY(zero_async(ctx, ctx->rcb_hist, sizeof(uint32_t) * RCB_BINS * (size_t)nseg, s));
         launch(s, g, 256, 0, k_rcb_box, n, L, leaf, cur, ctx->q_tmp, ctx->rcb_a, ctx->rcb_id, ctx->rcb_lo,
                ctx->rcb_hi, ctx->rcb_size);
         launch(s, g, 256, 0, k_rcb_hist, n, cur, ctx->q_tmp, ctx->rcb_id, ctx->rcb_lo, ctx->rcb_hi, ctx->rcb_bin,
@@ -566,7 +566,7 @@ static int rcb_refine(crk_ctx *ctx, int n, cudaStream_t s) {
         int32_t *t = cur; cur = nxt; nxt = t;
     }
     if (cur != ctx->idx_a)
-        copy_async(ctx, ctx->idx_a, cur, sizeof(int32_t) * n, s);
+        CRK_TRY(copy_async(ctx, ctx->idx_a, cur, sizeof(int32_t) * n, s));
     return CRK_OK;
 }
 
@@ -944,7 +944,7 @@ int rebuild_lists(crk_ctx *ctx, cudaStream_t s) {
     if (ctx->ntiles == 0) return CRK_OK;
     Tree32 T = tree32(ctx);
     if (T.cnt[T.top] > 32) return crk_set_error(ctx, CRK_ECAPACITY, "tile tree too deep");
-    zero_async(ctx, ctx->counters + CNT_GLIST, 3 * sizeof(unsigned long long), s);
+    CRK_TRY(zero_async(ctx, ctx->counters + CNT_GLIST, 3 * sizeof(unsigned long long), s));
     ctx->lists_valid = 0;
     const int count = ctx->act ? ctx->nact : ctx->ntiles;
     if (count == 0) return CRK_OK;
@@ -1015,7 +1015,7 @@ int build_cells_sorted(crk_ctx *ctx, int n, const float4 *pos, const int32_t *ba
     }
     ctx->nlevels = L;
     ctx->built = 0;
-    zero_async(ctx, ctx->counters + CNT_ERR_INPUT, 2 * sizeof(unsigned long long), s);
+    CRK_TRY(zero_async(ctx, ctx->counters + CNT_ERR_INPUT, 2 * sizeof(unsigned long long), s));
     if (n == 0) {
         ctx->built = 1;
         return CRK_OK;
@@ -1035,7 +1035,7 @@ int build_cells_sorted(crk_ctx *ctx, int n, const float4 *pos, const int32_t *ba
     if (box_of_input) {
         // batched boxes: stable sort by Morton key, then stable sort by box,
         // which leaves the order box-major and Morton within each box
-        copy_async(ctx, ctx->mkey, key0, sizeof(uint32_t) * n, s);
+        CRK_TRY(copy_async(ctx, ctx->mkey, key0, sizeof(uint32_t) * n, s));
         rc = radix_sort30(ctx, n, s);
         if (rc) return rc;
         launch(s, grid_for(n, 256), 256, 0, k_gather_u32, n, ctx->idx_a,
@@ -1043,7 +1043,7 @@ int build_cells_sorted(crk_ctx *ctx, int n, const float4 *pos, const int32_t *ba
         ++ctx->launches;
         rc = radix_sort16(ctx, n, s);
         if (rc) return rc;
-        copy_async(ctx, ctx->sbox, ctx->key_a, sizeof(int32_t) * n, s);
+        CRK_TRY(copy_async(ctx, ctx->sbox, ctx->key_a, sizeof(int32_t) * n, s));
         launch(s, grid_for(n, 256), 256, 0, k_gather_u32, n, ctx->idx_a, ctx->mkey, ctx->keys);
         ++ctx->launches;
         CRK_LAUNCH_CHECK(ctx, "box sort");
@@ -1063,7 +1063,7 @@ int build_cells_sorted(crk_ctx *ctx, int n, const float4 *pos, const int32_t *ba
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "gather sorted");
     if (perm != ctx->perm)
-        copy_async(ctx, ctx->perm, perm, sizeof(int32_t) * n, s);
+        CRK_TRY(copy_async(ctx, ctx->perm, perm, sizeof(int32_t) * n, s));
     if (!box_of_input && ctx->p.tile_order == 0) {   // the chaining-mesh table: one box, Morton order
         launch(s, grid_for(n + 1, 256), 256, 0, k_cell_start, n, ctx->keys, ctx->p.kmax, ctx->counters,
                ctx->cell_start);
@@ -1103,7 +1103,7 @@ int tile_order_by_length(crk_ctx *ctx, cudaStream_t s) {
     ++ctx->launches;
     int rc = radix_sort16(ctx, nt, s);
     if (rc) return rc;
-    copy_async(ctx, ctx->tile_order, ctx->idx_a, sizeof(int32_t) * (size_t)nt, s);
+    CRK_TRY(copy_async(ctx, ctx->tile_order, ctx->idx_a, sizeof(int32_t) * (size_t)nt, s));
     CRK_LAUNCH_CHECK(ctx, "tile order");
     return CRK_OK;
 }

@@ -390,8 +390,8 @@ namespace crk {
 // Zeros and device copies by kernels: a memset or copy between two kernels takes
 // 3.4 us of the stream, as it can neither start nor end under a neighbour, a
 // small kernel 1.3.
-void copy_async(crk_ctx *ctx, void *to, const void *from, size_t bytes, cudaStream_t s) {
-    if (bytes < 4) return;
+int copy_async(crk_ctx *ctx, void *to, const void *from, size_t bytes, cudaStream_t s) {
+    if (bytes < 4) return CRK_OK;
     const bool wide = (((uintptr_t)to | (uintptr_t)from | bytes) & 15) == 0;
     const long long count = (long long)(bytes / (wide ? 16 : 4));
     const long long want = (count + 255) / 256;
@@ -401,14 +401,18 @@ void copy_async(crk_ctx *ctx, void *to, const void *from, size_t bytes, cudaStre
     else
         launch(s, g, 256, 0, k_copy<uint32_t>, count, (uint32_t *)to, (const uint32_t *)from);
     ++ctx->launches;
+    CRK_LAUNCH_CHECK(ctx, "device copy");
+    return CRK_OK;
 }
 
-void zero_async(crk_ctx *ctx, void *p, size_t bytes, cudaStream_t s) {
+int zero_async(crk_ctx *ctx, void *p, size_t bytes, cudaStream_t s) {
     const long long words = (long long)(bytes / 4);
-    if (words == 0) return;
+    if (words == 0) return CRK_OK;
     const long long want = (words + 255) / 256;
     launch(s, want < 16384 ? (int)want : 16384, 256, 0, k_zero, words, (uint32_t *)p);
     ++ctx->launches;
+    CRK_LAUNCH_CHECK(ctx, "zeros");
+    return CRK_OK;
 }
 
 static int move_rows(crk_ctx *ctx, bool gather, std::initializer_list<Rows> rows, cudaStream_t s, const char *what) {
@@ -788,7 +792,7 @@ extern "C" int crk_cells(crk_ctx *ctx, uint32_t *keys, int32_t *perm, int32_t *c
         if (ctx->n)
             CRK_CUDA(ctx, cudaMemcpyAsync(cell_start, ctx->cell_start, 4 * cnt, cudaMemcpyDeviceToDevice, s));
         else
-            zero_async(ctx, cell_start, 4 * cnt, s);
+            CRK_TRY(zero_async(ctx, cell_start, 4 * cnt, s));
     }
     CRK_CUDA(ctx, cudaStreamSynchronize(s));
     return CRK_OK;

@@ -491,7 +491,7 @@ int flagged_tiles(crk_ctx *ctx, cudaStream_t s) {
         launch(s, 1, 1024, 0, k_compact_tiles<FlaggedTiles>, nt, ctx->n, FlaggedTiles{ctx->tflag}, ctx->tact,
                ctx->counters);
     } else {
-        zero_async(ctx, ctx->counters + CNT_NACT, 2 * sizeof(unsigned long long), s);
+        CRK_TRY(zero_async(ctx, ctx->counters + CNT_NACT, 2 * sizeof(unsigned long long), s));
         int rc = scan_u32(ctx, ctx->tflag, ctx->tscan, nt, s);
         if (rc) return rc;
         launch(s, grid_for(nt, 256), 256, 0, k_htb_compact, nt, ctx->n, ctx->tflag, ctx->tscan, ctx->tact,
@@ -544,7 +544,7 @@ static int limit(crk_ctx *ctx, const int32_t *act, int count, int f_l, int L, cu
     if (count == 0) return CRK_OK;
     const long long cap = (long long)ctx->ntiles * (L + 1) + 2;
     for (long long it = 0; it < cap; it += 4) {
-        zero_async(ctx, ctx->counters + CNT_CHANGED, sizeof(unsigned long long), s);
+        CRK_TRY(zero_async(ctx, ctx->counters + CNT_CHANGED, sizeof(unsigned long long), s));
         for (int k = 0; k < 4; k++) {
             launch(s, grid_for((long long)count * 32, 256), 256, 0, k_htb_limit, count, act, ctx->uofs, ctx->ulist,
                    f_l, ctx->tlev, ctx->counters + CNT_CHANGED);
@@ -611,7 +611,7 @@ static int cycle_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const flo
         if (!rc) rc = finish_build(ctx, s);
         if (!rc) rc = gather_rows(ctx, {{pos_h, ctx->st_pos, 4}, {vel_u, ctx->st_vel, 4}, {mass, ctx->mass, 1}}, s);
         if (rc) return rc;
-        copy_async(ctx, ctx->vel, ctx->st_vel, sizeof(float4) * n, s);
+        CRK_TRY(copy_async(ctx, ctx->vel, ctx->st_vel, sizeof(float4) * n, s));
         rc = evaluate(ctx, s);
         if (rc) return rc;
         ctx->rates_valid = 1;
@@ -631,7 +631,7 @@ static int cycle_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const flo
     rc = refit_lists(ctx, s);
     if (rc) return rc;
     // levels at the cycle start: requirement, then the limiter's fixed point
-    zero_async(ctx, ctx->counters + CNT_UNRES, 2 * sizeof(unsigned long long), s);
+    CRK_TRY(zero_async(ctx, ctx->counters + CNT_UNRES, 2 * sizeof(unsigned long long), s));
     launch(s, grid_for((long long)nt * 32, 256), 256, 0, k_htb_req, nt, nullptr, n, ctx->d_dt, c, 0, 0, ctx->tlev,
            ctx->counters);
     ++ctx->launches;
@@ -647,11 +647,11 @@ static int cycle_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const flo
         st->leaves = nt;
     }
     // every leaf opens its first step at tick 0 (t0 = len = 0 marks it active)
-    zero_async(ctx, ctx->tt0, sizeof(int32_t) * nt, s);
-    zero_async(ctx, ctx->tlen, sizeof(int32_t) * nt, s);
+    CRK_TRY(zero_async(ctx, ctx->tt0, sizeof(int32_t) * nt, s));
+    CRK_TRY(zero_async(ctx, ctx->tlen, sizeof(int32_t) * nt, s));
     std::vector<int32_t> none(nt, NO_LEVEL);
     CRK_CUDA(ctx, cudaMemcpyAsync(ctx->twake, none.data(), sizeof(int32_t) * nt, cudaMemcpyHostToDevice, s));
-    copy_async(ctx, ctx->st_half, ctx->st_vel, sizeof(float4) * n, s);
+    CRK_TRY(copy_async(ctx, ctx->st_half, ctx->st_vel, sizeof(float4) * n, s));
     launch(s, g, b, 0, k_htb_open, n, c, 0, ctx->tlev, ctx->tt0, ctx->tlen, ctx->st_half, ctx->acc, ctx->vel, ctx->vb,
            ctx->va);
     ++ctx->launches;
@@ -751,7 +751,7 @@ static int cycle_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const flo
     tp = ctx->st_pos; ctx->st_pos = ctx->st_tmp; ctx->st_tmp = tp;
     tp = ctx->vel; ctx->vel = ctx->vb; ctx->vb = tp;
     tp = ctx->st_half; ctx->st_half = ctx->va; ctx->va = tp;
-    copy_async(ctx, ctx->hc, ctx->st_tmp1, sizeof(float) * n, s);
+    CRK_TRY(copy_async(ctx, ctx->hc, ctx->st_tmp1, sizeof(float) * n, s));
     rc = gather_rows(ctx, {{mass, ctx->mass, 1}}, s);
     if (!rc) rc = evaluate(ctx, s);
     if (rc) return rc;
@@ -766,7 +766,7 @@ static int cycle_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const flo
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "finish cycle");
     rc = scatter_rows(ctx, {{ctx->st_pos, pos_h, 4}, {ctx->st_vel, vel_u, 4}}, s);
-    if (!rc) zero_async(ctx, ctx->counters + CNT_NEXT_OK, sizeof(unsigned long long), s);
+    if (!rc) rc = zero_async(ctx, ctx->counters + CNT_NEXT_OK, sizeof(unsigned long long), s);
     if (!rc) rc = crk_sync_counters(ctx, s);
     if (rc) return rc;
     ctx->rates_valid = 1;
@@ -816,7 +816,7 @@ extern "C" int crk_htb_levels(crk_ctx *ctx, int n, const float *pos_h, const flo
     ctx->rates_valid = 0;
     const HtbConsts c = htb_consts(ctx, Delta, L, f_l);
     const int nt = ctx->ntiles;
-    zero_async(ctx, ctx->counters + CNT_UNRES, sizeof(unsigned long long), s);
+    CRK_TRY(zero_async(ctx, ctx->counters + CNT_UNRES, sizeof(unsigned long long), s));
     launch(s, grid_for((long long)nt * 32, 256), 256, 0, k_htb_req, nt, nullptr, n, ctx->d_dt, c, 0, 0, ctx->tlev,
            ctx->counters);
     ++ctx->launches;

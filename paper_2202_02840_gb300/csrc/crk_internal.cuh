@@ -282,6 +282,12 @@ int crk_sync_counters(crk_ctx *ctx, cudaStream_t s);
         if (e_ != cudaSuccess) return crk_check_cuda((ctx), e_, #call);         \
     } while (0)
 
+#define CRK_TRY(call)                 \
+    do {                              \
+        const int rc_ = (call);       \
+        if (rc_) return rc_;          \
+    } while (0)
+
 #define CRK_LAUNCH_CHECK(ctx, what)                                              \
     do {                                                                         \
         cudaError_t e_ = cudaGetLastError();                                     \
@@ -355,8 +361,8 @@ int run_compatible_dual(crk_ctx *ctx, const double *dtn, const int32_t *sbox, cu
 int evaluate(crk_ctx *ctx, cudaStream_t s);   // P1..P4 and per-particle time steps (crk_step.cu)
 int propose_sorted(crk_ctx *ctx, int n, float4 *pos, const GvRec *gv, const float *Nn, float dt, float tol,
                    cudaStream_t s);   // learned h proposal in sorted order (crk_mlp.cu)
-void zero_async(crk_ctx *ctx, void *p, size_t bytes, cudaStream_t s);   // whole 32-bit words (crk_ctx.cu)
-void copy_async(crk_ctx *ctx, void *to, const void *from, size_t bytes, cudaStream_t s);
+int zero_async(crk_ctx *ctx, void *p, size_t bytes, cudaStream_t s);   // whole 32-bit words (crk_ctx.cu)
+int copy_async(crk_ctx *ctx, void *to, const void *from, size_t bytes, cudaStream_t s);
 struct Rows {   // of `words` 32-bit words
     const void *in;
     void *out;

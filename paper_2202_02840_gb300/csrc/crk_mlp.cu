@@ -806,8 +806,8 @@ bool feature_table(const crk_ctx *ctx, int n) { return n > wave_rows(ctx); }
 
 int count_cells(crk_ctx *ctx, int n, const float4 *pos, int kf, cudaStream_t s) {
     if (!ctx->fcnt) CRK_CUDA(ctx, cudaMalloc((void **)&ctx->fcnt, sizeof(int32_t) << 21));
-    zero_async(ctx, ctx->fcnt, sizeof(int32_t) << (3 * kf), s);
-    zero_async(ctx, ctx->counters + CNT_MLP_ERR, sizeof(unsigned long long), s);
+    CRK_TRY(zero_async(ctx, ctx->fcnt, sizeof(int32_t) << (3 * kf), s));
+    CRK_TRY(zero_async(ctx, ctx->counters + CNT_MLP_ERR, sizeof(unsigned long long), s));
     const int cells = 1 << (3 * kf);
     const bool table = feature_table(ctx, n);
     if (table && kf > ctx->ftab_level) {
@@ -964,8 +964,8 @@ extern "C" int crk_mlp_set_weights(crk_ctx *ctx, const float *w, void *stream) {
         }
     }
     CRK_CUDA(ctx, cudaMemcpyAsync(ctx->mlp_w, w, sizeof(float) * NP, cudaMemcpyDefault, s));
-    zero_async(ctx, ctx->mlp_m, sizeof(float) * NP, s);
-    zero_async(ctx, ctx->mlp_v, sizeof(float) * NP, s);
+    CRK_TRY(zero_async(ctx, ctx->mlp_m, sizeof(float) * NP, s));
+    CRK_TRY(zero_async(ctx, ctx->mlp_v, sizeof(float) * NP, s));
     ctx->mlp_t = 0;
     return CRK_OK;
 }

@@ -482,7 +482,7 @@ struct has_tma<P, std::void_t<decltype(P::TMA)>> : std::bool_constant<P::TMA> {}
 int tile_order_by_length(crk_ctx *ctx, cudaStream_t s);   // ctx->tile_order, longest pair-set list first
 
 template <class P, int WARPS, int U>
-static void launch_variant_u(crk_ctx *ctx, const ListGeom &g, const typename P::Params &prm, int ord,
+static int launch_variant_u(crk_ctx *ctx, const ListGeom &g, const typename P::Params &prm, int ord,
                              cudaStream_t s) {
     if (ord == ORD_SM) {
         static int per_sm = 0;
@@ -493,18 +493,19 @@ static void launch_variant_u(crk_ctx *ctx, const ListGeom &g, const typename P::
         }
         const int nrange = ctx->nsm > 0 ? (ctx->nsm < 1024 ? ctx->nsm : 1024) : 1;
         const int chunk = (ctx->ntiles + nrange - 1) / nrange;
-        zero_async(ctx, ctx->sm_next, sizeof(uint32_t) * nrange, s);
+        CRK_TRY(zero_async(ctx, ctx->sm_next, sizeof(uint32_t) * nrange, s));
         launch(s, nrange * per_sm, 32, 0, k_lpass_sm<P, U>, g, prm, ctx->sm_next, nrange, chunk);
     } else {
         launch(s, grid_for(ctx->ntiles, WARPS), WARPS * 32, 0, k_lpass<P, WARPS, U>, g, prm,
                ord == ORD_LONGEST ? ctx->tile_order : nullptr);
     }
+    return CRK_OK;
 }
 
 // per-SM tile ranges, the pass's own entries per iteration, records one
 // iteration ahead
 template <class P>
-static void launch_sm_rp(crk_ctx *ctx, const ListGeom &g, const typename P::Params &prm, cudaStream_t s) {
+static int launch_sm_rp(crk_ctx *ctx, const ListGeom &g, const typename P::Params &prm, cudaStream_t s) {
     constexpr int U = P::UNROLL;
     static int per_sm = 0;
     if (!per_sm) {
@@ -514,8 +515,9 @@ static void launch_sm_rp(crk_ctx *ctx, const ListGeom &g, const typename P::Para
     }
     const int nrange = ctx->nsm > 0 ? (ctx->nsm < 1024 ? ctx->nsm : 1024) : 1;
     const int chunk = (ctx->ntiles + nrange - 1) / nrange;
-    zero_async(ctx, ctx->sm_next, sizeof(uint32_t) * nrange, s);
+    CRK_TRY(zero_async(ctx, ctx->sm_next, sizeof(uint32_t) * nrange, s));
     launch(s, nrange * per_sm, 32, 0, k_lpass_sm<P, U, true>, g, prm, ctx->sm_next, nrange, chunk);
+    return CRK_OK;
 }
 
 template <class P, int W>
@@ -546,7 +548,7 @@ static int launch_variant(crk_ctx *ctx, const ListGeom &g, const typename P::Par
         return CRK_OK;
     }
     if (lv.rp && lv.ord == ORD_SM) {
-        if constexpr (!P::PREFETCH) launch_sm_rp<P>(ctx, g, prm, s);
+        if constexpr (!P::PREFETCH) return launch_sm_rp<P>(ctx, g, prm, s);
         return CRK_OK;
     }
     if (lv.rp) {   // records one iteration ahead (passes without their own prefetch)
@@ -572,15 +574,14 @@ static int launch_variant(crk_ctx *ctx, const ListGeom &g, const typename P::Par
         if (rc) return rc;
     }
     if constexpr (P::PREFETCH) {
-        launch_variant_u<P, WARPS, 1>(ctx, g, prm, lv.ord, s);
+        return launch_variant_u<P, WARPS, 1>(ctx, g, prm, lv.ord, s);
     } else {
         switch (lv.U) {
-        case 1: launch_variant_u<P, WARPS, 1>(ctx, g, prm, lv.ord, s); break;
-        case 2: launch_variant_u<P, WARPS, 2>(ctx, g, prm, lv.ord, s); break;
-        default: launch_variant_u<P, WARPS, 4>(ctx, g, prm, lv.ord, s); break;
+        case 1: return launch_variant_u<P, WARPS, 1>(ctx, g, prm, lv.ord, s);
+        case 2: return launch_variant_u<P, WARPS, 2>(ctx, g, prm, lv.ord, s);
+        default: return launch_variant_u<P, WARPS, 4>(ctx, g, prm, lv.ord, s);
         }
     }
-    return CRK_OK;
 }
 
 // the measured default of each pass (before or without tuning)

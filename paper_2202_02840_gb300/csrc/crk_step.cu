@@ -430,7 +430,7 @@ static int h_update(crk_ctx *ctx, const StepConsts &c, float tol, cudaStream_t s
     const int n = ctx->n;
     int rc = ensure_htb(ctx);
     if (rc) return rc;
-    zero_async(ctx, ctx->counters + CNT_NOTDONE, sizeof(unsigned long long), s);
+    CRK_TRY(zero_async(ctx, ctx->counters + CNT_NOTDONE, sizeof(unsigned long long), s));
     launch(s, grid_for(n, 256), 256, 0, k_h_iter, n, c, tol, ctx->Nn, ctx->hs, ctx->q4, ctx->flags, ctx->tflag,
            ctx->counters + CNT_NOTDONE);
     ++ctx->launches;
@@ -455,7 +455,7 @@ static int solve_h(crk_ctx *ctx, int n, const int32_t *idx, cudaStream_t s, int 
         ++ctx->launches;
         CRK_LAUNCH_CHECK(ctx, "permute grad v");
     }
-    zero_async(ctx, ctx->flags, sizeof(int32_t) * n, s);
+    CRK_TRY(zero_async(ctx, ctx->flags, sizeof(int32_t) * n, s));
     const int vo = ctx->volumes_only;
     ctx->volumes_only = 1;
     int it = 0;
@@ -518,7 +518,7 @@ static int step_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const floa
         if (rc) return rc;
         rc = gather_rows(ctx, {{pos_h, ctx->st_pos, 4}, {vel_u, ctx->st_vel, 4}, {mass, ctx->mass, 1}}, s);
         if (rc) return rc;
-        copy_async(ctx, ctx->vel, ctx->st_vel, sizeof(float4) * n, s);
+        CRK_TRY(copy_async(ctx, ctx->vel, ctx->st_vel, sizeof(float4) * n, s));
         rc = evaluate(ctx, s);
         if (rc) return rc;
         ctx->rates_valid = 1;
@@ -531,7 +531,7 @@ static int step_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const floa
     const int32_t *sbox = batched ? ctx->sbox : nullptr;
     double *dtb = batched ? ctx->dtb : ctx->d_scalars;
     double *dtn = batched ? ctx->dtb_next : ctx->d_scalars + 16;   // the next step's dt
-    if (fresh) zero_async(ctx, ctx->counters + CNT_NEXT_OK, 2 * sizeof(unsigned long long), s);
+    if (fresh) CRK_TRY(zero_async(ctx, ctx->counters + CNT_NEXT_OK, 2 * sizeof(unsigned long long), s));
     launch(s, grid_for(nb, 64), 64, 0, k_pick_dt, nb, dt_req, dt_box, c.dt_max,
            batched ? ctx->box_dtmin : ctx->counters + CNT_DTMIN, dtb);
     launch(s, 1, 256, 0, k_next_check, nb, dtb, dtn, ctx->counters);
@@ -548,7 +548,7 @@ static int step_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const floa
     ++ctx->launches;
     CRK_LAUNCH_CHECK(ctx, "drift");
     // rebuild at x1 (input order = current sorted order; boxes keep their particles)
-    if (batched) copy_async(ctx, ctx->sbox_tmp, ctx->sbox, sizeof(int32_t) * n, s);
+    if (batched) CRK_TRY(copy_async(ctx, ctx->sbox_tmp, ctx->sbox, sizeof(int32_t) * n, s));
     rc = build_cells_sorted(ctx, n, ctx->st_pos, ctx->perm, s, batched ? ctx->sbox_tmp : nullptr);
     if (!rc) rc = finish_build(ctx, s);
     if (rc) {
@@ -571,7 +571,7 @@ static int step_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const floa
             ctx->rates_valid = 0;
             return rc;
         }
-        copy_async(ctx, ctx->vel, ctx->st_vel, sizeof(float4) * n, s);
+        CRK_TRY(copy_async(ctx, ctx->vel, ctx->st_vel, sizeof(float4) * n, s));
     }
     // evaluation at (x1, p_p, u_p)
     rc = evaluate(ctx, s);
@@ -920,9 +920,9 @@ static int steps_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const flo
             CRK_CUDA(ctx, cudaEventCreateWithFlags(&ctx->gev[0], cudaEventDisableTiming));
             CRK_CUDA(ctx, cudaEventCreateWithFlags(&ctx->gev[1], cudaEventDisableTiming));
         }
-        copy_async(ctx, ctx->bk_pos, pos_h, sizeof(float4) * (size_t)n, s);
-        copy_async(ctx, ctx->bk_vel, vel_u, sizeof(float4) * (size_t)n, s);
-        zero_async(ctx, ctx->counters + CNT_GRAPH_ERR, sizeof(unsigned long long), s);
+        CRK_TRY(copy_async(ctx, ctx->bk_pos, pos_h, sizeof(float4) * (size_t)n, s));
+        CRK_TRY(copy_async(ctx, ctx->bk_vel, vel_u, sizeof(float4) * (size_t)n, s));
+        CRK_TRY(zero_async(ctx, ctx->counters + CNT_GRAPH_ERR, sizeof(unsigned long long), s));
         CRK_CUDA(ctx, cudaEventRecord(ctx->gev[0], s));
         CRK_CUDA(ctx, cudaStreamWaitEvent(ctx->gstream, ctx->gev[0], 0));
         bool eager = false;
@@ -960,8 +960,8 @@ static int steps_impl(crk_ctx *ctx, int n, float *pos_h, float *vel_u, const flo
             // positions and velocities this run of replays started from and redo
             // its steps eagerly (their first step evaluates the rates afresh there)
             ctx->grecoveries++;
-            copy_async(ctx, pos_h, ctx->bk_pos, sizeof(float4) * (size_t)n, s);
-            copy_async(ctx, vel_u, ctx->bk_vel, sizeof(float4) * (size_t)n, s);
+            CRK_TRY(copy_async(ctx, pos_h, ctx->bk_pos, sizeof(float4) * (size_t)n, s));
+            CRK_TRY(copy_async(ctx, vel_u, ctx->bk_vel, sizeof(float4) * (size_t)n, s));
             drop_graphs(ctx);
             ctx->rates_valid = 0;
             for (int k = done; k < nsteps; k++) {
@@ -1019,7 +1019,7 @@ static int h_iterate(crk_ctx *ctx, int n, float *pos_h, float tol, int max_it, i
     if (!rc) rc = finish_build(ctx, s);
     if (rc) return rc;
     StepConsts c = step_consts(ctx->p);
-    zero_async(ctx, ctx->flags, sizeof(int32_t) * n, s);
+    CRK_TRY(zero_async(ctx, ctx->flags, sizeof(int32_t) * n, s));
     int it = 0;
     unsigned long long nd = 1;
     for (it = 1; it <= max_it; it++) {

@@ -614,10 +614,10 @@ static int launch_walk(crk_ctx *ctx, cudaStream_t s) {
         int rc = crk_ensure_entries(ctx, (long long)ctx->ntiles * 32 * ctx->kcap, -1);
         if (rc) return rc;
     }
-    zero_async(ctx, ctx->counters + CNT_PAIRS_G, 5 * sizeof(unsigned long long), s);
+    CRK_TRY(zero_async(ctx, ctx->counters + CNT_PAIRS_G, 5 * sizeof(unsigned long long), s));
     if (ctx->act && !ctx->volumes_only) {   // tiles left out of the walk take no list columns and no stored forces
-        zero_async(ctx, ctx->len_g, sizeof(uint32_t) * ctx->ntiles, s);
-        zero_async(ctx, ctx->len_u, sizeof(uint32_t) * ctx->ntiles, s);
+        CRK_TRY(zero_async(ctx, ctx->len_g, sizeof(uint32_t) * ctx->ntiles, s));
+        CRK_TRY(zero_async(ctx, ctx->len_u, sizeof(uint32_t) * ctx->ntiles, s));
     }
     if (ctx->act && ctx->nact == 0) return CRK_OK;
     prof_begin(ctx, PROF_LISTS, s);

@@ -35,3 +35,17 @@ def test_every_kernel_waits_for_the_one_before():
 def test_no_launch_goes_round_the_rule():
     for path in sorted(glob.glob(os.path.join(CSRC, "*.cu*"))):
         assert "<<<" not in re.sub(r"//[^\n]*", "", open(path).read()), path
+
+
+def test_no_zeros_or_copies_go_unchecked():
+    """zero_async and copy_async return their launch's error: each call passes it on."""
+    calls = 0
+    for path in sorted(glob.glob(os.path.join(CSRC, "*.cu*"))):
+        src = re.sub(r"//[^\n]*", "", open(path).read())
+        for m in re.finditer(r"\b(zero|copy)_async\(", src):
+            line = src[src.rfind("\n", 0, m.start()) + 1:m.start()]
+            if line.strip() == "int":   # declarations, definitions
+                continue
+            calls += 1
+            assert line.endswith(("CRK_TRY(", "rc = ")), (path, src[m.start() - 40:m.start() + 40])
+    assert calls > 30
