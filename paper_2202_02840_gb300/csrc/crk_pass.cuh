@@ -395,7 +395,6 @@ __global__ void __launch_bounds__(S * 32) k_lpass_split(ListGeom g, typename P::
     const int end = count ? (int)*count : (int)blockIdx.x + 1;
     for (int t = blockIdx.x; t < end; t += gridDim.x) {
         const int tile = order ? order[t] : t;
-        if (g.heavy && g.len_u[tile] <= *g.heavy) continue;
         const int i = tile * TILE + lane;
         const bool valid = i < g.n;
         typename P::IState st;
@@ -403,6 +402,7 @@ __global__ void __launch_bounds__(S * 32) k_lpass_split(ListGeom g, typename P::
         if (w > 0) P::zero(st);
         const LaneList<P> ll(g, tile, lane, i, valid);
         const int bw = (int)((P::GATHER ? g.len_g[tile] : g.len_u[tile]) / LB);
+        if (g.heavy && g.len_u[tile] <= *g.heavy) continue;   // here: its loads and the particle's are in flight together
         const int chunk = (bw + S - 1) / S;
         const int b0 = w * chunk, b1 = min(bw, b0 + chunk);
         list_loop<P, U>(st, prm, ll, b0, min(ll.nb, b1), b1);
