@@ -159,8 +159,10 @@ struct PairOut {
 
 // One pair of the pair set seen from particle a.  Every operation on (a, b) has
 // its counterpart on (b, a): F_ba = -F_ab bitwise.  STATIC: a = 1, adot = 0 (the
-// same values without the factors of one and the terms of zero).
-template <bool STATIC>
+// same values without the factors of one and the terms of zero).  KEEP: eps^2 h^_a is
+// held in a register, not formed again for each pair (the same bits; P4 at 128^3:
+// compensated sums 7.49 ms held, 7.78 not, plain sums 7.95 and 7.73).
+template <bool STATIC, bool KEEP>
 __device__ __forceinline__ void pair_force(const FRec &a, const FOwn &oa, const FRec &b, const FParams &fp,
                                            PairOut &o) {
     const Sep d = separation((int)(fq(a, 0) - fq(b, 0)), (int)(fq(a, 1) - fq(b, 1)), (int)(fq(a, 2) - fq(b, 2)));
@@ -214,7 +216,7 @@ __device__ __forceinline__ void pair_force(const FRec &a, const FOwn &oa, const 
     // 1.61, 1.49, 1.73e-7 from (r/h)^2 and a plain quotient; 0.95, 1.26, 1.12, 1.19e-7 from
     // a record with h^ itself and IEEE roots).  P4 at 128^3 clustered 7.81 -> 7.53 ms; with
     // IEEE roots 7.92, with IEEE quotients 8.3.
-    const float mua = fminf(quotient(uxa, fmaf(d.r2, oa.ihh, oa.ehh)), 0.f);
+    const float mua = fminf(quotient(uxa, fmaf(d.r2, oa.ihh, KEEP ? oa.ehh : FDIV(fp.eps2_nh, a.w0.w))), 0.f);
     const float mub = fminf(quotient(uxa, fmaf(d.r2, fp.nh * b.w0.w, FDIV(fp.eps2_nh, b.w0.w))), 0.f);
     const float lcb = fp.Cl * sqrt_approx(fmaxf(fp.gamma * b.w7.w, 0.f));
     o.Q_a = __fmul_rn(a.w7.z * mua, fmaf(fp.Cq, mua, -oa.lc));
@@ -315,7 +317,7 @@ struct P4 {
     __device__ static Rec load(uint32_t j, size_t, const Params &p) { return ldg_frec(p.frec, j); }
     __device__ static void pair(IState &s, const Rec &r, uint32_t j, size_t pos, bool, const Params &p) {
         PairOut o;
-        pair_force<STATIC>(s.me, s.own, r, p.fp, o);
+        pair_force<STATIC, COMP>(s.me, s.own, r, p.fp, o);
         p.Fst[pos] = make_float4(o.F[0], o.F[1], o.F[2], __uint_as_float(j));   // F_ij, j
 #pragma unroll
         for (int g = 0; g < 3; g++) s.F[g].add(o.F[g]);
@@ -888,7 +890,7 @@ struct P4PO {
     __device__ static void pair(IState &s, const Rec &r, const Ent &e, size_t pos, const Params &p,
                                 float sh[NS]) {
         PairOut o;
-        pair_force<STATIC>(s.me, s.own, r, p.fp, o);
+        pair_force<STATIC, COMP>(s.me, s.own, r, p.fp, o);
         p.Fst[pos] = make_float4(o.F[0], o.F[1], o.F[2], __uint_as_float(e));   // F_ij, j
 #pragma unroll
         for (int g = 0; g < 3; g++) s.F[g].add(o.F[g]);
