@@ -324,9 +324,10 @@ __global__ void k_htb_compact(int ntiles, int n, const uint32_t *__restrict__ fl
 }
 
 // The same by one CTA straight from a predicate, without flags, scan and reset:
-// warp w takes 256 consecutive tiles of each 8192.  Up to COMPACT_ONE tiles (a
-// scan's three launches and the rest took 16 us a pass at 8192 tiles, this 4.3).
-constexpr int COMPACT_ONE = 65536;
+// warp w takes 256 consecutive tiles of each 8192.  Up to COMPACT_ONE tiles: a
+// pass of the h solve takes 2.8, 3.7, 2.5, 1.5 us less than with the scan's three
+// launches at 2000, 8192, 16000, 32197 tiles, 4.2 us more at 65536.
+constexpr int COMPACT_ONE = 32768;
 struct FlaggedTiles {
     const uint32_t *flag;
     __device__ bool operator()(int T) const { return flag[T] != 0u; }

@@ -381,3 +381,24 @@ def test_viscosity_keeps_its_digits(expansion):
     err = np.linalg.norm(q - o) / np.linalg.norm(o) * 2.0 ** 24
     print(expansion, "%.2f u" % err)
     assert err < 1.9, err
+
+
+@pytest.mark.parametrize("side", [102])
+def test_tiles_listed_by_a_scan(side):
+    """Beyond 32768 tiles the open and due tiles are listed by flags, a scan and a
+    compaction: the solve converges every particle, and the middle tick of a
+    two-level cycle evaluates the leaves of the deeper level, a ragged one among them."""
+    st = inputs.sedov(side)
+    g = dev(st["pos_h"] * np.float32([1, 1, 1, 0.9]))
+    ctx = crk.crk_create()
+    it, ok = crk.crk_h_iterate(ctx, g, tol=1e-4, max_it=60)
+    assert ok and it > 2
+    crk.crk_build_cells(ctx, g)
+    N = as_np(crk.crk_volumes(ctx)[1]).astype(np.float64)
+    assert np.all(np.abs(np.cbrt(268.0 / N) - 1.0) <= 1.01e-4)
+    n, pos, vel, mass = side ** 3, dev(st["pos_h"]), dev(st["vel_u"]), dev(st["mass"])
+    dt = crk.crk_step(ctx, pos, vel, mass, 0.0, diag=True)["dt_next"]
+    s = crk.crk_cycle(ctx, pos, vel, mass, 1.9 * dt, 1, f_l=1)
+    deep = s["level_count"][1]
+    assert s["ticks"] == 2 and 0 < deep < s["leaves"] == -(-n // 32)
+    assert s["evaluations"] - n in (32 * deep, 32 * deep - (-n % 32)), s
