@@ -4,7 +4,7 @@
 // assembled once per hydro step and reused by every hydro kernel).
 //
 // GB300 layout: 30-bit Morton keys of the fixed-point coordinates, a stable LSD
-// radix sort (8-bit digits, per-warp stable ranking with match_any), sorted
+// radix sort (10-bit digits, per-warp stable ranking with match_any), sorted
 // SoA particle records, tiles of 32 consecutive sorted particles (one warp),
 // an implicit binary tree over the Morton-ordered tiles, and per-tile lists of
 // neighbour tiles found by a depth-first walk of that tree with exact

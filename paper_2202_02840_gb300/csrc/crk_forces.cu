@@ -54,7 +54,8 @@ struct FParams {
 //
 // In memory the four sectors of record j stand in the order c ^ (j & 3): 32
 // lanes that read sector c of 32 records spread over the four sector columns
-// of the L1 data banks (18 cycles a load; 32 when all read the same column).
+// of the L1 data banks (17.4 cycles a load where the records are in L1, 31 from L2; 32
+// and 45 when all read the same column).
 struct FRec {
     float4 w0;      // qx, qy, qz (fixed-point bits), 1/h
     float4 w1;      // V, vx, vy, vz
@@ -160,8 +161,10 @@ struct PairOut {
 // One pair of the pair set seen from particle a.  Every operation on (a, b) has
 // its counterpart on (b, a): F_ba = -F_ab bitwise.  STATIC: a = 1, adot = 0 (the
 // same values without the factors of one and the terms of zero).  KEEP: eps^2 h^_a is
-// held in a register, not formed again for each pair (the same bits; P4 at 128^3:
-// compensated sums 7.49 ms held, 7.78 not, plain sums 7.95 and 7.73).
+// held in a register, not formed again for each pair (the same bits; P4 at 128^3,
+// ms, held / not: static with compensated sums 7.49/7.78, plain 7.95/7.73, comoving with
+// compensated sums 7.65/7.59, plain -/7.41; before the corrected viscosity 7.76, 7.72,
+// 7.46, 7.73).
 template <bool STATIC, bool KEEP>
 __device__ __forceinline__ void pair_force(const FRec &a, const FOwn &oa, const FRec &b, const FParams &fp,
                                            PairOut &o) {
@@ -317,7 +320,7 @@ struct P4 {
     __device__ static Rec load(uint32_t j, size_t, const Params &p) { return ldg_frec(p.frec, j); }
     __device__ static void pair(IState &s, const Rec &r, uint32_t j, size_t pos, bool, const Params &p) {
         PairOut o;
-        pair_force<STATIC, COMP>(s.me, s.own, r, p.fp, o);
+        pair_force<STATIC, COMP && STATIC>(s.me, s.own, r, p.fp, o);
         p.Fst[pos] = make_float4(o.F[0], o.F[1], o.F[2], __uint_as_float(j));   // F_ij, j
 #pragma unroll
         for (int g = 0; g < 3; g++) s.F[g].add(o.F[g]);
@@ -890,7 +893,7 @@ struct P4PO {
     __device__ static void pair(IState &s, const Rec &r, const Ent &e, size_t pos, const Params &p,
                                 float sh[NS]) {
         PairOut o;
-        pair_force<STATIC, COMP>(s.me, s.own, r, p.fp, o);
+        pair_force<STATIC, COMP && STATIC>(s.me, s.own, r, p.fp, o);
         p.Fst[pos] = make_float4(o.F[0], o.F[1], o.F[2], __uint_as_float(e));   // F_ij, j
 #pragma unroll
         for (int g = 0; g < 3; g++) s.F[g].add(o.F[g]);

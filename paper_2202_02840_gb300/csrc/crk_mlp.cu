@@ -54,8 +54,6 @@ __device__ __forceinline__ float tanh_sfu(float x) {
     return y;
 }
 
-__device__ __forceinline__ float logistic(float z) { return fmaf(0.5f, tanh_sfu(0.5f * z), 0.5f); }
-
 // Packed FP32 pairs (one instruction for two IEEE-rounded operations, the
 // same results as the scalar ones): the two columns of an mma accumulator
 // pair sit in adjacent registers.

@@ -18,7 +18,11 @@ namespace crk {
 constexpr int WALK_WARPS = 8;
 constexpr int WALK_WIDE = 8;       // fewer tiles than this per SM: CTAs of 32 warps
 constexpr int WALK_ALL = 20;       // fewer tiles than this per SM: every tile is shared by a CTA's warps
-constexpr int WALK_HEAVY = 384;    // candidate tiles above which a tile is shared
+// Candidate tiles above which a tile is shared.  The walk, us, with the line at 192, 256,
+// 384, 512, 768, none: clustered 64^3 (mean 134 candidates) 762, 698, 749, 838, 912, 1086;
+// 128^3 (126) 4629, 4396, 4285, 4340, 4482, 6068; Sedov 80^3 after 400 steps (160) 2748, 2710,
+// 2512, 2473, 2494, 8048; no tile of the Hilbert order is near it.
+constexpr int WALK_HEAVY = 384;
 
 struct WalkArgs {
     int n, ntiles, kcap;
