@@ -383,7 +383,7 @@ constexpr int split_warps() {   // as many as their sums fit static shared memor
 }
 
 // count null: block b takes tile order[b] (order null: tile b); else the blocks
-// share the tiles order[0 .. *count).
+// share those of the tiles order[0 .. *count) that have more than *g.heavy rows.
 template <class P, int S, int U>
 __global__ void __launch_bounds__(S * 32) k_lpass_split(ListGeom g, typename P::Params prm, const int32_t *order,
                                                         const unsigned long long *count) {
@@ -392,9 +392,7 @@ __global__ void __launch_bounds__(S * 32) k_lpass_split(ListGeom g, typename P::
     __shared__ __align__(16) unsigned char part[(S - 1) * 32 * sizeof(Sums)];
     if (pass_skipped<P>(prm)) return;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int end = count ? (int)*count : (int)blockIdx.x + 1;
-    for (int t = blockIdx.x; t < end; t += gridDim.x) {
-        const int tile = order ? order[t] : t;
+    auto take = [&](int tile) {
         const int i = tile * TILE + lane;
         const bool valid = i < g.n;
         typename P::IState st;
@@ -402,7 +400,6 @@ __global__ void __launch_bounds__(S * 32) k_lpass_split(ListGeom g, typename P::
         if (w > 0) P::zero(st);
         const LaneList<P> ll(g, tile, lane, i, valid);
         const int bw = (int)((P::GATHER ? g.len_g[tile] : g.len_u[tile]) / LB);
-        if (g.heavy && g.len_u[tile] <= *g.heavy) continue;   // here: its loads and the particle's are in flight together
         const int chunk = (bw + S - 1) / S;
         const int b0 = w * chunk, b1 = min(bw, b0 + chunk);
         list_loop<P, U>(st, prm, ll, b0, min(ll.nb, b1), b1);
@@ -415,6 +412,17 @@ __global__ void __launch_bounds__(S * 32) k_lpass_split(ListGeom g, typename P::
             if (valid) P::finish(st, i, prm);
         }
         __syncthreads();
+    };
+    if (!count) {
+        take(order ? order[blockIdx.x] : (int)blockIdx.x);
+        return;
+    }
+    // 32 of the block's listed tiles at a time: those above the line
+    const int end = (int)*count;
+    for (int t0 = blockIdx.x; t0 < end; t0 += 32 * gridDim.x) {
+        const int t = t0 + lane * (int)gridDim.x, mine = t < end ? order[t] : 0;
+        unsigned todo = __ballot_sync(0xffffffffu, t < end && g.len_u[mine] > *g.heavy);
+        for (; todo; todo &= todo - 1u) take(__shfl_sync(0xffffffffu, mine, __ffs(todo) - 1));
     }
 }
 
