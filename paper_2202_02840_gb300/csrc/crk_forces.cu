@@ -271,6 +271,7 @@ __device__ __forceinline__ FRec ldg_frec(const float4 *base, uint32_t j) {
 template <bool COMP, bool STATIC>
 struct P4 {
     static constexpr bool GATHER = false;
+    static constexpr int SPLIT_WARPS = 16;   // registers of the split form (split_blocks)
     static constexpr int UNROLL = 1;
     static constexpr bool ENTRIES = true;
     static constexpr bool PERSISTENT = true;

@@ -392,6 +392,7 @@ __device__ __forceinline__ void merge_acc(AccFF &d, const AccFF &o) { d.add(FF{o
 
 struct P2X {
     static constexpr bool GATHER = true;
+    static constexpr int SPLIT_WARPS = 16;   // registers of the split form (split_blocks)
     static constexpr int UNROLL = 2;
     static constexpr bool ENTRIES = true;
     static constexpr bool PERSISTENT = false;
@@ -599,6 +600,7 @@ struct P3 {
 // m_j / V_j, exact for constant and linear fields.
 struct PD {
     static constexpr bool GATHER = true;
+    static constexpr int SPLIT_WARPS = 16;   // registers of the split form (split_blocks)
     static constexpr int UNROLL = 4;
     static constexpr bool ENTRIES = true;
     static constexpr bool PERSISTENT = false;

@@ -382,47 +382,70 @@ constexpr int split_warps() {   // as many as their sums fit static shared memor
            : ((3 * 32 * sizeof(typename P::Sums) <= 44 * 1024) ? 4 : 2);
 }
 
-// count null: block b takes tile order[b] (order null: tile b); else the blocks
-// share those of the tiles order[0 .. *count) that have more than *g.heavy rows.
+// Blocks of the split form per SM that the compiler is told to leave registers for
+// (0: its own choice).  With 16 warps' worth it keeps more of a block's records in
+// flight, which P4, the float-float P2 and the density pass gain from (44^3 P4 383 -> 376 us,
+// 40^3 P2 546 -> 518, 24^3 density 22 -> 19) and P3 and P5 lose by (48^3 119 -> 135, 134 -> 146).
+template <class P, class = void>
+struct split_blocks : std::integral_constant<int, 0> {};
+template <class P>
+struct split_blocks<P, std::void_t<decltype(P::SPLIT_WARPS)>>
+    : std::integral_constant<int, P::SPLIT_WARPS / split_warps<P>()> {};
+
+// One tile, by the S warps of the block.
 template <class P, int S, int U>
-__global__ void __launch_bounds__(S * 32) k_lpass_split(ListGeom g, typename P::Params prm, const int32_t *order,
-                                                        const unsigned long long *count) {
-    grid_wait();
-    using Sums = typename P::Sums;
-    __shared__ __align__(16) unsigned char part[(S - 1) * 32 * sizeof(Sums)];
-    if (pass_skipped<P>(prm)) return;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    auto take = [&](int tile) {
-        const int i = tile * TILE + lane;
-        const bool valid = i < g.n;
-        typename P::IState st;
-        P::init(st, i, valid, prm);
-        if (w > 0) P::zero(st);
-        const LaneList<P> ll(g, tile, lane, i, valid);
-        const int bw = (int)((P::GATHER ? g.len_g[tile] : g.len_u[tile]) / LB);
-        const int chunk = (bw + S - 1) / S;
-        const int b0 = w * chunk, b1 = min(bw, b0 + chunk);
-        list_loop<P, U>(st, prm, ll, b0, min(ll.nb, b1), b1);
-        Sums *sp = reinterpret_cast<Sums *>(part);
-        if (w > 0) sp[(w - 1) * 32 + lane] = P::sums(st);
-        __syncthreads();
-        if (w == 0) {
+__device__ __forceinline__ void split_tile(const ListGeom &g, const typename P::Params &prm, int tile, int lane, int w,
+                                           typename P::Sums *part) {
+    const int i = tile * TILE + lane;
+    const bool valid = i < g.n;
+    typename P::IState st;
+    P::init(st, i, valid, prm);
+    if (w > 0) P::zero(st);
+    const LaneList<P> ll(g, tile, lane, i, valid);
+    const int bw = (int)((P::GATHER ? g.len_g[tile] : g.len_u[tile]) / LB);
+    const int chunk = (bw + S - 1) / S;
+    const int b0 = w * chunk, b1 = min(bw, b0 + chunk);
+    list_loop<P, U>(st, prm, ll, b0, min(ll.nb, b1), b1);
+    if (w > 0) part[(w - 1) * 32 + lane] = P::sums(st);
+    __syncthreads();
+    if (w == 0) {
 #pragma unroll 1
-            for (int v = 1; v < S; v++) P::merge(st, sp[(v - 1) * 32 + lane]);
-            if (valid) P::finish(st, i, prm);
-        }
-        __syncthreads();
-    };
-    if (!count) {
-        take(order ? order[blockIdx.x] : (int)blockIdx.x);
-        return;
+        for (int v = 1; v < S; v++) P::merge(st, part[(v - 1) * 32 + lane]);
+        if (valid) P::finish(st, i, prm);
     }
-    // 32 of the block's listed tiles at a time: those above the line
-    const int end = (int)*count;
+}
+
+// Block b takes tile order[b] (order null: tile b).
+template <class P, int S, int U>
+__global__ void __launch_bounds__(S * 32, split_blocks<P>::value)
+k_lpass_split(ListGeom g, typename P::Params prm, const int32_t *order) {
+    grid_wait();
+    __shared__ __align__(16) unsigned char part[(S - 1) * 32 * sizeof(typename P::Sums)];
+    if (pass_skipped<P>(prm)) return;
+    split_tile<P, S, U>(g, prm, order ? order[blockIdx.x] : (int)blockIdx.x, threadIdx.x & 31, threadIdx.x >> 5,
+                        reinterpret_cast<typename P::Sums *>(part));
+}
+
+// The blocks share those of the tiles listed[0 .. *count) that have more than
+// *g.heavy rows, looking at 32 of them at a time.  As few blocks run as there are long
+// tiles, so each needs its loads in flight more than neighbours: with registers for 16
+// warps an SM, Sedov 64^3 after 250 plain steps P2 84 -> 59 us, P3 73 -> 37, P4 120 -> 104,
+// P5 57 -> 38.
+template <class P, int S, int U>
+__global__ void __launch_bounds__(S * 32, 16 / S) k_lpass_long(ListGeom g, typename P::Params prm, const int32_t *listed,
+                                                       const unsigned long long *count) {
+    grid_wait();
+    __shared__ __align__(16) unsigned char part[(S - 1) * 32 * sizeof(typename P::Sums)];
+    if (pass_skipped<P>(prm)) return;
+    const int lane = threadIdx.x & 31, end = (int)*count;
     for (int t0 = blockIdx.x; t0 < end; t0 += 32 * gridDim.x) {
-        const int t = t0 + lane * (int)gridDim.x, mine = t < end ? order[t] : 0;
+        const int t = t0 + lane * (int)gridDim.x, mine = t < end ? listed[t] : 0;
         unsigned todo = __ballot_sync(0xffffffffu, t < end && g.len_u[mine] > *g.heavy);
-        for (; todo; todo &= todo - 1u) take(__shfl_sync(0xffffffffu, mine, __ffs(todo) - 1));
+        for (; todo; todo &= todo - 1u) {
+            split_tile<P, S, U>(g, prm, __shfl_sync(0xffffffffu, mine, __ffs(todo) - 1), lane, threadIdx.x >> 5,
+                                reinterpret_cast<typename P::Sums *>(part));
+            __syncthreads();   // `part` is free for the next tile
+        }
     }
 }
 
@@ -670,13 +693,13 @@ int launch_lpass(crk_ctx *ctx, int prof_id, const typename P::Params &prm, cudaS
     constexpr int S = split_warps<P>();
     if (split) {
         if (tuning) CRK_CUDA(ctx, cudaEventRecord(ctx->tune_ev[0], s));
-        launch(s, g.ntiles, S * 32, 0, k_lpass_split<P, S, U>, g, prm, ctx->act, nullptr);
+        launch(s, g.ntiles, S * 32, 0, k_lpass_split<P, S, U>, g, prm, ctx->act);
         if (tuning) CRK_CUDA(ctx, cudaEventRecord(ctx->tune_ev[1], s));
     } else if (ctx->act) {
         launch(s, grid_for(g.ntiles, WARPS), WARPS * 32, 0, k_lpass<P, WARPS, U>, g, prm, ctx->act);
     } else {
         if (heavy) {
-            launch(s, 2 * nsm, S * 32, 0, k_lpass_split<P, S, U>, g, prm, ctx->heavy, ctx->counters + CNT_HEAVY);
+            launch(s, 2 * nsm, S * 32, 0, k_lpass_long<P, S, U>, g, prm, ctx->heavy, ctx->counters + CNT_HEAVY);
             ++ctx->launches;
             CRK_LAUNCH_CHECK(ctx, what);
         }
