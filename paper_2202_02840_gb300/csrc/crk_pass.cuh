@@ -140,9 +140,11 @@ struct ListGeom {
 // (CNT_LONG_ROWS) is shared by the warps of a CTA: a warp that walks the 1000 to
 // 2000 neighbours of a particle in an evacuated region runs on alone when the
 // others are done.  P1 to P5 of Sedov 64^3 after 500 steps (mean 320 entries, longest
-// 1460): no tile shared 2.96 ms, beyond 576 rows and 1, 1.25, 1.5, 2, 2.5, 3 means
-// 3.54, 2.67, 2.60, 2.61, 2.66, 2.89; beyond 1.5 means and 384 to 800 rows within 2%.  Where all lists are long the warps are even, and sharing every tile
-// only costs: 80^3 with 600 neighbours each 6.80 ms, 9.64 with a fixed line of 576.
+// 1460): no tile shared 2.90 ms, beyond 576 rows and 1, 1.25, 1.5, 2, 2.5, 3 means
+// 2.49, 2.48, 2.49, 2.49, 2.54, 2.78; beyond 1.5 means and 384 to 800 rows within 1%.
+// (Clustered 64^3 after 60 steps, longest lists milder: 2.33 unshared, 2.42 at 1.5.)
+// Where all lists are long the warps are even, and sharing every tile only costs:
+// 80^3 with 600 neighbours each 6.76 ms, 9.15 with a fixed line of 576.
 constexpr int HEAVY_ROWS = 576;
 
 // The blocks of lists stream once from HBM (or L2, just written by the walk),
@@ -452,11 +454,11 @@ __global__ void __launch_bounds__(S * 32, 16 / S) k_lpass_long(ListGeom g, typen
 // Tiles per SM below which a pass splits them: a warp per tile then leaves the
 // SMs short of warps, or the last wave of warps nearly empty.  P1 to P5 together,
 // us, a warp per tile (long lists by CTAs) / split:
-//   jittered lattice, tiles per SM   8: 447/343   15: 649/568   26: 942/928   38: 1295/1337
-//   Sedov after 400 to 500 steps    13: 1163/669  23: 1430/1073 36: 1978/1606
-//                                   54: 2640/2341 105: 4102/4146
-// On an even lattice the passes cross one by one, P2 and P3 from 10 tiles per SM
-// (at 26: 142/174 and 111/150, P4 518/424); a run leaves that state within a few
+//   jittered lattice, tiles per SM   8: 449/326   15: 643/558   26: 924/894   38: 1276/1286
+//   Sedov after 400 to 500 steps    13: 1112/658  23: 1360/1035 36: 1888/1541
+//                                   54: 2494/2252 105: 3937/3982
+// On an even lattice the passes cross one by one, P2 and P3 from 10 to 15 tiles per SM
+// (at 26: 144/158 and 113/141, P4 500/426); a run leaves that state within a few
 // steps, and then a line of 10 to 25 for P1 to P3 costs 4% of the whole step at 23.
 constexpr int SPLIT_TILES = 40;
 
